@@ -31,7 +31,7 @@ def _nvcc() -> str:
 def _compile(src: str, extra: list, verbose: bool) -> str:
     obj = os.path.join(BUILD, src + ".o")
     path = os.path.join(CSRC, src)
-    deps = [path, os.path.join(CSRC, "akv_internal.h"), os.path.join(ROOT, "include", "akv.h")]
+    deps = [path, os.path.join(CSRC, "akv_internal.h"), os.path.join(CSRC, "akv_device.cuh"), os.path.join(ROOT, "include", "akv.h")]
     if os.path.exists(obj) and all(os.path.getmtime(obj) >= os.path.getmtime(d) for d in deps):
         return obj
     cmd = [_nvcc(), *ARCH, *COMMON, *extra, "-c", path, "-o", obj]

@@ -10,21 +10,25 @@
 //   enc_hash       anchor-selection hashes of the non-window positions
 //   enc_anchors    select the k - W smallest hashes, number anchor slots by position
 //   enc_rows       copy anchor rows into the arena (16-byte chunks swizzled), squared norms
-//   enc_assign     Eq. 1 nearest anchor, Eq. 2 gamma, residual energies (per position)
+//   enc_assign_tc  Eq. 1: the one or two anchors that can be a position's nearest, on tensor cores
+//   enc_finish     Eq. 1 decided, Eq. 2 gamma, residual energies (per position)
 //   enc_slots      top-N residual energies per side -> residual flags and slot list
 //   enc_order      stored order: stable counting sort of positions by value anchor slot
 //   enc_tile_count residual records per tile and side
 //   enc_tile_table tile block offsets
 //   enc_tile_fill  streams, bitmaps and rank words of every tile block
 //   enc_quant      Eq. 12 rotation and 2-bit quantization of every slot, into its tile
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 #include <vector>
 
+#include "akv_device.cuh"
 #include "akv_internal.h"
 
 namespace akv {
@@ -36,17 +40,23 @@ constexpr double kLloydT = 0.98046875;
 
 // Per-unit scratch pointers, derived from the workspace table the host writes.
 struct EncUnitWs {
-  uint64_t* key0;     // [S] anchor hashes, then key residual energies
-  uint64_t* key1;     // [S] value residual energies
+  // [S] each: anchor hashes or selector scores; then (plain encoder) the first half holds the
+  // residual energies per side as fp32 bits + 1, anchors 0, or (full selection, and slots that need
+  // fp64 energies) the whole the fp64 bits + 1
+  uint64_t* key0;
+  uint64_t* key1;
   int32_t* slot_of;   // [S] anchor slot or -1
   int32_t* res_pos;   // [N_K + N_V] residual positions (keys, then values)
   double* n2[2];      // [k] squared anchor norms per side
-  double* rn[2];      // [k] their square roots
-  uint32_t* ctrl;     // [0]: side 0 has a nonzero anchor, [1]: side 1
+  // [side]: the side has a nonzero anchor; [2 + side]: full selection's residual counts; [4 + side]:
+  // an anchor norm outside the filter's range; [6 + side]: an energy outside the fp32 range, or a
+  // band too wide, so that the slots are chosen from fp64 energies
+  uint32_t* ctrl;
   uint32_t* st[2];    // [S] stream word (slot | fp16 gamma << 16) per position and side
-  uint8_t* flag;      // [S] bit 0: key residual, bit 1: value residual
+  uint8_t* flag[2];   // [S] residual flag per side (values: over slot_of, which is read no more by then)
+  float* inv[2];      // [k to a multiple of 32] 1 / anchor norm, 0 for a zero anchor (over perm and inv)
   int32_t* perm;      // [S] position of stored token t
-  int32_t* inv;       // [S] stored index of position i
+  int32_t* at;        // [S] stored index of position i
   uint32_t* cursor;   // [k + 1] value-anchor counts, then start of each run
   uint32_t* tcnt;     // [2 * n_tiles] residual records per tile (keys, values)
   double* alpha;      // full selection: [m][S] observation rows' attention
@@ -94,9 +104,7 @@ __device__ EncUnitWs unit_ws(const EncArgs& A, int u, const akv_unit_desc* d) {
   p += au(n * 4 + 16, 256);
   for (int s = 0; s < 2; ++s) {
     w.n2[s] = (double*)p;
-    p += au(k * 8, 256);
-    w.rn[s] = (double*)p;
-    p += au(k * 8, 256);
+    p += 2 * au(k * 8, 256);
   }
   w.ctrl = (uint32_t*)p;
   p += 256;
@@ -104,11 +112,14 @@ __device__ EncUnitWs unit_ws(const EncArgs& A, int u, const akv_unit_desc* d) {
     w.st[s] = (uint32_t*)p;
     p += au(S * 4, 256);
   }
-  w.flag = p;
+  w.flag[0] = p;
+  w.flag[1] = reinterpret_cast<uint8_t*>(w.slot_of);
   p += au(S, 256);
   w.perm = (int32_t*)p;
+  w.inv[0] = (float*)p;
   p += au(S * 4, 256);
-  w.inv = (int32_t*)p;
+  w.at = (int32_t*)p;
+  w.inv[1] = (float*)p;
   p += au(S * 4, 256);
   w.cursor = (uint32_t*)p;
   p += au((k + 1) * 4, 256);
@@ -285,173 +296,798 @@ __global__ void __launch_bounds__(1024) enc_anchors(const EncArgs A) {
     }
     base += tot;
   }
-  if (threadIdx.x < 2) w.ctrl[threadIdx.x] = 0;
+  if (threadIdx.x < 8) w.ctrl[threadIdx.x] = 0;
 }
 
-// One warp per anchor: copy rows, squared norms (sequential in j) per side.
-__global__ void enc_rows(const EncArgs A) {
-  const int u = blockIdx.y;
-  const akv_unit_desc* d = unit_desc(A, u);
-  const int k = d->n_anchors;
-  const int a = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (a >= k) return;
-  EncUnitWs w = unit_ws(A, u, d);
-  const int pos = reinterpret_cast<const int32_t*>(A.arena_c + d->off_anchor_pos)[a];
-  for (int side = 0; side < 2; ++side) {
-    const __nv_bfloat16* X = (side ? A.V : A.K) + ((size_t)u * A.s_max + pos) * 128;
-    __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(A.arena + (side ? d->off_anchor_v : d->off_anchor_k)) +
-                         (size_t)a * 128;
-    // dim j is in chunk j / 8, stored at chunk place (j / 8) ^ (a % 8)
-    for (int j = lane; j < 128; j += 32) dst[8 * ((j >> 3) ^ (a & 7)) + (j & 7)] = X[j];
-    if (lane == 0) {
-      double n = 0.0;
-      for (int j = 0; j < 128; ++j) {
-        const double t = bf16_to_f64(X[j]);
-        n = __dadd_rn(n, __dmul_rn(t, t));
-      }
-      w.n2[side][a] = n;
-      w.rn[side][a] = __dsqrt_rn(n);
-      if (n != 0.0) atomicOr(&w.ctrl[side], 1u);
-    }
-  }
+// Bytes of one bf16 pair as two floats.
+__device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
+
+// fp16 bits of a float, round to nearest even, saturating like f64_to_fp16_bits.
+__device__ __forceinline__ uint32_t f32_to_fp16_bits(float x) {
+  const uint32_t b = __half_as_ushort(__float2half_rn(x));
+  if ((b & 0x7FFFu) < 0x7C00u) return b;
+  return (b & 0x3FFu) ? 0x7E00u : ((b & 0x8000u) | 0x7BFFu);
 }
 
-constexpr int AS_POS = 64;  // positions per assignment block
-constexpr int AS_ANC = 32;  // anchors per smem chunk
-constexpr int AS_THREADS = 256;
-constexpr size_t AS_SMEM = (size_t)128 * AS_POS * 8 + (size_t)AS_ANC * 128 * 8 + 4 * AS_POS * (8 + 8 + 4) + 64;
+// Anchor norms the fp32 filter handles: every product and sum of enc_assign_tc and enc_finish then
+// stays inside the fp32 range.
+constexpr double kNormLo = 0x1p-60, kNormHi = 0x1p60;  // of squared norms
 
-__global__ void __launch_bounds__(AS_THREADS) enc_assign(const EncArgs A) {
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  double* xs = reinterpret_cast<double*>(sm_raw);                 // [128][64] positions, transposed
-  double* xa = xs + 128 * AS_POS;                                 // [32][128] anchor chunk
-  double* bcv = xa + AS_ANC * 128;                                // [4][64]
-  double* bdv = bcv + 4 * AS_POS;                                 // [4][64]
-  int* bav = reinterpret_cast<int*>(bdv + 4 * AS_POS);            // [4][64]
-
+// 32 anchors of one side per block: rows copied into the arena, squared norms (sequential in j; the
+// square of a bf16 is exact, so a fused multiply-add rounds like the separate steps).  The rows pass
+// through shared memory so that one lane per anchor runs the serial fp64 chain: with one lane per
+// warp reading its row from global memory the same sums took 289 us for 8 units of 656 anchors.
+__global__ void __launch_bounds__(256) enc_rows(const EncArgs A) {
+  __shared__ __align__(16) uint4 rows[32][17];
   const int u = blockIdx.y, side = blockIdx.z;
   const akv_unit_desc* d = unit_desc(A, u);
-  const int S = d->len, k = d->n_anchors;
-  const int p0 = blockIdx.x * AS_POS;
-  if (p0 >= S) return;
+  const int k = d->n_anchors, a0 = blockIdx.x * 32, tid = threadIdx.x;
+  if (a0 >= k) return;
   EncUnitWs w = unit_ws(A, u, d);
-  const __nv_bfloat16* X = (side ? A.V : A.K) + (size_t)u * A.s_max * 128;
   const int32_t* apos = reinterpret_cast<const int32_t*>(A.arena_c + d->off_anchor_pos);
-  const double* n2 = w.n2[side];
-  const double* rn = w.rn[side];
-  const int tid = threadIdx.x;
-
-  for (int e = tid; e < AS_POS * 128; e += AS_THREADS) {
-    const int pi = e >> 7, j = e & 127;
-    const int p = p0 + pi;
-    xs[j * AS_POS + pi] = (p < S) ? bf16_to_f64(X[(size_t)p * 128 + j]) : 0.0;
+  uint8_t* dst = A.arena + (side ? d->off_anchor_v : d->off_anchor_k);
+  for (int e = tid; e < 32 * 16; e += 256) {
+    const int r = e >> 4, c = e & 15, a = a0 + r;
+    if (a >= k) continue;
+    const uint4 v = reinterpret_cast<const uint4*>(anchor_src(A, u, side, apos, a))[c];
+    rows[r][c] = v;
+    // chunk c (dims 8 c .. 8 c + 7) at chunk place c ^ (a % 8)
+    *reinterpret_cast<uint4*>(dst + (size_t)a * 256 + 16 * (c ^ (a & 7))) = v;
   }
-  const int pi = tid % AS_POS, ag = tid / AS_POS;
-  double bestc = -1.0, bestd = 0.0;
-  int besta = -1;
-  for (int ac = 0; ac < k; ac += AS_ANC) {
-    __syncthreads();
-    for (int e = tid; e < AS_ANC * 128; e += AS_THREADS) {
-      const int t = e >> 7, j = e & 127;
-      xa[e] = (ac + t < k) ? bf16_to_f64(anchor_src(A, u, side, apos, ac + t)[j]) : 0.0;
+  __syncthreads();
+  if (tid >= 32) return;
+  const int a = a0 + tid;
+  double n = 0.0;
+  if (a < k) {
+    for (int c = 0; c < 16; ++c) {
+      const uint4 v = rows[tid][c];
+      const uint32_t wd[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const double lo = (double)bf_lo(wd[e]), hi = (double)bf_hi(wd[e]);
+        n = __fma_rn(lo, lo, n);
+        n = __fma_rn(hi, hi, n);
+      }
     }
-    __syncthreads();
-    double dd[8];
+    w.n2[side][a] = n;
+  }
+  const bool safe = n >= kNormLo && n <= kNormHi;
+  w.inv[side][a] = a < k && safe ? (float)__ddiv_rn(1.0, __dsqrt_rn(n)) : 0.0f;  // (a < k rounded up to 32)
+  if (__any_sync(0xffffffffu, a < k && n != 0.0) && tid == 0) atomicOr(&w.ctrl[side], 1u);
+  if (__any_sync(0xffffffffu, a < k && n != 0.0 && !safe) && tid == 0) atomicOr(&w.ctrl[4 + side], 1u);
+}
+
+// ---- Eq. 1 on tensor cores ------------------------------------------------------------
+// The nearest anchor of a position is the one with the largest |x . x_a| / |x_a|, decided in fp64.
+// As a GEMM (positions x anchors x 128) the fp64 units need 81 ms for a layer of 8 x 32768 positions
+// and 656 anchors; the tensor cores' fp32 sums of the exact bf16 products take the same scores to
+// within 2^-14 |x| (128 exact products, fp32 accumulation; the margin is 8 times the worst bound of
+// truncated accumulation), so only the anchors within 2 x 2^-14 |x| of a position's largest
+// score can be its nearest.  That leaves one anchor for about 99 % of positions; enc_finish decides the
+// rest in fp64.  The candidate word of a position: first candidate in bits 0-15, second in bits 16-31
+// (0xFFFF: none), or 0xFFFFFFFF: any anchor may be the nearest.
+//
+// One persistent CTA per SM takes items of 256 positions of one unit and side (two M = 128 tiles
+// that share every anchor chunk, which halves the L2 reads of the anchors), anchor chunks of 192.
+// Warp 8 copies (three position tiles and two anchor chunks in flight), warp 9 issues the
+// products (two accumulators of 192 TMEM columns), warps 0-3 and 4-7 are the two tiles' epilogues:
+// a thread owns one position, scales 32 columns at a time by 1 / |x_a|, takes the largest of
+// each eight and looks at single columns only where that comes within the margin of the running
+// maximum.  Waits are bounded; after a failure every remaining position gets the word that lets
+// enc_finish decide it alone, so the result stays right.
+constexpr int kAtN = 192;
+constexpr int kAtA = 3, kAtB = 2;  // stages
+constexpr uint32_t kAtHalfA = 128 * 128, kAtHalfB = kAtN * 128;  // bytes of 64 of the 128 dimensions
+constexpr uint32_t kAtSmem = kAtA * 2 * kAtHalfA + kAtB * 2 * kAtHalfB + 1024;
+constexpr int kAtThreads = 320;
+constexpr float kAtMargin = 0x1p-13f;  // 2 x 2^-14, relative to |x|
+
+__device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&v)[32]) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr)
+      : "memory");
 #pragma unroll
-    for (int t = 0; t < 8; ++t) dd[t] = 0.0;
-    const double* xr = xa + (ag * 8) * 128;
-    for (int j = 0; j < 128; ++j) {
-      const double x = xs[j * AS_POS + pi];
-#pragma unroll
-      for (int t = 0; t < 8; ++t) dd[t] = __fma_rn(x, xr[t * 128 + j], dd[t]);  // product of two bf16: exact
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__global__ void __launch_bounds__(kAtThreads, 1)
+    enc_assign_tc(const __grid_constant__ EncArgs A, const __grid_constant__ CUtensorMap tmK,
+                  const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmA, long long items,
+                  int max_t) {
+  extern __shared__ __align__(1024) uint8_t as_dyn[];
+  __shared__ __align__(8) uint64_t bars[2 * kAtA + 2 * kAtB + 4];
+  __shared__ uint32_t tmem_sh;
+  __shared__ int failed_sh;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t sA = (smem_u32(as_dyn) + 1023u) & ~1023u, sB = sA + kAtA * 2 * kAtHalfA;
+  auto a_full = [&](int s) { return smem_u32(bars + s); };
+  auto a_free = [&](int s) { return smem_u32(bars + kAtA + s); };
+  auto b_full = [&](int s) { return smem_u32(bars + 2 * kAtA + s); };
+  auto b_free = [&](int s) { return smem_u32(bars + 2 * kAtA + kAtB + s); };
+  auto acc_full = [&](int m) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + m); };
+  auto acc_empty = [&](int m) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + 2 + m); };
+  volatile int* failed = &failed_sh;
+  if (tid == 0) {
+    for (int i = 0; i < 2 * kAtA + 2 * kAtB + 2; ++i) mbar_init(smem_u32(bars + i), 1);
+    for (int m = 0; m < 2; ++m) mbar_init(acc_empty(m), 4);  // one arrival per epilogue warp
+    *failed = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) tc_alloc(smem_u32(&tmem_sh), 512);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_sh;
+
+  // item (unit u, side, tile t): positions 256 t .. of the unit; every role walks the same items
+  struct Item {
+    int u, side, t, S, k;
+  };
+  auto next_item = [&](long long& i, Item& it) {  // the item at or after i that holds positions
+    for (; i < items; i += gridDim.x) {
+      it.t = (int)(i % max_t);
+      it.side = (int)((i / max_t) & 1);
+      it.u = (int)(i / max_t / 2);
+      const int2 sk = __ldg(reinterpret_cast<const int2*>(unit_desc(A, it.u)));
+      it.S = sk.x;
+      it.k = sk.y;
+      if (it.t * 256 < it.S) return true;
     }
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      const int a = ac + ag * 8 + t;
-      if (a < k && n2[a] != 0.0) {
-        const double c = __ddiv_rn(fabs(dd[t]), rn[a]);
-        if (c > bestc) {
-          bestc = c;
-          besta = a;
-          bestd = dd[t];
+    return false;
+  };
+  auto n_tiles = [](const Item& it) { return it.S - it.t * 256 > 128 ? 2 : 1; };
+
+  if (warp == 8) {
+    if (lane == 0) {  // ---- copies
+      int na = 0, nb = 0;
+      auto load_a = [&](const Item& it, int m) {
+        const int s = na % kAtA;
+        if (!mbar_wait(a_free(s), (uint32_t)((na / kAtA) & 1) ^ 1u)) return false;
+        const CUtensorMap* tm = it.side ? &tmV : &tmK;
+        const int row = it.u * A.s_max + it.t * 256 + 128 * m;
+        mbar_expect_tx(a_full(s), 2 * kAtHalfA);
+        tma_load_2d(sA + s * 2 * kAtHalfA, tm, 0, row, a_full(s));
+        tma_load_2d(sA + s * 2 * kAtHalfA + kAtHalfA, tm, 64, row, a_full(s));
+        ++na;
+        return true;
+      };
+      bool ok = true;
+      Item it;
+      for (long long i = blockIdx.x; ok && next_item(i, it); i += gridDim.x) {
+        const akv_unit_desc* d = unit_desc(A, it.u);
+        const int row0 = (int)((it.side ? d->off_anchor_v : d->off_anchor_k) >> 8);
+        ok = load_a(it, 0);
+        for (int c0 = 0; ok && c0 < it.k; c0 += kAtN) {
+          const int s = nb % kAtB, nr = (min(kAtN, it.k - c0) + 63) / 64;  // boxes of 64 anchor rows
+          if (*failed || !mbar_wait(b_free(s), (uint32_t)((nb / kAtB) & 1) ^ 1u)) {
+            ok = false;
+            break;
+          }
+          mbar_expect_tx(b_full(s), (uint32_t)nr * 2 * 64 * 128);
+          for (int r = 0; r < nr; ++r) {
+            tma_load_2d(sB + s * 2 * kAtHalfB + r * 64 * 128, &tmA, 0, row0 + c0 + 64 * r, b_full(s));
+            tma_load_2d(sB + s * 2 * kAtHalfB + kAtHalfB + r * 64 * 128, &tmA, 64, row0 + c0 + 64 * r, b_full(s));
+          }
+          ++nb;
+          if (c0 == 0 && n_tiles(it) == 2) ok = load_a(it, 1);
         }
+      }
+      if (!ok) *failed = 1;
+      // (bounded) every copy has landed before the CTA may exit
+      for (int j = max(0, na - kAtA); j < na; ++j) mbar_wait(a_full(j % kAtA), (uint32_t)(j / kAtA) & 1u);
+      for (int j = max(0, nb - kAtB); j < nb; ++j) mbar_wait(b_full(j % kAtB), (uint32_t)(j / kAtB) & 1u);
+    }
+    __syncwarp();
+  } else if (warp == 9) {
+    if (lane == 0) {  // ---- products
+      int na = 0, nb = 0, nacc[2] = {0, 0};
+      bool ok = true;
+      Item it;
+      for (long long i = blockIdx.x; ok && next_item(i, it); i += gridDim.x) {
+        const int nm = n_tiles(it);
+        for (int c0 = 0; ok && c0 < it.k; c0 += kAtN, ++nb) {
+          const int sb = nb % kAtB;
+          const uint32_t n = (uint32_t)min(kAtN, (it.k - c0 + 15) & ~15);
+          const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((128u >> 4) << 24);
+          ok = !*failed && mbar_wait(b_full(sb), (uint32_t)(nb / kAtB) & 1u);
+          for (int m = 0; ok && m < nm; ++m) {
+            const int sa = (na + m) % kAtA;
+            ok = (c0 > 0 || mbar_wait(a_full(sa), (uint32_t)((na + m) / kAtA) & 1u)) &&
+                 mbar_wait(acc_empty(m), (uint32_t)(nacc[m] & 1) ^ 1u);
+            if (!ok) break;
+            tc_fence_after();
+            const uint32_t a = sA + sa * 2 * kAtHalfA, b = sB + sb * 2 * kAtHalfB;
+#pragma unroll
+            for (int kk = 0; kk < 8; ++kk) {
+              const uint32_t ka = (uint32_t)(kk >> 2) * kAtHalfA + (uint32_t)(kk & 3) * 32;
+              const uint32_t kb = (uint32_t)(kk >> 2) * kAtHalfB + (uint32_t)(kk & 3) * 32;
+              tc_mma(tmem + 256u * (uint32_t)m, sw128_desc(a + ka), sw128_desc(b + kb), idesc, kk > 0 ? 1u : 0u);
+            }
+            ++nacc[m];
+            tc_commit(acc_full(m));
+            if (c0 + kAtN >= it.k) tc_commit(a_free(sa));
+          }
+          if (ok) tc_commit(b_free(sb));
+        }
+        na += nm;
+      }
+      if (!ok) *failed = 1;
+      // (bounded) every product has completed before the CTA may exit: the last commits have arrived
+      for (int m = 0; m < 2; ++m)
+        if (nacc[m] > 0) mbar_wait(acc_full(m), (uint32_t)(nacc[m] - 1) & 1u);
+    }
+    __syncwarp();
+  } else {  // ---- epilogue of tile m
+    const int m = warp >> 2, q = warp & 3;
+    int nacc = 0;
+    bool ok = true;
+    Item it;
+    for (long long i = blockIdx.x; next_item(i, it); i += gridDim.x) {
+      if (m >= n_tiles(it)) continue;
+      const int p = it.t * 256 + 128 * m + 32 * q + lane;
+      const EncUnitWs w = unit_ws(A, it.u, unit_desc(A, it.u));
+      const float* inv = w.inv[it.side];
+      float nx2 = 0.f;
+      if (p < it.S) {
+        const uint4* X = reinterpret_cast<const uint4*>((it.side ? A.V : A.K) + ((size_t)it.u * A.s_max + p) * 128);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          const uint4 v = __ldg(X + c);
+          const uint32_t wd[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            nx2 = __fmaf_rn(bf_lo(wd[e]), bf_lo(wd[e]), nx2);
+            nx2 = __fmaf_rn(bf_hi(wd[e]), bf_hi(wd[e]), nx2);
+          }
+        }
+      }
+      const bool usable = nx2 >= (float)kNormLo && nx2 <= (float)kNormHi && w.ctrl[4 + it.side] == 0u;
+      const float marg = kAtMargin * 1.001f * __fsqrt_rn(nx2);
+      float m1 = 0.f, thr = 0.f;  // the largest score so far; what a candidate must exceed
+      int i1 = 0xFFFF, i2 = 0xFFFF, cnt = 0;
+      for (int c0 = 0; c0 < it.k; c0 += kAtN) {
+        __syncwarp();
+        ok = ok && __shfl_sync(0xffffffffu, *failed, 0) == 0 && mbar_wait_w(acc_full(m), (uint32_t)nacc & 1u);
+        if (!ok) break;  // (the same for the whole warp)
+        ++nacc;
+        tc_fence_after();
+        const int n = min(kAtN, it.k - c0);
+        for (int sc = 0; sc < n; sc += 32) {
+          float s[32];
+          __syncwarp();
+          tc_ld32(tmem + ((uint32_t)(32 * q) << 16) + 256u * (uint32_t)m + (uint32_t)sc, s);
+          if (sc + 32 >= n) {  // the tile's last read of the accumulator
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty(m));
+          }
+          const float4* iv = reinterpret_cast<const float4*>(inv + c0 + sc);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            const float4 f = __ldg(iv + e);
+            s[4 * e] = fabsf(s[4 * e]) * f.x;
+            s[4 * e + 1] = fabsf(s[4 * e + 1]) * f.y;
+            s[4 * e + 2] = fabsf(s[4 * e + 2]) * f.z;
+            s[4 * e + 3] = fabsf(s[4 * e + 3]) * f.w;
+          }
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            const float* t = s + 8 * g;
+            const float mx = fmaxf(fmaxf(fmaxf(t[0], t[1]), fmaxf(t[2], t[3])), fmaxf(fmaxf(t[4], t[5]), fmaxf(t[6], t[7])));
+            if (mx > thr) {  // (NaN: no candidate)
+#pragma unroll
+              for (int e = 0; e < 8; ++e) {
+                if (t[e] > thr) {
+                  const int a = c0 + sc + 8 * g + e;
+                  if (t[e] > m1 + marg) {
+                    i1 = a;
+                    cnt = 1;
+                  } else {
+                    if (cnt == 0) i1 = a;
+                    else i2 = a;
+                    ++cnt;
+                  }
+                  m1 = fmaxf(m1, t[e]);
+                  thr = fmaxf(m1 - marg, 0.f);
+                }
+              }
+            }
+          }
+        }
+      }
+      if (p < it.S) {
+        const bool one = cnt == 1, two = cnt == 2;
+        const uint32_t word = (uint32_t)i1 | ((one ? 0xFFFFu : (uint32_t)i2) << 16);
+        w.st[it.side][p] = ok && usable && m1 > marg && (one || two) ? word : 0xFFFFFFFFu;
+      }
+    }
+    if (!ok) *failed = 1;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 0) tc_dealloc(tmem, 512);
+}
+
+// Exact x . x_a, summed j = 0 .. 127 in order (a product of two bf16 is exact, so the fused
+// step rounds once, like a separate add).
+__device__ double exact_dot(const uint4* x, const uint4* row, int a) {
+  double s = 0.0;
+  for (int c = 0; c < 16; ++c) {
+    const uint4 xv = __ldg(x + c), av = __ldg(row + (c ^ (a & 7)));
+    const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w}, aw[4] = {av.x, av.y, av.z, av.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      s = __fma_rn((double)bf_lo(xw[e]), (double)bf_lo(aw[e]), s);
+      s = __fma_rn((double)bf_hi(xw[e]), (double)bf_hi(aw[e]), s);
+    }
+  }
+  return s;
+}
+
+// Whether x == gamma x_a holds exactly in every dimension (a duplicate of its anchor): the
+// fp32 products are exact when they are 0 or not below 2^-100.
+__device__ bool exactly_zero_residual(const uint4* x, const uint4* row, int a, float g) {
+  for (int c = 0; c < 16; ++c) {
+    const uint4 xv = __ldg(x + c), av = __ldg(row + (c ^ (a & 7)));
+    const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w}, aw[4] = {av.x, av.y, av.z, av.w};
+    for (int e = 0; e < 8; ++e) {
+      const float xe = (e & 1) ? bf_hi(xw[e >> 1]) : bf_lo(xw[e >> 1]);
+      const float ae = (e & 1) ? bf_hi(aw[e >> 1]) : bf_lo(aw[e >> 1]);
+      const float pe = __fmul_rn(g, ae);
+      if (pe != xe || (fabsf(pe) < 0x1p-100f && g != 0.f && ae != 0.f)) return false;
+    }
+  }
+  return true;
+}
+
+// Exact residual energy (Eq. 5's r in fp64, squares summed in order) of position row x under
+// stream word st; the key that the slots are ranked by.
+__device__ uint64_t exact_energy_key(const uint4* x, const uint4* row, uint32_t st, bool valid) {
+  const int a = (int)(st & 0xFFFFu);
+  const double g = fp16_bits_to_f64(st >> 16);
+  double e = 0.0;
+  for (int c = 0; c < 16; ++c) {
+    const uint4 xv = __ldg(x + c), av = __ldg(row + (c ^ (a & 7)));
+    const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w}, aw[4] = {av.x, av.y, av.z, av.w};
+    for (int h = 0; h < 8; ++h) {
+      const float xe = (h & 1) ? bf_hi(xw[h >> 1]) : bf_lo(xw[h >> 1]);
+      const float ae = (h & 1) ? bf_hi(aw[h >> 1]) : bf_lo(aw[h >> 1]);
+      const double pj = valid ? __dmul_rn(g, (double)ae) : 0.0;
+      const double r = __dsub_rn((double)xe, pj);
+      e = __dadd_rn(e, __dmul_rn(r, r));
+    }
+  }
+  return (uint64_t)__double_as_longlong(e) + 1ull;
+}
+
+// Residual energy in fp32 as a key (bits + 1).  r = x - gamma x_a is one exactly rounded step and
+// every square is positive, so the sum is within 2^-19 of the exact energy while it lies in
+// [2^-90, 2^100]; an energy outside (and not exactly 0) sets the unit's fp64 flag.
+constexpr float kEnLo = 0x1p-90f, kEnHi = 0x1p100f;
+__device__ __forceinline__ uint32_t energy_key(float e, const uint4* x, const uint4* row, int a, float g, uint32_t* inexact) {
+  if (!(e >= kEnLo && e <= kEnHi) && !(e == 0.f && exactly_zero_residual(x, row, a, g))) atomicOr(inexact, 1u);
+  return __float_as_uint(e) + 1u;
+}
+
+// Eq. 1 decided and Eq. 2: gamma = fp16(x . x_a / |x_a|^2), and the residual energy of every
+// position.  Eight lanes take a position (16 dimensions each).  With one candidate anchor, x . x_a in
+// fp32 fixes gamma's fp16 rounding unless the quotient lies within its error (2^-19 sum |x x_a| /
+// |x_a|^2) of a rounding boundary; those positions, and the ones with two candidates, go to a list
+// that the block's threads finish with fp64 chains, one position each; positions where any anchor may be
+// the nearest take a warp each.  fp64 work for every position would bound this kernel (the energies
+// alone are 335 M operations, 0.55 ms at 0.6 T/s, for 2 x 8 x 32768 positions).
+constexpr int kFinPos = 256;  // positions per block
+__global__ void __launch_bounds__(256) enc_finish(const EncArgs A) {
+  __shared__ int todo[kFinPos], full[kFinPos];
+  __shared__ int n_todo, n_full;
+  __shared__ __align__(16) float xs[8][128];
+  const int u = blockIdx.y, side = blockIdx.z;
+  const akv_unit_desc* d = unit_desc(A, u);
+  const int S = d->len, k = d->n_anchors, p0 = blockIdx.x * kFinPos;
+  if (p0 >= S) return;
+  const EncUnitWs w = unit_ws(A, u, d);
+  const uint4* X = reinterpret_cast<const uint4*>((side ? A.V : A.K) + (size_t)u * A.s_max * 128);
+  const uint4* AR = reinterpret_cast<const uint4*>(A.arena_c + (side ? d->off_anchor_v : d->off_anchor_k));
+  uint32_t* stream = w.st[side];
+  const double* n2 = w.n2[side];
+  uint32_t* key = reinterpret_cast<uint32_t*>(side ? w.key1 : w.key0);
+  uint32_t* inexact = &w.ctrl[6 + side];
+  const bool want_e = A.m_obs == 0;  // (the full selection ranks by its own utilities)
+  const int tid = threadIdx.x, sub = tid & 7, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) n_todo = n_full = 0;
+  __syncthreads();
+  for (int q = tid >> 3; q < kFinPos; q += 32) {
+    const int p = p0 + q;
+    const bool in = p < S;
+    const int sl = in ? w.slot_of[p] : 0;
+    const uint32_t word = in ? stream[p] : 0u;
+    const int a = (int)(word & 0xFFFFu);
+    const bool one = in && sl < 0 && (word >> 16) == 0xFFFFu && a != 0xFFFF;
+    uint32_t xw[8] = {}, aw[8] = {};
+    if (one) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const uint4 xv = __ldg(X + (size_t)p * 16 + 2 * sub + c), av = __ldg(AR + (size_t)a * 16 + ((2 * sub + c) ^ (a & 7)));
+        xw[4 * c] = xv.x; xw[4 * c + 1] = xv.y; xw[4 * c + 2] = xv.z; xw[4 * c + 3] = xv.w;
+        aw[4 * c] = av.x; aw[4 * c + 1] = av.y; aw[4 * c + 2] = av.z; aw[4 * c + 3] = av.w;
+      }
+    }
+    float dd = 0.f, ab = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      dd = __fmaf_rn(bf_lo(xw[c]), bf_lo(aw[c]), dd);
+      dd = __fmaf_rn(bf_hi(xw[c]), bf_hi(aw[c]), dd);
+      ab = __fmaf_rn(fabsf(bf_lo(xw[c])), fabsf(bf_lo(aw[c])), ab);
+      ab = __fmaf_rn(fabsf(bf_hi(xw[c])), fabsf(bf_hi(aw[c])), ab);
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+      dd += __shfl_xor_sync(0xffffffffu, dd, o);
+      ab += __shfl_xor_sync(0xffffffffu, ab, o);
+    }
+    const float nf = one ? (float)n2[a] : 1.f;
+    const float gq = __fdiv_rn(dd, nf), ge = __fdiv_rn(ab, nf) * 0x1p-19f;
+    const uint32_t gh = f32_to_fp16_bits(gq - ge);
+    const bool fixed = one && ab >= 0x1p-80f && ab <= 0x1p100f && gh == f32_to_fp16_bits(gq + ge);
+    const float g = __half2float(__ushort_as_half((unsigned short)gh));
+    float e = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const float r0 = __fmaf_rn(-g, bf_lo(aw[c]), bf_lo(xw[c])), r1 = __fmaf_rn(-g, bf_hi(aw[c]), bf_hi(xw[c]));
+      e = __fmaf_rn(r0, r0, e);
+      e = __fmaf_rn(r1, r1, e);
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (sub == 0 && in) {
+      if (sl >= 0) {  // an anchor: its own slot, coefficient 1
+        stream[p] = (uint32_t)sl | (0x3C00u << 16);
+        if (want_e) key[p] = 0u;
+      } else if (fixed) {
+        stream[p] = (uint32_t)a | (gh << 16);
+        if (want_e) key[p] = energy_key(e, X + (size_t)p * 16, AR + (size_t)a * 16, a, g, inexact);
+      } else if (word == 0xFFFFFFFFu) {
+        full[atomicAdd(&n_full, 1)] = p;
+      } else {
+        todo[atomicAdd(&n_todo, 1)] = p;
       }
     }
   }
-  bcv[ag * AS_POS + pi] = bestc;
-  bdv[ag * AS_POS + pi] = bestd;
-  bav[ag * AS_POS + pi] = besta;
   __syncthreads();
-  if (tid >= AS_POS) return;
-  const int p = p0 + tid;
-  if (p >= S) return;
-  double c = -1.0, dbest = 0.0;
-  int a = -1;
-  for (int g = 0; g < 4; ++g) {
-    const int ga = bav[g * AS_POS + tid];
-    if (ga < 0) continue;
-    const double gc = bcv[g * AS_POS + tid];
-    if (a < 0 || gc > c || (gc == c && ga < a)) {
-      c = gc;
-      a = ga;
-      dbest = bdv[g * AS_POS + tid];
+  auto finish = [&](int p, int a, double dot) {  // the position's nearest anchor a (-1: none) is known
+    const uint32_t gh = a >= 0 ? f64_to_fp16_bits(__ddiv_rn(dot, n2[a])) : 0u;
+    const int as = a >= 0 ? a : 0;
+    stream[p] = (uint32_t)as | (gh << 16);
+    if (!want_e) return;
+    const float g = a >= 0 ? __half2float(__ushort_as_half((unsigned short)gh)) : 0.f;
+    const uint4 *x = X + (size_t)p * 16, *row = AR + (size_t)as * 16;
+    float e = 0.f;
+    for (int c = 0; c < 16; ++c) {
+      const uint4 xv = __ldg(x + c), av = __ldg(row + (c ^ (as & 7)));
+      const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w}, aw[4] = {av.x, av.y, av.z, av.w};
+      float ec = 0.f;  // (a sum per chunk keeps the rounding errors of the chain at 24)
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const float r0 = a >= 0 ? __fmaf_rn(-g, bf_lo(aw[h]), bf_lo(xw[h])) : bf_lo(xw[h]);
+        const float r1 = a >= 0 ? __fmaf_rn(-g, bf_hi(aw[h]), bf_hi(xw[h])) : bf_hi(xw[h]);
+        ec = __fmaf_rn(r0, r0, ec);
+        ec = __fmaf_rn(r1, r1, ec);
+      }
+      e += ec;
     }
+    key[p] = energy_key(e, x, row, as, g, inexact);
+  };
+  if (tid < n_todo) {
+    const int p = todo[tid];
+    const uint32_t word = stream[p];
+    const int a1 = (int)(word & 0xFFFFu), a2 = (int)(word >> 16);
+    int a = a1;
+    double dot = exact_dot(X + (size_t)p * 16, AR + (size_t)a1 * 16, a1);
+    if (a2 != 0xFFFF) {
+      const double dot2 = exact_dot(X + (size_t)p * 16, AR + (size_t)a2 * 16, a2);
+      const double c1 = __ddiv_rn(fabs(dot), __dsqrt_rn(n2[a1])), c2 = __ddiv_rn(fabs(dot2), __dsqrt_rn(n2[a2]));
+      if (c2 > c1 || (c2 == c1 && a2 < a1)) {
+        a = a2;
+        dot = dot2;
+      }
+    }
+    finish(p, a, dot);
   }
-  uint32_t* stream = w.st[side];
-  uint64_t* key = side ? w.key1 : w.key0;
-  const int sl = w.slot_of[p];
-  if (sl >= 0) {
-    stream[p] = (uint32_t)sl | (0x3C00u << 16);
-    key[p] = 0;
-    return;
+  for (int t = warp; t < n_full; t += 8) {  // any anchor: a lane takes every 32nd one
+    const int p = full[t];
+    const uint4* x = X + (size_t)p * 16;
+    __syncwarp();
+    if (lane < 16) {
+      const uint4 v = __ldg(x + lane);
+      float* o = xs[warp] + 8 * lane;
+      o[0] = bf_lo(v.x); o[1] = bf_hi(v.x); o[2] = bf_lo(v.y); o[3] = bf_hi(v.y);
+      o[4] = bf_lo(v.z); o[5] = bf_hi(v.z); o[6] = bf_lo(v.w); o[7] = bf_hi(v.w);
+    }
+    __syncwarp();
+    float nx2 = 0.f;
+    bool zero = true;
+    for (int j = 0; j < 4; ++j) {
+      const float v = xs[warp][4 * lane + j];
+      nx2 = __fmaf_rn(v, v, nx2);
+      zero = zero && v == 0.f;
+    }
+    for (int o = 16; o > 0; o >>= 1) nx2 += __shfl_xor_sync(0xffffffffu, nx2, o);
+    zero = __all_sync(0xffffffffu, zero);
+    const bool filter = !zero && nx2 >= (float)kNormLo && nx2 <= (float)kNormHi && w.ctrl[4 + side] == 0u;
+    const float marg = kAtMargin * 1.001f * __fsqrt_rn(nx2);
+    auto score = [&](int a) {  // fp32, within 2^-16 |x| of |x . x_a| / |x_a|
+      const uint4* row = AR + (size_t)a * 16;
+      float s = 0.f;
+      for (int c = 0; c < 16; ++c) {
+        const uint4 v = __ldg(row + (c ^ (a & 7)));
+        const float* xc = xs[warp] + 8 * c;
+        s = __fmaf_rn(xc[0], bf_lo(v.x), s);
+        s = __fmaf_rn(xc[1], bf_hi(v.x), s);
+        s = __fmaf_rn(xc[2], bf_lo(v.y), s);
+        s = __fmaf_rn(xc[3], bf_hi(v.y), s);
+        s = __fmaf_rn(xc[4], bf_lo(v.z), s);
+        s = __fmaf_rn(xc[5], bf_hi(v.z), s);
+        s = __fmaf_rn(xc[6], bf_lo(v.w), s);
+        s = __fmaf_rn(xc[7], bf_hi(v.w), s);
+      }
+      return fabsf(s) * w.inv[side][a];
+    };
+    float mx = 0.f;
+    if (filter) {
+      for (int a = lane; a < k; a += 32) mx = fmaxf(mx, score(a));
+      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    double bc = -1.0, bd = 0.0;
+    int ba = -1;
+    for (int a = lane; a < k; a += 32) {
+      const double na = n2[a];
+      if (na == 0.0 || (filter && score(a) < mx - marg)) continue;
+      if (zero && ba >= 0) continue;  // every usable anchor scores 0: the lane's first stands
+      const double dot = exact_dot(x, AR + (size_t)a * 16, a);
+      const double c = __ddiv_rn(fabs(dot), __dsqrt_rn(na));
+      if (c > bc) {
+        bc = c;
+        bd = dot;
+        ba = a;
+      }
+    }
+    for (int o = 16; o > 0; o >>= 1) {  // the largest, ties to the lowest slot
+      const double oc = __shfl_xor_sync(0xffffffffu, bc, o), od = __shfl_xor_sync(0xffffffffu, bd, o);
+      const int oa = __shfl_xor_sync(0xffffffffu, ba, o);
+      if (oa >= 0 && (ba < 0 || oc > bc || (oc == bc && oa < ba))) {
+        bc = oc;
+        bd = od;
+        ba = oa;
+      }
+    }
+    if (lane == 0) finish(p, ba, bd);
   }
-  const uint32_t gh = (a >= 0) ? f64_to_fp16_bits(__ddiv_rn(dbest, n2[a])) : 0u;
-  stream[p] = (uint32_t)(a >= 0 ? a : 0) | (gh << 16);
-  const double g = fp16_bits_to_f64(gh);
-  const __nv_bfloat16* xar = anchor_src(A, u, side, apos, a >= 0 ? a : 0);
-  double e = 0.0;
-  for (int j = 0; j < 128; ++j) {
-    const double pj = (a >= 0) ? __dmul_rn(g, bf16_to_f64(xar[j])) : 0.0;
-    const double r = __dsub_rn(xs[j * AS_POS + tid], pj);
-    e = __dadd_rn(e, __dmul_rn(r, r));
-  }
-  key[p] = (uint64_t)__double_as_longlong(e) + 1ull;
 }
 
-// Per (unit, side): the N largest keys (ties: lower position) -> flags and the
-// ascending slot list.
-__global__ void __launch_bounds__(1024) enc_slots(const EncArgs A, int side) {
+// ---- residual slots (plain encoder) ---------------------------------------------------
+// Per unit and side the N positions with the largest energies (ties: lower position), by a cluster
+// of kSelCtas CTAs that share out the positions and exchange counts through distributed shared
+// memory.  A radix select (digits of 11, 11 and 10 bits) finds the N-th largest of the fp32 energies;
+// those are within 2^-19 of the fp64 ones, so a position above (1 + 2^-16) of it is in, one below
+// (1 - 2^-16) of it is out, and the few between are ranked by their exact fp64 energies.  (One CTA per
+// unit over 64-bit keys took 84 + 99 us for the two sides of 8 x 32768 positions.)
+constexpr int kSelCtas = 8, kSelThreads = 512, kSelBand = 512;
+
+// The CTA's share [lo, hi) of n items, of a multiple of 4 items.
+__device__ __forceinline__ void cluster_share(int n, int rank, int& lo, int& hi) {
+  const int per = (int)((((long long)n + kSelCtas - 1) / kSelCtas + 3) & ~3ll);
+  lo = (int)min((long long)n, (long long)rank * per);
+  hi = (int)min((long long)n, (long long)lo + per);
+}
+
+__global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) enc_slots(const EncArgs A) {
+  namespace cg = cooperative_groups;
+  __shared__ uint32_t hist[3][2048];
+  __shared__ uint32_t wsum[kSelThreads / 32];
+  __shared__ uint32_t found[2];           // digit, and what is still wanted inside it
+  __shared__ uint32_t cnt_hi, cnt_band;   // this CTA's positions above the band, and inside it
+  __shared__ uint32_t n_app, n_list;      // slots written by this CTA; entries of the cluster's list (CTA 0)
+  __shared__ int band[kSelBand];          // this CTA's positions inside the band
+  __shared__ uint64_t lkey[kSelBand];     // CTA 0: every band position's exact key ...
+  __shared__ int lpos[kSelBand];          // ... and position
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int u = blockIdx.x / kSelCtas, side = blockIdx.y;
+  const akv_unit_desc* d = unit_desc(A, u);
+  const int S = d->len, N = side ? d->n_res_v : d->n_res_k;
+  const EncUnitWs w = unit_ws(A, u, d);
+  const uint32_t* key = reinterpret_cast<const uint32_t*>(side ? w.key1 : w.key0);
+  uint8_t* flag = w.flag[side];
+  int32_t* rp = w.res_pos + (side ? d->n_res_k : 0);
+  int lo, hi;
+  cluster_share(S, rank, lo, hi);
+  if (N == 0) {  // (the whole cluster)
+    for (int p = lo + tid; p < hi; p += kSelThreads) flag[p] = 0;
+    return;
+  }
+  if (w.ctrl[6 + side]) return;  // energies outside the fp32 range: enc_slots_exact
+  for (int i = tid; i < 3 * 2048; i += kSelThreads) (&hist[0][0])[i] = 0u;
+  if (tid == 0) cnt_hi = cnt_band = n_app = n_list = 0u;
+  __syncthreads();
+  uint32_t prefix = 0, want = (uint32_t)N;
+#pragma unroll 1
+  for (int dg = 0; dg < 3; ++dg) {
+    const int sh = dg == 0 ? 21 : (dg == 1 ? 10 : 0), bits = dg == 2 ? 10 : 11;
+    for (int p = lo + tid; p < hi; p += kSelThreads) {
+      const uint32_t v = key[p];
+      if (dg == 0 || (v >> (sh + bits)) == prefix) atomicAdd(&hist[dg][(v >> sh) & ((1u << bits) - 1u)], 1u);
+    }
+    cl.sync();
+    // four digits per thread, from the largest down: thread t holds digits 2047 - 4 t .. 2044 - 4 t
+    uint32_t c[4], sum = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) c[e] = 0;
+    for (int r = 0; r < kSelCtas; ++r) {
+      const uint4 v = *reinterpret_cast<const uint4*>(cl.map_shared_rank(&hist[dg][0], r) + 2044 - 4 * tid);
+      c[0] += v.w; c[1] += v.z; c[2] += v.y; c[3] += v.x;
+    }
+    sum = c[0] + c[1] + c[2] + c[3];
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    uint32_t before = incl - sum;
+    for (int x = 0; x < warp; ++x) before += wsum[x];
+    if (before < want && want <= before + sum) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (before < want && want <= before + c[e]) {
+          found[0] = (uint32_t)(2047 - 4 * tid - e);
+          found[1] = want - before;
+        }
+        before += c[e];
+      }
+    }
+    __syncthreads();
+    prefix = (prefix << bits) | found[0];
+    want = found[1];
+    __syncthreads();
+  }
+  const uint32_t T = prefix;  // the N-th largest key; N <= S - k, so it is no anchor's (T >= 1)
+  const float eT = __uint_as_float(T - 1u);
+  const uint32_t k_lo = __float_as_uint(__fmul_rn(eT, 1.0f - 0x1p-16f)) + 1u;
+  const uint32_t k_hi = __float_as_uint(__fmul_rn(eT, 1.0f + 0x1p-16f)) + 1u;
+  for (int p0 = lo; p0 < hi; p0 += kSelThreads) {
+    const int p = p0 + tid;
+    const uint32_t v = p < hi ? key[p] : 0u;
+    const unsigned above = __ballot_sync(0xffffffffu, v > k_hi);
+    if (lane == 0 && above) atomicAdd(&cnt_hi, (uint32_t)__popc(above));
+    if (v >= k_lo && v <= k_hi) {
+      const uint32_t i = atomicAdd(&cnt_band, 1u);
+      if (i < kSelBand) band[i] = p;
+    }
+  }
+  cl.sync();
+  uint32_t n_hi = 0, n_band = 0, hi_before = 0, band_before = 0;
+  for (int r = 0; r < kSelCtas; ++r) {
+    const uint32_t h = *cl.map_shared_rank(&cnt_hi, r), b = *cl.map_shared_rank(&cnt_band, r);
+    if (r < rank) {
+      hi_before += h;
+      band_before += b;
+    }
+    n_hi += h;
+    n_band += b;
+  }
+  const uint32_t need = (uint32_t)N - n_hi;  // of the band
+  const bool all = need == n_band;           // the whole band is in
+  const bool tied = eT == 0.f;               // every band energy is exactly 0: the lowest positions are in
+  if (!all && !tied && n_band > kSelBand) {  // (the whole cluster) too many to rank here
+    if (rank == 0 && tid == 0) atomicOr(&w.ctrl[6 + side], 1u);
+    cl.sync();  // no CTA leaves while another may still read its counts
+    return;
+  }
+  const uint32_t k_in = all ? k_lo : k_hi + 1u;
+  const uint32_t at = all ? hi_before + band_before : hi_before;
+  for (int p0 = lo; p0 < hi; p0 += kSelThreads) {
+    const int p = p0 + tid;
+    const bool sel = p < hi && key[p] >= k_in;
+    const unsigned bal = __ballot_sync(0xffffffffu, sel);
+    uint32_t i = 0;
+    if (lane == 0 && bal) i = atomicAdd(&n_app, (uint32_t)__popc(bal));
+    i = __shfl_sync(0xffffffffu, i, 0);
+    if (p < hi) flag[p] = sel ? 1 : 0;
+    if (sel) rp[at + i + __popc(bal & ((1u << lane) - 1u))] = p;
+  }
+  if (!all && tied) {  // in position order
+    __syncthreads();
+    if (tid == 0) {
+      uint32_t i = band_before;
+      for (int p = lo; p < hi && i < need; ++p)
+        if (key[p] >= k_lo && key[p] <= k_hi) {
+          flag[p] = 1;
+          rp[n_hi + i++] = p;
+        }
+    }
+  } else if (!all) {  // ranked by exact energies, ties to the lower position
+    uint32_t* n0 = cl.map_shared_rank(&n_list, 0);
+    uint64_t* k0 = cl.map_shared_rank(&lkey[0], 0);
+    int* p0 = cl.map_shared_rank(&lpos[0], 0);
+    const uint4* X = reinterpret_cast<const uint4*>((side ? A.V : A.K) + (size_t)u * A.s_max * 128);
+    const uint4* AR = reinterpret_cast<const uint4*>(A.arena_c + (side ? d->off_anchor_v : d->off_anchor_k));
+    const bool valid = w.ctrl[side] != 0u;
+    const int mine = (int)cnt_band;
+    uint64_t my_key = 0;
+    int my_pos = -1;
+    if (tid < mine) {  // (at most kSelBand = kSelThreads)
+      my_pos = band[tid];
+      const uint32_t st = w.st[side][my_pos];
+      my_key = exact_energy_key(X + (size_t)my_pos * 16, AR + (size_t)(st & 0xFFFFu) * 16, st, valid);
+      const uint32_t i = atomicAdd(n0, 1u);
+      k0[i] = my_key;
+      p0[i] = my_pos;
+    }
+    cl.sync();
+    if (my_pos >= 0) {
+      uint32_t before = 0;
+      for (uint32_t i = 0; i < n_band; ++i) before += k0[i] > my_key || (k0[i] == my_key && p0[i] < my_pos);
+      if (before < need) {
+        flag[my_pos] = 1;
+        rp[n_hi + before] = my_pos;
+      }
+    }
+  }
+  cl.sync();  // no CTA leaves while another may still read its shared memory
+}
+static_assert(kSelBand == kSelThreads, "a thread ranks one band position");
+
+// The same from fp64 energies of every position, for the units and sides that enc_slots left (energies
+// outside the fp32 range, or a band of more than kSelBand positions): one block each, else nothing.
+__global__ void __launch_bounds__(1024) enc_slots_exact(const EncArgs A) {
   __shared__ uint32_t hist[256];
   __shared__ uint32_t bc[2];
   __shared__ int wt[33];
-  const int u = blockIdx.x;
+  const int u = blockIdx.x, side = blockIdx.y;
   const akv_unit_desc* d = unit_desc(A, u);
   const int S = d->len, N = side ? d->n_res_v : d->n_res_k;
-  EncUnitWs w = unit_ws(A, u, d);
-  const uint64_t* key = side ? w.key1 : w.key0;
+  const EncUnitWs w = unit_ws(A, u, d);
+  if (N == 0 || w.ctrl[6 + side] == 0u) return;
+  uint64_t* key = side ? w.key1 : w.key0;
+  // the fp32 keys lie where the first half of the fp64 ones go, so which positions are anchors (key 0;
+  // the same for both sides) is taken from the stream words: an anchor's position is its slot's
+  const int32_t* apos = reinterpret_cast<const int32_t*>(A.arena_c + d->off_anchor_pos);
+  const uint4* X = reinterpret_cast<const uint4*>((side ? A.V : A.K) + (size_t)u * A.s_max * 128);
+  const uint4* AR = reinterpret_cast<const uint4*>(A.arena_c + (side ? d->off_anchor_v : d->off_anchor_k));
+  const bool valid = w.ctrl[side] != 0u;
+  for (int p = threadIdx.x; p < S; p += blockDim.x) {
+    const uint32_t st = w.st[side][p];
+    key[p] = apos[st & 0xFFFFu] == p ? 0ull : exact_energy_key(X + (size_t)p * 16, AR + (size_t)(st & 0xFFFFu) * 16, st, valid);
+  }
+  __syncthreads();
   int32_t* rp = w.res_pos + (side ? d->n_res_k : 0);
-  uint64_t thr = ~0ull;
   uint32_t need = 0;
-  if (N > 0) thr = block_select(key, S, (uint32_t)N, true, hist, bc, &need);
+  const uint64_t thr = block_select(key, S, (uint32_t)N, true, hist, bc, &need);
   int base = 0, eq_seen = 0;
   for (int c0 = 0; c0 < S; c0 += 1024) {
     const int p = c0 + threadIdx.x;
     const uint64_t kv = (p < S) ? key[p] : 0ull;
-    const int is_eq = (N > 0 && p < S && kv == thr) ? 1 : 0;
+    const int is_eq = (p < S && kv == thr) ? 1 : 0;
     int eq_tot;
     const int eq_pre = block_scan_flag(is_eq, wt, &eq_tot);
-    const int sel = (N > 0 && p < S) && (kv > thr || (is_eq && (uint32_t)(eq_seen + eq_pre) < need));
+    const int sel = p < S && (kv > thr || (is_eq && (uint32_t)(eq_seen + eq_pre) < need));
     eq_seen += eq_tot;
     int tot;
     const int pre = block_scan_flag(sel, wt, &tot);
     if (sel) rp[base + pre] = p;
-    // flags of both sides share bytes: the side-0 launch writes them, the side-1 launch
-    // (ordered after it on the stream) ORs its bit in
-    if (p < S) {
-      if (side == 0) w.flag[p] = (uint8_t)sel;
-      else if (sel) w.flag[p] |= 2u;
-    }
+    if (p < S) w.flag[side][p] = (uint8_t)sel;
     base += tot;
     __syncthreads();
   }
@@ -520,7 +1156,7 @@ __global__ void __launch_bounds__(1024) enc_order(const EncArgs A) {
     const int rank = __popc(peers & ((1u << lane) - 1u));
     if (p < S) {
       w.perm[base + rank] = p;
-      w.inv[p] = (int32_t)(base + rank);
+      w.at[p] = (int32_t)(base + rank);
       if (rank == 0) w.cursor[a] = base + (uint32_t)__popc(peers);
     }
     __syncwarp();
@@ -536,7 +1172,8 @@ __global__ void __launch_bounds__(kTile) enc_tile_count(const EncArgs A) {
   if (j >= d->n_tiles) return;
   EncUnitWs w = unit_ws(A, u, d);
   const int t = j * kTile + threadIdx.x;
-  const uint32_t f = t < d->len ? w.flag[w.perm[t]] : 0u;
+  const int i = t < d->len ? w.perm[t] : -1;
+  const uint32_t f = i >= 0 ? (w.flag[0][i] | (w.flag[1][i] << 1)) : 0u;
   const int nk = __syncthreads_count(f & 1u), nv = __syncthreads_count(f & 2u);
   if (threadIdx.x == 0) {
     w.tcnt[2 * j] = (uint32_t)nk;
@@ -580,7 +1217,7 @@ __global__ void __launch_bounds__(kTile) enc_tile_fill(const EncArgs A) {
     const int i = w.perm[j * kTile + t];
     kst[t] = w.st[0][i];
     vst[t] = w.st[1][i];
-    f = w.flag[i];
+    f = w.flag[0][i] | (w.flag[1][i] << 1);
     if (d->off_pos) reinterpret_cast<uint32_t*>(A.arena + d->off_pos)[j * kTile + t] = (uint32_t)i;  // RoPE positions
   }
   const unsigned bk = __ballot_sync(0xffffffffu, f & 1u), bv = __ballot_sync(0xffffffffu, f & 2u);
@@ -694,7 +1331,7 @@ __global__ void enc_quant(const EncArgs A) {
     }
   }
   // record r of its tile: the rank of the token among the tile's tokens with this side's bit
-  const int ts = w.inv[p], j = ts / kTile, tl = ts % kTile;
+  const int ts = w.at[p], j = ts / kTile, tl = ts % kTile;
   const int n = tile_len(d->len, j), nw = (int)tile_words(n), n64 = 64 * nw;
   const int nkj = (int)w.tcnt[2 * j], nvj = (int)w.tcnt[2 * j + 1];
   const uint8_t* blkc = A.arena_c + d->off_tiles + reinterpret_cast<const uint32_t*>(A.arena_c + d->off_tile_table)[j];
@@ -942,7 +1579,7 @@ __global__ void __launch_bounds__(1024) enc_pool(const EncArgs A, int side) {
     keys[h] = side ? w.key1 : w.key0;
     lists[h] = w.res_pos + (side ? d->n_res_k : 0);
     ctrls[h] = w.ctrl;
-    flags[h] = w.flag;
+    flags[h] = w.flag[side];
   }
   __syncthreads();
   const int64_t N = budget_residuals(A.theta, S, H, A.window, k);
@@ -968,11 +1605,7 @@ __global__ void __launch_bounds__(1024) enc_pool(const EncArgs A, int side) {
       int tot;
       const int pre = block_scan_flag(sel, wt, &tot);
       if (sel) lists[h][base + pre] = p;
-      // flags of both sides share bytes: the side-0 launch writes them, side 1 ORs its bit in
-      if (p < S) {
-        if (side == 0) flags[h][p] = (uint8_t)sel;
-        else if (sel) flags[h][p] |= 2u;
-      }
+      if (p < S) flags[h][p] = (uint8_t)sel;
       base += tot;
       __syncthreads();
     }
@@ -1065,17 +1698,29 @@ int launch_encode(const Layout& L, const EncodeWs& W, const akv_params& p, const
   }
   enc_hash<<<dim3((maxS + 255) / 256, units), 256, 0, st>>>(A);
   enc_anchors<<<units, 1024, 0, st>>>(A);
-  enc_rows<<<dim3((unsigned)(L.max_k + 7) / 8, units), 256, 0, st>>>(A);
-  if ((e = cudaFuncSetAttribute(enc_assign, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)AS_SMEM)) != cudaSuccess)
+  enc_rows<<<dim3((unsigned)(L.max_k + 31) / 32, units, 2), 256, 0, st>>>(A);
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return (int)e;
+  if ((e = cudaFuncSetAttribute(enc_assign_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAtSmem)) !=
+      cudaSuccess)
     return (int)e;
-  enc_assign<<<dim3((maxS + AS_POS - 1) / AS_POS, units, 2), AS_THREADS, AS_SMEM, st>>>(A);
+  CUtensorMap tmK, tmV, tmA;
+  if (!encode_row_map(&tmK, K, (uint64_t)units * (uint64_t)s_max, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_row_map(&tmV, V, (uint64_t)units * (uint64_t)s_max, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
+      !encode_row_map(&tmA, arena, (uint64_t)L.total_bytes / 256, 64, CU_TENSOR_MAP_SWIZZLE_NONE))
+    return (int)cudaErrorNotSupported;
+  const int max_t = (int)((maxS + 255) / 256);
+  const long long items = 2ll * units * max_t;
+  enc_assign_tc<<<(unsigned)std::min<long long>(items, sms), kAtThreads, kAtSmem, st>>>(A, tmK, tmV, tmA, items, max_t);
+  enc_finish<<<dim3((maxS + kFinPos - 1) / kFinPos, units, 2), 256, 0, st>>>(A);
   if (full) {  // Eq. 6 utilities, then each side's pooled top-N per request
     enc_util<<<dim3((maxS + 127) / 128, units), 128, 0, st>>>(A);
-    enc_pool<<<units / p.n_kv_heads, 1024, 0, st>>>(A, 0);  // writes the flag bytes
-    enc_pool<<<units / p.n_kv_heads, 1024, 0, st>>>(A, 1);  // ORs the value bit in
+    enc_pool<<<units / p.n_kv_heads, 1024, 0, st>>>(A, 0);
+    enc_pool<<<units / p.n_kv_heads, 1024, 0, st>>>(A, 1);
   } else {
-    enc_slots<<<units, 1024, 0, st>>>(A, 0);  // writes the flag bytes
-    enc_slots<<<units, 1024, 0, st>>>(A, 1);  // ORs the value bit in
+    enc_slots<<<dim3(kSelCtas * (unsigned)units, 2), kSelThreads, 0, st>>>(A);
+    enc_slots_exact<<<dim3(units, 2), 1024, 0, st>>>(A);
   }
   enc_order<<<units, 1024, 0, st>>>(A);
   enc_tile_count<<<dim3((unsigned)L.max_tiles, units), kTile, 0, st>>>(A);
