@@ -7,7 +7,6 @@
 // twice gives the same result.
 //
 // Kernels, in launch order, each over all units of the batch:
-//   enc_hash       anchor-selection hashes of the non-window positions
 //   enc_anchors    select the k - W smallest hashes, number anchor slots by position
 //   enc_rows       copy anchor rows into the arena (16-byte chunks swizzled), squared norms
 //   enc_assign_tc  Eq. 1: the one or two anchors that can be a position's nearest, on tensor cores
@@ -40,9 +39,9 @@ constexpr double kLloydT = 0.98046875;
 
 // Per-unit scratch pointers, derived from the workspace table the host writes.
 struct EncUnitWs {
-  // [S] each: anchor hashes or selector scores; then (plain encoder) the first half holds the
-  // residual energies per side as fp32 bits + 1, anchors 0, or (full selection, and slots that need
-  // fp64 energies) the whole the fp64 bits + 1
+  // [S] each: selector scores; then (plain encoder) the first half holds the residual energies per
+  // side as fp32 bits + 1, anchors 0, or (full selection, and slots that need fp64 energies) the
+  // whole the fp64 bits + 1; then the counting sort's rows
   uint64_t* key0;
   uint64_t* key1;
   int32_t* slot_of;   // [S] anchor slot or -1
@@ -250,53 +249,148 @@ __device__ __forceinline__ int n_scored(const EncArgs& A, int rest) {
   return (A.m_obs > 0 && rest > 0) ? (int)floor((double)A.rho * (double)rest) : 0;
 }
 
-__global__ void enc_hash(const EncArgs A) {
-  const int u = blockIdx.y;
-  const akv_unit_desc* d = unit_desc(A, u);
-  const int S = d->len;
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= S) return;
-  EncUnitWs w = unit_ws(A, u, d);
-  const int win = min(A.window, S);
-  const uint64_t base = A.seed ^ ((uint64_t)d->b << 40) ^ ((uint64_t)d->h << 32);
-  // (full selection: positions already chosen by their score take no part in the sampling)
-  const bool scored = A.m_obs > 0 && w.slot_of[p] == -2;
-  w.key0[p] = (p < S - win && !scored) ? splitmix64_dev(base ^ (uint64_t)p) : ~0ull;
+// Clusters of kSelCtas CTAs take one unit (and side): they share out its positions and exchange
+// counts through distributed shared memory.
+constexpr int kSelCtas = 8, kSelThreads = 512, kSelBand = 512;
+
+// The CTA's share [lo, hi) of n items, of a multiple of 4 items.
+__device__ __forceinline__ void cluster_share(int n, int rank, int& lo, int& hi) {
+  const int per = (int)((((long long)n + kSelCtas - 1) / kSelCtas + 3) & ~3ll);
+  lo = (int)min((long long)n, (long long)rank * per);
+  hi = (int)min((long long)n, (long long)lo + per);
 }
 
-__global__ void __launch_bounds__(1024) enc_anchors(const EncArgs A) {
-  __shared__ uint32_t hist[256];
-  __shared__ uint32_t bc[2];
-  __shared__ int wt[33];
-  const int u = blockIdx.x;
+// One digit of a radix select over the cluster, called by all its CTAs after the cluster barrier that
+// ends the counting: of the 2048 digits counted in every CTA's `hist` (taken from the largest down,
+// or from the smallest up) the one that holds the want-th key; want becomes the rank inside it.  The
+// number of keys with that digit goes to *inside.
+template <bool DOWN>
+__device__ uint32_t cluster_digit(cooperative_groups::cluster_group cl, uint32_t* hist, uint32_t* wsum, uint32_t* found,
+                                  uint32_t& want, uint32_t* inside) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t c[4] = {0u, 0u, 0u, 0u};  // four digits per thread, in order
+  for (int r = 0; r < kSelCtas; ++r) {
+    const uint4 v = *reinterpret_cast<const uint4*>(cl.map_shared_rank(hist, r) + (DOWN ? 2044 - 4 * tid : 4 * tid));
+    c[0] += DOWN ? v.w : v.x;
+    c[1] += DOWN ? v.z : v.y;
+    c[2] += DOWN ? v.y : v.z;
+    c[3] += DOWN ? v.x : v.w;
+  }
+  const uint32_t sum = c[0] + c[1] + c[2] + c[3];
+  uint32_t incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) wsum[warp] = incl;
+  __syncthreads();
+  uint32_t before = incl - sum;
+  for (int x = 0; x < warp; ++x) before += wsum[x];
+  if (before < want && want <= before + sum) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      if (before < want && want <= before + c[e]) {
+        found[0] = (uint32_t)(DOWN ? 2047 - 4 * tid - e : 4 * tid + e);
+        found[1] = want - before;
+        found[2] = c[e];
+      }
+      before += c[e];
+    }
+  }
+  __syncthreads();
+  const uint32_t digit = found[0];
+  want = found[1];
+  *inside = found[2];
+  __syncthreads();
+  return digit;
+}
+static_assert(kSelThreads * 4 == 2048, "four digits per thread");
+
+// The unit's anchors: the last min(W, S) positions, the positions the full selection scored, and the
+// `rest` smallest hashes of the others; slots numbered by position.  A radix select over the cluster
+// finds the hash that bounds the rest (hashes are distinct, so it ends at the first digit whose keys
+// are all wanted: two or three digits); hashes are computed where they are needed.  (One CTA per unit
+// and eight digits of stored hashes took 72 us for 8 x 32768 positions and 232 us for 2 x 131072.)
+__global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) enc_anchors(const EncArgs A) {
+  namespace cg = cooperative_groups;
+  __shared__ __align__(16) uint32_t hist[3][2048];
+  __shared__ uint32_t wsum[kSelThreads / 32];
+  __shared__ uint32_t found[3];
+  __shared__ uint32_t total;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int u = blockIdx.x / kSelCtas;
   const akv_unit_desc* d = unit_desc(A, u);
   const int S = d->len, k = d->n_anchors;
-  EncUnitWs w = unit_ws(A, u, d);
-  const int win = min(A.window, S);
-  const int pool = S - win;
+  const EncUnitWs w = unit_ws(A, u, d);
+  const int win = min(A.window, S), pool = S - win;
+  const bool full = A.m_obs > 0;
   // the sampled share: all k - w non-window anchors, less those the full selection scored
-  const int rest = k - win - n_scored(A, k - win);
-  uint64_t thr = 0;
-  bool any = rest > 0;
-  if (any) {
-    uint32_t req;
-    thr = block_select(w.key0, pool, (uint32_t)rest, false, hist, bc, &req);
-  }
-  int32_t* apos = reinterpret_cast<int32_t*>(A.arena + d->off_anchor_pos);
-  int base = 0;
-  for (int c0 = 0; c0 < S; c0 += 1024) {
-    const int p = c0 + threadIdx.x;
-    int flag = 0;
-    if (p < S) flag = (p >= pool) || (A.m_obs > 0 && w.slot_of[p] == -2) || (any && w.key0[p] <= thr);
-    int tot;
-    const int pre = block_scan_flag(flag, wt, &tot);
-    if (p < S) {
-      w.slot_of[p] = flag ? base + pre : -1;
-      if (flag) apos[base + pre] = p;
+  const uint32_t rest = (uint32_t)(k - win - n_scored(A, k - win));
+  const uint64_t base = A.seed ^ ((uint64_t)d->b << 40) ^ ((uint64_t)d->h << 32);
+  int lo, hi;
+  cluster_share(S, rank, lo, hi);
+  for (int i = tid; i < 3 * 2048; i += kSelThreads) (&hist[0][0])[i] = 0u;
+  __syncthreads();
+  int sh = 64;          // the keys taken are those with key >> sh <= prefix
+  uint64_t prefix = 0;
+  if (rest > 0) {
+    uint32_t want = rest;
+#pragma unroll 1
+    for (int dg = 0;; ++dg) {
+      const int ns = max(0, sh - 11), bits = sh - ns;
+      uint32_t* h = hist[dg % 3];
+      for (int p = lo + tid; p < min(hi, pool); p += kSelThreads) {
+        if (full && w.slot_of[p] == -2) continue;  // already chosen by its score
+        const uint64_t v = splitmix64_dev(base ^ (uint64_t)p);
+        if (dg == 0 || (v >> sh) == prefix) atomicAdd(&h[(uint32_t)(v >> ns) & ((1u << bits) - 1u)], 1u);
+      }
+      cl.sync();
+      // (the third buffer's last readers passed the barrier before this one)
+      if (dg > 0)
+        for (int i = tid; i < 2048; i += kSelThreads) hist[(dg + 2) % 3][i] = 0u;
+      uint32_t inside;
+      const uint32_t digit = cluster_digit<false>(cl, h, wsum, found, want, &inside);
+      prefix = (prefix << bits) | digit;
+      sh = ns;
+      if (want == inside || sh == 0) break;
     }
-    base += tot;
   }
-  if (threadIdx.x < 8) w.ctrl[threadIdx.x] = 0;
+  auto is_anchor = [&](int p) {
+    return p >= pool || (full && w.slot_of[p] == -2) || (rest > 0 && (splitmix64_dev(base ^ (uint64_t)p) >> sh) <= prefix);
+  };
+  // slots by position: a warp takes a contiguous share of the CTA's, 32 positions at a time
+  const int per = (((hi - lo) + kSelThreads - 1) / kSelThreads) * 32;
+  const int wlo = min(hi, lo + warp * per), whi = min(hi, wlo + per);
+  uint32_t n = 0;
+  for (int p0 = wlo; p0 < whi; p0 += 32) {
+    const int p = p0 + lane;
+    n += (uint32_t)__popc(__ballot_sync(0xffffffffu, p < whi && is_anchor(p)));
+  }
+  if (lane == 0) wsum[warp] = n;
+  __syncthreads();
+  if (tid == 0) {
+    uint32_t t = 0;
+    for (int x = 0; x < kSelThreads / 32; ++x) t += wsum[x];
+    total = t;
+  }
+  cl.sync();
+  uint32_t at = 0;
+  for (int r = 0; r < rank; ++r) at += *cl.map_shared_rank(&total, r);
+  for (int x = 0; x < warp; ++x) at += wsum[x];
+  int32_t* apos = reinterpret_cast<int32_t*>(A.arena + d->off_anchor_pos);
+  for (int p0 = wlo; p0 < whi; p0 += 32) {
+    const int p = p0 + lane;
+    const bool is = p < whi && is_anchor(p);
+    const unsigned bal = __ballot_sync(0xffffffffu, is);
+    const uint32_t slot = at + (uint32_t)__popc(bal & ((1u << lane) - 1u));
+    if (p < whi) w.slot_of[p] = is ? (int32_t)slot : -1;
+    if (is) apos[slot] = p;
+    at += (uint32_t)__popc(bal);
+  }
+  if (rank == 0 && tid < 8) w.ctrl[tid] = 0;
+  cl.sync();  // no CTA leaves while another may still read its counts
 }
 
 // Bytes of one bf16 pair as two floats.
@@ -881,20 +975,11 @@ __global__ void __launch_bounds__(256) enc_finish(const EncArgs A) {
 // those are within 2^-19 of the fp64 ones, so a position above (1 + 2^-16) of it is in, one below
 // (1 - 2^-16) of it is out, and the few between are ranked by their exact fp64 energies.  (One CTA per
 // unit over 64-bit keys took 84 + 99 us for the two sides of 8 x 32768 positions.)
-constexpr int kSelCtas = 8, kSelThreads = 512, kSelBand = 512;
-
-// The CTA's share [lo, hi) of n items, of a multiple of 4 items.
-__device__ __forceinline__ void cluster_share(int n, int rank, int& lo, int& hi) {
-  const int per = (int)((((long long)n + kSelCtas - 1) / kSelCtas + 3) & ~3ll);
-  lo = (int)min((long long)n, (long long)rank * per);
-  hi = (int)min((long long)n, (long long)lo + per);
-}
-
 __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) enc_slots(const EncArgs A) {
   namespace cg = cooperative_groups;
-  __shared__ uint32_t hist[3][2048];
+  __shared__ __align__(16) uint32_t hist[3][2048];
   __shared__ uint32_t wsum[kSelThreads / 32];
-  __shared__ uint32_t found[2];           // digit, and what is still wanted inside it
+  __shared__ uint32_t found[3];
   __shared__ uint32_t cnt_hi, cnt_band;   // this CTA's positions above the band, and inside it
   __shared__ uint32_t n_app, n_list;      // slots written by this CTA; entries of the cluster's list (CTA 0)
   __shared__ int band[kSelBand];          // this CTA's positions inside the band
@@ -928,39 +1013,8 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) 
       if (dg == 0 || (v >> (sh + bits)) == prefix) atomicAdd(&hist[dg][(v >> sh) & ((1u << bits) - 1u)], 1u);
     }
     cl.sync();
-    // four digits per thread, from the largest down: thread t holds digits 2047 - 4 t .. 2044 - 4 t
-    uint32_t c[4], sum = 0;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) c[e] = 0;
-    for (int r = 0; r < kSelCtas; ++r) {
-      const uint4 v = *reinterpret_cast<const uint4*>(cl.map_shared_rank(&hist[dg][0], r) + 2044 - 4 * tid);
-      c[0] += v.w; c[1] += v.z; c[2] += v.y; c[3] += v.x;
-    }
-    sum = c[0] + c[1] + c[2] + c[3];
-    uint32_t incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    uint32_t before = incl - sum;
-    for (int x = 0; x < warp; ++x) before += wsum[x];
-    if (before < want && want <= before + sum) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (before < want && want <= before + c[e]) {
-          found[0] = (uint32_t)(2047 - 4 * tid - e);
-          found[1] = want - before;
-        }
-        before += c[e];
-      }
-    }
-    __syncthreads();
-    prefix = (prefix << bits) | found[0];
-    want = found[1];
-    __syncthreads();
+    uint32_t inside;
+    prefix = (prefix << bits) | cluster_digit<true>(cl, hist[dg], wsum, found, want, &inside);
   }
   const uint32_t T = prefix;  // the N-th largest key; N <= S - k, so it is no anchor's (T >= 1)
   const float eT = __uint_as_float(T - 1u);
@@ -1122,45 +1176,111 @@ __device__ uint32_t block_scan_u32(uint32_t v, uint32_t* warp_tot, uint32_t* tot
   return pre;
 }
 
-// Stored order of one unit: positions sorted by value anchor slot, ties by position
-// (a stable counting sort).  One block per unit; the scatter is done by one warp in
-// position order, 32 positions at a time, so equal slots keep their position order.
-__global__ void __launch_bounds__(1024) enc_order(const EncArgs A) {
-  __shared__ uint32_t wt[33];
-  const int u = blockIdx.x;
+// Stored order of one unit: positions sorted by value anchor slot, ties by position (a stable
+// counting sort), by a cluster per unit.  Up to 128 warps take contiguous shares of the positions and
+// count them by slot into a row of their own (rows [n_rows][k] over the energies, which are read no
+// more; n_rows k 4 <= 16 S bytes); the rows' columns are then prefix-summed, and every warp scatters its share
+// in order, 32 positions at a time, equal slots of a warp ranked by lane.  (One warp per unit doing
+// the scatter took 357 us for 32768 positions and 1650 us for 131072.)
+constexpr int kOrdWarps = kSelThreads / 32;  // per CTA
+__global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) enc_order(const EncArgs A) {
+  namespace cg = cooperative_groups;
+  __shared__ uint32_t part[8][64];
+  __shared__ uint32_t cta_total;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int u = blockIdx.x / kSelCtas;
   const akv_unit_desc* d = unit_desc(A, u);
   const int S = d->len, k = d->n_anchors;
-  EncUnitWs w = unit_ws(A, u, d);
-  for (int a = threadIdx.x; a <= k; a += blockDim.x) w.cursor[a] = 0u;
-  __syncthreads();
-  for (int p = threadIdx.x; p < S; p += blockDim.x) atomicAdd(&w.cursor[w.st[1][p] & 0xFFFFu], 1u);
-  __syncthreads();
-  uint32_t run = 0;
-  for (int c0 = 0; c0 < k; c0 += 1024) {
-    const int a = c0 + threadIdx.x;
-    const uint32_t v = a < k ? w.cursor[a] : 0u;
-    uint32_t tot;
-    const uint32_t pre = block_scan_u32(v, wt, &tot);
-    if (a < k) w.cursor[a] = run + pre;
-    run += tot;
-  }
-  __syncthreads();
-  if (threadIdx.x >= 32) return;
-  const int lane = threadIdx.x;
-  for (int c0 = 0; c0 < S; c0 += 32) {
-    const int p = c0 + lane;
-    const uint32_t a = p < S ? (w.st[1][p] & 0xFFFFu) : 0xFFFFFFFFu;
-    const unsigned peers = __match_any_sync(0xffffffffu, a);
-    const uint32_t base = p < S ? w.cursor[a] : 0u;
+  const EncUnitWs w = unit_ws(A, u, d);
+  const uint32_t* st = w.st[1];
+  uint32_t* mat = reinterpret_cast<uint32_t*>(w.key0);
+  const int n_rows = (int)min((long long)(kSelCtas * kOrdWarps), 4ll * S / k);
+  const int row = rank * kOrdWarps + warp;
+  const int per = (int)((((long long)S + n_rows - 1) / n_rows + 31) & ~31ll);
+  const int lo = row < n_rows ? (int)min((long long)S, (long long)row * per) : S;
+  const int hi = (int)min((long long)S, (long long)lo + per);
+  uint32_t* mine = mat + (size_t)row * k;
+  if (row < n_rows) {
+    for (int a = lane; a < k; a += 32) mine[a] = 0u;
+    __threadfence();
     __syncwarp();
-    const int rank = __popc(peers & ((1u << lane) - 1u));
-    if (p < S) {
-      w.perm[base + rank] = p;
-      w.at[p] = (int32_t)(base + rank);
-      if (rank == 0) w.cursor[a] = base + (uint32_t)__popc(peers);
+    for (int p0 = lo; p0 < hi; p0 += 32) {
+      const int p = p0 + lane;
+      const uint32_t a = p < hi ? (st[p] & 0xFFFFu) : 0xFFFFFFFFu;
+      const unsigned peers = __match_any_sync(0xffffffffu, a);
+      if (p < hi && (peers & ((1u << lane) - 1u)) == 0u) atomicAdd(&mine[a], (uint32_t)__popc(peers));
     }
-    __syncwarp();
   }
+  cl.sync();
+  // this CTA's slots [rank kper, ..): 64 at a time, eight threads per slot over the rows
+  const int kper = (k + kSelCtas - 1) / kSelCtas, a_lo = min(k, rank * kper), a_hi = min(k, a_lo + kper);
+  const int rper = (n_rows + 7) / 8;  // rows per thread, at most 16
+  uint32_t base = 0;                  // tokens of the CTA's slots so far
+  for (int a0 = a_lo; a0 < a_hi; a0 += 64) {
+    const int a = a0 + (tid & 63), g = tid >> 6;
+    uint32_t v[16], sum = 0;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const int r = g * rper + j;
+      v[j] = j < rper && r < n_rows && a < a_hi ? __ldcg(mat + (size_t)r * k + a) : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < 16; ++j) sum += v[j];
+    part[g][tid & 63] = sum;
+    __syncthreads();
+    uint32_t before = 0, tot = 0;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+      const uint32_t c = part[x][tid & 63];
+      before += x < g ? c : 0u;
+      tot += c;
+    }
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const int r = g * rper + j;
+      if (j < rper && r < n_rows && a < a_hi) __stcg(mat + (size_t)r * k + a, before);
+      before += v[j];
+    }
+    // slot starts: the 64 totals scanned by the first two warps
+    uint32_t incl = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    __syncthreads();
+    if (warp < 2 && lane == 31) part[0][warp] = incl;
+    __syncthreads();
+    if (warp < 2 && a < a_hi) __stcg(w.cursor + a, base + (warp == 1 ? part[0][0] : 0u) + incl - tot);
+    base += part[0][0] + part[0][1];
+    __syncthreads();
+  }
+  if (tid == 0) cta_total = base;
+  cl.sync();
+  if (tid == 0) {
+    uint32_t t = 0;
+    for (int r = 0; r < kSelCtas; ++r) {
+      part[1][r] = t;
+      t += *cl.map_shared_rank(&cta_total, r);
+    }
+  }
+  __syncthreads();
+  for (int p0 = lo; p0 < hi; p0 += 32) {
+    const int p = p0 + lane;
+    const uint32_t a = p < hi ? (st[p] & 0xFFFFu) : 0xFFFFFFFFu;
+    const unsigned peers = __match_any_sync(0xffffffffu, a);
+    const int before = __popc(peers & ((1u << lane) - 1u));
+    uint32_t at = 0;
+    if (p < hi && before == 0) at = atomicAdd(&mine[a], (uint32_t)__popc(peers)) + __ldcg(w.cursor + a) + part[1][a / kper];
+    at = __shfl_sync(0xffffffffu, at, __ffs(peers) - 1) + (uint32_t)before;
+    if (p < hi) {
+      w.perm[at] = p;
+      w.at[p] = (int32_t)at;
+    }
+    __syncwarp();  // (orders the rows' updates of successive steps)
+  }
+  cl.sync();  // no CTA leaves while another may still read its total
 }
 
 __device__ __forceinline__ int tile_len(int S, int j) { return min(kTile, S - j * kTile); }
@@ -1181,22 +1301,30 @@ __global__ void __launch_bounds__(kTile) enc_tile_count(const EncArgs A) {
   }
 }
 
-// Tile block offsets of every unit (one thread per unit).
-__global__ void enc_tile_table(const EncArgs A, int units) {
-  const int u = blockIdx.x * blockDim.x + threadIdx.x;
-  if (u >= units) return;
+// Tile block offsets of every unit (one block per unit, a thread per tile).
+__global__ void __launch_bounds__(1024) enc_tile_table(const EncArgs A) {
+  __shared__ uint32_t wt[33];
+  const int u = blockIdx.x;
   const akv_unit_desc* d = unit_desc(A, u);
-  EncUnitWs w = unit_ws(A, u, d);
+  const EncUnitWs w = unit_ws(A, u, d);
   uint32_t* table = reinterpret_cast<uint32_t*>(A.arena + d->off_tile_table);
-  uint32_t off = 0;
-  for (int j = 0; j < d->n_tiles; ++j) {
-    table[j] = off;
-    off += tile_block_bytes(tile_len(d->len, j), (int)w.tcnt[2 * j], (int)w.tcnt[2 * j + 1]);
-    // value slots of the tile's first and last stored tokens
-    const int t0 = j * kTile, t1 = t0 + tile_len(d->len, j) - 1;
-    table[d->n_tiles + 1 + j] = (w.st[1][w.perm[t0]] & 0xFFFFu) | ((w.st[1][w.perm[t1]] & 0xFFFFu) << 16);
+  uint32_t run = 0;
+  for (int j0 = 0; j0 < d->n_tiles; j0 += 1024) {
+    const int j = j0 + threadIdx.x;
+    const bool in = j < d->n_tiles;
+    const int n = in ? tile_len(d->len, j) : 0;
+    const uint32_t bytes = in ? tile_block_bytes(n, (int)w.tcnt[2 * j], (int)w.tcnt[2 * j + 1]) : 0u;
+    uint32_t tot;
+    const uint32_t pre = block_scan_u32(bytes, wt, &tot);
+    if (in) {
+      table[j] = run + pre;
+      // value slots of the tile's first and last stored tokens
+      const int t0 = j * kTile, t1 = t0 + n - 1;
+      table[d->n_tiles + 1 + j] = (w.st[1][w.perm[t0]] & 0xFFFFu) | ((w.st[1][w.perm[t1]] & 0xFFFFu) << 16);
+    }
+    run += tot;
   }
-  table[d->n_tiles] = off;
+  if (threadIdx.x == 0) table[d->n_tiles] = run;
 }
 
 // Streams, bitmaps and rank words of one tile block (one thread per stored token).
@@ -1467,7 +1595,7 @@ __global__ void enc_score_pool(const EncArgs A) {
 }
 
 // The floor(rho (k - w)) highest scores (ties: lower position) become anchors: slot_of = -2
-// marks them for enc_hash and enc_anchors, every other position gets -1.
+// marks them for enc_anchors, every other position gets -1.
 __global__ void __launch_bounds__(1024) enc_score_pick(const EncArgs A) {
   __shared__ uint32_t hist[256];
   __shared__ uint32_t bc[2];
@@ -1696,8 +1824,7 @@ int launch_encode(const Layout& L, const EncodeWs& W, const akv_params& p, const
     enc_score_pool<<<dim3((maxS + 255) / 256, units), 256, 0, st>>>(A);
     enc_score_pick<<<units, 1024, 0, st>>>(A);
   }
-  enc_hash<<<dim3((maxS + 255) / 256, units), 256, 0, st>>>(A);
-  enc_anchors<<<units, 1024, 0, st>>>(A);
+  enc_anchors<<<kSelCtas * (unsigned)units, kSelThreads, 0, st>>>(A);
   enc_rows<<<dim3((unsigned)(L.max_k + 31) / 32, units, 2), 256, 0, st>>>(A);
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -1722,9 +1849,9 @@ int launch_encode(const Layout& L, const EncodeWs& W, const akv_params& p, const
     enc_slots<<<dim3(kSelCtas * (unsigned)units, 2), kSelThreads, 0, st>>>(A);
     enc_slots_exact<<<dim3(units, 2), 1024, 0, st>>>(A);
   }
-  enc_order<<<units, 1024, 0, st>>>(A);
+  enc_order<<<kSelCtas * (unsigned)units, kSelThreads, 0, st>>>(A);
   enc_tile_count<<<dim3((unsigned)L.max_tiles, units), kTile, 0, st>>>(A);
-  enc_tile_table<<<(units + 127) / 128, 128, 0, st>>>(A, units);
+  enc_tile_table<<<units, 1024, 0, st>>>(A);
   enc_tile_fill<<<dim3((unsigned)L.max_tiles, units), kTile, 0, st>>>(A);
   const int maxN = std::max(L.max_nk, L.max_nv);
   if (maxN > 0) enc_quant<<<dim3((unsigned)(maxN + 7) / 8, units, 2), 256, 0, st>>>(A);
