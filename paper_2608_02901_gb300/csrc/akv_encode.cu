@@ -1366,25 +1366,15 @@ __global__ void __launch_bounds__(kTile) enc_tile_fill(const EncArgs A) {
   }
 }
 
-// One warp per residual slot: r = x - gamma x_a (fp64), v = H(s o r), quantize.
-__global__ void enc_quant(const EncArgs A) {
-  __shared__ double vbuf[8][128];
-  const int u = blockIdx.y, side = blockIdx.z;
-  const akv_unit_desc* d = unit_desc(A, u);
-  EncUnitWs w = unit_ws(A, u, d);
-  // slots of this unit: the parameters' count, or the count the full selection chose
-  const int N = A.m_obs > 0 ? (int)w.ctrl[2 + side] : (side ? d->n_res_v : d->n_res_k);
-  const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int s = blockIdx.x * 8 + wi;
-  if (s >= N) return;
-  const int p = w.res_pos[(side ? d->n_res_k : 0) + s];
-  const uint32_t st = w.st[side][p];
-  const int a = (int)(st & 0xFFFFu);
-  const double g = fp16_bits_to_f64(st >> 16);
-  const bool valid = w.ctrl[side] != 0u;
-  const __nv_bfloat16* X = (side ? A.V : A.K) + ((size_t)u * A.s_max + p) * 128;
-  const __nv_bfloat16* XA = anchor_src(A, u, side, reinterpret_cast<const int32_t*>(A.arena_c + d->off_anchor_pos), a);
-  double* v = vbuf[wi];
+// Scale, min and codes of one record, by a warp; lane l's four codes are those of dims 4 l .. 4 l + 3.
+struct Quantized {
+  uint32_t scale, min, byte;
+};
+
+// Quantized record in fp64: r = x - gamma x_a, v = H(s o r), quantize.  v: 128 doubles of shared memory.
+__device__ Quantized quantize_exact(const EncArgs& A, const __nv_bfloat16* X, const __nv_bfloat16* XA, double g, bool valid,
+                                    double* v) {
+  const int lane = threadIdx.x & 31;
   for (int j = lane; j < 128; j += 32) {
     const double pj = valid ? __dmul_rn(g, bf16_to_f64(XA[j])) : 0.0;
     double r = __dsub_rn(bf16_to_f64(X[j]), pj);
@@ -1458,6 +1448,130 @@ __global__ void enc_quant(const EncArgs A) {
       byte |= (uint32_t)code << (2 * c);
     }
   }
+  return Quantized{sch, mnh, byte};
+}
+
+// The same in fp32, where its error bounds decide every rounding; false (for the whole warp) where one does
+// not.  r is one exactly rounded step; each of the seven butterfly stages rounds values whose sum of
+// magnitudes is at most L1 = sum |r|, so v is within 8 x 2^-24 L1 of the exact transform: err = 2^-20 L1
+// below is twice that.  A value within err of a rounding boundary (fp16 min and scale, code regions) leaves
+// the record to quantize_exact, about one record in a hundred.  (fp64 for every record took 457 us for
+// 52,000 records: the fp64 units issue one warp instruction in 64 cycles.)
+__device__ bool quantize_fast(const EncArgs& A, const uint2 xr, const uint2 ar, float g, bool valid, Quantized* q) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t xw[4] = {xr.x << 16, xr.x & 0xFFFF0000u, xr.y << 16, xr.y & 0xFFFF0000u};
+  const uint32_t aw[4] = {ar.x << 16, ar.x & 0xFFFF0000u, ar.y << 16, ar.y & 0xFFFF0000u};
+  float v[4], l1 = 0.f;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    v[e] = __uint_as_float(xw[e]);
+    if (valid) v[e] = __fmaf_rn(-g, __uint_as_float(aw[e]), v[e]);
+    l1 += fabsf(v[e]);
+    if (A.rotate) {
+      const unsigned long long sb = lane < 16 ? A.sign_lo : A.sign_hi;
+      if ((sb >> ((4 * lane + e) & 63)) & 1ull) v[e] = -v[e];
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) l1 += __shfl_xor_sync(0xffffffffu, l1, o);
+  if (!(l1 >= 0x1p-60f && l1 <= 0x1p60f)) return false;
+  const float err = l1 * 0x1p-20f;
+  if (A.rotate) {
+    const float b0 = v[0] + v[1], b1 = v[0] - v[1], b2 = v[2] + v[3], b3 = v[2] - v[3];
+    v[0] = b0 + b2;
+    v[1] = b1 + b3;
+    v[2] = b0 - b2;
+    v[3] = b1 - b3;
+#pragma unroll
+    for (int m = 1; m < 32; m <<= 1) {
+      const float sg = (lane & m) ? -1.f : 1.f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] = __fmaf_rn(sg, v[e], __shfl_xor_sync(0xffffffffu, v[e], m));
+    }
+  }
+  bool sure = true;
+  q->byte = 0;
+  if (A.lloyd) {
+    float ss = 0.f, sa = 0.f;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      ss = __fmaf_rn(v[e], v[e], ss);
+      sa += fabsf(v[e]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      ss += __shfl_xor_sync(0xffffffffu, ss, o);
+      sa += __shfl_xor_sync(0xffffffffu, sa, o);
+    }
+    // sum v^2 off by 2 err sum |v| + 128 err^2 and ten roundings; the root adds two more
+    const float es = 2.001f * err * sa + 128.f * err * err + ss * 0x1p-20f;
+    q->min = 0u;
+    q->scale = f32_to_fp16_bits(__fsqrt_rn(fmaxf(ss - es, 0.f) * 0.0078125f) * (1.f - 0x1p-22f));
+    sure = q->scale == f32_to_fp16_bits(__fsqrt_rn((ss + es) * 0.0078125f) * (1.f + 0x1p-22f));
+    const float sc = __half2float(__ushort_as_half((unsigned short)q->scale));
+    const float T = (float)kLloydT;
+    if (sc == 0.f) {
+      q->byte = 0xAAu;  // a zero scale: code 2 everywhere
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float t = __fdiv_rn(v[e], sc), et = __fdiv_rn(err, sc) + fabsf(t) * 0x1p-22f;
+        sure = sure && fabsf(fabsf(t) - T) > et && fabsf(t) > et;
+        q->byte |= (t < -T ? 0u : (t < 0.f ? 1u : (t < T ? 2u : 3u))) << (2 * e);
+      }
+    }
+  } else {
+    float mn = fminf(fminf(v[0], v[1]), fminf(v[2], v[3])), mx = fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    q->min = f32_to_fp16_bits(mn - err);
+    sure = q->min == f32_to_fp16_bits(mn + err);
+    const float m16 = __half2float(__ushort_as_half((unsigned short)q->min));
+    const float t = __fdiv_rn(mx - m16, 3.f), et = err + fabsf(t) * 0x1p-22f;  // (a third of err, rounded up)
+    sure = sure && t > et;
+    q->scale = f32_to_fp16_bits(t - et);
+    sure = sure && q->scale == f32_to_fp16_bits(t + et);
+    const float sc = __half2float(__ushort_as_half((unsigned short)q->scale));
+    if (sc != 0.f) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float c = __fdiv_rn(v[e] - m16, sc), ec = __fdiv_rn(err, sc) + (fabsf(c) + fabsf(__fdiv_rn(m16, sc))) * 0x1p-22f;
+        const float f = floorf(c);
+        sure = sure && fabsf(c - f - 0.5f) > ec;
+        q->byte |= (uint32_t)fminf(fmaxf(rintf(c), 0.f), 3.f) << (2 * e);
+      }
+    }
+  }
+  return __all_sync(0xffffffffu, sure);
+}
+
+// One warp per residual slot: its scale, min and codes into its tile.
+__global__ void __launch_bounds__(256) enc_quant(const EncArgs A) {
+  __shared__ double vbuf[8][128];
+  const int u = blockIdx.y, side = blockIdx.z;
+  const akv_unit_desc* d = unit_desc(A, u);
+  EncUnitWs w = unit_ws(A, u, d);
+  // slots of this unit: the parameters' count, or the count the full selection chose
+  const int N = A.m_obs > 0 ? (int)w.ctrl[2 + side] : (side ? d->n_res_v : d->n_res_k);
+  const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int s = blockIdx.x * 8 + wi;
+  if (s >= N) return;
+  const int p = w.res_pos[(side ? d->n_res_k : 0) + s];
+  const uint32_t st = w.st[side][p];
+  const int a = (int)(st & 0xFFFFu);
+  const bool valid = w.ctrl[side] != 0u;
+  const __nv_bfloat16* X = (side ? A.V : A.K) + ((size_t)u * A.s_max + p) * 128;
+  const uint8_t* row = A.arena_c + (side ? d->off_anchor_v : d->off_anchor_k) + (size_t)a * 256;
+  Quantized q;
+  if (!quantize_fast(A, *reinterpret_cast<const uint2*>(X + 4 * lane),
+                     *reinterpret_cast<const uint2*>(row + 16 * ((lane >> 1) ^ (a & 7)) + 8 * (lane & 1)),
+                     __half2float(__ushort_as_half((unsigned short)(st >> 16))), valid, &q))
+    q = quantize_exact(A, X, anchor_src(A, u, side, reinterpret_cast<const int32_t*>(A.arena_c + d->off_anchor_pos), a),
+                       fp16_bits_to_f64(st >> 16), valid, vbuf[wi]);
+  const uint32_t mnh = q.min, sch = q.scale, byte = q.byte;
   // record r of its tile: the rank of the token among the tile's tokens with this side's bit
   const int ts = w.at[p], j = ts / kTile, tl = ts % kTile;
   const int n = tile_len(d->len, j), nw = (int)tile_words(n), n64 = 64 * nw;
