@@ -10,7 +10,8 @@
 //   enc_anchors    select the k - W smallest hashes, number anchor slots by position
 //   enc_rows       copy anchor rows into the arena (16-byte chunks swizzled), squared norms
 //   enc_assign_tc  Eq. 1: the one or two anchors that can be a position's nearest, on tensor cores
-//   enc_finish     Eq. 1 decided, Eq. 2 gamma, residual energies (per position)
+//   enc_finish     Eq. 2 gamma, residual energies (per position), as far as fp32 decides them
+//   enc_undecided  the rest in fp64
 //   enc_slots      top-N residual energies per side -> residual flags and slot list
 //   enc_order      stored order: stable counting sort of positions by value anchor slot
 //   enc_tile_count residual records per tile and side
@@ -49,7 +50,8 @@ struct EncUnitWs {
   double* n2[2];      // [k] squared anchor norms per side
   // [side]: the side has a nonzero anchor; [2 + side]: full selection's residual counts; [4 + side]:
   // an anchor norm outside the filter's range; [6 + side]: an energy outside the fp32 range, or a
-  // band too wide, so that the slots are chosen from fp64 energies
+  // band too wide, so that the slots are chosen from fp64 energies; [8 + side]: positions left to fp64,
+  // [10 + side]: positions where any anchor may be the nearest (lists behind the energies)
   uint32_t* ctrl;
   uint32_t* st[2];    // [S] stream word (slot | fp16 gamma << 16) per position and side
   uint8_t* flag[2];   // [S] residual flag per side (values: over slot_of, which is read no more by then)
@@ -389,13 +391,21 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) 
     if (is) apos[slot] = p;
     at += (uint32_t)__popc(bal);
   }
-  if (rank == 0 && tid < 8) w.ctrl[tid] = 0;
+  if (rank == 0 && tid < 16) w.ctrl[tid] = 0;
   cl.sync();  // no CTA leaves while another may still read its counts
 }
 
 // Bytes of one bf16 pair as two floats.
 __device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
+
+// A bf16 value, as the bits of a float, in fp64, on the integer pipe: the fp64 unit of an SM sub-partition
+// takes 64 cycles for one warp instruction, conversions included.
+__device__ __forceinline__ double bf_f64(uint32_t f) {
+  const uint32_t mag = f & 0x7FFFFFFFu;
+  if (mag - 0x00800000u >= 0x7F000000u) return (double)__uint_as_float(f);  // 0, subnormal, inf, NaN
+  return __hiloint2double((int)((f & 0x80000000u) | ((mag >> 3) + 0x38000000u)), 0);
+}
 
 // fp16 bits of a float, round to nearest even, saturating like f64_to_fp16_bits.
 __device__ __forceinline__ uint32_t f32_to_fp16_bits(float x) {
@@ -439,7 +449,7 @@ __global__ void __launch_bounds__(256) enc_rows(const EncArgs A) {
       const uint32_t wd[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const double lo = (double)bf_lo(wd[e]), hi = (double)bf_hi(wd[e]);
+        const double lo = bf_f64(wd[e] << 16), hi = bf_f64(wd[e] & 0xFFFF0000u);
         n = __fma_rn(lo, lo, n);
         n = __fma_rn(hi, hi, n);
       }
@@ -456,41 +466,56 @@ __global__ void __launch_bounds__(256) enc_rows(const EncArgs A) {
 // The nearest anchor of a position is the one with the largest |x . x_a| / |x_a|, decided in fp64.
 // As a GEMM (positions x anchors x 128) the fp64 units need 81 ms for a layer of 8 x 32768 positions
 // and 656 anchors; the tensor cores' fp32 sums of the exact bf16 products take the same scores to
-// within 2^-14 |x| (128 exact products, fp32 accumulation; the margin is 8 times the worst bound of
-// truncated accumulation), so only the anchors within 2 x 2^-14 |x| of a position's largest
-// score can be its nearest.  That leaves one anchor for about 99 % of positions; enc_finish decides the
-// rest in fp64.  The candidate word of a position: first candidate in bits 0-15, second in bits 16-31
-// (0xFFFF: none), or 0xFFFFFFFF: any anchor may be the nearest.
+// within 2^-15 |x| (128 exact products, fp32 accumulation; 4 times the worst bound of eight truncated
+// steps, the column bits below included), so only the anchors within 2 x 2^-15 |x| of a position's
+// largest score can be its nearest.  That leaves one anchor for about 99 % of positions; enc_finish and
+// enc_undecided decide the rest.  The candidate word of a position: first candidate in bits 0-15, second
+// in bits 16-31 (0xFFFF: none; the first again: the anchors of its group of 32), or 0xFFFFFFFF: any
+// anchor may be the nearest.
 //
 // One persistent CTA per SM takes items of 256 positions of one unit and side (two M = 128 tiles
 // that share every anchor chunk, which halves the L2 reads of the anchors), anchor chunks of 192.
 // Warp 8 copies (three position tiles and two anchor chunks in flight), warp 9 issues the
-// products (two accumulators of 192 TMEM columns), warps 0-3 and 4-7 are the two tiles' epilogues:
-// a thread owns one position, scales 32 columns at a time by 1 / |x_a|, takes the largest of
-// each eight and looks at single columns only where that comes within the margin of the running
-// maximum.  Waits are bounded; after a failure every remaining position gets the word that lets
+// products (two accumulators of 192 TMEM columns), warps 10 and 11 take the positions' norms one
+// item ahead, warps 0-3 and 4-7 are the two tiles' epilogues:
+// a thread owns one position and takes 32 columns at a time without branches on single columns (those
+// diverge: in the first chunks nearly every column is some lane's new maximum, and the kernel took
+// 293 us that way): scores with the column number in their lowest bits give the largest and its
+// column, and a clamped sum how many come near it.  Waits are bounded; after a failure every remaining position gets the word that lets
 // enc_finish decide it alone, so the result stays right.
 constexpr int kAtN = 192;
 constexpr int kAtA = 3, kAtB = 2;  // stages
 constexpr uint32_t kAtHalfA = 128 * 128, kAtHalfB = kAtN * 128;  // bytes of 64 of the 128 dimensions
-constexpr uint32_t kAtSmem = kAtA * 2 * kAtHalfA + kAtB * 2 * kAtHalfB + 1024;
-constexpr int kAtThreads = 320;
-constexpr float kAtMargin = 0x1p-13f;  // 2 x 2^-14, relative to |x|
+constexpr int kAtI = 4;  // chunks of inverse norms in flight
+constexpr uint32_t kAtSmem = kAtA * 2 * kAtHalfA + kAtB * 2 * kAtHalfB + kAtI * kAtN * 4 + 2 * 256 * 4 + 1024;
+constexpr int kAtThreads = 384;
+constexpr float kAtMargin = 0x1p-14f;  // 2 x 2^-15, relative to |x|
 
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+// a b + c clamped to [0, 1] (NaN: 0)
+__device__ __forceinline__ float fma_sat(float a, float b, float c) {
+  float r;
+  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+// 32 columns of the thread's TMEM lane: the load is started, and waited for through the registers it fills,
+// so that nothing can read them in between.
+__device__ __forceinline__ void tc_ld32_start(uint32_t taddr, float2 (&v)[16]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
-      "tcgen05.wait::ld.sync.aligned;\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[2].x), "=f"(v[2].y), "=f"(v[3].x), "=f"(v[3].y), "=f"(v[4].x), "=f"(v[4].y), "=f"(v[5].x), "=f"(v[5].y), "=f"(v[6].x), "=f"(v[6].y), "=f"(v[7].x), "=f"(v[7].y), "=f"(v[8].x), "=f"(v[8].y), "=f"(v[9].x), "=f"(v[9].y), "=f"(v[10].x), "=f"(v[10].y), "=f"(v[11].x), "=f"(v[11].y), "=f"(v[12].x), "=f"(v[12].y), "=f"(v[13].x), "=f"(v[13].y), "=f"(v[14].x), "=f"(v[14].y), "=f"(v[15].x), "=f"(v[15].y)
       : "r"(taddr)
       : "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tc_ld32_wait(float2 (&v)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+f"(v[0].x), "+f"(v[0].y), "+f"(v[1].x), "+f"(v[1].y), "+f"(v[2].x), "+f"(v[2].y), "+f"(v[3].x), "+f"(v[3].y), "+f"(v[4].x), "+f"(v[4].y), "+f"(v[5].x), "+f"(v[5].y), "+f"(v[6].x), "+f"(v[6].y), "+f"(v[7].x), "+f"(v[7].y), "+f"(v[8].x), "+f"(v[8].y), "+f"(v[9].x), "+f"(v[9].y), "+f"(v[10].x), "+f"(v[10].y), "+f"(v[11].x), "+f"(v[11].y), "+f"(v[12].x), "+f"(v[12].y), "+f"(v[13].x), "+f"(v[13].y), "+f"(v[14].x), "+f"(v[14].y), "+f"(v[15].x), "+f"(v[15].y)
+               :
+               : "memory");
 }
 
 __global__ void __launch_bounds__(kAtThreads, 1)
@@ -498,7 +523,7 @@ __global__ void __launch_bounds__(kAtThreads, 1)
                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmA, long long items,
                   int max_t) {
   extern __shared__ __align__(1024) uint8_t as_dyn[];
-  __shared__ __align__(8) uint64_t bars[2 * kAtA + 2 * kAtB + 4];
+  __shared__ __align__(8) uint64_t bars[2 * kAtA + 2 * kAtB + 8 + kAtI];
   __shared__ uint32_t tmem_sh;
   __shared__ int failed_sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -509,10 +534,21 @@ __global__ void __launch_bounds__(kAtThreads, 1)
   auto b_free = [&](int s) { return smem_u32(bars + 2 * kAtA + kAtB + s); };
   auto acc_full = [&](int m) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + m); };
   auto acc_empty = [&](int m) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + 2 + m); };
+  auto nrm_full = [&](int b) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + 4 + b); };
+  auto nrm_free = [&](int b) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + 6 + b); };
+  auto inv_free = [&](int s) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + 8 + s); };
+  const uint32_t sI = sB + kAtB * 2 * kAtHalfB;
+  float* inv_sm = reinterpret_cast<float*>(as_dyn + (sI - smem_u32(as_dyn)));  // [kAtI][kAtN]
+  float* nrm_sm = inv_sm + kAtI * kAtN;                                        // [2][256] squared norms
   volatile int* failed = &failed_sh;
   if (tid == 0) {
     for (int i = 0; i < 2 * kAtA + 2 * kAtB + 2; ++i) mbar_init(smem_u32(bars + i), 1);
-    for (int m = 0; m < 2; ++m) mbar_init(acc_empty(m), 4);  // one arrival per epilogue warp
+    for (int m = 0; m < 2; ++m) {
+      mbar_init(acc_empty(m), 4);  // one arrival per epilogue warp
+      mbar_init(nrm_full(m), 2);   // per norm warp
+      mbar_init(nrm_free(m), 8);   // per epilogue warp
+    }
+    for (int s = 0; s < kAtI; ++s) mbar_init(inv_free(s), 8);
     *failed = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -558,15 +594,20 @@ __global__ void __launch_bounds__(kAtThreads, 1)
       Item it;
       for (long long i = blockIdx.x; ok && next_item(i, it); i += gridDim.x) {
         const akv_unit_desc* d = unit_desc(A, it.u);
+        const EncUnitWs w = unit_ws(A, it.u, d);
+        const float* inv = it.side ? w.inv[1] : w.inv[0];
         const int row0 = (int)((it.side ? d->off_anchor_v : d->off_anchor_k) >> 8);
         ok = load_a(it, 0);
         for (int c0 = 0; ok && c0 < it.k; c0 += kAtN) {
           const int s = nb % kAtB, nr = (min(kAtN, it.k - c0) + 63) / 64;  // boxes of 64 anchor rows
-          if (*failed || !mbar_wait(b_free(s), (uint32_t)((nb / kAtB) & 1) ^ 1u)) {
+          if (*failed || !mbar_wait(b_free(s), (uint32_t)((nb / kAtB) & 1) ^ 1u) ||
+              !mbar_wait(inv_free(nb % kAtI), (uint32_t)((nb / kAtI) & 1) ^ 1u)) {
             ok = false;
             break;
           }
-          mbar_expect_tx(b_full(s), (uint32_t)nr * 2 * 64 * 128);
+          const uint32_t ib = (uint32_t)min(kAtN, (it.k - c0 + 31) & ~31) * 4u;
+          mbar_expect_tx(b_full(s), (uint32_t)nr * 2 * 64 * 128 + ib);
+          bulk_g2s(sI + (uint32_t)(nb % kAtI) * kAtN * 4u, inv + c0, ib, b_full(s));
           for (int r = 0; r < nr; ++r) {
             tma_load_2d(sB + s * 2 * kAtHalfB + r * 64 * 128, &tmA, 0, row0 + c0 + 64 * r, b_full(s));
             tma_load_2d(sB + s * 2 * kAtHalfB + kAtHalfB + r * 64 * 128, &tmA, 64, row0 + c0 + 64 * r, b_full(s));
@@ -620,89 +661,127 @@ __global__ void __launch_bounds__(kAtThreads, 1)
         if (nacc[m] > 0) mbar_wait(acc_full(m), (uint32_t)(nacc[m] - 1) & 1u);
     }
     __syncwarp();
-  } else {  // ---- epilogue of tile m
-    const int m = warp >> 2, q = warp & 3;
-    int nacc = 0;
-    bool ok = true;
+  } else if (warp >= 10) {  // ---- squared norms of the item's 256 positions, four per thread
+    int j = 0;
     Item it;
-    for (long long i = blockIdx.x; next_item(i, it); i += gridDim.x) {
-      if (m >= n_tiles(it)) continue;
-      const int p = it.t * 256 + 128 * m + 32 * q + lane;
-      const EncUnitWs w = unit_ws(A, it.u, unit_desc(A, it.u));
-      const float* inv = w.inv[it.side];
-      float nx2 = 0.f;
-      if (p < it.S) {
-        const uint4* X = reinterpret_cast<const uint4*>((it.side ? A.V : A.K) + ((size_t)it.u * A.s_max + p) * 128);
+    for (long long i = blockIdx.x; next_item(i, it); i += gridDim.x, ++j) {
+      const int t = tid - 320, b = j & 1;
+      const uint4* X = reinterpret_cast<const uint4*>((it.side ? A.V : A.K) + ((size_t)it.u * A.s_max + it.t * 256) * 128);
+      float nx2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        if (it.t * 256 + t + 64 * h >= it.S) continue;
 #pragma unroll
         for (int c = 0; c < 16; ++c) {
-          const uint4 v = __ldg(X + c);
+          const uint4 v = __ldg(X + (size_t)(t + 64 * h) * 16 + c);
           const uint32_t wd[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
-            nx2 = __fmaf_rn(bf_lo(wd[e]), bf_lo(wd[e]), nx2);
-            nx2 = __fmaf_rn(bf_hi(wd[e]), bf_hi(wd[e]), nx2);
+            nx2[h] = __fmaf_rn(bf_lo(wd[e]), bf_lo(wd[e]), nx2[h]);
+            nx2[h] = __fmaf_rn(bf_hi(wd[e]), bf_hi(wd[e]), nx2[h]);
           }
         }
       }
+      __syncwarp();
+      if (__shfl_sync(0xffffffffu, *failed, 0) != 0 || !mbar_wait_w(nrm_free(b), (uint32_t)((j >> 1) & 1) ^ 1u)) {
+        *failed = 1;
+        break;
+      }
+#pragma unroll
+      for (int h = 0; h < 4; ++h) nrm_sm[256 * b + 64 * h + t] = nx2[h];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(nrm_full(b));
+    }
+  } else {  // ---- epilogue of tile m
+    const int m = warp >> 2, q = warp & 3;
+    int nacc = 0, ni = 0, nc = 0;  // accumulators, items and anchor chunks so far
+    bool ok = true;
+    Item it;
+    for (long long i = blockIdx.x; next_item(i, it); i += gridDim.x, ++ni) {
+      const int p = it.t * 256 + 128 * m + 32 * q + lane;
+      const EncUnitWs w = unit_ws(A, it.u, unit_desc(A, it.u));
+      __syncwarp();
+      ok = ok && __shfl_sync(0xffffffffu, *failed, 0) == 0 && mbar_wait_w(nrm_full(ni & 1), (uint32_t)(ni >> 1) & 1u);
+      const float nx2 = ok ? nrm_sm[256 * (ni & 1) + 128 * m + 32 * q + lane] : 0.f;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(nrm_free(ni & 1));
+      if (m >= n_tiles(it)) {  // no positions of this tile: its chunks pass by
+        for (int c0 = 0; c0 < it.k; c0 += kAtN, ++nc) {
+          if (ok && nc >= kAtI) ok = mbar_wait_w(inv_free(nc % kAtI), (uint32_t)(nc / kAtI - 1) & 1u);
+          if (lane == 0) mbar_arrive(inv_free(nc % kAtI));
+        }
+        continue;
+      }
       const bool usable = nx2 >= (float)kNormLo && nx2 <= (float)kNormHi && w.ctrl[4 + it.side] == 0u;
       const float marg = kAtMargin * 1.001f * __fsqrt_rn(nx2);
-      float m1 = 0.f, thr = 0.f;  // the largest score so far; what a candidate must exceed
-      int i1 = 0xFFFF, i2 = 0xFFFF, cnt = 0;
-      for (int c0 = 0; c0 < it.k; c0 += kAtN) {
+      const float rm = 1.f / marg;  // (an unusable row may give anything here: its word is not used)
+      float m1 = 0.f;               // the largest score so far
+      uint32_t i1 = 0xFFFFu, i2 = 0xFFFFu;  // its anchor; a second one within the margin, or i1: its group
+      bool more = false;                    // candidates beyond these
+      // 32 columns at a time: scores with the column in the five lowest bits (2^-18 relative), their
+      // largest, and how many lie within the margin of it (s / margin, shifted so that 1 is reached
+      // there, clamped to [0, 1])
+      auto step = [&](const float2 (&s)[16], const float* iv, uint32_t a0) {
+        float v[32];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const float4 f = *reinterpret_cast<const float4*>(iv + 4 * e);
+          const float2 x = __fmul2_rn(s[2 * e], make_float2(f.x, f.y)), y = __fmul2_rn(s[2 * e + 1], make_float2(f.z, f.w));
+          v[4 * e] = __uint_as_float((__float_as_uint(x.x) & 0x7FFFFFE0u) | (uint32_t)(4 * e));
+          v[4 * e + 1] = __uint_as_float((__float_as_uint(x.y) & 0x7FFFFFE0u) | (uint32_t)(4 * e + 1));
+          v[4 * e + 2] = __uint_as_float((__float_as_uint(y.x) & 0x7FFFFFE0u) | (uint32_t)(4 * e + 2));
+          v[4 * e + 3] = __uint_as_float((__float_as_uint(y.y) & 0x7FFFFFE0u) | (uint32_t)(4 * e + 3));
+        }
+        float mx[11];
+#pragma unroll
+        for (int e = 0; e < 10; ++e) mx[e] = max3(v[3 * e], v[3 * e + 1], v[3 * e + 2]);
+        mx[10] = fmaxf(v[30], v[31]);
+        const float c1 = max3(max3(max3(mx[0], mx[1], mx[2]), max3(mx[3], mx[4], mx[5]), max3(mx[6], mx[7], mx[8])), mx[9], mx[10]);
+        const float top = fmaxf(m1, c1), off = __fmaf_rn(-top, rm, 2.f);
+        float2 near2[4] = {};
+#pragma unroll
+        for (int e = 0; e < 32; e += 2)
+          near2[(e / 2) & 3] = __fadd2_rn(near2[(e / 2) & 3], make_float2(fma_sat(v[e], rm, off), fma_sat(v[e + 1], rm, off)));
+        const float2 nr = __fadd2_rn(__fadd2_rn(near2[0], near2[1]), __fadd2_rn(near2[2], near2[3]));
+        const bool several = nr.x + nr.y > 1.004f;
+        const bool here = c1 >= m1 - marg, alone = c1 > m1 + marg;  // alone: nothing before comes near
+        const uint32_t idx = a0 + (__float_as_uint(c1) & 31u);
+        more = here ? !alone && (more || several || i2 != 0xFFFFu) : more;
+        i2 = here ? (alone ? (several ? idx : 0xFFFFu) : idx) : i2;
+        i1 = alone ? idx : i1;
+        m1 = top;
+      };
+      for (int c0 = 0; c0 < it.k; c0 += kAtN, ++nc) {
         __syncwarp();
         ok = ok && __shfl_sync(0xffffffffu, *failed, 0) == 0 && mbar_wait_w(acc_full(m), (uint32_t)nacc & 1u);
         if (!ok) break;  // (the same for the whole warp)
         ++nacc;
         tc_fence_after();
         const int n = min(kAtN, it.k - c0);
-        for (int sc = 0; sc < n; sc += 32) {
-          float s[32];
+        const uint32_t tcol = tmem + ((uint32_t)(32 * q) << 16) + 256u * (uint32_t)m;
+        const float* iv = inv_sm + (nc % kAtI) * kAtN;
+        auto done = [&]() {  // the tile's last read of the accumulator has come back
+          tc_fence_before();
           __syncwarp();
-          tc_ld32(tmem + ((uint32_t)(32 * q) << 16) + 256u * (uint32_t)m + (uint32_t)sc, s);
-          if (sc + 32 >= n) {  // the tile's last read of the accumulator
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty(m));
-          }
-          const float4* iv = reinterpret_cast<const float4*>(inv + c0 + sc);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const float4 f = __ldg(iv + e);
-            s[4 * e] = fabsf(s[4 * e]) * f.x;
-            s[4 * e + 1] = fabsf(s[4 * e + 1]) * f.y;
-            s[4 * e + 2] = fabsf(s[4 * e + 2]) * f.z;
-            s[4 * e + 3] = fabsf(s[4 * e + 3]) * f.w;
-          }
-#pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            const float* t = s + 8 * g;
-            const float mx = fmaxf(fmaxf(fmaxf(t[0], t[1]), fmaxf(t[2], t[3])), fmaxf(fmaxf(t[4], t[5]), fmaxf(t[6], t[7])));
-            if (mx > thr) {  // (NaN: no candidate)
-#pragma unroll
-              for (int e = 0; e < 8; ++e) {
-                if (t[e] > thr) {
-                  const int a = c0 + sc + 8 * g + e;
-                  if (t[e] > m1 + marg) {
-                    i1 = a;
-                    cnt = 1;
-                  } else {
-                    if (cnt == 0) i1 = a;
-                    else i2 = a;
-                    ++cnt;
-                  }
-                  m1 = fmaxf(m1, t[e]);
-                  thr = fmaxf(m1 - marg, 0.f);
-                }
-              }
-            }
-          }
+          if (lane == 0) mbar_arrive(acc_empty(m));
+        };
+        float2 sa[16], sb[16];
+        tc_ld32_start(tcol, sa);
+        for (int sc = 0; sc < n; sc += 64) {
+          tc_ld32_wait(sa);
+          if (sc + 32 < n) tc_ld32_start(tcol + (uint32_t)(sc + 32), sb);
+          else done();
+          step(sa, iv + sc, (uint32_t)(c0 + sc));
+          if (sc + 32 >= n) break;
+          tc_ld32_wait(sb);
+          if (sc + 64 < n) tc_ld32_start(tcol + (uint32_t)(sc + 64), sa);
+          else done();
+          step(sb, iv + sc + 32, (uint32_t)(c0 + sc + 32));
         }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(inv_free(nc % kAtI));
       }
-      if (p < it.S) {
-        const bool one = cnt == 1, two = cnt == 2;
-        const uint32_t word = (uint32_t)i1 | ((one ? 0xFFFFu : (uint32_t)i2) << 16);
-        w.st[it.side][p] = ok && usable && m1 > marg && (one || two) ? word : 0xFFFFFFFFu;
-      }
+      if (p < it.S) (it.side ? w.st[1] : w.st[0])[p] = ok && usable && m1 > marg && !more ? i1 | (i2 << 16) : 0xFFFFFFFFu;
     }
     if (!ok) *failed = 1;
   }
@@ -716,13 +795,21 @@ __global__ void __launch_bounds__(kAtThreads, 1)
 // step rounds once, like a separate add).
 __device__ double exact_dot(const uint4* x, const uint4* row, int a) {
   double s = 0.0;
-  for (int c = 0; c < 16; ++c) {
-    const uint4 xv = __ldg(x + c), av = __ldg(row + (c ^ (a & 7)));
-    const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w}, aw[4] = {av.x, av.y, av.z, av.w};
+  for (int c0 = 0; c0 < 16; c0 += 8) {
+    uint4 xv[8], av[8];  // (loads in flight together)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      s = __fma_rn((double)bf_lo(xw[e]), (double)bf_lo(aw[e]), s);
-      s = __fma_rn((double)bf_hi(xw[e]), (double)bf_hi(aw[e]), s);
+    for (int c = 0; c < 8; ++c) {
+      xv[c] = __ldg(x + c0 + c);
+      av[c] = __ldg(row + ((c0 + c) ^ (a & 7)));
+    }
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const uint32_t xw[4] = {xv[c].x, xv[c].y, xv[c].z, xv[c].w}, aw[4] = {av[c].x, av[c].y, av[c].z, av[c].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        s = __fma_rn(bf_f64(xw[e] << 16), bf_f64(aw[e] << 16), s);
+        s = __fma_rn(bf_f64(xw[e] & 0xFFFF0000u), bf_f64(aw[e] & 0xFFFF0000u), s);
+      }
     }
   }
   return s;
@@ -754,10 +841,10 @@ __device__ uint64_t exact_energy_key(const uint4* x, const uint4* row, uint32_t 
     const uint4 xv = __ldg(x + c), av = __ldg(row + (c ^ (a & 7)));
     const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w}, aw[4] = {av.x, av.y, av.z, av.w};
     for (int h = 0; h < 8; ++h) {
-      const float xe = (h & 1) ? bf_hi(xw[h >> 1]) : bf_lo(xw[h >> 1]);
-      const float ae = (h & 1) ? bf_hi(aw[h >> 1]) : bf_lo(aw[h >> 1]);
-      const double pj = valid ? __dmul_rn(g, (double)ae) : 0.0;
-      const double r = __dsub_rn((double)xe, pj);
+      const uint32_t xe = (h & 1) ? xw[h >> 1] & 0xFFFF0000u : xw[h >> 1] << 16;
+      const uint32_t ae = (h & 1) ? aw[h >> 1] & 0xFFFF0000u : aw[h >> 1] << 16;
+      const double pj = valid ? __dmul_rn(g, bf_f64(ae)) : 0.0;
+      const double r = __dsub_rn(bf_f64(xe), pj);
       e = __dadd_rn(e, __dmul_rn(r, r));
     }
   }
@@ -773,50 +860,67 @@ __device__ __forceinline__ uint32_t energy_key(float e, const uint4* x, const ui
   return __float_as_uint(e) + 1u;
 }
 
+// s + c += p with the rounding error kept in c (Knuth's two-sum): the sum of exact products in twice
+// the precision of fp32.
+__device__ __forceinline__ void two_sum_add(float& s, float& c, float p) {
+  const float t = s + p, z = t - s;
+  c += (s - (t - z)) + (p - z);
+  s = t;
+}
+
+// gamma's fp16 bits where the fp32 quotient gq is within ge of one rounding boundary, the one between
+// the neighbours gh and gh2 (at or below gq - ge and gq + ge): x . x_a = s + c against the boundary times
+// |x_a|^2, both in twice the precision of fp32; false if even that does not decide.
+__device__ bool gamma_at_edge(float s, float c, float ab, double n2, uint32_t gh2, uint32_t& gh) {
+  const float nh = (float)n2, nl = (float)(n2 - (double)nh);
+  const float mid = 0.5f * (__half2float(__ushort_as_half((unsigned short)gh)) + __half2float(__ushort_as_half((unsigned short)gh2)));
+  const float pm = mid * nh, pe = __fmaf_rn(mid, nl, __fmaf_rn(mid, nh, -pm));
+  const float diff = (s - pm) + (c - pe);
+  // (errors of the sum, the product and the fp64 result that this stands for: below 2^-37 of each)
+  if (!(fabsf(diff) > (ab + fabsf(pm)) * 0x1p-35f)) return false;
+  if (diff > 0.f) gh = gh2;
+  return true;
+}
+
 // Eq. 1 decided and Eq. 2: gamma = fp16(x . x_a / |x_a|^2), and the residual energy of every
-// position.  Eight lanes take a position (16 dimensions each).  With one candidate anchor, x . x_a in
-// fp32 fixes gamma's fp16 rounding unless the quotient lies within its error (2^-19 sum |x x_a| /
-// |x_a|^2) of a rounding boundary; those positions, and the ones with two candidates, go to a list
-// that the block's threads finish with fp64 chains, one position each; positions where any anchor may be
-// the nearest take a warp each.  fp64 work for every position would bound this kernel (the energies
-// alone are 335 M operations, 0.55 ms at 0.6 T/s, for 2 x 8 x 32768 positions).
+// position.  Eight lanes take a position (16 dimensions each).  Two candidate anchors are told apart by
+// their scores in fp32 unless those lie within their error (24 roundings of sum |x x_a|).  x . x_a in
+// fp32 fixes gamma's fp16 rounding unless the quotient comes within its error of a rounding boundary;
+// there the products are summed again in twice the precision and compared with the boundary times
+// |x_a|^2.  What even that leaves (equal scores of duplicate anchors, mostly) and the positions with more
+// candidates go to the unit's lists, which enc_undecided finishes in fp64.  fp64 for every position
+// would be 335 M operations for the energies alone, 0.55 ms for 2 x 8 x 32768 positions, and a few fp64
+// chains in every block (271 us for the kernel) cost as much as full warps of them.
 constexpr int kFinPos = 256;  // positions per block
 __global__ void __launch_bounds__(256) enc_finish(const EncArgs A) {
   __shared__ int todo[kFinPos], full[kFinPos];
-  __shared__ int n_todo, n_full;
-  __shared__ __align__(16) float xs[8][128];
+  __shared__ int n_todo, n_full, at_todo, at_full;
   const int u = blockIdx.y, side = blockIdx.z;
   const akv_unit_desc* d = unit_desc(A, u);
-  const int S = d->len, k = d->n_anchors, p0 = blockIdx.x * kFinPos;
+  const int S = d->len, p0 = blockIdx.x * kFinPos;
   if (p0 >= S) return;
   const EncUnitWs w = unit_ws(A, u, d);
   const uint4* X = reinterpret_cast<const uint4*>((side ? A.V : A.K) + (size_t)u * A.s_max * 128);
   const uint4* AR = reinterpret_cast<const uint4*>(A.arena_c + (side ? d->off_anchor_v : d->off_anchor_k));
   uint32_t* stream = w.st[side];
+  const float* inv = w.inv[side];
   const double* n2 = w.n2[side];
   uint32_t* key = reinterpret_cast<uint32_t*>(side ? w.key1 : w.key0);
   uint32_t* inexact = &w.ctrl[6 + side];
   const bool want_e = A.m_obs == 0;  // (the full selection ranks by its own utilities)
-  const int tid = threadIdx.x, sub = tid & 7, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, sub = tid & 7;
   if (tid == 0) n_todo = n_full = 0;
   __syncthreads();
-  for (int q = tid >> 3; q < kFinPos; q += 32) {
-    const int p = p0 + q;
-    const bool in = p < S;
-    const int sl = in ? w.slot_of[p] : 0;
-    const uint32_t word = in ? stream[p] : 0u;
-    const int a = (int)(word & 0xFFFFu);
-    const bool one = in && sl < 0 && (word >> 16) == 0xFFFFu && a != 0xFFFF;
-    uint32_t xw[8] = {}, aw[8] = {};
-    if (one) {
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const uint4 xv = __ldg(X + (size_t)p * 16 + 2 * sub + c), av = __ldg(AR + (size_t)a * 16 + ((2 * sub + c) ^ (a & 7)));
-        xw[4 * c] = xv.x; xw[4 * c + 1] = xv.y; xw[4 * c + 2] = xv.z; xw[4 * c + 3] = xv.w;
-        aw[4 * c] = av.x; aw[4 * c + 1] = av.y; aw[4 * c + 2] = av.z; aw[4 * c + 3] = av.w;
-      }
-    }
-    float dd = 0.f, ab = 0.f;
+  auto load16 = [](const uint4* lo, const uint4* hi, uint32_t (&o)[8]) {
+    const uint4 v = __ldg(lo), t = __ldg(hi);
+    o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
+    o[4] = t.x; o[5] = t.y; o[6] = t.z; o[7] = t.w;
+  };
+  auto load_anchor = [&](int a, uint32_t (&o)[8]) {
+    load16(AR + (size_t)a * 16 + ((2 * sub) ^ (a & 7)), AR + (size_t)a * 16 + ((2 * sub + 1) ^ (a & 7)), o);
+  };
+  auto dot = [](const uint32_t (&xw)[8], const uint32_t (&aw)[8], float& dd, float& ab) {  // and sum |x x_a|
+    dd = ab = 0.f;
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
       dd = __fmaf_rn(bf_lo(xw[c]), bf_lo(aw[c]), dd);
@@ -829,10 +933,69 @@ __global__ void __launch_bounds__(256) enc_finish(const EncArgs A) {
       dd += __shfl_xor_sync(0xffffffffu, dd, o);
       ab += __shfl_xor_sync(0xffffffffu, ab, o);
     }
-    const float nf = one ? (float)n2[a] : 1.f;
-    const float gq = __fdiv_rn(dd, nf), ge = __fdiv_rn(ab, nf) * 0x1p-19f;
-    const uint32_t gh = f32_to_fp16_bits(gq - ge);
-    const bool fixed = one && ab >= 0x1p-80f && ab <= 0x1p100f && gh == f32_to_fp16_bits(gq + ge);
+  };
+  for (int q = tid >> 3; q < kFinPos; q += 32) {
+    const int p = p0 + q;
+    const bool in = p < S;
+    const int sl = in ? w.slot_of[p] : 0;
+    const uint32_t word = in ? stream[p] : 0u;
+    int a = (int)(word & 0xFFFFu);
+    const int a2 = (int)(word >> 16);
+    const bool some = in && sl < 0, lone = some && a2 != a;  // lone: one candidate, or two
+    bool one = lone && a2 == 0xFFFF;
+    uint32_t xw[8] = {}, aw[8] = {};
+    if (lone) {
+      load16(X + (size_t)p * 16 + 2 * sub, X + (size_t)p * 16 + 2 * sub + 1, xw);
+      load_anchor(a, aw);
+    }
+    float iv = lone ? inv[a] : 0.f;
+    float dd, ab;
+    dot(xw, aw, dd, ab);
+    const bool two = lone && a2 != 0xFFFF;
+    if (__any_sync(0xffffffffu, two)) {
+      uint32_t bw[8] = {};
+      if (two) load_anchor(a2, bw);
+      const float iv2 = two ? inv[a2] : 0.f;
+      float dd2, ab2;
+      dot(xw, bw, dd2, ab2);
+      // 19 roundings in a sum, two in its score
+      const float gap = fabsf(dd) * iv - fabsf(dd2) * iv2, tol = (ab * iv + ab2 * iv2) * 0x1p-19f;
+      if (two) {
+        one = fabsf(gap) > tol;
+        if (gap < 0.f) {
+          a = a2;
+          dd = dd2;
+          ab = ab2;
+          iv = iv2;
+#pragma unroll
+          for (int c = 0; c < 8; ++c) aw[c] = bw[c];
+        }
+      }
+    }
+    // gamma: 1 / |x_a|^2 from the inverse norm (dd 19 roundings, the quotient 5 more)
+    const float i2 = iv * iv, gq = dd * i2, ge = ab * i2 * 0x1p-19f;
+    uint32_t gh = f32_to_fp16_bits(gq - ge);
+    const uint32_t gh2 = f32_to_fp16_bits(gq + ge);
+    one = one && ab >= 0x1p-80f && ab <= 0x1p100f;
+    bool fixed = one && gh == gh2;
+    const bool edge = one && !fixed && (gq < 0.f ? gh == gh2 + 1u : gh2 == gh + 1u);  // one boundary in reach
+    if (__any_sync(0xffffffffu, edge)) {
+      float hs = 0.f, hc = 0.f;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        two_sum_add(hs, hc, bf_lo(xw[c]) * bf_lo(aw[c]));  // (16-bit products: exact)
+        two_sum_add(hs, hc, bf_hi(xw[c]) * bf_hi(aw[c]));
+      }
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) {
+        const float os = __shfl_xor_sync(0xffffffffu, hs, o), oc = __shfl_xor_sync(0xffffffffu, hc, o);
+        two_sum_add(hs, hc, os);
+        hc += oc;
+      }
+      if (edge) {
+        fixed = gamma_at_edge(hs, hc, ab, n2[a], gh2, gh);
+      }
+    }
     const float g = __half2float(__ushort_as_half((unsigned short)gh));
     float e = 0.f;
 #pragma unroll
@@ -850,7 +1013,7 @@ __global__ void __launch_bounds__(256) enc_finish(const EncArgs A) {
       } else if (fixed) {
         stream[p] = (uint32_t)a | (gh << 16);
         if (want_e) key[p] = energy_key(e, X + (size_t)p * 16, AR + (size_t)a * 16, a, g, inexact);
-      } else if (word == 0xFFFFFFFFu) {
+      } else if (!lone) {
         full[atomicAdd(&n_full, 1)] = p;
       } else {
         todo[atomicAdd(&n_todo, 1)] = p;
@@ -858,14 +1021,78 @@ __global__ void __launch_bounds__(256) enc_finish(const EncArgs A) {
     }
   }
   __syncthreads();
-  auto finish = [&](int p, int a, double dot) {  // the position's nearest anchor a (-1: none) is known
-    const uint32_t gh = a >= 0 ? f64_to_fp16_bits(__ddiv_rn(dot, n2[a])) : 0u;
+  // the lists lie behind the energies: undecided positions from the front, the others from the back
+  int* list = reinterpret_cast<int*>(key + S);
+  if (tid == 0) {
+    at_todo = n_todo ? (int)atomicAdd(&w.ctrl[8 + side], (uint32_t)n_todo) : 0;
+    at_full = n_full ? (int)atomicAdd(&w.ctrl[10 + side], (uint32_t)n_full) : 0;
+  }
+  __syncthreads();
+  for (int i = tid; i < n_todo; i += 256) list[at_todo + i] = todo[i];
+  for (int i = tid; i < n_full; i += 256) list[S - 1 - (at_full + i)] = full[i];
+}
+
+// x . x_a by one thread in twice the precision of fp32 (s + c, within 2^-38 sum |x x_a|), and that sum.
+__device__ void paired_dot(const uint4* x, const uint4* row, int a, float& s, float& c, float& ab) {
+  s = c = ab = 0.f;
+  for (int c0 = 0; c0 < 16; c0 += 8) {
+    uint4 xv[8], av[8];  // (loads in flight together)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      xv[i] = __ldg(x + c0 + i);
+      av[i] = __ldg(row + ((c0 + i) ^ (a & 7)));
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t xw[4] = {xv[i].x, xv[i].y, xv[i].z, xv[i].w}, aw[4] = {av[i].x, av[i].y, av[i].z, av[i].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float p0 = bf_lo(xw[e]) * bf_lo(aw[e]), p1 = bf_hi(xw[e]) * bf_hi(aw[e]);  // (exact)
+        two_sum_add(s, c, p0);
+        two_sum_add(s, c, p1);
+        ab += fabsf(p0) + fabsf(p1);
+      }
+    }
+  }
+}
+
+// The positions that enc_finish left.  First list: one or two candidate anchors, a thread each; second list: any
+// anchor of a group of 32, or any at all, a block each.  Scores are told apart in fp32, then in twice its
+// precision (as squares: dot^2 |other|^2), duplicates by their bytes; fp64 chains run only for what is
+// left, since one of 128 steps takes about 10 us here.
+constexpr int kUndFirst = 8, kUndBlocks = 72, kUndThreads = 128;  // blocks of the first list; blocks per unit and side
+__global__ void __launch_bounds__(kUndThreads) enc_undecided(const EncArgs A) {
+  __shared__ __align__(16) float xs[128];
+  __shared__ float red[kUndThreads / 32];
+  __shared__ int lowest;
+  __shared__ double bcs[kUndThreads], bds[kUndThreads];
+  __shared__ int bas[kUndThreads];
+  const int u = blockIdx.y, side = blockIdx.z;
+  const akv_unit_desc* d = unit_desc(A, u);
+  const int S = d->len, k = d->n_anchors;
+  const EncUnitWs w = unit_ws(A, u, d);
+  const int n_todo = (int)w.ctrl[8 + side], n_full = (int)w.ctrl[10 + side];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const bool second = blockIdx.x >= kUndFirst;
+  if (second ? n_full <= (int)blockIdx.x - kUndFirst : n_todo <= (int)blockIdx.x * kUndThreads) return;
+  const uint4* X = reinterpret_cast<const uint4*>((side ? A.V : A.K) + (size_t)u * A.s_max * 128);
+  const uint4* AR = reinterpret_cast<const uint4*>(A.arena_c + (side ? d->off_anchor_v : d->off_anchor_k));
+  uint32_t* stream = w.st[side];
+  const double* n2 = w.n2[side];
+  const float* inv = w.inv[side];
+  uint32_t* key = reinterpret_cast<uint32_t*>(side ? w.key1 : w.key0);
+  const int* list = reinterpret_cast<const int*>(key + S);
+  uint32_t* inexact = &w.ctrl[6 + side];
+  const bool want_e = A.m_obs == 0;
+
+  auto store = [&](int p, int a, uint32_t gh) {  // nearest anchor a (-1: none) and gamma are known
     const int as = a >= 0 ? a : 0;
     stream[p] = (uint32_t)as | (gh << 16);
     if (!want_e) return;
     const float g = a >= 0 ? __half2float(__ushort_as_half((unsigned short)gh)) : 0.f;
     const uint4 *x = X + (size_t)p * 16, *row = AR + (size_t)as * 16;
     float e = 0.f;
+#pragma unroll 4
     for (int c = 0; c < 16; ++c) {
       const uint4 xv = __ldg(x + c), av = __ldg(row + (c ^ (as & 7)));
       const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w}, aw[4] = {av.x, av.y, av.z, av.w};
@@ -881,90 +1108,183 @@ __global__ void __launch_bounds__(256) enc_finish(const EncArgs A) {
     }
     key[p] = energy_key(e, x, row, as, g, inexact);
   };
-  if (tid < n_todo) {
-    const int p = todo[tid];
-    const uint32_t word = stream[p];
-    const int a1 = (int)(word & 0xFFFFu), a2 = (int)(word >> 16);
-    int a = a1;
-    double dot = exact_dot(X + (size_t)p * 16, AR + (size_t)a1 * 16, a1);
-    if (a2 != 0xFFFF) {
-      const double dot2 = exact_dot(X + (size_t)p * 16, AR + (size_t)a2 * 16, a2);
-      const double c1 = __ddiv_rn(fabs(dot), __dsqrt_rn(n2[a1])), c2 = __ddiv_rn(fabs(dot2), __dsqrt_rn(n2[a2]));
-      if (c2 > c1 || (c2 == c1 && a2 < a1)) {
-        a = a2;
-        dot = dot2;
+  auto finish = [&](int p, int a, double dot) { store(p, a, a >= 0 ? f64_to_fp16_bits(__ddiv_rn(dot, n2[a])) : 0u); };
+  auto in_range = [](float ab) { return ab >= 0x1p-80f && ab <= 0x1p100f; };
+  // gamma and energy for nearest anchor a, x . x_a = hs + hc
+  auto settle = [&](int p, int a, float hs, float hc, float ab) {
+    const float iv = inv[a], i2 = iv * iv, gq = (hs + hc) * i2, ge = fabsf(gq) * 0x1p-20f + ab * i2 * 0x1p-36f;
+    uint32_t gh = f32_to_fp16_bits(gq - ge);
+    const uint32_t gh2 = f32_to_fp16_bits(gq + ge);
+    bool fixed = in_range(ab) && iv > 0.f;
+    if (fixed && gh != gh2) fixed = (gq < 0.f ? gh == gh2 + 1u : gh2 == gh + 1u) && gamma_at_edge(hs, hc, ab, n2[a], gh2, gh);
+    if (fixed) store(p, a, gh);
+    else finish(p, a, exact_dot(X + (size_t)p * 16, AR + (size_t)a * 16, a));
+  };
+  auto same_rows = [&](int a, int b) {
+    bool same = true;
+    for (int c = 0; c < 16; ++c) {
+      const uint4 v = __ldg(AR + (size_t)a * 16 + (c ^ (a & 7))), o = __ldg(AR + (size_t)b * 16 + (c ^ (b & 7)));
+      same = same && v.x == o.x && v.y == o.y && v.z == o.z && v.w == o.w;
+    }
+    return same;
+  };
+  if (!second) {
+    for (int t = blockIdx.x * kUndThreads + tid; t < n_todo; t += kUndFirst * kUndThreads) {
+      const int p = list[t];
+      const uint32_t word = stream[p];
+      const int a1 = (int)(word & 0xFFFFu), a2 = (int)(word >> 16);
+      const uint4* x = X + (size_t)p * 16;
+      float s1, c1, ab1;
+      paired_dot(x, AR + (size_t)a1 * 16, a1, s1, c1, ab1);
+      if (a2 == 0xFFFF) {
+        settle(p, a1, s1, c1, ab1);
+        continue;
       }
+      float s2, c2, ab2;
+      paired_dot(x, AR + (size_t)a2 * 16, a2, s2, c2, ab2);
+      const double d1 = (double)s1 + (double)c1, d2 = (double)s2 + (double)c2;
+      const double q1 = d1 * d1 * n2[a2], q2 = d2 * d2 * n2[a1];
+      // squares off by 2^-37 (|x||x_a|)^2 |other|^2 each; scores are above 2^-14 |x|, so 2^-9 of that is left
+      const bool told = in_range(ab1) && in_range(ab2) && fabs(q1 - q2) > 0x1p-34 * (fabs(d1) * (double)ab1 * n2[a2] + fabs(d2) * (double)ab2 * n2[a1]);
+      if (told || same_rows(a1, a2)) {
+        const bool first = told ? q1 > q2 : a1 < a2;
+        settle(p, first ? a1 : a2, first ? s1 : s2, first ? c1 : c2, first ? ab1 : ab2);
+        continue;
+      }
+      const double e1 = exact_dot(x, AR + (size_t)a1 * 16, a1), e2 = exact_dot(x, AR + (size_t)a2 * 16, a2);
+      const double r1 = __ddiv_rn(fabs(e1), __dsqrt_rn(n2[a1])), r2 = __ddiv_rn(fabs(e2), __dsqrt_rn(n2[a2]));
+      const bool first = r1 > r2 || (r1 == r2 && a1 < a2);
+      finish(p, first ? a1 : a2, first ? e1 : e2);
     }
-    finish(p, a, dot);
+    return;
   }
-  for (int t = warp; t < n_full; t += 8) {  // any anchor: a lane takes every 32nd one
-    const int p = full[t];
+  for (int t = (int)blockIdx.x - kUndFirst; t < n_full; t += kUndBlocks - kUndFirst) {
+    const int p = list[S - 1 - t];
+    const uint32_t word = stream[p];
+    const int a_lo = word == 0xFFFFFFFFu ? 0 : (int)(word & 0xFFE0u), a_hi = word == 0xFFFFFFFFu ? k : min(k, a_lo + 32);
     const uint4* x = X + (size_t)p * 16;
-    __syncwarp();
-    if (lane < 16) {
-      const uint4 v = __ldg(x + lane);
-      float* o = xs[warp] + 8 * lane;
-      o[0] = bf_lo(v.x); o[1] = bf_hi(v.x); o[2] = bf_lo(v.y); o[3] = bf_hi(v.y);
-      o[4] = bf_lo(v.z); o[5] = bf_hi(v.z); o[6] = bf_lo(v.w); o[7] = bf_hi(v.w);
-    }
-    __syncwarp();
-    float nx2 = 0.f;
-    bool zero = true;
-    for (int j = 0; j < 4; ++j) {
-      const float v = xs[warp][4 * lane + j];
-      nx2 = __fmaf_rn(v, v, nx2);
-      zero = zero && v == 0.f;
-    }
+    __syncthreads();
+    xs[tid] = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(x)[tid] << 16);
+    if (tid == 0) lowest = 0x7FFFFFFF;
+    float nx2 = xs[tid] * xs[tid];
+    const bool zero = __syncthreads_and(xs[tid] == 0.f);
     for (int o = 16; o > 0; o >>= 1) nx2 += __shfl_xor_sync(0xffffffffu, nx2, o);
-    zero = __all_sync(0xffffffffu, zero);
+    if (lane == 0) red[warp] = nx2;
+    __syncthreads();
+    nx2 = (red[0] + red[1]) + (red[2] + red[3]);
     const bool filter = !zero && nx2 >= (float)kNormLo && nx2 <= (float)kNormHi && w.ctrl[4 + side] == 0u;
-    const float marg = kAtMargin * 1.001f * __fsqrt_rn(nx2);
-    auto score = [&](int a) {  // fp32, within 2^-16 |x| of |x . x_a| / |x_a|
+    auto score = [&](int a) {  // fp32, within 2^-19 |x| of |x . x_a| / |x_a| (sums per chunk: 26 roundings)
       const uint4* row = AR + (size_t)a * 16;
       float s = 0.f;
+#pragma unroll 8
       for (int c = 0; c < 16; ++c) {
         const uint4 v = __ldg(row + (c ^ (a & 7)));
-        const float* xc = xs[warp] + 8 * c;
-        s = __fmaf_rn(xc[0], bf_lo(v.x), s);
-        s = __fmaf_rn(xc[1], bf_hi(v.x), s);
-        s = __fmaf_rn(xc[2], bf_lo(v.y), s);
-        s = __fmaf_rn(xc[3], bf_hi(v.y), s);
-        s = __fmaf_rn(xc[4], bf_lo(v.z), s);
-        s = __fmaf_rn(xc[5], bf_hi(v.z), s);
-        s = __fmaf_rn(xc[6], bf_lo(v.w), s);
-        s = __fmaf_rn(xc[7], bf_hi(v.w), s);
+        const float* xc = xs + 8 * c;
+        float e = xc[0] * bf_lo(v.x);
+        e = __fmaf_rn(xc[1], bf_hi(v.x), e);
+        e = __fmaf_rn(xc[2], bf_lo(v.y), e);
+        e = __fmaf_rn(xc[3], bf_hi(v.y), e);
+        e = __fmaf_rn(xc[4], bf_lo(v.z), e);
+        e = __fmaf_rn(xc[5], bf_hi(v.z), e);
+        e = __fmaf_rn(xc[6], bf_lo(v.w), e);
+        e = __fmaf_rn(xc[7], bf_hi(v.w), e);
+        s += e;
       }
-      return fabsf(s) * w.inv[side][a];
+      return fabsf(s) * inv[a];
     };
-    float mx = 0.f;
+    // a thread's two largest scores, and its third; the block's largest and what comes near it
+    float b1 = -1.f, b2 = -1.f, b3 = -1.f, near = 0.f;
+    int j1 = -1, j2 = -1;
     if (filter) {
-      for (int a = lane; a < k; a += 32) mx = fmaxf(mx, score(a));
+      for (int a = a_lo + tid; a < a_hi; a += kUndThreads) {
+        const float v = score(a);
+        if (v > b1) {
+          b3 = b2; b2 = b1; b1 = v;
+          j2 = j1; j1 = a;
+        } else if (v > b2) {
+          b3 = b2; b2 = v;
+          j2 = a;
+        } else {
+          b3 = fmaxf(b3, v);
+        }
+      }
+      float mx = b1;
       for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      __syncthreads();
+      if (lane == 0) red[warp] = mx;
+      __syncthreads();
+      mx = fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3]));
+      near = mx - 0x1p-17f * 1.001f * __fsqrt_rn(nx2);
+      if (mx > 0x1p-14f * __fsqrt_rn(nx2)) {
+        // a thread with three near the largest looks at all its anchors again, else at its two
+        const bool crowd = b3 >= near;
+        if (b1 < near) j1 = -1;
+        if (b2 < near) j2 = -1;
+        auto each = [&](auto&& f) {  // f(anchor) for the thread's near anchors
+          if (crowd) {
+            for (int a = a_lo + tid; a < a_hi; a += kUndThreads)
+              if (score(a) >= near) f(a);
+          } else {
+            if (j1 >= 0) f(j1);
+            if (j2 >= 0) f(j2);
+          }
+        };
+        each([&](int a) { atomicMin(&lowest, a); });
+        __syncthreads();
+        const int a0 = lowest;
+        bool same = true;  // one left, or copies of one row: the lowest slot is the nearest
+        each([&](int a) { same = same && (a == a0 || same_rows(a, a0)); });
+        if (__syncthreads_and(same)) {
+          if (tid == 0) {
+            float s, c, ab;
+            paired_dot(x, AR + (size_t)a0 * 16, a0, s, c, ab);
+            settle(p, a0, s, c, ab);
+          }
+          continue;
+        }
+        if (crowd) j1 = -3;
+      } else {
+        j1 = -2;  // every anchor of the thread
+      }
+    } else {
+      j1 = -2;
     }
     double bc = -1.0, bd = 0.0;
     int ba = -1;
-    for (int a = lane; a < k; a += 32) {
+    auto try_anchor = [&](int a) {
       const double na = n2[a];
-      if (na == 0.0 || (filter && score(a) < mx - marg)) continue;
-      if (zero && ba >= 0) continue;  // every usable anchor scores 0: the lane's first stands
+      if (na == 0.0) return;
       const double dot = exact_dot(x, AR + (size_t)a * 16, a);
       const double c = __ddiv_rn(fabs(dot), __dsqrt_rn(na));
-      if (c > bc) {
+      if (c > bc || (c == bc && a < ba)) {
         bc = c;
         bd = dot;
         ba = a;
       }
+    };
+    if (j1 == -3) {
+      for (int a = a_lo + tid; a < a_hi; a += kUndThreads)
+        if (score(a) >= near) try_anchor(a);
+    } else if (j1 == -2) {
+      // (every usable anchor scores 0 against a zero row: the thread's first one stands for it)
+      for (int a = a_lo + tid; a < a_hi && !(zero && ba >= 0); a += kUndThreads) try_anchor(a);
+    } else {
+      if (j1 >= 0) try_anchor(j1);
+      if (j2 >= 0) try_anchor(j2);
     }
-    for (int o = 16; o > 0; o >>= 1) {  // the largest, ties to the lowest slot
-      const double oc = __shfl_xor_sync(0xffffffffu, bc, o), od = __shfl_xor_sync(0xffffffffu, bd, o);
-      const int oa = __shfl_xor_sync(0xffffffffu, ba, o);
-      if (oa >= 0 && (ba < 0 || oc > bc || (oc == bc && oa < ba))) {
-        bc = oc;
-        bd = od;
-        ba = oa;
-      }
+    bcs[tid] = bc;
+    bds[tid] = bd;
+    bas[tid] = ba;
+    __syncthreads();
+    if (tid == 0) {  // the largest, ties to the lowest slot
+      for (int i = 1; i < kUndThreads; ++i)
+        if (bas[i] >= 0 && (ba < 0 || bcs[i] > bc || (bcs[i] == bc && bas[i] < ba))) {
+          bc = bcs[i];
+          bd = bds[i];
+          ba = bas[i];
+        }
+      finish(p, ba, bd);
     }
-    if (lane == 0) finish(p, ba, bd);
   }
 }
 
@@ -1010,7 +1330,14 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) 
     const int sh = dg == 0 ? 21 : (dg == 1 ? 10 : 0), bits = dg == 2 ? 10 : 11;
     for (int p = lo + tid; p < hi; p += kSelThreads) {
       const uint32_t v = key[p];
-      if (dg == 0 || (v >> (sh + bits)) == prefix) atomicAdd(&hist[dg][(v >> sh) & ((1u << bits) - 1u)], 1u);
+      const bool in = dg == 0 || (v >> (sh + bits)) == prefix;
+      const uint32_t digit = (v >> sh) & ((1u << bits) - 1u);
+      if (dg == 0) {  // a few digits hold all the energies: equal ones of a warp are counted at once
+        const unsigned peers = __match_any_sync(__activemask(), digit);
+        if ((peers & ((1u << lane) - 1u)) == 0u) atomicAdd(&hist[dg][digit], (uint32_t)__popc(peers));
+      } else if (in) {
+        atomicAdd(&hist[dg][digit], 1u);
+      }
     }
     cl.sync();
     uint32_t inside;
@@ -1078,16 +1405,38 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) 
     const uint4* X = reinterpret_cast<const uint4*>((side ? A.V : A.K) + (size_t)u * A.s_max * 128);
     const uint4* AR = reinterpret_cast<const uint4*>(A.arena_c + (side ? d->off_anchor_v : d->off_anchor_k));
     const bool valid = w.ctrl[side] != 0u;
-    const int mine = (int)cnt_band;
+    const int mine = (int)cnt_band;  // (at most kSelBand = kSelThreads)
     uint64_t my_key = 0;
-    int my_pos = -1;
-    if (tid < mine) {  // (at most kSelBand = kSelThreads)
-      my_pos = band[tid];
-      const uint32_t st = w.st[side][my_pos];
-      my_key = exact_energy_key(X + (size_t)my_pos * 16, AR + (size_t)(st & 0xFFFFu) * 16, st, valid);
-      const uint32_t i = atomicAdd(n0, 1u);
-      k0[i] = my_key;
-      p0[i] = my_pos;
+    const int my_pos = tid < mine ? band[tid] : -1;
+    // 16 positions at a time: a warp squares a position's residual (four dimensions per lane), a lane sums
+    // it in order, so that the serial part is 128 fp64 additions
+    double* sq = reinterpret_cast<double*>(&hist[0][0]);  // [16][129]
+    for (int b0 = 0; b0 < mine; b0 += kSelThreads / 32) {
+      __syncthreads();
+      if (b0 + warp < mine) {
+        const int p = band[b0 + warp];
+        const uint32_t st = w.st[side][p];
+        const int a = (int)(st & 0xFFFFu);
+        const double g = fp16_bits_to_f64(st >> 16);
+        const uint2 xv = reinterpret_cast<const uint2*>(X + (size_t)p * 16)[lane];
+        const uint2 av = reinterpret_cast<const uint2*>(AR + (size_t)a * 16 + ((lane >> 1) ^ (a & 7)))[lane & 1];
+        const uint32_t xe[4] = {xv.x << 16, xv.x & 0xFFFF0000u, xv.y << 16, xv.y & 0xFFFF0000u};
+        const uint32_t ae[4] = {av.x << 16, av.x & 0xFFFF0000u, av.y << 16, av.y & 0xFFFF0000u};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const double r = __dsub_rn(bf_f64(xe[e]), valid ? __dmul_rn(g, bf_f64(ae[e])) : 0.0);
+          sq[warp * 129 + 4 * lane + e] = __dmul_rn(r, r);
+        }
+      }
+      __syncthreads();
+      if (tid >= b0 && tid < b0 + kSelThreads / 32 && tid < mine) {
+        double e = 0.0;
+        for (int j = 0; j < 128; ++j) e = __dadd_rn(e, sq[(tid - b0) * 129 + j]);
+        my_key = (uint64_t)__double_as_longlong(e) + 1ull;
+        const uint32_t i = atomicAdd(n0, 1u);
+        k0[i] = my_key;
+        p0[i] = my_pos;
+      }
     }
     cl.sync();
     if (my_pos >= 0) {
@@ -1955,6 +2304,7 @@ int launch_encode(const Layout& L, const EncodeWs& W, const akv_params& p, const
   const long long items = 2ll * units * max_t;
   enc_assign_tc<<<(unsigned)std::min<long long>(items, sms), kAtThreads, kAtSmem, st>>>(A, tmK, tmV, tmA, items, max_t);
   enc_finish<<<dim3((maxS + kFinPos - 1) / kFinPos, units, 2), 256, 0, st>>>(A);
+  enc_undecided<<<dim3(kUndBlocks, units, 2), kUndThreads, 0, st>>>(A);
   if (full) {  // Eq. 6 utilities, then each side's pooled top-N per request
     enc_util<<<dim3((maxS + 127) / 128, units), 128, 0, st>>>(A);
     enc_pool<<<units / p.n_kv_heads, 1024, 0, st>>>(A, 0);
