@@ -876,8 +876,8 @@ __device__ bool gamma_at_edge(float s, float c, float ab, double n2, uint32_t gh
   const float mid = 0.5f * (__half2float(__ushort_as_half((unsigned short)gh)) + __half2float(__ushort_as_half((unsigned short)gh2)));
   const float pm = mid * nh, pe = __fmaf_rn(mid, nl, __fmaf_rn(mid, nh, -pm));
   const float diff = (s - pm) + (c - pe);
-  // (errors of the sum, the product and the fp64 result that this stands for: below 2^-37 of each)
-  if (!(fabsf(diff) > (ab + fabsf(pm)) * 0x1p-35f)) return false;
+  // (errors of the sum, the product and the fp64 result that this stands for: below 2^-33 of each)
+  if (!(fabsf(diff) > (ab + fabsf(pm)) * 0x1p-32f)) return false;
   if (diff > 0.f) gh = gh2;
   return true;
 }
@@ -1032,7 +1032,7 @@ __global__ void __launch_bounds__(256) enc_finish(const EncArgs A) {
   for (int i = tid; i < n_full; i += 256) list[S - 1 - (at_full + i)] = full[i];
 }
 
-// x . x_a by one thread in twice the precision of fp32 (s + c, within 2^-38 sum |x x_a|), and that sum.
+// x . x_a by one thread in twice the precision of fp32 (s + c, within 128^2 2^-48 sum |x x_a|), and that sum.
 __device__ void paired_dot(const uint4* x, const uint4* row, int a, float& s, float& c, float& ab) {
   s = c = ab = 0.f;
   for (int c0 = 0; c0 < 16; c0 += 8) {
@@ -1112,7 +1112,7 @@ __global__ void __launch_bounds__(kUndThreads) enc_undecided(const EncArgs A) {
   auto in_range = [](float ab) { return ab >= 0x1p-80f && ab <= 0x1p100f; };
   // gamma and energy for nearest anchor a, x . x_a = hs + hc
   auto settle = [&](int p, int a, float hs, float hc, float ab) {
-    const float iv = inv[a], i2 = iv * iv, gq = (hs + hc) * i2, ge = fabsf(gq) * 0x1p-20f + ab * i2 * 0x1p-36f;
+    const float iv = inv[a], i2 = iv * iv, gq = (hs + hc) * i2, ge = fabsf(gq) * 0x1p-20f + ab * i2 * 0x1p-33f;
     uint32_t gh = f32_to_fp16_bits(gq - ge);
     const uint32_t gh2 = f32_to_fp16_bits(gq + ge);
     bool fixed = in_range(ab) && iv > 0.f;
@@ -1144,8 +1144,8 @@ __global__ void __launch_bounds__(kUndThreads) enc_undecided(const EncArgs A) {
       paired_dot(x, AR + (size_t)a2 * 16, a2, s2, c2, ab2);
       const double d1 = (double)s1 + (double)c1, d2 = (double)s2 + (double)c2;
       const double q1 = d1 * d1 * n2[a2], q2 = d2 * d2 * n2[a1];
-      // squares off by 2^-37 (|x||x_a|)^2 |other|^2 each; scores are above 2^-14 |x|, so 2^-9 of that is left
-      const bool told = in_range(ab1) && in_range(ab2) && fabs(q1 - q2) > 0x1p-34 * (fabs(d1) * (double)ab1 * n2[a2] + fabs(d2) * (double)ab2 * n2[a1]);
+      // (a square is off by twice the dot's error times the dot)
+      const bool told = in_range(ab1) && in_range(ab2) && fabs(q1 - q2) > 0x1p-31 * (fabs(d1) * (double)ab1 * n2[a2] + fabs(d2) * (double)ab2 * n2[a1]);
       if (told || same_rows(a1, a2)) {
         const bool first = told ? q1 > q2 : a1 < a2;
         settle(p, first ? a1 : a2, first ? s1 : s2, first ? c1 : c2, first ? ab1 : ab2);
@@ -1963,29 +1963,573 @@ __device__ double exp_neg_dev(double x) {
   return ldexp(y, (int)n);
 }
 
+// ---- the full selection's sums in paired fp32 -------------------------------------------
+// Scores and utilities only rank positions, so they are first taken with known errors: the inner
+// products over 128 dimensions in twice the precision of fp32 (two_sum_add: the fp64 unit would need 64
+// cycles per warp instruction for 1.6 G of them per 8 heads x 4096 positions x 128 rows), the rest in
+// fp64.  A chain of n paired steps is within n^2 2^-48 of the sum of the terms' magnitudes (2^-34 for
+// n = 128).  A ranking stands if the lowest selected value less its error exceeds the largest unselected
+// one plus its own; else the unit's or request's flag has the exact kernels below repeat it (equal
+// values, in practice).  ctrl[16]: scores undecided, [17 .. 19]: the largest squared norm of the
+// observation rows, keys and values (fp32 bits), [12 + side] of a request's first unit: utilities undecided.
+constexpr int kObsRows = 32;  // rows per block of the logits
+
+// the largest squared norms and the outputs' sums start at zero
+__global__ void __launch_bounds__(256) enc_obs_init(const EncArgs A) {
+  const int u = blockIdx.x;
+  const EncUnitWs w = unit_ws(A, u, unit_desc(A, u));
+  if (threadIdx.x < 16) w.ctrl[16 + threadIdx.x] = 0u;
+  for (int e = threadIdx.x; e < A.m_obs * 128; e += 256) w.yobs[e] = 0.0;
+}
+
+__device__ __forceinline__ double pair_f64(float s, float c) { return (double)s + (double)c; }
+// The relative error of the observation rows' attention: twice a logit's error, for numerator and sum.
+__device__ __forceinline__ float alpha_error(const EncUnitWs& w) {
+  return 4.f * 0x1p-34f * 0.0885f * __fsqrt_rn(__uint_as_float(w.ctrl[17])) * __fsqrt_rn(__uint_as_float(w.ctrl[18])) + 0x1p-34f;
+}
+// Squared norms that keep every fp32 product of the kernels below inside the range.
+__device__ __forceinline__ bool norm_ok(float n2) { return n2 >= 0x1p-80f && n2 <= 0x1p60f; }
+
+// Logits q_w . K_t / sqrt(D): a thread takes one position and eight rows at a time.
+__global__ void __launch_bounds__(128) enc_obs_logit_f(const EncArgs A) {
+  __shared__ __align__(16) uint4 ks[128][17];
+  __shared__ __align__(16) float qs[8][128];
+  const int u = blockIdx.y;
+  const akv_unit_desc* d = unit_desc(A, u);
+  const int S = d->len, t0 = blockIdx.x * 128, tid = threadIdx.x, t = t0 + tid;
+  if (t0 >= S) return;
+  const EncUnitWs w = unit_ws(A, u, d);
+  const uint4* K = reinterpret_cast<const uint4*>(A.K + (size_t)u * A.s_max * 128);
+  for (int e = tid; e < 128 * 16; e += 128)
+    ks[e >> 4][e & 15] = t0 + (e >> 4) < S ? __ldg(K + (size_t)t0 * 16 + e) : make_uint4(0u, 0u, 0u, 0u);
+  const double rs = __ddiv_rn(1.0, __dsqrt_rn(128.0));
+  const int w1 = min(A.m_obs, (int)(blockIdx.z + 1) * kObsRows);
+  float kn = 0.f;
+  for (int w0 = blockIdx.z * kObsRows; w0 < w1; w0 += 8) {
+    __syncthreads();
+    for (int e = tid; e < 8 * 128; e += 128)
+      qs[e >> 7][e & 127] = w0 + (e >> 7) < w1 ? __bfloat162float(A.Q[((size_t)u * A.m_obs + w0) * 128 + e]) : 0.f;
+    __syncthreads();
+    float s[8] = {}, c[8] = {};
+    kn = 0.f;
+    for (int g = 0; g < 16; ++g) {
+      const uint4 v = ks[tid][g];
+      const float k[8] = {bf_lo(v.x), bf_hi(v.x), bf_lo(v.y), bf_hi(v.y), bf_lo(v.z), bf_hi(v.z), bf_lo(v.w), bf_hi(v.w)};
+#pragma unroll
+      for (int j = 0; j < 8; ++j) kn = __fmaf_rn(k[j], k[j], kn);
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        const float4 a = *reinterpret_cast<const float4*>(&qs[r][8 * g]), b = *reinterpret_cast<const float4*>(&qs[r][8 * g + 4]);
+        const float q[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int j = 0; j < 8; ++j) two_sum_add(s[r], c[r], q[j] * k[j]);
+      }
+    }
+    if (t < S)
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (w0 + r < w1) w.alpha[(size_t)(w0 + r) * S + t] = pair_f64(s[r], c[r]) * rs;
+    if (tid < 8) {
+      float qn = 0.f;
+      for (int j = 0; j < 128; ++j) qn = __fmaf_rn(qs[tid][j], qs[tid][j], qn);
+      atomicMax(&w.ctrl[17], __float_as_uint(qn < INFINITY ? qn : INFINITY));
+    }
+  }
+  if (blockIdx.z == 0) atomicMax(&w.ctrl[18], __float_as_uint(kn < INFINITY ? kn : INFINITY));
+}
+
+// e^x for x <= 0 to 2^-40: n = rint(x / ln 2), a degree-10 Taylor series of e^(x - n ln 2), scaled by 2^n.
+__device__ __forceinline__ double exp_neg_f(double x) {
+  if (!(x >= -700.0)) return 0.0;
+  const double n = rint(x * 1.4426950408889634074);
+  const double r = fma(n, -0.69314718055994530942, x);
+  double y = 1.0 / 3628800.0;
+  y = fma(y, r, 1.0 / 362880.0);
+  y = fma(y, r, 1.0 / 40320.0);
+  y = fma(y, r, 1.0 / 5040.0);
+  y = fma(y, r, 1.0 / 720.0);
+  y = fma(y, r, 1.0 / 120.0);
+  y = fma(y, r, 1.0 / 24.0);
+  y = fma(y, r, 1.0 / 6.0);
+  y = fma(y, r, 0.5);
+  y = fma(y, r, 1.0);
+  y = fma(y, r, 1.0);
+  return __hiloint2double(__double2hiint(y) + (__double2int_rn(n) << 20), __double2loint(y));
+}
+
+// Softmax of each observation row over all positions (one block per row, sums as a tree).
+__global__ void __launch_bounds__(512) enc_obs_softmax_f(const EncArgs A) {
+  __shared__ double red[16];
+  const int u = blockIdx.y, wr = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const akv_unit_desc* d = unit_desc(A, u);
+  const int S = d->len;
+  double* a = unit_ws(A, u, d).alpha + (size_t)wr * S;
+  // (a maximum good to fp32 keeps e^(x - max) below e^1: the quotient does not depend on it)
+  float mf = -INFINITY;
+  for (int t = threadIdx.x; t < S; t += 512) mf = fmaxf(mf, (float)a[t]);
+  for (int o = 16; o > 0; o >>= 1) mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
+  if (lane == 0) red[warp] = (double)mf;
+  __syncthreads();
+  double mx = red[0];
+  for (int i = 1; i < 16; ++i) mx = red[i] > mx ? red[i] : mx;
+  __syncthreads();
+  double sum = 0.0;
+  for (int t = threadIdx.x; t < S; t += 512) {
+    const double e = exp_neg_f(a[t] - mx);
+    a[t] = e;
+    sum += e;
+  }
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (lane == 0) red[warp] = sum;
+  __syncthreads();
+  sum = 0.0;
+  for (int i = 0; i < 16; ++i) sum += red[i];
+  const double f = 1.0 / sum;
+  for (int t = threadIdx.x; t < S; t += 512) a[t] *= f;
+}
+
+// Outputs y_w = sum_t alpha_wt V_t: a block takes 256 positions and eight rows, a thread one dimension.
+constexpr int kObsChunk = 256;
+__global__ void __launch_bounds__(128) enc_obs_y_f(const EncArgs A) {
+  __shared__ __align__(16) float2 as[kObsChunk][8];
+  __shared__ float vn[4];
+  const int u = blockIdx.z, tid = threadIdx.x, t0 = blockIdx.x * kObsChunk, w0 = blockIdx.y * 8;
+  const akv_unit_desc* d = unit_desc(A, u);
+  const int S = d->len;
+  if (t0 >= S) return;
+  const EncUnitWs w = unit_ws(A, u, d);
+  const int n = min(kObsChunk, S - t0);
+  for (int r = 0; r < 8; ++r)
+    for (int t = tid; t < kObsChunk; t += 128) {
+      const double a = t < n && w0 + r < A.m_obs ? w.alpha[(size_t)(w0 + r) * S + t0 + t] : 0.0;
+      const float hi = (float)a;
+      as[t][r] = make_float2(hi, (float)(a - (double)hi));
+    }
+  __syncthreads();
+  const __nv_bfloat16* V = A.V + ((size_t)u * A.s_max + t0) * 128 + tid;
+  float s[8] = {}, c[8] = {};
+#pragma unroll 4
+  for (int t = 0; t < n; ++t) {
+    const float v = __bfloat162float(V[(size_t)t * 128]);
+#pragma unroll
+    for (int r = 0; r < 8; r += 2) {
+      const float4 a = *reinterpret_cast<const float4*>(&as[t][r]);
+      const float p0 = a.x * v, p1 = a.z * v;
+      c[r] += __fmaf_rn(a.x, v, -p0);
+      c[r + 1] += __fmaf_rn(a.z, v, -p1);
+      two_sum_add(s[r], c[r], p0);
+      two_sum_add(s[r + 1], c[r + 1], p1);
+      c[r] = __fmaf_rn(a.y, v, c[r]);
+      c[r + 1] = __fmaf_rn(a.w, v, c[r + 1]);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+    if (w0 + r < A.m_obs) atomicAdd(&w.yobs[(w0 + r) * 128 + tid], pair_f64(s[r], c[r]));
+  if (w0 == 0) {  // the largest squared norm of the values
+    float mx = 0.f;
+    for (int t = tid >> 5; t < n; t += 4) {
+      const uint2 x = *reinterpret_cast<const uint2*>(A.V + ((size_t)u * A.s_max + t0 + t) * 128 + 4 * (tid & 31));
+      float q = bf_lo(x.x) * bf_lo(x.x) + bf_hi(x.x) * bf_hi(x.x) + bf_lo(x.y) * bf_lo(x.y) + bf_hi(x.y) * bf_hi(x.y);
+      for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+      mx = fmaxf(mx, q < INFINITY ? q : INFINITY);
+    }
+    if ((tid & 31) == 0) vn[tid >> 5] = mx;
+    __syncthreads();
+    if (tid == 0) atomicMax(&w.ctrl[19], __float_as_uint(fmaxf(fmaxf(vn[0], vn[1]), fmaxf(vn[2], vn[3]))));
+  }
+}
+
+// Eq. 6 utilities of 32 positions: key0 = bits(u^K) + 1, key1 = bits(u^V) + 1, anchors 0, and the relative error
+// of u^K (fp32, over perm).  Thread (position, group g of eight): rows g and g + 8 of every sixteen.  With r the
+// key residual as an exact pair, u^K sums alpha^2 (q . r)^2 / D (|V|^2 - 2 V . y + |y|^2).
+constexpr int kUtPos = 32, kUtRows = 16;
+struct UtilSmem {
+  float rh[128][kUtPos], rl[128][kUtPos], v[128][kUtPos];  // residual pairs and values, by dimension
+  float q[kUtRows][128], yh[kUtRows][128], yl[kUtRows][128];
+  double y2[kUtRows];
+  float qn[kUtRows], yn[kUtRows];
+  double red[8][kUtPos][3];
+  float red_n[2][kUtPos];
+};
+__global__ void __launch_bounds__(256) enc_util_f(const EncArgs A) {
+  extern __shared__ __align__(16) uint8_t ut_dyn[];
+  UtilSmem& s = *reinterpret_cast<UtilSmem*>(ut_dyn);
+  const int u = blockIdx.y;
+  const akv_unit_desc* d = unit_desc(A, u);
+  const int S = d->len, p0 = blockIdx.x * kUtPos, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (p0 >= S) return;
+  const EncUnitWs w = unit_ws(A, u, d);
+  const uint4* AK = reinterpret_cast<const uint4*>(A.arena_c + d->off_anchor_k);
+  const uint4* AV = reinterpret_cast<const uint4*>(A.arena_c + d->off_anchor_v);
+  // residuals: eight threads per position, 16 dimensions each
+  const int lp = tid >> 3, sub = tid & 7, pl = p0 + lp;
+  const bool in = pl < S && w.slot_of[pl] < 0;
+  float rn = 0.f, vn = 0.f, es = 0.f, ec = 0.f, vs = 0.f, vc = 0.f;
+  {
+    const uint32_t sk = in ? w.st[0][pl] : 0u, sv = in ? w.st[1][pl] : 0u;
+    const int ak = (int)(sk & 0xFFFFu), av = (int)(sv & 0xFFFFu);
+    const float gk = __half2float(__ushort_as_half((unsigned short)(sk >> 16)));
+    const float gv = __half2float(__ushort_as_half((unsigned short)(sv >> 16)));
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int ch = 2 * sub + c;
+      const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+      const uint4 xk = in ? __ldg(reinterpret_cast<const uint4*>(A.K + ((size_t)u * A.s_max + pl) * 128) + ch) : z;
+      const uint4 xv = in ? __ldg(reinterpret_cast<const uint4*>(A.V + ((size_t)u * A.s_max + pl) * 128) + ch) : z;
+      const uint4 yk = in ? __ldg(AK + (size_t)ak * 16 + (ch ^ (ak & 7))) : z, yv = in ? __ldg(AV + (size_t)av * 16 + (ch ^ (av & 7))) : z;
+      const uint32_t kw[4] = {xk.x, xk.y, xk.z, xk.w}, vw[4] = {xv.x, xv.y, xv.z, xv.w};
+      const uint32_t ka[4] = {yk.x, yk.y, yk.z, yk.w}, va[4] = {yv.x, yv.y, yv.z, yv.w};
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const float x = (e & 1) ? bf_hi(kw[e >> 1]) : bf_lo(kw[e >> 1]), a = (e & 1) ? bf_hi(ka[e >> 1]) : bf_lo(ka[e >> 1]);
+        float h = x, l = 0.f;
+        two_sum_add(h, l, -(gk * a));  // (the product is exact)
+        s.rh[8 * ch + e][lp] = h;
+        s.rl[8 * ch + e][lp] = l;
+        rn = __fmaf_rn(h, h, rn);
+        const float v = (e & 1) ? bf_hi(vw[e >> 1]) : bf_lo(vw[e >> 1]), b = (e & 1) ? bf_hi(va[e >> 1]) : bf_lo(va[e >> 1]);
+        s.v[8 * ch + e][lp] = v;
+        two_sum_add(vs, vc, v * v);
+        float rvh = v, rvl = 0.f;
+        two_sum_add(rvh, rvl, -(gv * b));
+        const float pp = rvh * rvh;
+        ec += __fmaf_rn(2.f * rvh, rvl, __fmaf_rn(rvh, rvh, -pp));
+        two_sum_add(es, ec, pp);
+      }
+    }
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+      rn += __shfl_xor_sync(0xffffffffu, rn, o);
+      const float a = __shfl_xor_sync(0xffffffffu, vs, o), b = __shfl_xor_sync(0xffffffffu, vc, o);
+      two_sum_add(vs, vc, a);
+      vc += b;
+      const float a2 = __shfl_xor_sync(0xffffffffu, es, o), b2 = __shfl_xor_sync(0xffffffffu, ec, o);
+      two_sum_add(es, ec, a2);
+      ec += b2;
+    }
+    vn = vs;
+    if (sub == 0) {  // handed to the position's threads below through the sums' places
+      s.red[0][lp][0] = pair_f64(vs, vc);
+      s.red[1][lp][0] = pair_f64(es, ec);
+      s.red_n[0][lp] = rn;
+      s.red_n[1][lp] = vn;
+    }
+  }
+  __syncthreads();
+  const int p = p0 + lane, g = warp;
+  const double v2 = s.red[0][lane][0], ev = s.red[1][lane][0];
+  const float rnorm2 = s.red_n[0][lane], vnorm2 = s.red_n[1][lane];
+  __syncthreads();
+  const float ea = alpha_error(w), vmax = __fsqrt_rn(__uint_as_float(w.ctrl[19]));
+  const float ey = (0x1p-29f + ea) * vmax;  // |error of y| (256 paired steps of three additions, and alpha's)
+  const float rnorm = __fsqrt_rn(rnorm2), vnorm = __fsqrt_rn(vnorm2);
+  double uk = 0.0, uv = 0.0, ek = 0.0;
+  for (int w0 = 0; w0 < A.m_obs; w0 += kUtRows) {
+    const int nr = min(kUtRows, A.m_obs - w0);
+    __syncthreads();
+    for (int r = warp; r < kUtRows; r += 8) {  // a warp loads a row, and takes its norms
+      float ys = 0.f, yc = 0.f, qn = 0.f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int j = lane + 32 * e;
+        const float q = r < nr ? __bfloat162float(A.Q[((size_t)u * A.m_obs + w0 + r) * 128 + j]) : 0.f;
+        const double y = r < nr ? w.yobs[(w0 + r) * 128 + j] : 0.0;
+        const float yh = (float)y, yl = (float)(y - (double)yh), pp = yh * yh;
+        s.q[r][j] = q;
+        s.yh[r][j] = yh;
+        s.yl[r][j] = yl;
+        qn = __fmaf_rn(q, q, qn);
+        yc += __fmaf_rn(2.f * yh, yl, __fmaf_rn(yh, yh, -pp));
+        two_sum_add(ys, yc, pp);
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        qn += __shfl_xor_sync(0xffffffffu, qn, o);
+        const float a = __shfl_xor_sync(0xffffffffu, ys, o), b = __shfl_xor_sync(0xffffffffu, yc, o);
+        two_sum_add(ys, yc, a);
+        yc += b;
+      }
+      if (lane == 0) {
+        s.y2[r] = pair_f64(ys, yc);
+        s.qn[r] = __fsqrt_rn(qn);
+        s.yn[r] = __fsqrt_rn(ys);
+      }
+    }
+    __syncthreads();
+    float qs[2] = {}, qc[2] = {}, ys[2] = {}, yc[2] = {};  // q . r and V . y of the thread's two rows
+#pragma unroll 2
+    for (int j = 0; j < 128; j += 4) {
+      float rh[4], rl[4], v[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        rh[e] = s.rh[j + e][lane];
+        rl[e] = s.rl[j + e][lane];
+        v[e] = s.v[j + e][lane];
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int r = g + 8 * i;
+        const float4 q4 = *reinterpret_cast<const float4*>(&s.q[r][j]), h4 = *reinterpret_cast<const float4*>(&s.yh[r][j]),
+                     l4 = *reinterpret_cast<const float4*>(&s.yl[r][j]);
+        const float q[4] = {q4.x, q4.y, q4.z, q4.w}, yh[4] = {h4.x, h4.y, h4.z, h4.w}, yl[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float a = q[e] * rh[e], b = v[e] * yh[e];
+          qc[i] += __fmaf_rn(q[e], rl[e], __fmaf_rn(q[e], rh[e], -a));
+          two_sum_add(qs[i], qc[i], a);
+          yc[i] += __fmaf_rn(v[e], yl[e], __fmaf_rn(v[e], yh[e], -b));
+          two_sum_add(ys[i], yc[i], b);
+        }
+      }
+    }
+    if (p < S) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int r = g + 8 * i;
+        if (r >= nr) continue;
+        const double a = w.alpha[(size_t)(w0 + r) * S + p], a2 = a * a;
+        const double dq = pair_f64(qs[i], qc[i]), dv = fma(-2.0, pair_f64(ys[i], yc[i]), v2 + s.y2[r]);
+        const double aq = a2 * (dq * dq) * 0.0078125;
+        uk = fma(aq, dv, uk);
+        uv += a2;
+        // errors of q . r and of dv: paired chains of 128 steps, and y's
+        const float hq = 0x1p-32f * s.qn[r] * rnorm, sum = vnorm + s.yn[r] + ey;
+        const float hv = sum * (0x1p-31f * sum + 2.f * ey);
+        ek = fma(a2, (double)(0.0078125f * (2.f * fabsf((float)dq) + hq) * hq * ((float)dv + hv)), fma(aq, (double)hv, ek));
+      }
+    }
+  }
+  s.red[g][lane][0] = uk;
+  s.red[g][lane][1] = uv;
+  s.red[g][lane][2] = ek;
+  __syncthreads();
+  if (g != 0 || p >= S) return;
+  float* err = reinterpret_cast<float*>(w.perm);
+  if (w.slot_of[p] >= 0) {
+    w.key0[p] = w.key1[p] = 0ull;
+    err[p] = 0.f;
+    return;
+  }
+  for (int x = 1; x < 8; ++x) {
+    uk += s.red[x][lane][0];
+    uv += s.red[x][lane][1];
+    ek += s.red[x][lane][2];
+  }
+  const double rm = 1.0 / (double)A.m_obs;
+  uk *= rm;
+  uv *= ev * rm;
+  // fp32 norms outside the safe range (and not exactly 0): no bound
+  const bool bounded = (rnorm2 == 0.f || norm_ok(rnorm2)) && (vnorm2 == 0.f || norm_ok(vnorm2));
+  w.key0[p] = (uint64_t)__double_as_longlong(uk > 0.0 ? uk : 0.0) + 1ull;
+  w.key1[p] = (uint64_t)__double_as_longlong(uv > 0.0 ? uv : 0.0) + 1ull;
+  err[p] = !bounded ? INFINITY : (ek > 0.0 ? (float)(1.001 * ek * rm / uk) : 0.f);  // relative to u^K
+}
+
+// Whether a ranking by values v with errors e stands: the lowest selected v - e above the largest
+// unselected v + e.  Order-preserving 64-bit form of an fp64 value, for the maxima over the cluster.
+__device__ __forceinline__ uint64_t f64_order(double x) {
+  const uint64_t b = (uint64_t)__double_as_longlong(x);
+  return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
+}
+
+// Top `want` of n 64-bit keys over the cluster (each CTA holding keys i in [lo, hi) through key_at), from the
+// largest down: selected are those with key >> sh >= prefix.  False if equal keys straddle the cut.
+template <class KeyAt>
+__device__ bool cluster_top(cooperative_groups::cluster_group cl, KeyAt key_at, int64_t lo, int64_t hi, uint32_t want,
+                            uint32_t (*hist)[2048], uint32_t* wsum, uint32_t* found, int& sh, uint64_t& prefix) {
+  const int tid = threadIdx.x;
+  for (int i = tid; i < 3 * 2048; i += kSelThreads) (&hist[0][0])[i] = 0u;
+  __syncthreads();
+  sh = 64;
+  prefix = 0;
+#pragma unroll 1
+  for (int dg = 0;; ++dg) {
+    const int ns = max(0, sh - 11), bits = sh - ns;
+    uint32_t* h = hist[dg % 3];
+    for (int64_t i0 = lo; i0 < hi; i0 += kSelThreads) {
+      const int64_t i = i0 + tid;
+      const uint64_t v = i < hi ? key_at(i) : 0ull;
+      const bool in = i < hi && (dg == 0 || (v >> sh) == prefix);
+      const uint32_t digit = in ? (uint32_t)(v >> ns) & ((1u << bits) - 1u) : 0xFFFFFFFFu;
+      const unsigned peers = __match_any_sync(0xffffffffu, digit);
+      if (in && (peers & ((1u << (tid & 31)) - 1u)) == 0u) atomicAdd(&h[digit], (uint32_t)__popc(peers));
+    }
+    cl.sync();
+    if (dg > 0)
+      for (int i = tid; i < 2048; i += kSelThreads) hist[(dg + 2) % 3][i] = 0u;
+    uint32_t inside;
+    const uint32_t digit = cluster_digit<true>(cl, h, wsum, found, want, &inside);
+    prefix = (prefix << bits) | digit;
+    sh = ns;
+    if (want == inside) return true;
+    if (sh == 0) return false;
+  }
+}
+// Largest of a 64-bit value over the cluster.
+__device__ uint64_t cluster_max(cooperative_groups::cluster_group cl, uint64_t v, unsigned long long* slot) {
+  for (int o = 16; o > 0; o >>= 1) {
+    const uint64_t t = __shfl_xor_sync(0xffffffffu, v, o);
+    v = t > v ? t : v;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) *slot = 0ull;
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) atomicMax(slot, (unsigned long long)v);
+  cl.sync();
+  for (int r = 0; r < kSelCtas; ++r) {
+    const uint64_t t = *cl.map_shared_rank(slot, r);
+    v = t > v ? t : v;
+  }
+  return v;
+}
+
+// The floor(rho (k - w)) highest scores (ties: lower position) become anchors: slot_of = -2 marks them for
+// enc_anchors, every other position gets -1.
+__global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) enc_score_pick_f(const EncArgs A) {
+  namespace cg = cooperative_groups;
+  __shared__ __align__(16) uint32_t hist[3][2048];
+  __shared__ uint32_t wsum[kSelThreads / 32], found[3];
+  __shared__ unsigned long long slot[2];
+  cg::cluster_group cl = cg::this_cluster();
+  const int tid = threadIdx.x, u = blockIdx.x / kSelCtas;
+  const akv_unit_desc* d = unit_desc(A, u);
+  const int S = d->len, k = d->n_anchors, win = min(A.window, S), P = S - win;
+  const EncUnitWs w = unit_ws(A, u, d);
+  const int ns = n_scored(A, k - win);
+  int lo, hi, sh = 0;
+  cluster_share(S, (int)cl.block_rank(), lo, hi);
+  uint64_t prefix = ~0ull;
+  if (ns > 0) {
+    const int hp = min(hi, P);
+    bool ok = cluster_top(cl, [&](int64_t i) { return w.key0[i]; }, lo, hp, (uint32_t)ns, hist, wsum, found, sh, prefix);
+    const double e = 2.0 * (double)alpha_error(w);
+    uint64_t in_lo = 0, out_hi = 0;  // complement of the lowest selected bound; largest unselected one
+    for (int p = lo + tid; p < hp; p += kSelThreads) {
+      const uint64_t key = w.key0[p];
+      const double v = __longlong_as_double((long long)key);
+      if ((key >> sh) >= prefix) in_lo = max(in_lo, ~f64_order(v - e * v - 1e-290));
+      else out_hi = max(out_hi, f64_order(v + e * v + 1e-290));
+    }
+    in_lo = cluster_max(cl, in_lo, &slot[0]);
+    out_hi = cluster_max(cl, out_hi, &slot[1]);
+    ok = ok && ~in_lo > out_hi && __uint_as_float(w.ctrl[17]) <= 0x1p60f && __uint_as_float(w.ctrl[18]) <= 0x1p60f;
+    if (!ok && cl.block_rank() == 0 && tid == 0) w.ctrl[16] = 1u;
+  }
+  for (int p = lo + tid; p < hi; p += kSelThreads) w.slot_of[p] = ns > 0 && p < P && (w.key0[p] >> sh) >= prefix ? -2 : -1;
+  cl.sync();  // no CTA leaves while another may still read its counts
+}
+
+// A cluster per request and side: the side's Eq. 9 share of the budget goes to the highest utilities over all
+// KV heads of the request (ties: lower head, then lower position) -> per-unit flags, slot lists and counts
+// (ctrl[2 + side]).
+__global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) enc_pool_f(const EncArgs A) {
+  namespace cg = cooperative_groups;
+  __shared__ __align__(16) uint32_t hist[3][2048];
+  __shared__ uint32_t wsum[kSelThreads / 32], found[3];
+  __shared__ unsigned long long slot[2];
+  __shared__ const uint64_t* keys[256];
+  __shared__ const float* errs[256];
+  __shared__ float rel[256];
+  __shared__ int32_t* lists[256];
+  __shared__ uint32_t* ctrls[256];
+  __shared__ uint8_t* flags[256];
+  cg::cluster_group cl = cg::this_cluster();
+  const int tid = threadIdx.x, side = blockIdx.y, H = A.n_kv_heads, u0 = (int)(blockIdx.x / kSelCtas) * H;
+  const akv_unit_desc* d0 = unit_desc(A, u0);
+  const int S = d0->len, k = d0->n_anchors;
+  bool ok = true;
+  for (int h = tid; h < H; h += kSelThreads) {
+    const akv_unit_desc* d = unit_desc(A, u0 + h);
+    const EncUnitWs w = unit_ws(A, u0 + h, d);
+    keys[h] = side ? w.key1 : w.key0;
+    errs[h] = reinterpret_cast<const float*>(w.perm);
+    rel[h] = 2.5f * alpha_error(w) + 0x1p-30f;
+    lists[h] = w.res_pos + (side ? d->n_res_k : 0);
+    ctrls[h] = w.ctrl;
+    flags[h] = w.flag[side];
+    for (int i = 17; i < 20; ++i) ok = ok && __uint_as_float(w.ctrl[i]) <= 0x1p60f;
+  }
+  ok = __syncthreads_and(ok);
+  const int64_t N = budget_residuals(A.theta, S, H, A.window, k), cand = (int64_t)H * (S - k), n = (int64_t)H * S;
+  int64_t want = side ? N - N / 2 : N / 2;
+  if (want > cand) want = cand;
+  const int64_t per = (n + kSelCtas - 1) / kSelCtas, lo = min(n, (int64_t)cl.block_rank() * per), hi = min(n, lo + per);
+  int sh = 0;
+  uint64_t prefix = ~0ull;
+  if (want > 0) {
+    ok = cluster_top(cl, [&](int64_t i) { return keys[i / S][i % S]; }, lo, hi, (uint32_t)want, hist, wsum, found, sh, prefix) && ok;
+    uint64_t in_lo = 0, out_hi = 0;
+    for (int64_t i = lo + tid; i < hi; i += kSelThreads) {
+      const int h = (int)(i / S), p = (int)(i % S);
+      const uint64_t key = keys[h][p];
+      if (key == 0ull) continue;  // an anchor
+      const double v = __longlong_as_double((long long)(key - 1ull));
+      const double e = v * (double)(rel[h] + (side ? 0.f : errs[h][p])) + 1e-300;
+      if ((key >> sh) >= prefix) in_lo = max(in_lo, ~f64_order(v - e));
+      else out_hi = max(out_hi, f64_order(v + e));
+    }
+    in_lo = cluster_max(cl, in_lo, &slot[0]);
+    out_hi = cluster_max(cl, out_hi, &slot[1]);
+    // (every candidate in, or the cut clear of both sides' errors)
+    ok = want == cand || (ok && ~in_lo > out_hi);
+  }
+  if (!ok) {
+    if (cl.block_rank() == 0 && tid == 0) ctrls[0][12 + side] = 1u;
+    cl.sync();
+    return;
+  }
+  for (int64_t i0 = lo; i0 < hi; i0 += kSelThreads) {
+    const int64_t i = i0 + tid;
+    if (i >= hi) continue;
+    const int h = (int)(i / S), p = (int)(i % S);
+    const uint64_t key = keys[h][p];
+    const bool sel = want > 0 && (want == cand ? key != 0ull : (key >> sh) >= prefix);
+    flags[h][p] = sel ? 1 : 0;
+    if (sel) lists[h][atomicAdd(&ctrls[h][2 + side], 1u)] = p;
+  }
+  cl.sync();
+}
+
+// The exact forms, run only where the paired sums left a ranking undecided: GATE 1, of the unit's scores;
+// GATE 2, of the request's utilities (either side).
+template <int GATE>
+__device__ __forceinline__ bool gated(const EncArgs& A, int u) {
+  if (GATE == 1) return unit_ws(A, u, unit_desc(A, u)).ctrl[16] != 0u;
+  const int u0 = u / A.n_kv_heads * A.n_kv_heads;
+  const uint32_t* c = unit_ws(A, u0, unit_desc(A, u0)).ctrl;
+  return (c[12] | c[13]) != 0u;
+}
+
 // Logits q_w . K_t / sqrt(D) of every observation row and position (Eq. 4), into alpha.
+template <int GATE>
 __global__ void __launch_bounds__(128) enc_obs_logit(const EncArgs A) {
   __shared__ double qs[128];
-  const int u = blockIdx.z, wr = blockIdx.y;
+  const int u = blockIdx.y;
+  if (!gated<GATE>(A, u)) return;
   const akv_unit_desc* d = unit_desc(A, u);
   const int S = d->len;
   const int t = blockIdx.x * 128 + threadIdx.x;
   if (blockIdx.x * 128 >= S) return;
   EncUnitWs w = unit_ws(A, u, d);
-  qs[threadIdx.x] = bf16_to_f64(A.Q[((size_t)u * A.m_obs + wr) * 128 + threadIdx.x]);
-  __syncthreads();
-  if (t >= S) return;
-  const __nv_bfloat16* X = A.K + ((size_t)u * A.s_max + t) * 128;
-  double acc = 0.0;
-  for (int j = 0; j < 128; ++j) acc = __dadd_rn(acc, __dmul_rn(qs[j], bf16_to_f64(X[j])));
-  w.alpha[(size_t)wr * S + t] = __dmul_rn(acc, __ddiv_rn(1.0, __dsqrt_rn(128.0)));
+  const __nv_bfloat16* X = A.K + ((size_t)u * A.s_max + min(t, S - 1)) * 128;
+  for (int wr = 0; wr < A.m_obs; ++wr) {
+    __syncthreads();
+    qs[threadIdx.x] = bf16_to_f64(A.Q[((size_t)u * A.m_obs + wr) * 128 + threadIdx.x]);
+    __syncthreads();
+    double acc = 0.0;  // (a product of two bf16 is exact: the fused step rounds like a separate add)
+    for (int j = 0; j < 128; ++j) acc = __fma_rn(qs[j], bf16_to_f64(X[j]), acc);
+    if (t < S) w.alpha[(size_t)wr * S + t] = __dmul_rn(acc, __ddiv_rn(1.0, __dsqrt_rn(128.0)));
+  }
 }
 
 // Softmax of each observation row's logits over all S positions.
+template <int GATE>
 __global__ void __launch_bounds__(1024) enc_obs_softmax(const EncArgs A) {
   __shared__ double red[32];
   __shared__ double den_s;
   const int u = blockIdx.y, wr = blockIdx.x;
+  if (!gated<GATE>(A, u)) return;
   const akv_unit_desc* d = unit_desc(A, u);
   const int S = d->len;
   EncUnitWs w = unit_ws(A, u, d);
@@ -2017,6 +2561,7 @@ __global__ void __launch_bounds__(1024) enc_obs_softmax(const EncArgs A) {
 // Exact output y_w = sum_t alpha_wt V_t of each observation row (positions in order).
 __global__ void __launch_bounds__(128) enc_obs_y(const EncArgs A) {
   const int u = blockIdx.y, wr = blockIdx.x, j = threadIdx.x;
+  if (!gated<2>(A, u)) return;
   const akv_unit_desc* d = unit_desc(A, u);
   const int S = d->len;
   EncUnitWs w = unit_ws(A, u, d);
@@ -2028,8 +2573,10 @@ __global__ void __launch_bounds__(128) enc_obs_y(const EncArgs A) {
 }
 
 // Selector score, step 1: the rows' attention averaged over the m rows (into key1 as fp64).
+template <int GATE>
 __global__ void enc_score_mean(const EncArgs A) {
   const int u = blockIdx.y;
+  if (GATE && !gated<GATE>(A, u)) return;
   const akv_unit_desc* d = unit_desc(A, u);
   const int S = d->len, P = S - min(A.window, S);
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2043,8 +2590,10 @@ __global__ void enc_score_mean(const EncArgs A) {
 // Selector score, step 2: average pooling of width kappa centred on t over [0, P), zero
 // outside, divided by kappa (Appendix A.2); the score's bits into key0 (scores are >= 0,
 // so their bit patterns order like the values).
+template <int GATE>
 __global__ void enc_score_pool(const EncArgs A) {
   const int u = blockIdx.y;
+  if (GATE && !gated<GATE>(A, u)) return;
   const akv_unit_desc* d = unit_desc(A, u);
   const int S = d->len, P = S - min(A.window, S);
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -2064,6 +2613,7 @@ __global__ void __launch_bounds__(1024) enc_score_pick(const EncArgs A) {
   __shared__ uint32_t bc[2];
   __shared__ int wt[33];
   const int u = blockIdx.x;
+  if (!gated<1>(A, u)) return;
   const akv_unit_desc* d = unit_desc(A, u);
   const int S = d->len, k = d->n_anchors, win = min(A.window, S), P = S - win;
   EncUnitWs w = unit_ws(A, u, d);
@@ -2092,13 +2642,14 @@ __global__ void __launch_bounds__(128) enc_util(const EncArgs A) {
   __shared__ double qs[UT_ROWS][128];
   __shared__ double ys[UT_ROWS][128];
   const int u = blockIdx.y;
+  if (!gated<2>(A, u)) return;
   const akv_unit_desc* d = unit_desc(A, u);
   const int S = d->len;
   if (blockIdx.x * 128 >= S) return;
   EncUnitWs w = unit_ws(A, u, d);
   const int p = blockIdx.x * 128 + threadIdx.x;
-  const bool live = p < S && w.slot_of[p] < 0;
   const int32_t* apos = reinterpret_cast<const int32_t*>(A.arena_c + d->off_anchor_pos);
+  const bool live = p < S && apos[w.st[0][p] & 0xFFFFu] != p;  // (an anchor's position is its slot's)
   const __nv_bfloat16 *xk = nullptr, *xv = nullptr, *ak = nullptr, *av = nullptr;
   double gk = 0.0, gv = 0.0, ev = 0.0;
   if (live) {
@@ -2162,6 +2713,7 @@ __global__ void __launch_bounds__(1024) enc_pool(const EncArgs A, int side) {
   __shared__ uint32_t* ctrls[256];
   __shared__ uint8_t* flags[256];
   const int H = A.n_kv_heads, u0 = blockIdx.x * H;
+  if (unit_ws(A, u0, unit_desc(A, u0)).ctrl[12 + side] == 0u) return;
   const akv_unit_desc* d0 = unit_desc(A, u0);
   const int S = d0->len, k = d0->n_anchors;
   for (int h = threadIdx.x; h < H; h += blockDim.x) {
@@ -2280,11 +2832,18 @@ int launch_encode(const Layout& L, const EncodeWs& W, const akv_params& p, const
   const unsigned maxS = (unsigned)L.max_len;
   if (full) {  // observation rows' attention, selector scores, the scored anchors
     const unsigned m = (unsigned)m_obs;
-    enc_obs_logit<<<dim3((maxS + 127) / 128, m, units), 128, 0, st>>>(A);
-    enc_obs_softmax<<<dim3(m, units), 1024, 0, st>>>(A);
-    enc_obs_y<<<dim3(m, units), 128, 0, st>>>(A);
-    enc_score_mean<<<dim3((maxS + 255) / 256, units), 256, 0, st>>>(A);
-    enc_score_pool<<<dim3((maxS + 255) / 256, units), 256, 0, st>>>(A);
+    enc_obs_init<<<units, 256, 0, st>>>(A);
+    enc_obs_logit_f<<<dim3((maxS + 127) / 128, units, (m + kObsRows - 1) / kObsRows), 128, 0, st>>>(A);
+    enc_obs_softmax_f<<<dim3(m, units), 512, 0, st>>>(A);
+    enc_obs_y_f<<<dim3((maxS + kObsChunk - 1) / kObsChunk, (m + 7) / 8, units), 128, 0, st>>>(A);
+    enc_score_mean<0><<<dim3((maxS + 255) / 256, units), 256, 0, st>>>(A);
+    enc_score_pool<0><<<dim3((maxS + 255) / 256, units), 256, 0, st>>>(A);
+    enc_score_pick_f<<<kSelCtas * (unsigned)units, kSelThreads, 0, st>>>(A);
+    // the units whose scores the errors leave undecided
+    enc_obs_logit<1><<<dim3((maxS + 127) / 128, units), 128, 0, st>>>(A);
+    enc_obs_softmax<1><<<dim3(m, units), 1024, 0, st>>>(A);
+    enc_score_mean<1><<<dim3((maxS + 255) / 256, units), 256, 0, st>>>(A);
+    enc_score_pool<1><<<dim3((maxS + 255) / 256, units), 256, 0, st>>>(A);
     enc_score_pick<<<units, 1024, 0, st>>>(A);
   }
   enc_anchors<<<kSelCtas * (unsigned)units, kSelThreads, 0, st>>>(A);
@@ -2306,6 +2865,16 @@ int launch_encode(const Layout& L, const EncodeWs& W, const akv_params& p, const
   enc_finish<<<dim3((maxS + kFinPos - 1) / kFinPos, units, 2), 256, 0, st>>>(A);
   enc_undecided<<<dim3(kUndBlocks, units, 2), kUndThreads, 0, st>>>(A);
   if (full) {  // Eq. 6 utilities, then each side's pooled top-N per request
+    const unsigned m = (unsigned)m_obs;
+    if ((e = cudaFuncSetAttribute(enc_util_f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(UtilSmem))) !=
+        cudaSuccess)
+      return (int)e;
+    enc_util_f<<<dim3((maxS + kUtPos - 1) / kUtPos, units), 256, sizeof(UtilSmem), st>>>(A);
+    enc_pool_f<<<dim3(kSelCtas * (unsigned)(units / p.n_kv_heads), 2), kSelThreads, 0, st>>>(A);
+    // the requests whose utilities the errors leave undecided
+    enc_obs_logit<2><<<dim3((maxS + 127) / 128, units), 128, 0, st>>>(A);
+    enc_obs_softmax<2><<<dim3(m, units), 1024, 0, st>>>(A);
+    enc_obs_y<<<dim3(m, units), 128, 0, st>>>(A);
     enc_util<<<dim3((maxS + 127) / 128, units), 128, 0, st>>>(A);
     enc_pool<<<units / p.n_kv_heads, 1024, 0, st>>>(A, 0);
     enc_pool<<<units / p.n_kv_heads, 1024, 0, st>>>(A, 1);

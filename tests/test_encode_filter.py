@@ -46,3 +46,33 @@ def test_equal_rows(dev, kinds, k1):  # noqa: F811
     K, V = gen.clustered_batch(1, 1, [S], seed=10)
     pick = np.random.Generator(np.random.PCG64(3)).integers(0, kinds, size=S)
     _encode_both(dev, p, [S], K[:, :, pick], V[:, :, pick])
+
+
+@pytest.mark.parametrize("kinds,e", [(30, 0), (0, 40), (300, 0)])
+def test_selection_left_to_fp64(dev, kinds, e):  # noqa: F811
+    """The full selection where the paired sums cannot rank: positions drawn from a few distinct rows (equal scores
+    and utilities, ties to the lower head and position), and keys whose norms leave the fp32 range."""
+    import oracle
+    import torch
+    from helpers import assert_same_unit, stored_order, to_dev_u16
+    lens, H, G, W = [900, 333], 2, 2, 16
+    p = akv.Params(batch=2, n_kv_heads=H, n_q_heads=H * G, anchor_frac=0.06, res_frac_k=0.0, res_frac_v=0.0, window=W,
+                   seed=12, rot_seed=13)
+    sel = akv.SelectParams(theta=0.3, rho=0.7, kappa=3)
+    K, V = gen.clustered_batch(2, H, lens, seed=14)
+    if kinds:
+        pick = np.random.Generator(np.random.PCG64(4)).integers(0, min(kinds, 300), size=K.shape[2])
+        K, V = K[:, :, pick].copy(), V[:, :, pick].copy()
+        for b, S in enumerate(lens):
+            K[b, :, S:] = V[b, :, S:] = 0
+    K = _scaled(K, e)
+    Q = gen.observation_queries(_scaled(K, -e), lens, W * G, seed=15)
+    a_bytes, w_bytes = akv.akv_cache_size_select(p, sel, lens)
+    arena = torch.empty(a_bytes, dtype=torch.uint8, device=dev)
+    ws = torch.full((w_bytes,), 0xAB, dtype=torch.uint8, device=dev)
+    akv.akv_encode_select(p, sel, lens, to_dev_u16(K, torch, dev), to_dev_u16(V, torch, dev), to_dev_u16(Q, torch, dev), arena, ws)
+    got = oracle.unpack_arena(arena.cpu().numpy())
+    want = oracle.encode_select(K, V, Q, lens, H, p.anchor_frac, W, sel.theta, sel.rho, sel.kappa, p.seed, p.rot_seed, True)
+    for u, (g, w) in enumerate(zip(got, want)):
+        assert (g.S, g.k, g.nk, g.nv) == (w.S, w.k, w.nk, w.nv), u
+        assert_same_unit(g, stored_order(w), f"unit {u}")
