@@ -93,6 +93,7 @@ constexpr uint32_t kScTmemCols = 32;                     // two accumulators of 
 // Instruction descriptor of kind::f16: fp32 accumulator (bits 4-5 = 1), bf16 A and B (7-9 = 1,
 // 10-12 = 1), both K-major (15, 16 = 0), N / 8 (17-22), M / 16 (24-28).
 constexpr uint32_t kScIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((16u >> 3) << 17) | ((uint32_t)(kScTile >> 4) << 24);
+constexpr int kEnds = 2 * WPG;       // a tile's runs that may go on in a neighbour warp: each warp's first and last
 constexpr int kOvl = 32;            // a tile's entries per overflow list (value records, anchor-value runs)
 constexpr int kRingSlack = 4096;    // shared memory after the ring: the masked rows of the last
                                     // 16-row block of staged anchor values are read from here
@@ -177,7 +178,7 @@ struct DecodeParams {
   int cap;         // staged bytes of a tile block at most
   int ring_bytes, drop_last, smem_sa;
   int o_bar, o_meta, o_misc, o_sa, o_ovf, o_grp, grp_bytes, o_ring;
-  int g_qp, g_rows, g_red, g_wb, g_pv, g_qf, g_ovl;  // offsets inside a group's block
+  int g_qp, g_rows, g_red, g_wb, g_vs, g_sum, g_pv, g_qf, g_ovl;  // offsets inside a group's block
   const float* lg;         // RoPE at decode: logits [units][s_stride][G] in stored order (else null)
   int s_stride;
   const float* suf_part;   // dense suffix partials [units][n_sch][suf_floats] (null: no suffix)
@@ -1431,7 +1432,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
     *segcnt = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int e = tid; e < 2 * GS * 128 + 16; e += NT) ovf[e] = 0.f;  // (the CTA's sums start at zero)
+  for (int e = tid; e < 2 * GS * 128; e += NT) ovf[e] = 0.f;  // (the overflow's sums start at zero)
   // zeroed p rows: rows past a tile's records are read (and multiplied by zero codes)
   for (int gi = 0; gi < NG; ++gi) {
     float* pvz = reinterpret_cast<float*>(smem + P.o_grp + gi * P.grp_bytes + P.g_pv);
@@ -1469,10 +1470,21 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
     return true;
   };
 
-  // the first unit's anchor-score table (later ones: the group that finishes the previous unit last)
-  auto start_table = [&](int u) {
+  // the first unit's anchor-score table and both groups' copies of its query header (later units: the
+  // group that finishes the previous unit last, which has read the sums kept where the headers go)
+  auto start_unit = [&](int u) {
     const int k = unit_desc(P.arena, u)->n_anchors;
-    if (P.smem_sa && !*failed) {
+    const bool ok = !*failed;
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    for (int g = 0; g < NG; ++g) {
+      if (ok && !ROPE) {  // (RoPE: no key-side header is needed)
+        mbar_expect_tx(bar_hdr(g), (uint32_t)hdr_bytes(GS));
+        bulk_g2s(smem_u32(smem + P.o_grp + g * P.grp_bytes + P.g_qp), P.uh + (size_t)u * P.uh_stride, (uint32_t)hdr_bytes(GS), bar_hdr(g));
+      } else {
+        mbar_arrive(bar_hdr(g));
+      }
+    }
+    if (P.smem_sa && ok) {
       const float* src = P.sa + (size_t)u * P.ka_stride * GS;
       if (GS == 8) {  // the two four-head arrays, k rows of each
         const uint32_t half = 16u * (uint32_t)k;
@@ -1488,7 +1500,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
       mbar_arrive(bar_sa_full);  // the unit's start, for the warps that wait on it
     }
   };
-  if (tid == 0) start_table(P.cta_unit[c]);
+  if (tid == 0) start_unit(P.cta_unit[c]);
   const int n_cta_tiles = (int)(B1 - B0);
 
   // =========================== compute groups ==================================
@@ -1498,7 +1510,9 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
   float* sq = qp + GS * 128;                              // [8] sums of q' per head
   float* rows = reinterpret_cast<float*>(GB + P.g_rows);  // [0,8): -m, [8,16): -inf, [24,32): m
   int* lastf = reinterpret_cast<int*>(GB + P.g_red);
-  float* wb = reinterpret_cast<float*>(GB + P.g_wb);      // [2][X][GS] value weights of a tile's slots
+  float* wb = reinterpret_cast<float*>(GB + P.g_wb);      // [2][X + kEnds][GS] value weights of a tile's slots, then of the warps' first and last runs
+  int* vsl = reinterpret_cast<int*>(GB + P.g_vs);          // [2][kEnds] the slots of those, from the tile's first (-1: none)
+  float* gsum = reinterpret_cast<float*>(GB + P.g_sum);   // [WPG][16] a segment's normaliser and sum of p min per warp and head
   float* pv = reinterpret_cast<float*>(GB + P.g_pv);      // [R][8] p rows of the value records, then A operands
   int* ovl_n = reinterpret_cast<int*>(GB + P.g_ovl);       // [2] entries in the two overflow lists
   float* ovl = reinterpret_cast<float*>(GB + P.g_ovl + 16);  // [2][kOvl][9]: index bits, then p (or weights) per head
@@ -1597,17 +1611,9 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
   for (;; ++sigma) {
     const UnitView U = unit_view(P.arena, sg.u);
     const int k = U.k;
-    // ---- segment set-up: the unit's query header (q', its sums, key-residual fragments, from
-    // the score kernel) by one bulk copy; meanwhile the reference m of each head from the chunk
+    // ---- segment set-up: the unit's query header (q', its sums, key-residual fragments, from the score
+    // kernel) and score table are on their way; meanwhile the reference m of each head from the chunk
     // maxima (warp wg: heads wg, wg + 4) ----
-    if (wg == 0 && lane == 0) {
-      if (!*failed && !ROPE) {  // (RoPE: no key-side header is needed)
-        mbar_expect_tx(bar_hdr(grp), (uint32_t)hdr_bytes(GS));
-        bulk_g2s(smem_u32(qp), P.uh + (size_t)sg.u * P.uh_stride, (uint32_t)hdr_bytes(GS), bar_hdr(grp));
-      } else {
-        mbar_arrive(bar_hdr(grp));
-      }
-    }
     for (int g = wg; g < GS; g += WPG) {
       float m = -INFINITY;
       // the largest anchor score (a lower bound of the largest logit), or with RoPE the largest logit
@@ -1648,7 +1654,8 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
       TileView tv;
       int nKs = 0, nVs = 0;
       bool fast_tile = false;
-      float* W = wb + (lt & 1) * P.X * GS;
+      float* W = wb + (lt & 1) * (P.X + kEnds) * GS;
+      int* vs = vsl + (lt & 1) * kEnds;
       if (go) {
         tv = tile_view(st, mt, U);
         const uint32_t codes_staged = tv.staged > tv.cd_k ? (tv.staged - tv.cd_k) / 32u : 0u;
@@ -1656,8 +1663,9 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
         nVs = min(tv.nv, P.R);
         fast_tile = (ROPE || nKs == tv.nk) && nVs == tv.nv &&
                     (int)(((reinterpret_cast<const uint32_t*>(st + 4 * tv.n64))[tv.n - 1] & 0xFFFFu) - mt.lo) < (int)mt.nrows;
-        for (int e = gt; e < P.X * GS; e += WPG * 32) W[e] = 0.f;
+        for (int e = gt; e < (P.X + kEnds) * GS; e += WPG * 32) W[e] = 0.f;
         if (gt < 2) ovl_n[gt] = 0;
+        if (gt < kEnds) vs[gt] = -1;
         // ---- key residuals: q' . c of the staged key records, tensor cores; the terms
         // scale (q' . c) + min sum(q') - m are written over the records' codes ----
         float* rsb = reinterpret_cast<float*>(const_cast<uint8_t*>(st) + tv.cd_k);
@@ -1843,15 +1851,15 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
                                           __shfl_down_sync(0xffffffffu, hs[i2].y, 1));
             acc[i2] = __ffma2_rn(nh, tn2, acc[i2]);
           }
+          // the warp's first run may continue the previous warp's last one and its last run go on in the
+          // next: both get rows of their own past the slots' (a shared-memory float addition is a
+          // compare-and-swap loop, and would meet the neighbour's)
+          float* w_ends = W + (P.X + 2 * wg) * GS;
           if (multi && !(lane > 0 && ptk == hk)) {
-            float* w = W + (int)(hk - lo) * GS;
-            if (lane == 0) {  // may continue the previous warp's last run
-#pragma unroll
-              for (int g = 0; g < GS; ++g) red_local(w + g, (g & 1) ? hs[g >> 1].y : hs[g >> 1].x);
-            } else {
-              store_row<GS>(w, hs);
-            }
+            if (lane == 0) vs[2 * wg] = (int)(hk - lo);
+            store_row<GS>(lane == 0 ? w_ends : W + (int)(hk - lo) * GS, hs);
           }
+          const bool multi0 = __shfl_sync(0xffffffffu, (int)multi, 0) != 0;
           // segmented inclusive scan of the last runs over lanes with equal slots
 #pragma unroll
           for (int d = 1; d < 32; d <<= 1) {
@@ -1868,13 +1876,11 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
           const uint32_t nkey = __shfl_down_sync(0xffffffffu, key, 1);
           const uint32_t key0 = __shfl_sync(0xffffffffu, key, 0);
           if (lane == 31 || nkey != key) {  // the last lane of a segment holds its total
-            float* w = W + (int)(key - lo) * GS;
-            if (lane == 31 || key == key0) {  // the warp's first or last run: shared with a neighbour warp
-#pragma unroll
-              for (int g = 0; g < GS; ++g) red_local(w + g, (g & 1) ? acc[g >> 1].y : acc[g >> 1].x);
-            } else {
-              store_row<GS>(w, acc);
-            }
+            // (a single run over the whole warp counts as its last)
+            const bool first = !multi0 && key == key0, last = lane == 31;
+            if (last) vs[2 * wg + 1] = (int)(key - lo);
+            else if (first) vs[2 * wg] = (int)(key - lo);
+            store_row<GS>(last ? w_ends + GS : (first ? w_ends : W + (int)(key - lo) * GS), acc);
           }
         } else if (t0 < tv.n) {
           const auto ls = token_chunk_general<GS>(TokTile{tv, mt.lo, mt.nrows, SAt, rows, qp, pv, W, ovf, U.AV,
@@ -1984,6 +1990,27 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
             mma_bf16(accA[2 * hf + 1], ah0, al0, ah2, al2, b10, b11);
           }
         }
+        {  // the warps' first and last runs: rows picked by their slots (k places 8 .. 15 are empty)
+          uint32_t ah0 = 0, al0 = 0;
+          if (r8 < GS) {
+            __nv_bfloat16 hi[2], lo_[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) split_b(W[(P.X + 2 * c4 + e) * GS + r8], hi[e], lo_[e]);
+            ah0 = pack_b2(hi[0], hi[1]);
+            al0 = pack_b2(lo_[0], lo_[1]);
+          }
+          const int2 vc = *reinterpret_cast<const int2*>(vs + 2 * c4);
+          const uint32_t m0 = (vc.x >= 0 ? 0xFFFFu : 0u) | (vc.y >= 0 ? 0xFFFF0000u : 0u);
+          const int slot = max(vs[ri], 0);
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            const int cc = (4 * wg + 2 * hf + (mi >> 1)) ^ (int)((mt.lo + (uint32_t)slot) & 7u);
+            uint32_t b00, b01, b10, b11;
+            ldsm_x4_trans(smem_u32(Vr + slot * 256 + 16 * cc), b00, b01, b10, b11);
+            mma_bf16(accA[2 * hf], ah0, al0, 0u, 0u, b00 & m0, 0u);
+            mma_bf16(accA[2 * hf + 1], ah0, al0, 0u, 0u, b10 & m0, 0u);
+          }
+        }
       }
       gsync();  // (C) every value operand is built
       if (go) {
@@ -2017,43 +2044,39 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
       }
     }
 
-    // ---- the group's sums for this unit into the CTA's sums in shared memory (anchor-value and
-    // rotated value-residual numerators, normaliser, sum of p min); the overflow paths added there
-    // already.  Adds of the two groups meet only element by element. ----
-    float* cl = ovf + 2 * GS * 128;  // [8] normaliser, then [8] sum of p min, per head
-    {
-      if (r8 < GS) {
+    // ---- the group's sums for this unit into shared memory, where its query header was (anchor-value
+    // and rotated value-residual numerators [2][GS][128]; normaliser and sum of p min per warp) ----
+    static_assert(2 * GS * 512 <= hdr_bytes(GS), "a group's sums fit its header's place");
+    gsync();  // every warp is done with the header
+    if (r8 < GS) {
 #pragma unroll
-        for (int nb = 0; nb < 4; ++nb) {
-          const int col = 32 * wg + 8 * nb + 2 * c4;
-          red_local(ovf + r8 * 128 + col, accA[nb][0] + accA[nb][2]);
-          red_local(ovf + r8 * 128 + col + 1, accA[nb][1] + accA[nb][3]);
-          red_local(ovf + GS * 128 + r8 * 128 + col, accR[nb][0] + accR[nb][2]);
-          red_local(ovf + GS * 128 + r8 * 128 + col + 1, accR[nb][1] + accR[nb][3]);
-        }
+      for (int nb = 0; nb < 4; ++nb) {
+        const int col = 32 * wg + 8 * nb + 2 * c4;
+        *reinterpret_cast<float2*>(qp + r8 * 128 + col) = make_float2(accA[nb][0] + accA[nb][2], accA[nb][1] + accA[nb][3]);
+        *reinterpret_cast<float2*>(qp + (GS + r8) * 128 + col) = make_float2(accR[nb][0] + accR[nb][2], accR[nb][1] + accR[nb][3]);
       }
+    }
 #pragma unroll
-      for (int g = 0; g < GS; ++g) {
-        const float sl = warp_sum((g & 1) ? l2[g >> 1].y : l2[g >> 1].x);
-        if (lane == 0) red_local(cl + g, sl);
-      }
+    for (int g = 0; g < GS; ++g) {
+      const float sl = warp_sum((g & 1) ? l2[g >> 1].y : l2[g >> 1].x);
+      if (lane == 0) gsum[wg * 16 + g] = sl;
+    }
 #pragma unroll
-      for (int i2 = 0; i2 < HPL; ++i2) {
-        float v = pminv[i2];
+    for (int i2 = 0; i2 < HPL; ++i2) {
+      float v = pminv[i2];
 #pragma unroll
-        for (int o = 1; o < 16; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        const int g = (lane >> 4) + 2 * i2;
-        if ((lane & 15) == 0 && g < GS) red_local(cl + 8 + g, v);
-      }
+      for (int o = 1; o < 16; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      const int g = (lane >> 4) + 2 * i2;
+      if ((lane & 15) == 0 && g < GS) gsum[wg * 16 + 8 + g] = v;
     }
     if (wg == 0) {  // the segment's last tile is done with: top the ring up
       release_to(lt);
       issue_more();
     }
-    // ---- the group that finishes the segment last (the other has added its sums) turns the
-    // CTA's sums into its slot of the unit: the value-residual part gets its sum of p min and the
-    // inverse rotation (s o H(.) / 128, once per head and CTA), the anchor-value part is added;
-    // then it clears the sums, counts the slot in, and starts the next unit's anchor scores ----
+    // ---- the group that finishes the segment last (the other has stored its sums) turns both
+    // groups' sums and the overflow's into the CTA's slot of the unit: the value-residual part gets its sum
+    // of p min and the inverse rotation (s o H(.) / 128, once per head and CTA), the anchor-value part
+    // is added; then it counts the slot in, and starts the next unit ----
     gsync();
     if (gt == 0) {
       __threadfence_block();
@@ -2064,11 +2087,28 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
     const bool has_next = sg.t0 + sg.je < B1;
     if (lastf[1]) {
       float* dst = P.part + (size_t)(c + sg.u) * PF;
+      const uint8_t* G0 = smem + P.o_grp;  // the groups' blocks, summed in their order
+      auto group_sum = [&](int off, int i) {
+        float v = 0.f;
+#pragma unroll
+        for (int g = 0; g < NG; ++g)
+#pragma unroll
+          for (int x = 0; x < WPG; ++x) v += reinterpret_cast<const float*>(G0 + g * P.grp_bytes + off)[x * 16 + i];
+        return v;
+      };
       for (int h = wg; h < GS; h += WPG) {
         float4* oa = reinterpret_cast<float4*>(ovf + h * 128 + 4 * lane);
         float4* orr = reinterpret_cast<float4*>(ovf + GS * 128 + h * 128 + 4 * lane);
-        const float4 va = *oa, vr = *orr;
-        const float pm = cl[8 + h];
+        float4 va = *oa, vr = *orr;
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+          const float* sums = reinterpret_cast<const float*>(G0 + g * P.grp_bytes + P.g_qp);
+          const float4 a = *reinterpret_cast<const float4*>(sums + h * 128 + 4 * lane);
+          const float4 r = *reinterpret_cast<const float4*>(sums + (GS + h) * 128 + 4 * lane);
+          va.x += a.x; va.y += a.y; va.z += a.z; va.w += a.w;
+          vr.x += r.x; vr.y += r.y; vr.z += r.z; vr.w += r.w;
+        }
+        const float pm = group_sum(P.g_sum, 8 + h);
         float x[4] = {vr.x + pm, vr.y + pm, vr.z + pm, vr.w + pm};
         if (P.rotate) {
           warp_wht128(x, lane);
@@ -2080,17 +2120,12 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
         *oa = make_float4(0.f, 0.f, 0.f, 0.f);
         *orr = make_float4(0.f, 0.f, 0.f, 0.f);
       }
-      gsync();
-      if (gt < GS) {
-        dst[part_l(GS) + gt] = cl[gt];
-        cl[gt] = 0.f;
-        cl[8 + gt] = 0.f;
-      }
+      if (gt < GS) dst[part_l(GS) + gt] = group_sum(P.g_sum, gt);
       gsync();
       if (gt == 0) {
         dst[part_flag(GS)] = *failed ? 1.f : 0.f;
         lastf[0] = count_in(P, sg.u, sg.nseg) ? 1 : 0;
-        if (has_next) start_table(sg.u + 1);  // the CTA's sums are clear for it
+        if (has_next) start_unit(sg.u + 1);  // both groups' sums are read
       }
       gsync();
       if (lastf[0]) {
@@ -2189,7 +2224,7 @@ bool make_plan_rx(const Layout& L, int GS, int R, int X, bool smem_sa, int smem_
   P.o_meta = take(NG * NSG * sizeof(Meta));
   P.o_misc = take(16);
   P.o_sa = take(smem_sa ? (size_t)P.ka_stride * GS * 4 : 0);
-  P.o_ovf = take((size_t)2 * GS * 128 * 4 + 2 * 8 * 4);  // + normaliser and sum of p min per head
+  P.o_ovf = take((size_t)2 * GS * 128 * 4);
   // a group's block: q' rows, small rows, last flag, two weight tables, p rows / A operands
   size_t g = 0;
   auto gtake = [&](size_t bytes) {
@@ -2201,7 +2236,9 @@ bool make_plan_rx(const Layout& L, int GS, int R, int X, bool smem_sa, int smem_
   P.g_qf = P.g_qp + GS * 512 + 32;
   P.g_rows = gtake(32 * 4);
   P.g_red = gtake(16);
-  P.g_wb = gtake((size_t)2 * X * GS * 4);
+  P.g_wb = gtake((size_t)2 * (X + kEnds) * GS * 4);  // the slots' rows, then the warps' first and last runs
+  P.g_vs = gtake((size_t)2 * kEnds * 4);
+  P.g_sum = gtake((size_t)WPG * 16 * 4);
   P.g_pv = gtake((size_t)R * 32);
   P.g_ovl = gtake((size_t)(16 + 2 * kOvl * 9 * 4));  // the tile's overflow lists (counts, then entries)
   P.grp_bytes = (int)g;
