@@ -67,7 +67,7 @@ DEFAULT_LAYERS = {"8b-32k": 32, "8b-128k": 8, "70b-128k": 4}
 DEFAULT_LAYERS.update({n: 2 for n in SWEEP_POINTS})
 # graph replays of (N_TOKENS x layers) steps timed by default, about ten seconds or less of device time
 DEFAULT_REPLAYS = {"8b-32k": 100, "8b-128k": 40, "70b-128k": 40}
-DEC_KERNEL_SRC = os.path.join(ROOT, "paper_2608_02901_gb300", "csrc", "akv_decode.cu")
+DEC_KERNEL_SRC = os.path.join(ROOT, "paper_2608_02901_gb300", "csrc", "akv_decode.cuh")
 
 
 def parse():

@@ -17,6 +17,10 @@ COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", os.path
 SOURCES = {
     "akv_api.cpp": [],
     "akv_decode.cu": [],
+    "akv_decode_g1.cu": [],  # the decode kernels per query-group size, compiled in parallel
+    "akv_decode_g2.cu": [],
+    "akv_decode_g4.cu": [],
+    "akv_decode_g8.cu": [],
     "akv_encode.cu": ["--fmad=false"],  # fp64 decisions: no contraction
 }
 
@@ -31,7 +35,8 @@ def _nvcc() -> str:
 def _compile(src: str, extra: list, verbose: bool) -> str:
     obj = os.path.join(BUILD, src + ".o")
     path = os.path.join(CSRC, src)
-    deps = [path, os.path.join(CSRC, "akv_internal.h"), os.path.join(CSRC, "akv_device.cuh"), os.path.join(ROOT, "include", "akv.h")]
+    deps = [path, os.path.join(ROOT, "include", "akv.h")]
+    deps += [os.path.join(CSRC, h) for h in ("akv_internal.h", "akv_device.cuh", "akv_decode.cuh")]
     if os.path.exists(obj) and all(os.path.getmtime(obj) >= os.path.getmtime(d) for d in deps):
         return obj
     cmd = [_nvcc(), *ARCH, *COMMON, *extra, "-c", path, "-o", obj]

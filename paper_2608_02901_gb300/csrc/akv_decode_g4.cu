@@ -1,0 +1,7 @@
+// The decode kernels for four query heads per KV head.
+#include "akv_decode.cuh"
+
+namespace akv {
+template int launch_g<4>(const Layout&, const akv_params&, const void*, size_t, const void*, void*, float*, float,
+                         const DecodeSuffix&, void*, void*, std::string*);
+}  // namespace akv

@@ -130,6 +130,24 @@ struct DecodeSuffix {
 };
 // Tokens per suffix chunk (one score-launch CTA each, one partial slot each).
 constexpr int kSuffixChunk = 64;
+constexpr int kMaxGrid = 256;       // CTAs of the decode launch at most
+constexpr int CHA = 64;             // anchors per chunk maximum of the score launch
+// floats of one CTA's partial slot for a unit: numerator y [GS][128] (the inverse rotation already
+// applied), normaliser l [GS] (8 places), failure flag, pad to 16 bytes
+AKV_HD constexpr int part_floats(int GS) { return 128 * GS + 12; }
+AKV_HD constexpr int part_l(int GS) { return 128 * GS; }
+AKV_HD constexpr int part_flag(int GS) { return 128 * GS + 8; }
+
+// Bytes of a unit's query header (from the score kernel): the rotated query q' [GS][128] f32, its
+// sums [8] f32, and the key-residual mma B fragments [GS == 8 ? 2 : 1][8][32] uint2.
+AKV_HD constexpr int hdr_bytes(int GS) { return GS * 512 + 32 + (GS == 8 ? 2 : 1) * 2048; }
+
+// Dense suffix: tokens per chunk, and the floats of a chunk's partial slot: the value sum
+// o [GS][128] under the chunk's own maximum, its normaliser l [8] and that maximum m [8] (log2 units).
+AKV_HD constexpr int suf_floats(int GS) { return 128 * GS + 16; }
+AKV_HD constexpr int suf_l(int GS) { return 128 * GS; }
+AKV_HD constexpr int suf_m(int GS) { return 128 * GS + 8; }
+
 // Workspace of a decode call whose suffix holds at most `suffix_cap` tokens per request.
 DecodeWs decode_ws_layout(const Layout& L, int32_t suffix_cap = 0);
 int launch_decode(const Layout& L, const akv_params& p, const void* arena, size_t arena_bytes, const void* q, void* out, float* out_f32,
@@ -143,6 +161,7 @@ extern std::atomic<int> g_debug_cluster, g_debug_withhold;
 // Timing aid of the decode launch (akv_decode_set_events): events recorded after each of
 // its two launches; both null = off.
 void set_decode_events(void* after_scores, void* after_decode);
+void get_decode_events(void** after_scores, void** after_decode);
 // Device address of the library's static encode scratch on the current device
 // and context (looked up on every call); returns a cudaError_t as int.
 int noalloc_scratch(void** ptr, size_t* bytes);
