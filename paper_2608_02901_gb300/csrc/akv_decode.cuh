@@ -2,43 +2,50 @@
 // Eq. 4: no key or value row is ever rebuilt in memory).  Two launches per call, in stream
 // order (three with a dense suffix, whose chunks take a launch of their own between them):
 //
-// 1. akv_scores_tc_kernel.  The anchor scores S_A[a][g] = q_g . k_a of every anchor of every
-//    unit, once per anchor (Eq. 2-3), in log2 units with sm_scale folded in, into the
-//    workspace, with the largest score per query head of each chunk of 64 anchors: tiles of
-//    128 anchors brought by tensor copies (TMA) into shared memory, products by tcgen05.mma
-//    into tensor memory, one persistent warp-specialised CTA per SM.  It streams the anchor
-//    keys, a fifth of the compressed bytes.  It also writes each unit's query header (the
-//    rotated query q' = H(s o q)/128 of Appendix A.1 Eq. 12, its sums per head, and q' as
-//    tensor-core fragments for the key residuals) and zeroes the unit's arrival counter.
-//    (With RoPE at decode akv_rope_logits_kernel takes its place.)
+// 1. The anchor scores S_A[a][g] = q_g . k_a of every anchor of every unit, once per anchor (Eq. 2-3),
+//    in log2 units with sm_scale folded in, into the workspace, with the largest score per query head of
+//    each chunk of 64 anchors; also each unit's query header (the rotated query q' = H(s o q)/128 of
+//    Appendix A.1 Eq. 12, its sums per head, and q' as tensor-core fragments for the key residuals) and
+//    zeroed arrival counters behind it.  akv_scores_tc_kernel: tiles of 128 anchors brought by tensor
+//    copies (TMA), products by tcgen05.mma into tensor memory, one persistent warp-specialised CTA per SM.
+//    akv_scores_small_kernel, for calls of at most kSmallChunks chunks: one short-lived CTA per chunk, beside
+//    which the decode sets itself up (programmatic dependent launch).  (With RoPE at decode
+//    akv_rope_logits_kernel takes their place.)
 //
 // 2. akv_decode_kernel.  Persistent: one CTA per SM.  The tile blocks of all units, in unit
 //    order, are split into equal contiguous ranges, one per CTA (stream-K): a unit's tiles may
-//    lie in several CTAs and a CTA's range may cross units (its segments).  A CTA has two
-//    groups of four warps; each group takes every other tile of the range, end to end:
-//      staging        the group's warp 0 issues its own tiles into its half of a byte ring of
-//                     shared memory: one bulk asynchronous copy of the tile block and one of
-//                     the anchor-value rows of the value slots the tile covers (the tile
-//                     table records the range), completing a transaction-counted mbarrier;
-//                     table entries are read one issue ahead;
-//      key residuals  q' . c of the tile's staged key records on tensor cores, the terms
-//                     scale (q' . c) + min sum(q') written over the records' own codes;
-//      tokens         each lane 8 consecutive stored tokens, every head: logits
+//    lie in several CTAs and a CTA's range may cross units (its segments).  A CTA has eight token warps
+//    and eight product warps (four warps per SM sub-partition at 128 registers), coupled by mbarriers, which
+//    work on neighbouring tiles at the same time:
+//      copies         a lane of token warp 0 brings the tiles into a byte ring of shared memory: one bulk
+//                     asynchronous copy of the tile block and one of the anchor-value rows of the value
+//                     slots the tile covers (the tile table records the range); table entries are read
+//                     one tile ahead;
+//      key residuals  (product warps, one tile ahead of the values) q' . c of the tile's staged key records
+//                     on tensor cores, the terms scale (q' . c) + min sum(q') written over the records' own
+//                     codes;
+//      tokens         (token warps) each lane 4 consecutive stored tokens, every head: logits
 //                     gamma_i S_A[a(i)] + residual term, p = 2^(l - m), the normaliser, p
 //                     rows of the value records, and the value weights w[a] = sum_i p_i
 //                     gamma_i (Eq. 3): tokens are stored sorted by value anchor, so runs
 //                     inside a lane are summed in registers and stored, and runs across
 //                     lanes merged by a warp segmented scan, without shared atomics;
-//      value side     the value-residual sum (p scale) c over the records and the anchor-
+//      value side     (product warps) the value-residual sum (p scale) c over the records and the anchor-
 //                     value product w^T V_A over the tile's slots, both on tensor cores
-//                     (weights and p scale as bf16 high + low parts, codes exact),
-//                     accumulated in registers across the segment's tiles.
-//    At the end of a segment both groups add their sums into the CTA's shared sums; the group
-//    that finishes last applies the inverse rotation once (Appendix E.1), stores the CTA's
-//    partial numerator and normaliser into its workspace slot for the unit, and counts it in
-//    on the unit's counter; the CTA that completes the count sums the unit's slots in a fixed
+//                     (weights and p scale as bf16 high + low parts, built once per tile as operands in
+//                     place; codes exact), accumulated in registers across the segment's tiles.
+//    At the end of a segment a warp per query head applies the inverse rotation once (Appendix E.1), stores
+//    the CTA's partial numerator and normaliser into its workspace slot for the unit, and counts it in
+//    on the head's counter; the warp that completes the count sums the head's slots in a fixed
 //    order and writes the output.  Tiles denser than the staged counts, and runs on value
 //    slots beyond a tile's staged anchor-value rows, take CUDA-core paths.
+//
+// What bounds the decode (70B shape, 128K: 54 tiles per SM): shared-memory wavefronts (about 3100 per tile, the
+// gathers of score rows by random slots a quarter of them) and issue slots (about 11000 warp instructions
+// per tile), each about half used; the rest is the latency of the phases' dependent chains.  Two groups
+// of four warps that took a tile through all phases (255 registers, two warps per sub-partition) spent
+// 2.8 us per tile pair-wise; token and product warps side by side spend 2.7 us and leave each other's
+// latencies covered where tiles are few (8B shape, 32K: 24.6 -> 18.9 us per call with the small score launch).
 //
 // The exponent reference m is the largest anchor score of each query row.  Anchors are
 // tokens of the unit, so it is a lower bound of the largest logit (sums cannot overflow unless
@@ -71,14 +78,14 @@
 namespace akv {
 namespace {
 
-constexpr int NG = 2;               // tile groups per CTA: tiles in processing at once
-constexpr int WPG = 4;              // warps per group
-constexpr int NCW = NG * WPG;       // warps 0 .. 7; two per SM sub-partition, so 255 registers each
-constexpr int NT = NCW * 32;        // 256 threads
+constexpr int NTW = 8;              // token warps
+constexpr int NMW = 8;              // product warps
+constexpr int NCW = NTW + NMW;      // four per SM sub-partition, so 128 registers each
+constexpr int NT = NCW * 32;        // 512 threads
 constexpr int T = kTile;            // tokens per tile block
-constexpr int LCH = T / (WPG * 32); // consecutive stored tokens per lane
-static_assert(LCH == 8, "a lane's tokens are one byte of a bitmap word");
-constexpr int NSG = 4;              // tiles a group has in flight at most (its stage descriptors)
+constexpr int LCH = T / (NTW * 32); // consecutive stored tokens per lane
+static_assert(LCH == 4, "a lane's tokens are half a byte of a bitmap word and 16 bytes of a stream");
+constexpr int NSG = 6;              // tiles in flight at most (their descriptors)
 // Score launch on tensor cores: a tile of 128 anchors (TMEM lanes) x 16 query rows (columns),
 // anchor rows and query rows brought by tensor copies into two 128-byte halves each
 constexpr int kScTile = 128;
@@ -93,8 +100,9 @@ constexpr uint32_t kScTmemCols = 32;                     // two accumulators of 
 // Instruction descriptor of kind::f16: fp32 accumulator (bits 4-5 = 1), bf16 A and B (7-9 = 1,
 // 10-12 = 1), both K-major (15, 16 = 0), N / 8 (17-22), M / 16 (24-28).
 constexpr uint32_t kScIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((16u >> 3) << 17) | ((uint32_t)(kScTile >> 4) << 24);
-constexpr int kEnds = 2 * WPG;       // a tile's runs that may go on in a neighbour warp: each warp's first and last
+constexpr int kEnds = 2 * NTW;       // a tile's runs that may go on in a neighbour warp: each warp's first and last
 constexpr int kOvl = 32;            // a tile's entries per overflow list (value records, anchor-value runs)
+constexpr int kOvlBytes = 16 + 2 * kOvl * 9 * 4;  // a tile's two lists: counts, then entries
 constexpr int kRingSlack = 4096;    // shared memory after the ring: the masked rows of the last
                                     // 16-row block of staged anchor values are read from here
 constexpr float kLog2e = 1.4426950408889634f;
@@ -110,7 +118,6 @@ struct ScoreParams {
   unsigned long long sign_lo, sign_hi;
   float* sa;      // [units][ka_stride][G] anchor scores (log2 units)
   float* cmax;    // [units][n_ch][G] largest score of each chunk of CHA anchors
-  unsigned* cnt;  // [units] arrival counters of the decode launch, zeroed here
   int n_kv_heads, n_q_heads, G, ka_stride, n_ch;
   float scale_log2;
   // dense suffix (null ksuf: none): rows [units][suf_cap][128], lengths per request, n_sch
@@ -132,15 +139,34 @@ struct RopeParams {
   const __nv_bfloat16* q;
   float* lg;      // [units][s_stride][G] logits (log2 units, sm_scale folded in), stored order
   float* cmax;    // [units][n_tch][G] largest logit of each chunk of 64 stored tokens
-  unsigned* cnt;  // [units] arrival counters of the decode launch, zeroed here
+  const uint8_t* uh;  // query headers: only their arrival counters are used (zeroed here)
+  int uh_stride;
   int n_kv_heads, n_q_heads, rotate, lloyd, s_stride, n_tch;
   float scale_log2;
   unsigned long long sign_lo, sign_hi;
   unsigned long long turn[64];  // theta_j / (2 pi) as a 64-bit binary fraction of a turn
 };
 
-struct Meta {  // a staged tile, as the producer recorded it
-  uint32_t ring_off, blk_off, blk_bytes, staged, lo, nrows, j, pad;
+struct __align__(16) Meta {  // a staged tile: as it was copied, then its shape (product warp 0, before the key terms are announced)
+  uint32_t ring_off, blk_off, staged, lo, nrows, j, bytes, pad;
+  uint32_t sm_v, cd_k, cd_v, sm_k;  // byte offsets of scales and codes in the block
+  int n, nKs, nVs;                  // tokens; key records with terms, value records on tensor cores
+  uint32_t fast;                    // every record and anchor-value row staged: the token path without rare cases; bit 1: value records staged
+};
+struct Seg {  // a CTA's tiles of one unit
+  int u, jb, je, ib;  // unit, its tiles [jb, je), CTA-local index of tile jb
+  long long t0;       // global index of the unit's tile 0
+  int nt, first, nseg, pad;
+};
+// What the copying lane keeps (in shared memory: no register of the other threads waits for it).
+struct Prod {
+  Seg s;                      // segment of the next tile to copy
+  const uint8_t *tiles, *av;  // its unit's tile blocks, anchor values,
+  const uint32_t* table;      // tile table
+  int end;                    // CTA-local index past the segment
+  int ii;                     // CTA-local index of the next tile to copy: so many are issued
+  int nrel;                   // tiles released
+  uint32_t head, used;        // ring bytes: next free place, bytes in flight
 };
 
 struct DecodeParams {
@@ -151,8 +177,7 @@ struct DecodeParams {
   const float* sa;
   const float* cmax;
   float* part;
-  unsigned* cnt;
-  const uint8_t* uh;  // query headers (score kernel)
+  const uint8_t* uh;  // query headers (score launch), each with its unit's arrival counters behind it
   int uh_stride;
   long long ttot;  // tiles of all units
   int grid, n_kv_heads, n_q_heads, rotate, ka_stride, n_ch;
@@ -162,8 +187,7 @@ struct DecodeParams {
   int X;           // anchor-value rows per tile that are staged (the weight table's rows)
   int cap;         // staged bytes of a tile block at most
   int ring_bytes, drop_last, smem_sa;
-  int o_bar, o_meta, o_misc, o_sa, o_ovf, o_grp, grp_bytes, o_ring;
-  int g_qp, g_rows, g_red, g_wb, g_vs, g_sum, g_pv, g_qf, g_ovl;  // offsets inside a group's block
+  int o_bar, o_meta, o_misc, o_sa, o_ovf, o_qp, o_rows, o_gsum, o_wb, o_vs, o_pv, o_ovl, o_prod, o_ring;
   const float* lg;         // RoPE at decode: logits [units][s_stride][G] in stored order (else null)
   int s_stride;
   const float* suf_part;   // dense suffix partials [units][n_sch][suf_floats] (null: no suffix)
@@ -326,34 +350,18 @@ __device__ __forceinline__ size_t qrow_base(int u, int n_kv_heads, int n_q_heads
   return ((size_t)b * n_q_heads + (size_t)h * G) * 128;
 }
 
-// Sections of one unit.
-struct UnitView {
-  int S, k, nt;
-  const uint8_t* AV;
-  const uint32_t* table;  // [nt + 1] block offsets, then [nt] value-slot ranges
-  const uint8_t* tiles;
-};
-__device__ __forceinline__ UnitView unit_view(const uint8_t* A, int u) {
-  const akv_unit_desc* d = unit_desc(A, u);
-  UnitView v;
-  v.S = d->len;
-  v.k = d->n_anchors;
-  v.nt = d->n_tiles;
-  v.AV = A + d->off_anchor_v;
-  v.table = reinterpret_cast<const uint32_t*>(A + d->off_tile_table);
-  v.tiles = A + d->off_tiles;
-  return v;
-}
-
 // Geometry of one staged tile block: the first `staged` bytes are in shared memory, the
 // rest is read from global memory (a tile with more records than the stage holds).
 struct TileView {
   const uint8_t* st;   // stage
-  const uint8_t* gb;   // the block in global memory
+  uint32_t blk_off;    // the block in global memory, from the unit's tiles
   uint32_t staged;
+  int u;
   int n, nw, n64, nk, nv;
   uint32_t sm_k, sm_v, cd_k, cd_v;  // byte offsets of scales and codes in the block
-  __device__ __forceinline__ const uint8_t* at(uint32_t off) const { return off < staged ? st + off : gb + off; }
+  // (the descriptor is read again where a byte past the stage is wanted: rare, and no register waits for it)
+  __device__ __forceinline__ const uint8_t* gb(const uint8_t* A) const { return A + unit_desc(A, u)->off_tiles + blk_off; }
+  __device__ __forceinline__ const uint8_t* at(const uint8_t* A, uint32_t off) const { return off < staged ? st + off : gb(A) + off; }
   __device__ __forceinline__ uint64_t bm(int side, int w) const {
     return reinterpret_cast<const uint64_t*>(st + 8 * n64)[side * nw + w];
   }
@@ -361,12 +369,14 @@ struct TileView {
     return reinterpret_cast<const uint16_t*>(st + 8 * n64 + 16 * nw + side * round16(2u * nw))[w];
   }
 };
-__device__ __forceinline__ TileView tile_view(const uint8_t* st, const Meta& mt, const UnitView& U) {
+// The shape of a tile from its bitmaps and rank words.
+__device__ __forceinline__ TileView tile_view(const uint8_t* st, const Meta& mt, int u, int S) {
   TileView v;
   v.st = st;
-  v.gb = U.tiles + mt.blk_off;
+  v.blk_off = mt.blk_off;
   v.staged = mt.staged;
-  v.n = min(T, U.S - (int)mt.j * T);
+  v.u = u;
+  v.n = min(T, S - (int)mt.j * T);
   v.nw = (int)tile_words(v.n);
   v.n64 = 64 * v.nw;
   v.nk = v.rk(0, v.nw - 1) + __popcll(v.bm(0, v.nw - 1));
@@ -376,6 +386,23 @@ __device__ __forceinline__ TileView tile_view(const uint8_t* st, const Meta& mt,
   v.sm_v = F + round16(4u * (uint32_t)v.nk);
   v.cd_k = v.sm_v + round16(4u * (uint32_t)v.nv);
   v.cd_v = v.cd_k + 32u * (uint32_t)v.nk;
+  return v;
+}
+// The same as product warp 0 left it in the tile's descriptor.
+__device__ __forceinline__ TileView tile_view(const uint8_t* st, const Meta& mt, int u) {
+  TileView v;
+  v.st = st;
+  v.blk_off = mt.blk_off;
+  v.staged = mt.staged;
+  v.u = u;
+  v.n = mt.n;
+  v.nw = (int)tile_words(v.n);
+  v.n64 = 64 * v.nw;
+  v.nk = v.nv = 0;  // (not kept)
+  v.sm_k = mt.sm_k;
+  v.sm_v = mt.sm_v;
+  v.cd_k = mt.cd_k;
+  v.cd_v = mt.cd_v;
   return v;
 }
 
@@ -654,8 +681,14 @@ __device__ __forceinline__ void suffix_chunk(const ScoreParams& P, int u, int sc
 template <int GS, bool ROPE>
 __global__ void __launch_bounds__(128) akv_suffix_kernel(const ScoreParams P) {
   extern __shared__ __align__(16) uint8_t score_dyn[];  // the chunk's value rows
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (a decode that waits for it where it needs it)
   suffix_chunk<GS, ROPE>(P, blockIdx.x / P.n_sch, blockIdx.x % P.n_sch,
                          reinterpret_cast<__nv_bfloat16 (*)[128]>(score_dyn));
+}
+
+// The arrival counters of unit u's query heads, behind its query header.
+__device__ __forceinline__ unsigned* unit_counters(const uint8_t* uh, int uh_stride, int u, int GS) {
+  return reinterpret_cast<unsigned*>(const_cast<uint8_t*>(uh) + (size_t)u * uh_stride + hdr_bytes(GS));
 }
 
 // The unit's query header, by one warp: the rotated query q' = H(s o q) / 128 scaled to log2 units
@@ -857,7 +890,7 @@ __global__ void __launch_bounds__(kScThreads) akv_scores_tc_kernel(const __grid_
   } else if (warp == 5) {  // ---- query headers
     for (int T = (int)blockIdx.x; T < n_tiles; T += (int)gridDim.x) {
       if (T % P.n_t) continue;
-      if (lane == 0) P.cnt[T / P.n_t] = 0u;
+      if (lane < 8) unit_counters(P.uh, P.uh_stride, T / P.n_t, GS)[lane] = 0u;
       unit_query_header_warp<GS>(P, T / P.n_t, hdr_q);
     }
   } else {  // ---- epilogue, warps 0-3
@@ -919,100 +952,139 @@ __global__ void __launch_bounds__(kScThreads) akv_scores_tc_kernel(const __grid_
   if (warp == 0) tc_dealloc(tmem, kScTmemCols);
 }
 
-// ============================ the unit's output ====================================
-// Sum of the unit's partial slots in a fixed order (CTAs, then groups and the overflow slot),
-// the inverse rotation of the value-residual part once, the normalisation, bf16 RNE output.
-// Run by nw warps (index widx); warp widx takes heads widx, widx + nw, ...
+// Anchor scores of small calls: CTA b < units writes unit b's query header and zeroes its counters; the others
+// take 64 anchors of a unit each (warp w rows 16 w .. 16 w + 15), straight from global memory into bf16 mma A
+// fragments (rows are stored swizzled in 16-byte chunks by slot % 8; the k order is permuted the same way in
+// A and B, so that a thread's dims are contiguous).  It holds no tensor memory and little else, so it starts
+// and ends in about 3 us where the persistent launch above takes 7 us whatever its size (8 x 656 anchors),
+// and the decode, its programmatic dependent, sets itself up beside it.
 template <int GS>
-__device__ void combine_unit(const DecodeParams& P, int u, int first, int nseg, int widx, int nw) {
-  const int lane = threadIdx.x & 31;
-  constexpr int PF = part_floats(GS);
-  const size_t ob = qrow_base(u, P.n_kv_heads, P.n_q_heads);
-  auto slot = [&](int s) { return P.part + (size_t)(first + s + u) * PF; };  // CTA first + s
-  // normalisers and failure flags of every slot: lanes in parallel, then a fixed-order reduction
-  float Lh[GS];
-#pragma unroll
-  for (int g = 0; g < GS; ++g) Lh[g] = 0.f;
-  bool bad = false;
-  for (int s = lane; s < nseg; s += 32) {
-    const float* sp = slot(s);
-    bad |= __ldcg(sp + part_flag(GS)) != 0.f;
-#pragma unroll
-    for (int g = 0; g < GS; ++g) Lh[g] += __ldcg(sp + part_l(GS) + g);
+__global__ void __launch_bounds__(128) akv_scores_small_kernel(const ScoreParams P) {
+  __shared__ __align__(16) float hdr_q[8 * 128];
+  __shared__ float wm[4][8];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, r8 = lane >> 2, c4 = lane & 3;
+  if ((int)blockIdx.x < P.units) {
+    if (tid < 8) unit_counters(P.uh, P.uh_stride, blockIdx.x, GS)[tid] = 0u;
+    if (warp == 0) unit_query_header_warp<GS>(P, blockIdx.x, hdr_q);
+    return;
   }
-  bad = __any_sync(0xffffffffu, bad);
+  const int u = ((int)blockIdx.x - P.units) / P.n_ch, ch = ((int)blockIdx.x - P.units) % P.n_ch;
+  const akv_unit_desc* d = unit_desc(P.arena, u);
+  const int k = d->n_anchors;
+  if (ch * CHA >= k) return;
+  const uint64_t off = d->off_anchor_k;
+  const bool inside = (long long)(off >> 8) + k <= P.arena_rows;
+  const uint8_t* AK = P.arena + off;
+  const size_t qb = qrow_base(u, P.n_kv_heads, P.n_q_heads);
+  uint2 bq[8];
 #pragma unroll
-  for (int g = 0; g < GS; ++g) Lh[g] = warp_sum(Lh[g]);
-  for (int h = widx; h < GS; h += nw) {
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s0 = 0; s0 < nseg; s0 += 8) {  // eight slots' loads in flight at a time
-      float4 xa[8];
+  for (int ks = 0; ks < 8; ++ks)
+    bq[ks] = r8 < GS ? *reinterpret_cast<const uint2*>(P.q + qb + (size_t)r8 * 128 + 32 * (ks >> 1) + 8 * c4 + 4 * (ks & 1))
+                     : make_uint2(0u, 0u);
+  const int g0 = 2 * c4, a0 = ch * CHA + 16 * warp + r8;
+  const int ra = inside ? min(a0, k - 1) : 0, rb = inside ? min(a0 + 8, k - 1) : 0;
+  uint4 lo[4] = {}, hi[4] = {};
+  if (inside) {
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        xa[j] = s0 + j < nseg ? __ldcg(reinterpret_cast<const float4*>(slot(s0 + j) + h * 128 + 4 * lane))
-                              : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        a.x += xa[j].x; a.y += xa[j].y; a.z += xa[j].z; a.w += xa[j].w;
-      }
+    for (int j = 0; j < 4; ++j) {
+      lo[j] = ldg_stream(AK + (size_t)ra * 256 + 16 * ((4 * j + c4) ^ (ra & 7)));
+      hi[j] = ldg_stream(AK + (size_t)rb * 256 + 16 * ((4 * j + c4) ^ (rb & 7)));
     }
-    float L = 0.f;
-#pragma unroll
-    for (int g = 0; g < GS; ++g)
-      if (g == h) L = Lh[g];
-    if (P.suf_part) {  // the dense suffix joins the same softmax (Appendix E.1 and E.2)
-      const int len = max(0, min(P.suf_len[u / P.n_kv_heads], P.suf_cap));
-      if (len > 0) {
-        // the compressed part's reference m (the unit's largest anchor score), the common maximum
-        // M over it and the chunks' maxima, and every part rescaled to M
-        // (with RoPE at decode: the chunk maxima are those of every token's logit)
-        const int nch = P.lg ? (unit_desc(P.arena, u)->len + 63) / 64 : (unit_desc(P.arena, u)->n_anchors + CHA - 1) / CHA;
-        float m = -INFINITY;
-        for (int ch = lane; ch < nch; ch += 32) m = fmaxf(m, P.cmax[((size_t)u * P.n_ch + ch) * GS + h]);
-        m = warp_max(m);
-        const float* sp0 = P.suf_part + (size_t)u * P.n_sch * suf_floats(GS);
-        const int nsc = (len + SCH - 1) / SCH;
-        float M = m;
-        for (int c = lane; c < nsc; c += 32) M = fmaxf(M, sp0[(size_t)c * suf_floats(GS) + suf_m(GS) + h]);
-        M = warp_max(M);
-        const float f0 = exp2_approx(m - M);
-        a.x *= f0;
-        a.y *= f0;
-        a.z *= f0;
-        a.w *= f0;
-        L *= f0;
-        for (int c = 0; c < nsc; ++c) {
-          const float* sp = sp0 + (size_t)c * suf_floats(GS);
-          const float f = exp2_approx(sp[suf_m(GS) + h] - M);
-          const float4 o = *reinterpret_cast<const float4*>(sp + h * 128 + 4 * lane);
-          a.x = fmaf(f, o.x, a.x);
-          a.y = fmaf(f, o.y, a.y);
-          a.z = fmaf(f, o.z, a.z);
-          a.w = fmaf(f, o.w, a.w);
-          L = fmaf(f, sp[suf_l(GS) + h], L);
-        }
-      }
-    }
-    const bool badh = bad || !(L < INFINITY);  // a logit so far above the reference that the sums overflowed
-    const float yv[4] = {a.x, a.y, a.z, a.w};
-    const size_t o = ob + (size_t)h * 128 + 4 * lane;
-    float y[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) y[e] = badh ? __int_as_float(0x7FC00000) : yv[e] / L;
-    *reinterpret_cast<uint2*>(P.out + o) = make_uint2(pack_b2(__float2bfloat16_rn(y[0]), __float2bfloat16_rn(y[1])),
-                                                      pack_b2(__float2bfloat16_rn(y[2]), __float2bfloat16_rn(y[3])));
-    if (P.out_f32) *reinterpret_cast<float4*>(P.out_f32 + o) = make_float4(y[0], y[1], y[2], y[3]);
   }
+  float dd[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    mma_bf16(dd, lo[j].x, hi[j].x, lo[j].y, hi[j].y, bq[2 * j].x, bq[2 * j].y);
+    mma_bf16(dd, lo[j].z, hi[j].z, lo[j].w, hi[j].w, bq[2 * j + 1].x, bq[2 * j + 1].y);
+  }
+  float mx0 = -INFINITY, mx1 = -INFINITY;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int a = a0 + 8 * h;
+    if (a >= k || g0 >= GS) continue;
+    const float v0 = dd[2 * h] * P.scale_log2, v1 = dd[2 * h + 1] * P.scale_log2;
+    float* t = P.sa + (size_t)u * P.ka_stride * GS + sa_at<GS>(a, g0, P.ka_stride);
+    if constexpr (GS == 1) t[0] = v0;
+    else *reinterpret_cast<float2*>(t) = make_float2(v0, v1);
+    mx0 = fmaxf(mx0, v0);
+    mx1 = fmaxf(mx1, v1);
+  }
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) {
+    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, o));
+    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, o));
+  }
+  if (lane < 4) {
+    wm[warp][2 * lane] = mx0;
+    wm[warp][2 * lane + 1] = mx1;
+  }
+  __syncthreads();
+  if (tid < GS)  // (rows outside the arena: the unit's outputs become NaN)
+    P.cmax[((size_t)u * P.n_ch + ch) * GS + tid] =
+        inside ? fmaxf(fmaxf(wm[0][tid], wm[1][tid]), fmaxf(wm[2][tid], wm[3][tid])) : INFINITY;
 }
 
-// Counts one slot of unit u in (after this thread's group stored it); true if it completed the
-// unit, whose slots the caller then combines.
-__device__ __forceinline__ bool count_in(const DecodeParams& P, int u, int nseg) {
-  __threadfence();
-  const unsigned old = atomicAdd(P.cnt + u, 1u);
-  const bool last = old == (unsigned)(nseg - 1);
-  if (last) __threadfence();
-  return last;
+// ============================ the unit's output ====================================
+// One query head of unit u, by a warp: the sum of its partial slots in a fixed order, the dense suffix's chunks
+// (m: the unit's reference), the normalisation, bf16 RNE output.  A CTA that failed left a NaN normaliser.
+template <int GS>
+__device__ __noinline__ void combine_head(const DecodeParams& P, int u, int first, int nseg, int h, float m) {
+  const int lane = threadIdx.x & 31;
+  constexpr int PF = part_floats(GS);
+  auto slot = [&](int s) { return P.part + (size_t)(first + s + u) * PF; };  // CTA first + s
+  float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+  float L = 0.f;
+  for (int s0 = 0; s0 < nseg; s0 += 16) {  // sixteen slots' loads in flight at a time, their normalisers with them
+    const float l = lane < 16 && s0 + lane < nseg ? __ldcg(slot(s0 + lane) + part_l(GS) + h) : 0.f;
+    float4 xa[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      xa[j] = s0 + j < nseg ? __ldcg(reinterpret_cast<const float4*>(slot(s0 + j) + h * 128 + 4 * lane))
+                            : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      a.x += xa[j].x; a.y += xa[j].y; a.z += xa[j].z; a.w += xa[j].w;
+    }
+    L += warp_sum(l);
+  }
+  if (P.suf_part) {  // the dense suffix joins the same softmax (Appendix E.1 and E.2)
+    const int len = max(0, min(P.suf_len[u / P.n_kv_heads], P.suf_cap));
+    if (len > 0) {
+      // the compressed part's reference m, the common maximum M over it and the chunks' maxima, and every
+      // part rescaled to M
+      const float* sp0 = P.suf_part + (size_t)u * P.n_sch * suf_floats(GS);
+      const int nsc = (len + SCH - 1) / SCH;
+      float M = m;
+      for (int c = lane; c < nsc; c += 32) M = fmaxf(M, sp0[(size_t)c * suf_floats(GS) + suf_m(GS) + h]);
+      M = warp_max(M);
+      const float f0 = exp2_approx(m - M);
+      a.x *= f0;
+      a.y *= f0;
+      a.z *= f0;
+      a.w *= f0;
+      L *= f0;
+      for (int c = 0; c < nsc; ++c) {
+        const float* sp = sp0 + (size_t)c * suf_floats(GS);
+        const float f = exp2_approx(sp[suf_m(GS) + h] - M);
+        const float4 o = *reinterpret_cast<const float4*>(sp + h * 128 + 4 * lane);
+        a.x = fmaf(f, o.x, a.x);
+        a.y = fmaf(f, o.y, a.y);
+        a.z = fmaf(f, o.z, a.z);
+        a.w = fmaf(f, o.w, a.w);
+        L = fmaf(f, sp[suf_l(GS) + h], L);
+      }
+    }
+  }
+  const bool bad = !(L < INFINITY);  // a failure, or a logit so far above the reference that the sums overflowed
+  const float yv[4] = {a.x, a.y, a.z, a.w};
+  const size_t o = qrow_base(u, P.n_kv_heads, P.n_q_heads) + (size_t)h * 128 + 4 * lane;
+  float y[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) y[e] = bad ? __int_as_float(0x7FC00000) : yv[e] / L;
+  *reinterpret_cast<uint2*>(P.out + o) = make_uint2(pack_b2(__float2bfloat16_rn(y[0]), __float2bfloat16_rn(y[1])),
+                                                    pack_b2(__float2bfloat16_rn(y[2]), __float2bfloat16_rn(y[3])));
+  if (P.out_f32) *reinterpret_cast<float4*>(P.out_f32 + o) = make_float4(y[0], y[1], y[2], y[3]);
 }
 
 // Probabilities of one token for every head: p_g = 2^(gamma S_A[a][g] + rt_g) (rt: the key-residual
@@ -1055,7 +1127,7 @@ __global__ void __launch_bounds__(128) akv_rope_logits_kernel(const RopeParams P
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const akv_unit_desc* d = unit_desc(P.arena, u);
   const int S = d->len, k = d->n_anchors;
-  if (c == 0 && tid == 0) P.cnt[u] = 0u;
+  if (c == 0 && tid < 8) unit_counters(P.uh, P.uh_stride, u, GS)[tid] = 0u;
   const int ts0 = 64 * c;
   if (ts0 >= S) return;  // past this unit's end (a shorter request)
   const size_t qb = qrow_base(u, P.n_kv_heads, P.n_q_heads);
@@ -1226,6 +1298,7 @@ struct TokLane {
 // What the general token path reads of its tile.
 struct TokTile {
   TileView tv;
+  const uint8_t* gb;  // the block in global memory
   uint32_t lo, nrows;
   const float* SAt;   // anchor scores [k][GS]
   const float* rows;  // [0,8): -m, [8,16): -inf, [16,24): sum q'
@@ -1258,7 +1331,7 @@ __device__ __noinline__ LShare<(GS >= 2 ? GS / 2 : 1)> token_chunk_general(const
   const TokLane tl = tl_arg;
   const TileView tv = tt.tv;
   const uint8_t* st = tv.st;
-  const uint8_t* gb = tv.gb;
+  const uint8_t* gb = tt.gb;
   const uint32_t staged = tv.staged;
   const int t0 = tl.t0;
   const int nvalid = min(LCH, tv.n - t0);
@@ -1387,56 +1460,52 @@ __device__ __noinline__ LShare<(GS >= 2 ? GS / 2 : 1)> token_chunk_general(const
 
 // ================================ decode ============================================
 // CODEC: 0 = uniform codes (c^ = min + c scale), 1 = Lloyd-Max levels (c^ = scale L[c]).
-// ROPE: 1 = pre-RoPE keys: every token's logit comes from the RoPE logits launch (P.lg) instead
-// of gamma S_A plus its key-residual term; the key-residual phase has nothing to do.
-template <int GS, int CODEC, int ROPE>
+// MODE: where a unit's anchor scores are.  kTableSmem: copied from the score launch into shared memory;
+// kTableGlobal: read from global memory where the score launch left them; kRope: pre-RoPE keys, every
+// token's logit comes from the RoPE logits launch (P.lg) instead of gamma S_A plus its key-residual
+// term, and the key-residual phase has nothing to do.
+enum Mode { kTableSmem = 0, kTableGlobal = 1, kRope = 2 };
+template <int GS, int CODEC, int MODE>
 __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P) {
   extern __shared__ __align__(128) uint8_t smem[];
   constexpr int NP = GS >= 2 ? GS / 2 : 1;      // pairs of heads for the packed arithmetic
-  constexpr int HPL = GS >= 2 ? GS / 2 : 1;     // heads per lane when building value operands
+  constexpr bool ROPE = MODE == kRope, TABLE = MODE == kTableSmem;
   constexpr int PF = part_floats(GS);
+  constexpr int NBF = GS == 8 ? 2 : 1;  // key-residual fragment sets: GS = 8 keeps high and low parts apart
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int c4 = lane & 3, r8 = lane >> 2;
   const int c = blockIdx.x;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + P.o_bar);
   Meta* meta = reinterpret_cast<Meta*>(smem + P.o_meta);
   volatile int* failed = reinterpret_cast<volatile int*>(smem + P.o_misc);
+  Seg* sg = reinterpret_cast<Seg*>(smem + P.o_misc + 16);  // the segment in work
   float* SAs = reinterpret_cast<float*>(smem + P.o_sa);
   float* ovf = reinterpret_cast<float*>(smem + P.o_ovf);  // [2][GS][128]: anchor-value and value-residual overflow sums
+  float* qp = reinterpret_cast<float*>(smem + P.o_qp);    // [GS][128] rotated query q'; at a segment's end its sums [2][GS][128]
+  float* sq = qp + GS * 128;                              // [8] sums of q' per head
+  uint2* qf = reinterpret_cast<uint2*>(sq + 8);           // [NBF][8][32] key-residual B fragments
+  float* rows = reinterpret_cast<float*>(smem + P.o_rows);  // [0,8): -m, [8,16): -inf, [24,32): m
+  float* gsum = reinterpret_cast<float*>(smem + P.o_gsum);  // [8][8] normaliser per token warp, then [8][8] sum of p min per product warp
   uint8_t* ring = smem + P.o_ring;
-  // per group and slot: a tile block and its anchor-value rows landed (full); per unit: its
-  // anchor-score table landed (sa_full; a plain arrival when the table stays in global memory)
-  auto bar_full = [&](int g, int s) { return smem_u32(bars + g * NSG + s); };
-  const uint32_t bar_sa_full = smem_u32(bars + NG * NSG);
-  auto bar_hdr = [&](int g) { return smem_u32(bars + NG * NSG + 1 + g); };  // a group's query header landed
-  int* segcnt = reinterpret_cast<int*>(smem + P.o_misc + 4);  // groups done with a segment, in total
-
-  if (tid == 0) {
-    for (int s = 0; s < NG * NSG + 1 + NG; ++s) mbar_init(smem_u32(bars + s), 1);
-    *failed = 0;
-    *segcnt = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  for (int e = tid; e < 2 * GS * 128; e += NT) ovf[e] = 0.f;  // (the overflow's sums start at zero)
-  // zeroed p rows: rows past a tile's records are read (and multiplied by zero codes)
-  for (int gi = 0; gi < NG; ++gi) {
-    float* pvz = reinterpret_cast<float*>(smem + P.o_grp + gi * P.grp_bytes + P.g_pv);
-    for (int e = tid; e < P.R * 8; e += NT) pvz[e] = 0.f;
-  }
-  __syncthreads();
+  // per slot: a tile block and its anchor-value rows landed, and its place is free again; per tile parity: its key
+  // terms are written, its tokens are done; per unit: query header and score table landed
+  auto bar_full = [&](int s) { return smem_u32(bars + s); };
+  auto bar_empty = [&](int s) { return smem_u32(bars + NSG + s); };
+  auto bar_kdone = [&](int b) { return smem_u32(bars + 2 * NSG + b); };
+  auto bar_tdone = [&](int b) { return smem_u32(bars + 2 * NSG + 2 + b); };
+  const uint32_t bar_hdr = smem_u32(bars + 2 * NSG + 4), bar_sa_full = smem_u32(bars + 2 * NSG + 5);
 
   // This CTA's range of the concatenated tiles, walked as segments (one per unit it touches).
-  const long long B0 = (long long)c * P.ttot / P.grid, B1 = (long long)(c + 1) * P.ttot / P.grid;
-  struct Seg {
-    int u, jb, je, ib;  // unit, its tiles [jb, je), CTA-local index of tile jb
-    long long t0;       // global index of the unit's tile 0
-    int nt, first, nseg;
-  };
+  // (products of tile indexes and CTAs stay below 2^32 for all but the largest calls: 32-bit divisions)
+  const bool small = (unsigned long long)P.ttot * (unsigned)P.grid < (1ull << 32);
+  auto quot = [&](long long x, long long y) -> long long { return small ? (long long)((unsigned)x / (unsigned)y) : x / y; };
+  const long long B0 = quot((long long)c * P.ttot, P.grid), B1 = quot((long long)(c + 1) * P.ttot, P.grid);
+  const int n_cta_tiles = (int)(B1 - B0);
   auto seg_fill = [&](Seg& s) {
     s.nt = unit_desc(P.arena, s.u)->n_tiles;
     s.je = (int)min((long long)s.nt, B1 - s.t0);
-    s.first = (int)(((s.t0 + 1) * P.grid - 1) / P.ttot);
-    s.nseg = (int)(((s.t0 + s.nt) * P.grid - 1) / P.ttot) - s.first + 1;
+    s.first = (int)quot((s.t0 + 1) * P.grid - 1, P.ttot);
+    s.nseg = (int)quot((s.t0 + s.nt) * P.grid - 1, P.ttot) - s.first + 1;
   };
   auto seg_begin = [&](Seg& s) {
     s.u = P.cta_unit[c];
@@ -1445,31 +1514,26 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
     s.ib = 0;
     seg_fill(s);
   };
-  auto seg_next = [&](Seg& s) -> bool {  // false past the last segment
-    if (s.t0 + s.je >= B1) return false;
+  auto seg_next = [&](Seg& s) {  // (not past the last segment)
     s.ib += s.je - s.jb;
     s.t0 += s.nt;
     ++s.u;
     s.jb = 0;
     seg_fill(s);
-    return true;
   };
-
-  // the first unit's anchor-score table and both groups' copies of its query header (later units: the
-  // group that finishes the previous unit last, which has read the sums kept where the headers go)
+  // The unit's query header, and its anchor-score table where it comes from the score launch (one thread;
+  // the sums kept where the header goes have been read).
   auto start_unit = [&](int u) {
     const int k = unit_desc(P.arena, u)->n_anchors;
     const bool ok = !*failed;
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    for (int g = 0; g < NG; ++g) {
-      if (ok && !ROPE) {  // (RoPE: no key-side header is needed)
-        mbar_expect_tx(bar_hdr(g), (uint32_t)hdr_bytes(GS));
-        bulk_g2s(smem_u32(smem + P.o_grp + g * P.grp_bytes + P.g_qp), P.uh + (size_t)u * P.uh_stride, (uint32_t)hdr_bytes(GS), bar_hdr(g));
-      } else {
-        mbar_arrive(bar_hdr(g));
-      }
+    if (ok && !ROPE) {  // (RoPE: no key-side header is needed)
+      mbar_expect_tx(bar_hdr, (uint32_t)hdr_bytes(GS));
+      bulk_g2s(smem_u32(qp), P.uh + (size_t)u * P.uh_stride, (uint32_t)hdr_bytes(GS), bar_hdr);
+    } else {
+      mbar_arrive(bar_hdr);
     }
-    if (P.smem_sa && ok) {
+    if (MODE == kTableSmem && ok) {
       const float* src = P.sa + (size_t)u * P.ka_stride * GS;
       if (GS == 8) {  // the two four-head arrays, k rows of each
         const uint32_t half = 16u * (uint32_t)k;
@@ -1485,650 +1549,707 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
       mbar_arrive(bar_sa_full);  // the unit's start, for the warps that wait on it
     }
   };
-  if (tid == 0) start_unit(P.cta_unit[c]);
-  const int n_cta_tiles = (int)(B1 - B0);
 
-  // =========================== compute groups ==================================
-  const int grp = warp / WPG, wg = warp % WPG, gt = tid - grp * WPG * 32;
-  uint8_t* GB = smem + P.o_grp + grp * P.grp_bytes;
-  float* qp = reinterpret_cast<float*>(GB + P.g_qp);      // [GS][128] rotated query q'
-  float* sq = qp + GS * 128;                              // [8] sums of q' per head
-  float* rows = reinterpret_cast<float*>(GB + P.g_rows);  // [0,8): -m, [8,16): -inf, [24,32): m
-  int* lastf = reinterpret_cast<int*>(GB + P.g_red);
-  float* wb = reinterpret_cast<float*>(GB + P.g_wb);      // [2][X + kEnds][GS] value weights of a tile's slots, then of the warps' first and last runs
-  int* vsl = reinterpret_cast<int*>(GB + P.g_vs);          // [2][kEnds] the slots of those, from the tile's first (-1: none)
-  float* gsum = reinterpret_cast<float*>(GB + P.g_sum);   // [WPG][16] a segment's normaliser and sum of p min per warp and head
-  float* pv = reinterpret_cast<float*>(GB + P.g_pv);      // [R][8] p rows of the value records, then A operands
-  int* ovl_n = reinterpret_cast<int*>(GB + P.g_ovl);       // [2] entries in the two overflow lists
-  float* ovl = reinterpret_cast<float*>(GB + P.g_ovl + 16);  // [2][kOvl][9]: index bits, then p (or weights) per head
-  uint2* qf = reinterpret_cast<uint2*>(GB + P.g_qf);      // [NBF][8][32] key-residual B fragments
-  const int bar_id = 1 + grp;
-  auto gsync = [&]() { named_sync(bar_id, WPG * 32); };
-  constexpr int NBF = GS == 8 ? 2 : 1;  // key-residual fragment sets: GS = 8 keeps high and low parts apart
-
-  float accA[4][4], accR[4][4];  // anchor-value and value-residual sums, dims 32 wg .. 32 wg + 31
-  float2 l2[NP];
-  float pminv[HPL];
-  int lt = 0;  // this group's tiles so far (weight-table buffer parity, stage descriptor)
-
-  // ---- the group as its own producer (warp wg = 0; lane 0 issues the copies) ----
-  // Its tiles are the CTA's tiles i = grp, grp + NG, ...; each goes, with the anchor-value rows
-  // of the value slots it covers, into this group's half of the ring, oldest first: the tile
-  // table entries of the next tile to issue are read one issue ahead, so a copy never waits on
-  // a global load.
-  const uint32_t RH = ((uint32_t)P.ring_bytes / NG) & ~127u, rbase = (uint32_t)grp * RH;  // 128-byte aligned halves
-  Meta* gmeta = meta + grp * NSG;
-  Seg si{};                       // segment of the next tile to issue
-  int ii = grp;                   // CTA-local index of the next tile to issue
-  int nis = 0, nrel = 0;          // tiles issued, tiles released (group-local)
-  uint32_t head = 0, used = 0;    // ring bytes: next free place, bytes in flight
-  uint32_t pe0 = 0, pe1 = 0, pe2 = 0;  // table entries of tile ii: block offset, next offset, slot range
-  int pj = 0;
-  const uint8_t* ptiles = nullptr;
-  const uint8_t* pav = nullptr;
-  auto prefetch = [&]() {
+  // ---- copies: lane 0 of token warp 0.  Each tile goes, with the anchor-value rows of the value slots it
+  // covers, into the ring, oldest first, as places come free; the table entries of the next tile are read
+  // one tile ahead ----
+  Prod* pr = reinterpret_cast<Prod*>(smem + P.o_prod);
+  uint32_t pe0 = 0, pe1 = 0, pe2 = 0;  // table entries of the next tile to copy: block offset, next offset, slot range
+  auto read_entry = [&](int ii) {
     if (ii >= n_cta_tiles) return;
-    while (ii >= si.ib + (si.je - si.jb)) seg_next(si);
-    const UnitView V = unit_view(P.arena, si.u);
-    pj = si.jb + (ii - si.ib);
-    pe0 = V.table[pj];
-    pe1 = V.table[pj + 1];
-    pe2 = V.table[V.nt + 1 + pj];
-    ptiles = V.tiles;
-    pav = V.AV;
+    if (ii >= pr->end) {  // (and at the start)
+      Seg s = pr->s;
+      while (ii >= s.ib + (s.je - s.jb)) seg_next(s);
+      const akv_unit_desc* d = unit_desc(P.arena, s.u);
+      pr->s = s;
+      pr->end = s.ib + (s.je - s.jb);
+      pr->tiles = P.arena + d->off_tiles;
+      pr->av = P.arena + d->off_anchor_v;
+      pr->table = reinterpret_cast<const uint32_t*>(P.arena + d->off_tile_table);
+    }
+    const int pj = pr->s.jb + (ii - pr->s.ib);
+    const uint32_t* table = pr->table;
+    pe0 = table[pj];
+    pe1 = table[pj + 1];
+    pe2 = table[pr->s.nt + 1 + pj];
   };
-  auto issue_more = [&]() {
-    while (ii < n_cta_tiles && nis - nrel < NSG && !warp_failed(failed)) {
-      const uint32_t blkn = pe1 - pe0, lo = pe2 & 0xFFFFu, hi = pe2 >> 16;
-      const uint32_t staged = min(blkn, (uint32_t)P.cap);
+  // (one tile a call: the entries read after it are not waited for)
+  auto copy_more = [&]() {  // the next tile, if it fits now (never waits)
+    const int ii = pr->ii;
+    if (ii < n_cta_tiles && !*failed) {
+      const uint32_t RB = (uint32_t)P.ring_bytes;
+      const uint32_t lo = pe2 & 0xFFFFu, hi = pe2 >> 16;
+      const uint32_t staged = min(pe1 - pe0, (uint32_t)P.cap);
       const uint32_t nrows = min(hi - lo + 1u, (uint32_t)P.X);
       const uint32_t sz = staged + 256u * nrows;
+      int nrel = pr->nrel;
+      uint32_t used = pr->used;
+      while (nrel < ii && mbar_test(bar_empty(nrel % NSG), (uint32_t)(nrel / NSG) & 1u)) {
+        used -= meta[nrel % NSG].bytes;
+        ++nrel;
+      }
+      pr->nrel = nrel;
+      pr->used = used;
+      const uint32_t head = pr->head;
       uint32_t at = 0;
-      bool fits = true;
-      if (used == 0) {
-        at = 0;
-      } else {
-        const uint32_t tail = gmeta[nrel % NSG].ring_off - rbase;  // the oldest tile in flight
+      bool fits = ii - nrel < NSG;
+      if (used > 0) {
+        const uint32_t tail = meta[nrel % NSG].ring_off;  // the oldest tile in flight
         if (head > tail) {
-          if (head + sz <= RH) at = head;
-          else if (sz <= tail) at = 0;
-          else fits = false;
-        } else if (head < tail) {
+          if (head + sz <= RB) at = head;
+          else fits = fits && sz <= tail;
+        } else {
           at = head;
-          fits = head + sz <= tail;
-        } else {
-          fits = false;
+          fits = fits && head + sz <= tail;
         }
       }
-      if (!fits) break;
-      const int sl = nis % NSG;
-      if (lane == 0) {
-        gmeta[sl] = Meta{rbase + at, pe0, blkn, staged, lo, nrows, (uint32_t)pj, sz};
-        // (drop_last: a test withholds the last tile of the range)
-        if (P.drop_last > 0 && ii == n_cta_tiles - P.drop_last) {
-          gmeta[sl].nrows |= 0x80000000u;  // withheld: nothing in flight
-        } else {
-          const uint32_t bar = bar_full(grp, sl);
-          mbar_expect_tx(bar, sz);
-          bulk_g2s(smem_u32(ring + rbase + at), ptiles + pe0, staged, bar);
-          if (nrows) bulk_g2s(smem_u32(ring + rbase + at + staged), pav + (size_t)lo * 256, 256u * nrows, bar);
-        }
+      if (!fits) return;
+      const int sl = ii % NSG;
+      Meta& mt = meta[sl];
+      mt.ring_off = at;
+      mt.blk_off = pe0;
+      mt.staged = staged;
+      mt.lo = lo;
+      mt.nrows = nrows;
+      mt.j = (uint32_t)(pr->s.jb + (ii - pr->s.ib));
+      mt.bytes = sz;
+      // (drop_last: a test withholds the last tile of the range)
+      if (P.drop_last > 0 && ii == n_cta_tiles - P.drop_last) {
+        mt.nrows |= 0x80000000u;  // withheld: nothing in flight
+      } else {
+        mbar_expect_tx(bar_full(sl), sz);
+        bulk_g2s(smem_u32(ring + at), pr->tiles + pe0, staged, bar_full(sl));
+        if (nrows) bulk_g2s(smem_u32(ring + at + staged), pr->av + (size_t)lo * 256, 256u * nrows, bar_full(sl));
       }
-      __syncwarp();
-      head = at + sz;
-      used += sz;
-      ++nis;
-      ii += NG;
-      prefetch();
+      pr->head = at + sz;
+      pr->used = used + sz;
+      pr->ii = ii + 1;
+      read_entry(ii + 1);
     }
   };
-  auto release_to = [&](int upto) {  // this group's tiles before `upto` are done with
-    for (; nrel < upto; ++nrel) used -= gmeta[nrel % NSG].pad;
-  };
-  if (wg == 0) {
-    seg_begin(si);
-    prefetch();
-    issue_more();
+  if (tid == 0) {  // the first tile's table entries are on their way while shared memory is set up
+    Seg s;
+    seg_begin(s);
+    *sg = s;
+    pr->s = s;
+    pr->end = 0;
+    pr->ii = pr->nrel = 0;
+    pr->head = pr->used = 0;
+    read_entry(0);
   }
-  Seg sg;
-  seg_begin(sg);
-  int sigma = 0;
-  for (;; ++sigma) {
-    const UnitView U = unit_view(P.arena, sg.u);
-    const int k = U.k;
-    // ---- segment set-up: the unit's query header (q', its sums, key-residual fragments, from the score
-    // kernel) and score table are on their way; meanwhile the reference m of each head from the chunk
-    // maxima (warp wg: heads wg, wg + 4) ----
-    for (int g = wg; g < GS; g += WPG) {
-      float m = -INFINITY;
-      // the largest anchor score (a lower bound of the largest logit), or with RoPE the largest logit
-      const int nch = ROPE ? (U.S + 63) / 64 : (k + CHA - 1) / CHA;
-      for (int ch = lane; ch < nch; ch += 32) m = fmaxf(m, P.cmax[((size_t)sg.u * P.n_ch + ch) * GS + g]);
-      m = warp_max(m);
-      if (lane == 0) {
-        rows[g] = -m;
-        rows[8 + g] = -INFINITY;
-        rows[24 + g] = m;
-      }
+  if (tid == 0) {
+    for (int s = 0; s < NSG; ++s) {
+      mbar_init(bar_full(s), 1);
+      mbar_init(bar_empty(s), NMW);
     }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(bar_kdone(b), NMW);
+      mbar_init(bar_tdone(b), NTW);
+    }
+    mbar_init(bar_hdr, 1);
+    mbar_init(bar_sa_full, 1);
+    *failed = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int e = tid; e < 2 * GS * 128; e += NT) ovf[e] = 0.f;  // (the overflow's sums start at zero)
+  for (int e = tid; e < 2 * P.R * 8; e += NT) reinterpret_cast<float*>(smem + P.o_pv)[e] = 0.f;
+  __syncthreads();
+
+  if (tid == 0)
+    for (int i = 0; i < 3; ++i) copy_more();
+
+  // =========================== token warps, product warps ==========================
+  const bool tok = warp < NTW;
+  const int wi8 = tok ? warp : warp - NTW;  // index among the role's warps
+  const int mt_ = tid - NTW * 32;           // thread among the product warps
+  auto all_sync = [&]() { named_sync(1, NCW * 32); };
+  auto tok_sync = [&]() { named_sync(2, NTW * 32); };
+  auto prod_sync = [&]() { named_sync(3, NMW * 32); };
+  // (the launch before this one, and everything before it, is complete past this point)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (tid == 0) start_unit(sg->u);
+
+  int lt = 0;     // this CTA's tiles so far
+  int sigma = 0;  // segments so far
+  for (;; ++sigma) {
+    const int u = sg->u, S = unit_desc(P.arena, u)->len, k = unit_desc(P.arena, u)->n_anchors;
+    const int n_seg = sg->je - sg->jb;
+    // a bounded wait of the whole warp; after a failure nothing is waited for any more
+    auto wait_or_fail = [&](uint32_t bar, uint32_t parity) {
+      uint32_t done = mbar_try(bar, parity);
+      if (__all_sync(0xffffffffu, done)) return true;
+      unsigned long long t_0 = 0;
+      for (unsigned n = 0;; ++n) {
+        if (!done) done = mbar_try(bar, parity);
+        if (__all_sync(0xffffffffu, done)) return true;
+        if (warp_failed(failed)) return false;
+        if ((n & 63u) == 63u) {
+          const unsigned long long now = __shfl_sync(0xffffffffu, global_ns(), 0);
+          if (t_0 == 0) t_0 = now;
+          else if (now - t_0 >= kWaitNs) {
+            *failed = 1;
+            return false;
+          }
+        }
+      }
+    };
+
+    if (tok) {
+      // ---- the reference m of each head: the largest anchor score (a lower bound of the largest logit), or
+      // with RoPE the largest logit; from the chunk maxima ----
+      for (int g = wi8; g < GS; g += NTW) {
+        float m = -INFINITY;
+        const int nch = ROPE ? (S + 63) / 64 : (k + CHA - 1) / CHA;
+        for (int ch = lane; ch < nch; ch += 32) m = fmaxf(m, P.cmax[((size_t)u * P.n_ch + ch) * GS + g]);
+        m = warp_max(m);
+        if (lane == 0) {
+          rows[g] = -m;
+          rows[8 + g] = -INFINITY;
+          rows[24 + g] = m;
+        }
+      }
+      wait_or_fail(bar_hdr, (uint32_t)sigma & 1u);
+      wait_or_fail(bar_sa_full, (uint32_t)sigma & 1u);
+      tok_sync();  // m of every head written
+      const float* SAt = TABLE ? SAs : P.sa + (size_t)u * P.ka_stride * GS;
+      float2 l2[NP];
 #pragma unroll
-    for (int nb = 0; nb < 4; ++nb)
+      for (int i = 0; i < NP; ++i) l2[i] = make_float2(0.f, 0.f);
+      for (int i = 0; i < n_seg; ++i, ++lt) {
+        const int b = lt & 1;
+        // (the tile itself too: its bytes came through the asynchronous proxy)
+        if (warp == 0) {  // the copying lane's warp: the ring is topped up, and this tile certainly on its way
+          unsigned long long t_0 = 0;
+          for (unsigned n = 0;; ++n) {
+            if (lane == 0) copy_more();
+            __syncwarp();
+            if (__shfl_sync(0xffffffffu, pr->ii, 0) > lt || warp_failed(failed)) break;
+            if ((n & 63u) == 63u) {  // (bounded; the clock is read now and then)
+              const unsigned long long now = __shfl_sync(0xffffffffu, global_ns(), 0);
+              if (t_0 == 0) t_0 = now;
+              else if (now - t_0 >= kWaitNs) break;
+            }
+          }
+        }
+        const bool go = wait_or_fail(bar_kdone(b), (uint32_t)(lt >> 1) & 1u) && wait_or_fail(bar_full(lt % NSG), (uint32_t)(lt / NSG) & 1u);
+        if (go) {
+          const Meta mt = meta[lt % NSG];
+          const uint8_t* st = ring + mt.ring_off;
+          const TileView tv = tile_view(st, mt, u);
+          const bool fast_tile = mt.fast & 1u;
+          float* W = reinterpret_cast<float*>(smem + P.o_wb) + (lt % 3) * (P.X + kEnds) * GS;
+          int* vs = reinterpret_cast<int*>(smem + P.o_vs) + (lt % 3) * kEnds;
+          float* pv = reinterpret_cast<float*>(smem + P.o_pv) + b * P.R * 8;
+          // ---- tokens: lane -> stored tokens t0 .. t0 + 3, every head ----
+          const int t0 = wi8 * (32 * LCH) + LCH * lane;
+          TokLane tl;
+          tl.kbits = tl.vbits = 0u;
+          tl.rk = tl.rv = 0;
+          tl.t0 = t0;
+          if (t0 < tv.n) {
+            const int wi = t0 >> 6, sh = t0 & 63;
+            const uint64_t wk = tv.bm(0, wi), wv = tv.bm(1, wi);
+            tl.kbits = (uint32_t)(wk >> sh) & ((1u << LCH) - 1u);
+            tl.vbits = (uint32_t)(wv >> sh) & ((1u << LCH) - 1u);
+            tl.rk = tv.rk(0, wi) + __popcll(wk & ((1ull << sh) - 1ull));
+            tl.rv = tv.rk(1, wi) + __popcll(wv & ((1ull << sh) - 1ull));
+          }
+          if (fast_tile) {  // warp-uniform
+            // Every record staged, every run on a staged anchor-value row.  No shared atomics: a run
+            // that starts and ends inside a lane's tokens is stored as it is (no other lane has its
+            // slot); runs that cross lanes are merged by a segmented scan.  Places past the end of a unit's
+            // last tile join its last run with weight 0.
+            const int nval = min(LCH, max(0, tv.n - t0)), t0c = min(t0, tv.n64 - LCH);
+            const uint32_t last_key = reinterpret_cast<const uint32_t*>(st + 4 * tv.n64)[tv.n - 1] & 0xFFFFu;
+            const float* rsb = reinterpret_cast<const float*>(st + tv.cd_k);
+            const uint32_t lo = mt.lo;
+            const int km1 = k - 1;
+            int rk = tl.rk, rv = tl.rv;
+            uint32_t key = 0, hk = 0;  // the run in work; the lane's first run (its head), kept for the merge
+            bool multi = false;        // the lane's tokens hold more than one run
+            float2 acc[NP], hs[NP];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        accA[nb][e] = 0.f;
-        accR[nb][e] = 0.f;
+            for (int i2 = 0; i2 < NP; ++i2) acc[i2] = hs[i2] = make_float2(0.f, 0.f);
+            // RoPE: the lane's tokens' logit rows (global, stored order)
+            const float* lgt = ROPE ? P.lg + ((size_t)u * P.s_stride + (size_t)mt.j * T + t0c) * GS : nullptr;
+            // the table as shared memory (32-bit addressing, shared loads) or global memory (RoPE: not read)
+            const float* SAtab = TABLE ? SAs : P.sa + (size_t)u * P.ka_stride * GS;
+            float2 negm2[NP];  // -m: the logit offset of every token
+#pragma unroll
+            for (int i2 = 0; i2 < NP; ++i2) negm2[i2] = make_float2(rows[2 * i2], GS >= 2 ? rows[2 * i2 + 1] : 0.f);
+            auto token_loop = [&](auto tail_c) {
+              constexpr bool TAIL = decltype(tail_c)::value;  // some places of the tile hold no token
+              uint32_t ek[LCH], ev[LCH];
+              load_words<LCH>(st + 4 * t0c, ek);
+              load_words<LCH>(st + 4 * (tv.n64 + t0c), ev);
+              hk = key = !TAIL || nval > 0 ? ev[0] & 0xFFFFu : last_key;
+#pragma unroll
+              for (int e = 0; e < LCH; ++e) {
+                const bool valid = !TAIL || e < nval;
+                const float gv = valid ? half_hi(ev[e]) : 0.f;
+                float2 x[NP];
+                if constexpr (ROPE) {  // the token's logits from the RoPE logits launch, minus m
+                  float lr[GS];
+                  load_row<GS>(lgt + e * GS, lr);
+#pragma unroll
+                  for (int i2 = 0; i2 < NP; ++i2)
+                    x[i2] = __fadd2_rn(make_float2(lr[2 * i2], GS >= 2 ? lr[2 * i2 + 1] : 0.f), negm2[i2]);
+                } else {
+                  const int a = min((int)(ek[e] & 0xFFFFu), km1);  // indices are < k by construction
+                  float sa[GS];
+                  load_sa_row<GS>(SAtab, a, P.ka_stride, sa);
+                  const bool kb = (tl.kbits >> e) & 1u;
+                  const float gk = half_hi(ek[e]);
+                  // logits gamma S_A - m, plus the key-residual term for the lanes whose token has one
+                  const float2 gk2 = make_float2(gk, gk);
+#pragma unroll
+                  for (int i2 = 0; i2 < NP; ++i2)
+                    x[i2] = __ffma2_rn(gk2, make_float2(sa[2 * i2], GS >= 2 ? sa[2 * i2 + 1] : 0.f), negm2[i2]);
+                  if (kb) {
+                    float rs[GS];
+                    load_row<GS>(rsb + rk * 8, rs);
+#pragma unroll
+                    for (int i2 = 0; i2 < NP; ++i2)
+                      x[i2] = __fadd2_rn(x[i2], make_float2(rs[2 * i2], GS >= 2 ? rs[2 * i2 + 1] : 0.f));
+                  }
+                  rk += (int)kb;
+                }
+                if constexpr (TAIL) {
+#pragma unroll
+                  for (int i2 = 0; i2 < NP; ++i2) x[i2] = valid ? x[i2] : make_float2(-INFINITY, -INFINITY);
+                }
+                float2 pe[NP];
+#pragma unroll
+                for (int i2 = 0; i2 < NP; ++i2) {
+                  pe[i2] = make_float2(exp2_approx(x[i2].x), GS >= 2 ? exp2_approx(x[i2].y) : 0.f);
+                  l2[i2] = __fadd2_rn(l2[i2], pe[i2]);
+                }
+                const bool vb = (tl.vbits >> e) & 1u;
+                if (vb) store_row<GS>(pv + rv * 8, pe);
+                rv += (int)vb;
+                // the run of `key` ends here when the slot changes (branch-free): the lane's first
+                // run is kept as its head (it may continue the previous lane's); a later one started
+                // and ended in this lane, so its slot is this lane's alone and is stored as it is
+                const float2 gv2 = make_float2(gv, gv);
+                if (e == 0) {
+#pragma unroll
+                  for (int i2 = 0; i2 < NP; ++i2) acc[i2] = __fmul2_rn(pe[i2], gv2);
+                } else {
+                  const uint32_t av = valid ? ev[e] & 0xFFFFu : last_key;
+                  const bool chg = av != key;
+                  if (e > 1 && chg && multi) store_row<GS>(W + (int)(key - lo) * GS, acc);
+                  const float f_first = (chg && !multi) ? 1.f : 0.f, f_keep = chg ? 0.f : 1.f;
+                  const float2 first2 = make_float2(f_first, f_first), keep2 = make_float2(f_keep, f_keep);
+#pragma unroll
+                  for (int i2 = 0; i2 < NP; ++i2) {
+                    hs[i2] = __ffma2_rn(acc[i2], first2, hs[i2]);
+                    acc[i2] = __ffma2_rn(pe[i2], gv2, __fmul2_rn(acc[i2], keep2));
+                  }
+                  multi |= chg;
+                  key = av;
+                }
+              }
+            };
+            if (tv.n == T) token_loop(std::false_type{});
+            else token_loop(std::true_type{});
+            // merge across lanes: the next lane's head continues this lane's last run when their
+            // slots match; a head that does not continue the previous lane's run is complete
+            const uint32_t ptk = __shfl_up_sync(0xffffffffu, key, 1);
+            const uint32_t nhk = __shfl_down_sync(0xffffffffu, hk, 1);
+            const unsigned multis = __ballot_sync(0xffffffffu, multi);
+            if (multis) {  // (warp-uniform)
+              const bool nmulti = lane < 31 && ((multis >> (lane + 1)) & 1u);
+              const float f_tn = (nmulti && nhk == key) ? 1.f : 0.f;
+              const float2 tn2 = make_float2(f_tn, f_tn);
+#pragma unroll
+              for (int i2 = 0; i2 < NP; ++i2) {
+                const float2 nh = make_float2(__shfl_down_sync(0xffffffffu, hs[i2].x, 1),
+                                              __shfl_down_sync(0xffffffffu, hs[i2].y, 1));
+                acc[i2] = __ffma2_rn(nh, tn2, acc[i2]);
+              }
+            }
+            // the warp's first run may continue the previous warp's last one and its last run go on in the
+            // next: both get rows of their own past the slots' (a shared-memory float addition is a
+            // compare-and-swap loop, and would meet the neighbour's)
+            float* w_ends = W + (P.X + 2 * wi8) * GS;
+            if (multi && !(lane > 0 && ptk == hk)) {
+              if (lane == 0) vs[2 * wi8] = (int)(hk - lo);
+              store_row<GS>(lane == 0 ? w_ends : W + (int)(hk - lo) * GS, hs);
+            }
+            // segmented inclusive scan of the last runs over lanes with equal slots
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+              const uint32_t kd = __shfl_up_sync(0xffffffffu, key, d);
+              const float f_add = (lane >= d && kd == key) ? 1.f : 0.f;
+              const float2 add2 = make_float2(f_add, f_add);
+#pragma unroll
+              for (int i2 = 0; i2 < NP; ++i2) {
+                const float2 vd = make_float2(__shfl_up_sync(0xffffffffu, acc[i2].x, d),
+                                              __shfl_up_sync(0xffffffffu, acc[i2].y, d));
+                acc[i2] = __ffma2_rn(vd, add2, acc[i2]);
+              }
+            }
+            const uint32_t nkey = __shfl_down_sync(0xffffffffu, key, 1);
+            const uint32_t key0 = __shfl_sync(0xffffffffu, key, 0);
+            if (lane == 31 || nkey != key) {  // the last lane of a segment holds its total
+              // (a single run over the whole warp counts as its last)
+              const bool first = !(multis & 1u) && key == key0, last = lane == 31;
+              if (last) vs[2 * wi8 + 1] = (int)(key - lo);
+              else if (first) vs[2 * wi8] = (int)(key - lo);
+              store_row<GS>(last ? w_ends + GS : (first ? w_ends : W + (int)(key - lo) * GS), acc);
+            }
+          } else if (t0 < tv.n) {
+            int* ovl_n = reinterpret_cast<int*>(smem + P.o_ovl + b * kOvlBytes);
+            float* ovl = reinterpret_cast<float*>(ovl_n + 4);
+            const auto ls = token_chunk_general<GS>(
+                TokTile{tv, tv.gb(P.arena), mt.lo, mt.nrows, SAt, rows, qp, pv, W, ovf, P.arena + unit_desc(P.arena, u)->off_anchor_v,
+                        ROPE ? P.lg + ((size_t)u * P.s_stride + (size_t)mt.j * T) * GS : nullptr, ovl_n, ovl, k, mt.nKs, mt.nVs, P.ka_stride,
+                        CODEC}, tl);
+#pragma unroll
+            for (int i2 = 0; i2 < NP; ++i2) l2[i2] = __fadd2_rn(l2[i2], ls.v[i2]);
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_tdone(b));
       }
 #pragma unroll
-    for (int i = 0; i < NP; ++i) l2[i] = make_float2(0.f, 0.f);
+      for (int g = 0; g < GS; ++g) {
+        const float sl = warp_sum((g & 1) ? l2[g >> 1].y : l2[g >> 1].x);
+        if (lane == 0) gsum[wi8 * 8 + g] = sl;
+      }
+    } else {
+      // ================================ products ==================================
+      float accA[2][4] = {}, accR[2][4] = {};  // anchor-value and value-residual sums, dims 16 wi8 .. 16 wi8 + 15
+      float pminv = 0.f;                       // sum of p min, head r8 (a quarter per c4)
+      wait_or_fail(bar_hdr, (uint32_t)sigma & 1u);
+      uint2 bq[NBF][8];  // the unit's key-residual B fragments
+      float sqh[2];      // sums of q' of heads 2 c4, 2 c4 + 1
 #pragma unroll
-    for (int i = 0; i < HPL; ++i) pminv[i] = 0.f;
-    // the header, then the unit's anchor-score table (every warp waits on both, tiles or not, so
-    // the phase counts stay right)
-    if (!warp_failed(failed) && !mbar_wait_w(bar_hdr(grp), (uint32_t)sigma & 1u)) *failed = 1;
-    if (!warp_failed(failed) && !mbar_wait_w(bar_sa_full, (uint32_t)sigma & 1u)) *failed = 1;
-    gsync();  // m of every head written
-    const float* SAt = P.smem_sa ? SAs : P.sa + (size_t)sg.u * P.ka_stride * GS;
-
-    const int i_end = sg.ib + (sg.je - sg.jb);
-    int i0 = sg.ib + ((grp - sg.ib % NG) + NG) % NG;  // this group's first tile of the segment
-    for (int i = i0; i < i_end; i += NG, ++lt) {
-      const bool go = !warp_failed(failed) && mbar_wait_w(bar_full(grp, lt % NSG), (uint32_t)(lt / NSG) & 1u);
-      if (!go) *failed = 1;
-      const Meta mt = gmeta[lt % NSG];
-      const uint8_t* st = ring + mt.ring_off;
-      TileView tv;
-      int nKs = 0, nVs = 0;
-      bool fast_tile = false;
-      float* W = wb + (lt & 1) * (P.X + kEnds) * GS;
-      int* vs = vsl + (lt & 1) * kEnds;
-      if (go) {
-        tv = tile_view(st, mt, U);
-        const uint32_t codes_staged = tv.staged > tv.cd_k ? (tv.staged - tv.cd_k) / 32u : 0u;
-        nKs = ROPE ? 0 : min(tv.nk, (int)codes_staged);  // their terms go over their own codes: no cap but staging
-        nVs = min(tv.nv, P.R);
-        fast_tile = (ROPE || nKs == tv.nk) && nVs == tv.nv &&
-                    (int)(((reinterpret_cast<const uint32_t*>(st + 4 * tv.n64))[tv.n - 1] & 0xFFFFu) - mt.lo) < (int)mt.nrows;
-        for (int e = gt; e < (P.X + kEnds) * GS; e += WPG * 32) W[e] = 0.f;
-        if (gt < 2) ovl_n[gt] = 0;
-        if (gt < kEnds) vs[gt] = -1;
-        // ---- key residuals: q' . c of the staged key records, tensor cores; the terms
-        // scale (q' . c) + min sum(q') - m are written over the records' codes ----
-        float* rsb = reinterpret_cast<float*>(const_cast<uint8_t*>(st) + tv.cd_k);
-        for (int g16 = wg; g16 * 16 < nKs; g16 += 2 * WPG) {
-          uint32_t wd[2][2][8];  // [group][record r8 / r8 + 8][16-dim step]
+      for (int f = 0; f < NBF; ++f)
 #pragma unroll
-          for (int q = 0; q < 2; ++q)
+        for (int ks = 0; ks < 8; ++ks) bq[f][ks] = qf[(f * 8 + ks) * 32 + lane];
+      sqh[0] = sq[2 * c4];
+      sqh[1] = sq[2 * c4 + 1];
+      // ---- key residuals of tile t: q' . c of the staged key records, tensor cores; the terms
+      // scale (q' . c) + min sum(q') are written over the records' codes; the tile's weight rows zeroed.
+      // (Waits for the tile, unless `landed`.) ----
+      auto key_phase = [&](int t, bool landed) {
+        const int b = t & 1;
+        const bool go = landed || wait_or_fail(bar_full(t % NSG), (uint32_t)(t / NSG) & 1u);
+        if (go) {
+          const Meta mt = meta[t % NSG];
+          const uint8_t* st = ring + mt.ring_off;
+          const TileView tv = tile_view(st, mt, u, S);
+          const uint32_t codes_staged = tv.staged > tv.cd_k ? (tv.staged - tv.cd_k) / 32u : 0u;
+          const int nKs = ROPE ? 0 : min(tv.nk, (int)codes_staged);  // their terms go over their own codes: no cap but staging
+          if (wi8 == 0 && lane == 0) {
+            const int nVs = min(tv.nv, P.R);
+            const bool fast = (ROPE || nKs == tv.nk) && nVs == tv.nv &&
+                              (int)(((reinterpret_cast<const uint32_t*>(st + 4 * tv.n64))[tv.n - 1] & 0xFFFFu) - mt.lo) < (int)mt.nrows;
+            Meta& w = meta[t % NSG];
+            w.sm_v = tv.sm_v;
+            w.cd_k = tv.cd_k;
+            w.cd_v = tv.cd_v;
+            w.sm_k = tv.sm_k;
+            w.n = tv.n;
+            w.nKs = nKs;
+            w.nVs = nVs;
+            w.fast = (fast ? 1u : 0u) | (tv.cd_v + 512u * (uint32_t)((nVs + 15) / 16) <= tv.staged ? 2u : 0u);
+          }
+          float* W = reinterpret_cast<float*>(smem + P.o_wb) + (t % 3) * (P.X + kEnds) * GS;
+          for (int e = 4 * mt_; e < (P.X + kEnds) * GS; e += 4 * NMW * 32) *reinterpret_cast<float4*>(W + e) = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (mt_ < kEnds) reinterpret_cast<int*>(smem + P.o_vs)[(t % 3) * kEnds + mt_] = -1;
+          if (mt_ < 2) reinterpret_cast<int*>(smem + P.o_ovl + b * kOvlBytes)[mt_] = 0;
+          float* rsb = reinterpret_cast<float*>(const_cast<uint8_t*>(st) + tv.cd_k);
+          for (int g16 = wi8; g16 * 16 < nKs; g16 += NMW) {
+            uint32_t wd[2][8], smn[2];  // [record r8 / r8 + 8][16-dim step]; scale and min
 #pragma unroll
             for (int hr = 0; hr < 2; ++hr) {
-              const int sl = (g16 + q * WPG) * 16 + r8 + 8 * hr;
+              const int sl = g16 * 16 + r8 + 8 * hr;
               uint4 w0 = make_uint4(0u, 0u, 0u, 0u), w1 = w0;
+              smn[hr] = 0u;
               if (sl < nKs) {
                 w0 = *reinterpret_cast<const uint4*>(st + tv.cd_k + 32u * (uint32_t)sl);
                 w1 = *reinterpret_cast<const uint4*>(st + tv.cd_k + 32u * (uint32_t)sl + 16u);
+                smn[hr] = *reinterpret_cast<const uint32_t*>(st + tv.sm_k + 4u * (uint32_t)sl);
               }
-              wd[q][hr][0] = w0.x; wd[q][hr][1] = w0.y; wd[q][hr][2] = w0.z; wd[q][hr][3] = w0.w;
-              wd[q][hr][4] = w1.x; wd[q][hr][5] = w1.y; wd[q][hr][6] = w1.z; wd[q][hr][7] = w1.w;
+              wd[hr][0] = w0.x; wd[hr][1] = w0.y; wd[hr][2] = w0.z; wd[hr][3] = w0.w;
+              wd[hr][4] = w1.x; wd[hr][5] = w1.y; wd[hr][6] = w1.z; wd[hr][7] = w1.w;
             }
-          float d[2][2][4] = {};
+            float d[2][4] = {};
 #pragma unroll
-          for (int ks = 0; ks < 8; ++ks) {
-            const uint2 b0 = qf[ks * 32 + lane], b1 = qf[((NBF - 1) * 8 + ks) * 32 + lane];
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-              const uint32_t xa = wd[q][0][ks] >> (4 * c4), xb = wd[q][1][ks] >> (4 * c4);
+            for (int ks = 0; ks < 8; ++ks) {
+              const uint32_t xa = wd[0][ks] >> (4 * c4), xb = wd[1][ks] >> (4 * c4);
               const uint4 a = make_uint4(code_pair_h2<CODEC>(xa), code_pair_h2<CODEC>(xb), code_pair_h2<CODEC>(xa >> 2),
                                          code_pair_h2<CODEC>(xb >> 2));
               if constexpr (GS == 8) {
-                mma_f16(d[q][0], a, b0.x, b0.y);
-                mma_f16(d[q][1], a, b1.x, b1.y);
+                mma_f16(d[0], a, bq[0][ks].x, bq[0][ks].y);
+                mma_f16(d[1], a, bq[NBF - 1][ks].x, bq[NBF - 1][ks].y);
               } else {
-                mma_f16(d[q][ks & 1], a, b0.x, b0.y);
+                mma_f16(d[ks & 1], a, bq[0][ks].x, bq[0][ks].y);
               }
             }
-          }
-          __syncwarp();  // every lane has its codes before any term overwrites them
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
+            __syncwarp();  // every lane has its codes before any term overwrites them
             float v[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              v[e] = d[q][0][e] + d[q][1][e];
+              v[e] = d[0][e] + d[1][e];
               if constexpr (GS != 8) v[e] += __shfl_xor_sync(0xffffffffu, v[e], 2);
             }
             if (GS == 8 || c4 < 2) {
 #pragma unroll
               for (int hr = 0; hr < 2; ++hr) {
-                const int sl = (g16 + q * WPG) * 16 + r8 + 8 * hr;
-                if (sl < nKs) {
-                  const uint32_t smn = *reinterpret_cast<const uint32_t*>(st + tv.sm_k + 4u * (uint32_t)sl);
-#pragma unroll
-                  for (int e = 0; e < 2; ++e) {
-                    const int g = 2 * c4 + e;
-                    if (g < GS) rsb[sl * 8 + g] = half_hi(smn) * sq[g] + half_lo(smn) * v[2 * hr + e];
-                  }
+                const int sl = g16 * 16 + r8 + 8 * hr;
+                if (sl < nKs && 2 * c4 < GS) {  // (rows of eight floats; heads past GS are not read)
+                  const float sc = half_lo(smn[hr]), mn = half_hi(smn[hr]);
+                  *reinterpret_cast<float2*>(rsb + sl * 8 + 2 * c4) = make_float2(mn * sqh[0] + sc * v[2 * hr], mn * sqh[1] + sc * v[2 * hr + 1]);
                 }
               }
             }
           }
         }
-      }
-      gsync();  // (A) key-residual terms written, weight table zeroed
-      if (wg == 0) {  // every warp is done with the group's previous tile: its bytes take new ones
-        release_to(lt);
-        issue_more();
-        // the next tile did not fit beside this one (the ring's free bytes are split): it is
-        // issued once this tile is done (rare)
-        if (lane == 0) lastf[2] = (nis <= lt + 1 && ii < n_cta_tiles) ? 1 : 0;
-      }
-      if (go) {
-        // ---- tokens: lane -> stored tokens t0 .. t0 + 7, every head ----
-        const int t0 = wg * (32 * LCH) + LCH * lane;
-        TokLane tl;
-        if (t0 < tv.n) {
-          const int wi = t0 >> 6, sh = t0 & 63;
-          const uint64_t wk = tv.bm(0, wi), wv = tv.bm(1, wi);
-          tl.kbits = (uint32_t)(wk >> sh) & 0xFFu;
-          tl.vbits = (uint32_t)(wv >> sh) & 0xFFu;
-          tl.rk = tv.rk(0, wi) + __popcll(wk & ((1ull << sh) - 1ull));
-          tl.rv = tv.rk(1, wi) + __popcll(wv & ((1ull << sh) - 1ull));
-          tl.t0 = t0;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_kdone(b));
+      };
+      if (n_seg > 0) key_phase(lt, false);
+      for (int i = 0; i < n_seg; ++i, ++lt) {
+        const int b = lt & 1;
+        // the next tile's key terms first, if it is there, so that the token warps have work while this tile's
+        // values are summed (else after them: its place may be this tile's)
+        bool ahead = i + 1 >= n_seg;
+        if (!ahead && !warp_failed(failed) &&
+            __all_sync(0xffffffffu, mbar_test(bar_full((lt + 1) % NSG), (uint32_t)((lt + 1) / NSG) & 1u))) {
+          key_phase(lt + 1, true);
+          ahead = true;
         }
-        if (fast_tile && tv.n == T) {  // warp-uniform
-          // A full tile, every record staged, every run on a staged anchor-value row.  No shared
-          // atomics: a run that starts and ends inside a lane's tokens is stored as it is (no
-          // other lane has its slot); runs that cross lanes are merged by a segmented scan.
-          const float* rsb = reinterpret_cast<const float*>(st + tv.cd_k);
-          const uint32_t lo = mt.lo;
-          const int km1 = k - 1;
-          uint32_t kb8 = tl.kbits, vb8 = tl.vbits;
-          int rk = tl.rk, rv = tl.rv;
-          uint32_t key = *reinterpret_cast<const uint32_t*>(st + 4 * (tv.n64 + t0)) & 0xFFFFu;
-          uint32_t hk = key;  // the lane's first run (its head), kept for the merge
-          bool multi = false;  // the lane's tokens hold more than one run
-          float2 acc[NP], hs[NP];
+        const bool go = wait_or_fail(bar_tdone(b), (uint32_t)(lt >> 1) & 1u);
+        const Meta mt = meta[lt % NSG];
+        const uint8_t* st = ring + mt.ring_off;
+        float* W = reinterpret_cast<float*>(smem + P.o_wb) + (lt % 3) * (P.X + kEnds) * GS;
+        float* pv = reinterpret_cast<float*>(smem + P.o_pv) + b * P.R * 8;
+        const int nVs = mt.nVs, nr = (int)mt.nrows, nb16 = (nr + 15) / 16;
+        if (go) {
+          if (!(mt.fast & 1u)) {  // the overflow lists: thread mt_ takes dimension mt_ % 128 of every entry of one list
+            const TileView tv = tile_view(st, mt, u);
+            const int* ovl_n = reinterpret_cast<const int*>(smem + P.o_ovl + b * kOvlBytes);
+            const float* ovl = reinterpret_cast<const float*>(ovl_n + 4);
+            const int dim = mt_ & 127;
+            float av[GS];
 #pragma unroll
-          for (int i2 = 0; i2 < NP; ++i2) acc[i2] = hs[i2] = make_float2(0.f, 0.f);
-          float2 negm2[NP];  // -m: the logit offset of every token
+            for (int g = 0; g < GS; ++g) av[g] = 0.f;
+            if (mt_ < 128) {
+              const int nv_o = min(ovl_n[0], kOvl);
+              for (int e = 0; e < nv_o; ++e) {  // p (min + scale L(c)) of a value record, rotated domain
+                const float* en = ovl + e * 9;
+                const uint32_t r = (uint32_t)__float_as_int(en[0]);
+                const uint32_t smn = *reinterpret_cast<const uint32_t*>(tv.at(P.arena, tv.sm_v + 4u * r));
+                const uint32_t w = *reinterpret_cast<const uint32_t*>(tv.at(P.arena, tv.cd_v + 512u * (r / 16u) + 4u * value_code_word(dim)));
+                const float val = fmaf(half_lo(smn), code_level((w >> value_code_bit((int)(r % 16u))) & 3u, CODEC), half_hi(smn));
 #pragma unroll
-          for (int i2 = 0; i2 < NP; ++i2) negm2[i2] = make_float2(rows[2 * i2], GS >= 2 ? rows[2 * i2 + 1] : 0.f);
-          constexpr int TPI = 4;  // stream words per load (16 bytes)
-          // RoPE: the lane's tokens' logit rows (global, stored order)
-          const float* lgt = ROPE ? P.lg + ((size_t)sg.u * P.s_stride + (size_t)mt.j * T + t0) * GS : nullptr;
-          // the table pointer as shared memory (32-bit addressing, shared loads) or global memory
-          auto token_loop = [&](const float* SAtab) {
-#pragma unroll 1
-          for (int qd = 0; qd < LCH / TPI; ++qd) {
-            uint32_t ek[TPI], ev[TPI];
-            load_words<TPI>(st + 4 * (t0 + TPI * qd), ek);
-            load_words<TPI>(st + 4 * (tv.n64 + t0 + TPI * qd), ev);
+                for (int g = 0; g < GS; ++g) av[g] = fmaf(en[1 + g], val, av[g]);
+              }
+              if (nv_o)
 #pragma unroll
-            for (int e = 0; e < TPI; ++e) {
-              const float gv = half_hi(ev[e]);
-              float2 x[NP];
-              if constexpr (ROPE) {  // the token's logits from the RoPE logits launch, minus m
-                float lr[GS];
-                load_row<GS>(lgt + (TPI * qd + e) * GS, lr);
+                for (int g = 0; g < GS; ++g) red_local(ovf + GS * 128 + g * 128 + dim, av[g]);
+            } else {
+              const int na_o = min(ovl_n[1], kOvl);
+              for (int e = 0; e < na_o; ++e) {  // weight x the anchor's value row (global, swizzled by the slot)
+                const float* en = ovl + (kOvl + e) * 9;
+                const int kk = __float_as_int(en[0]);
+                const uint8_t* row = P.arena + unit_desc(P.arena, u)->off_anchor_v + (size_t)kk * 256;
+                const float x = __bfloat162float(
+                    *reinterpret_cast<const __nv_bfloat16*>(row + 16 * ((dim >> 3) ^ (kk & 7)) + 2 * (dim & 7)));
 #pragma unroll
-                for (int i2 = 0; i2 < NP; ++i2)
-                  x[i2] = __fadd2_rn(make_float2(lr[2 * i2], GS >= 2 ? lr[2 * i2 + 1] : 0.f), negm2[i2]);
+                for (int g = 0; g < GS; ++g) av[g] = fmaf(en[1 + g], x, av[g]);
+              }
+              if (na_o)
+#pragma unroll
+                for (int g = 0; g < GS; ++g) red_local(ovf + g * 128 + dim, av[g]);
+            }
+          }
+          // ---- operands of the value side, each built once by one warp, over the numbers it is made of, as the
+          // mma A fragments (lane 4 g + c4: k places 2 c4, 2 c4 + 1, then those + 8; bf16 high part, then
+          // low part): p scale of 16 value records (with the sum of p min per head), or 16 slots' weights ----
+          const int n_vg = (nVs + 15) / 16;
+          for (int x = wi8; x < n_vg + nb16 + 1; x += NMW) {
+            const bool val = x < n_vg;
+            const int blk = x - n_vg;  // block of slots; the last one: the token warps' first and last runs
+            float* src = val ? pv + 128 * x : (blk < nb16 ? W + 16 * GS * blk : W + P.X * GS);
+            const int stride = val ? 8 : GS;
+            const int lim = val ? nVs - 16 * x : (blk < nb16 ? nr - 16 * blk : kEnds);
+            const int kk[4] = {2 * c4, 2 * c4 + 1, 2 * c4 + 8, 2 * c4 + 9};
+            float f[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) f[e] = kk[e] < lim && r8 < GS ? src[kk[e] * stride + r8] : 0.f;
+            if (val) {
+              uint32_t smn[4];
+              const uint32_t so = mt.sm_v + 64u * (uint32_t)x;  // (padded to 16 bytes: pairs may be read together)
+              if (mt.fast & 2u) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) smn[e] = kk[e] < lim ? *reinterpret_cast<const uint32_t*>(st + so + 4u * (uint32_t)kk[e]) : 0u;
               } else {
-                const int a = min((int)(ek[e] & 0xFFFFu), km1);  // indices are < k by construction
-                float sa[GS];
-                load_sa_row<GS>(SAtab, a, P.ka_stride, sa);
-                const bool kb = kb8 & 1u;
-                kb8 >>= 1;
-                const float gk = half_hi(ek[e]);
-                // logits gamma S_A - m, plus the key-residual term for the lanes whose token has one
-                const float2 gk2 = make_float2(gk, gk);
+                const TileView tv = tile_view(st, mt, u);
 #pragma unroll
-                for (int i2 = 0; i2 < NP; ++i2)
-                  x[i2] = __ffma2_rn(gk2, make_float2(sa[2 * i2], GS >= 2 ? sa[2 * i2 + 1] : 0.f), negm2[i2]);
-                if (kb) {
-                  float rs[GS];
-                  load_row<GS>(rsb + rk * 8, rs);
-#pragma unroll
-                  for (int i2 = 0; i2 < NP; ++i2)
-                    x[i2] = __fadd2_rn(x[i2], make_float2(rs[2 * i2], GS >= 2 ? rs[2 * i2 + 1] : 0.f));
-                }
-                rk += (int)kb;
+                for (int e = 0; e < 4; ++e) smn[e] = kk[e] < lim ? *reinterpret_cast<const uint32_t*>(tv.at(P.arena, so + 4u * (uint32_t)kk[e])) : 0u;
               }
-              float2 pe[NP];
 #pragma unroll
-              for (int i2 = 0; i2 < NP; ++i2) {
-                pe[i2] = make_float2(exp2_approx(x[i2].x), GS >= 2 ? exp2_approx(x[i2].y) : 0.f);
-                l2[i2] = __fadd2_rn(l2[i2], pe[i2]);
+              for (int e = 0; e < 4; ++e) {
+                pminv = fmaf(f[e], half_hi(smn[e]), pminv);
+                f[e] *= half_lo(smn[e]);
               }
-              const bool vb = vb8 & 1u;
-              vb8 >>= 1;
-              if (vb) store_row<GS>(pv + rv * 8, pe);
-              rv += (int)vb;
-              // the run of `key` ends here when the slot changes (branch-free): the lane's first
-              // run is kept as its head (it may continue the previous lane's); a later one started
-              // and ended in this lane, so its slot is this lane's alone and is stored as it is
-              const uint32_t av = ev[e] & 0xFFFFu;
-              const bool chg = av != key;
-              if (chg && multi) store_row<GS>(W + (int)(key - lo) * GS, acc);
-              const float f_first = (chg && !multi) ? 1.f : 0.f, f_keep = chg ? 0.f : 1.f;
-              const float2 first2 = make_float2(f_first, f_first), keep2 = make_float2(f_keep, f_keep);
-              const float2 gv2 = make_float2(gv, gv);
-#pragma unroll
-              for (int i2 = 0; i2 < NP; ++i2) {
-                hs[i2] = __ffma2_rn(acc[i2], first2, hs[i2]);
-                acc[i2] = __ffma2_rn(pe[i2], gv2, __fmul2_rn(acc[i2], keep2));
-              }
-              multi |= chg;
-              key = av;
             }
-          }
-          };
-          if (ROPE || !P.smem_sa) token_loop(P.sa + (size_t)sg.u * P.ka_stride * GS);  // (RoPE: no table read)
-          else token_loop(SAs);
-          // merge across lanes: the next lane's head continues this lane's last run when their
-          // slots match; a head that does not continue the previous lane's run is complete
-          const uint32_t ptk = __shfl_up_sync(0xffffffffu, key, 1);
-          const uint32_t nhk = __shfl_down_sync(0xffffffffu, hk, 1);
-          const bool nmulti = __shfl_down_sync(0xffffffffu, (int)multi, 1) != 0;
-          const float f_tn = (lane < 31 && nmulti && nhk == key) ? 1.f : 0.f;
-          const float2 tn2 = make_float2(f_tn, f_tn);
-#pragma unroll
-          for (int i2 = 0; i2 < NP; ++i2) {
-            const float2 nh = make_float2(__shfl_down_sync(0xffffffffu, hs[i2].x, 1),
-                                          __shfl_down_sync(0xffffffffu, hs[i2].y, 1));
-            acc[i2] = __ffma2_rn(nh, tn2, acc[i2]);
-          }
-          // the warp's first run may continue the previous warp's last one and its last run go on in the
-          // next: both get rows of their own past the slots' (a shared-memory float addition is a
-          // compare-and-swap loop, and would meet the neighbour's)
-          float* w_ends = W + (P.X + 2 * wg) * GS;
-          if (multi && !(lane > 0 && ptk == hk)) {
-            if (lane == 0) vs[2 * wg] = (int)(hk - lo);
-            store_row<GS>(lane == 0 ? w_ends : W + (int)(hk - lo) * GS, hs);
-          }
-          const bool multi0 = __shfl_sync(0xffffffffu, (int)multi, 0) != 0;
-          // segmented inclusive scan of the last runs over lanes with equal slots
-#pragma unroll
-          for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t kd = __shfl_up_sync(0xffffffffu, key, d);
-            const float f_add = (lane >= d && kd == key) ? 1.f : 0.f;
-            const float2 add2 = make_float2(f_add, f_add);
-#pragma unroll
-            for (int i2 = 0; i2 < NP; ++i2) {
-              const float2 vd = make_float2(__shfl_up_sync(0xffffffffu, acc[i2].x, d),
-                                            __shfl_up_sync(0xffffffffu, acc[i2].y, d));
-              acc[i2] = __ffma2_rn(vd, add2, acc[i2]);
-            }
-          }
-          const uint32_t nkey = __shfl_down_sync(0xffffffffu, key, 1);
-          const uint32_t key0 = __shfl_sync(0xffffffffu, key, 0);
-          if (lane == 31 || nkey != key) {  // the last lane of a segment holds its total
-            // (a single run over the whole warp counts as its last)
-            const bool first = !multi0 && key == key0, last = lane == 31;
-            if (last) vs[2 * wg + 1] = (int)(key - lo);
-            else if (first) vs[2 * wg] = (int)(key - lo);
-            store_row<GS>(last ? w_ends + GS : (first ? w_ends : W + (int)(key - lo) * GS), acc);
-          }
-        } else if (t0 < tv.n) {
-          const auto ls = token_chunk_general<GS>(TokTile{tv, mt.lo, mt.nrows, SAt, rows, qp, pv, W, ovf, U.AV,
-                                                      ROPE ? P.lg + ((size_t)sg.u * P.s_stride + (size_t)mt.j * T) * GS : nullptr,
-                                                      ovl_n, ovl, k, nKs, nVs, P.ka_stride, CODEC}, tl);
-#pragma unroll
-          for (int i2 = 0; i2 < NP; ++i2) l2[i2] = __fadd2_rn(l2[i2], ls.v[i2]);
-        }
-      }
-      gsync();  // (B) the tile's weights and p rows are complete
-      if (go && !fast_tile) {  // the overflow lists: thread gt takes dimension gt of every entry
-        const int nv_o = min(ovl_n[0], kOvl), na_o = min(ovl_n[1], kOvl);
-        if (nv_o + na_o > 0) {
-          float av[GS], aa[GS];
-#pragma unroll
-          for (int g = 0; g < GS; ++g) av[g] = aa[g] = 0.f;
-          for (int e = 0; e < nv_o; ++e) {  // p (min + scale L(c)) of a value record, rotated domain
-            const float* en = ovl + e * 9;
-            const uint32_t r = (uint32_t)__float_as_int(en[0]);
-            const uint32_t smn = *reinterpret_cast<const uint32_t*>(tv.at(tv.sm_v + 4u * r));
-            const uint32_t w = *reinterpret_cast<const uint32_t*>(tv.at(tv.cd_v + 512u * (r / 16u) + 4u * value_code_word(gt)));
-            const float val = fmaf(half_lo(smn), code_level((w >> value_code_bit((int)(r % 16u))) & 3u, CODEC), half_hi(smn));
-#pragma unroll
-            for (int g = 0; g < GS; ++g) av[g] = fmaf(en[1 + g], val, av[g]);
-          }
-          for (int e = 0; e < na_o; ++e) {  // weight x the anchor's value row (global, swizzled by the slot)
-            const float* en = ovl + (kOvl + e) * 9;
-            const int kk = __float_as_int(en[0]);
-            const uint8_t* row = U.AV + (size_t)kk * 256;
-            const float x = __bfloat162float(
-                *reinterpret_cast<const __nv_bfloat16*>(row + 16 * ((gt >> 3) ^ (kk & 7)) + 2 * (gt & 7)));
-#pragma unroll
-            for (int g = 0; g < GS; ++g) aa[g] = fmaf(en[1 + g], x, aa[g]);
-          }
-#pragma unroll
-          for (int g = 0; g < GS; ++g) {
-            if (nv_o) red_local(ovf + GS * 128 + g * 128 + gt, av[g]);
-            if (na_o) red_local(ovf + g * 128 + gt, aa[g]);
-          }
-        }
-      }
-      if (go) {
-        // ---- value operands: p scale as bf16 high + low parts in the mma A layout, written
-        // over the p rows of the same 16 records; sum of p min per head ----
-        const int sl16 = lane & 15, hb = lane >> 4;
-        for (int grp16 = wg; grp16 * 16 < nVs; grp16 += WPG) {
-          const int r = grp16 * 16 + sl16;
-          const bool rec_ok = r < nVs;
-          uint32_t smn = 0u;
-          if (rec_ok) smn = *reinterpret_cast<const uint32_t*>(tv.at(tv.sm_v + 4u * (uint32_t)r));
-          const float scl = half_lo(smn), mn = half_hi(smn);
-          float pr[HPL];
-#pragma unroll
-          for (int i2 = 0; i2 < HPL; ++i2) {
-            const int g = hb + 2 * i2;
-            pr[i2] = (rec_ok && g < GS) ? pv[r * 8 + g] : 0.f;
-          }
-          __syncwarp();  // the group's p rows are read before they are overwritten
-#pragma unroll
-          for (int i2 = 0; i2 < HPL; ++i2) {
-            const int g = hb + 2 * i2;
-            if (g < GS) {
-              // A-operand place of (record r, head g): lane 4 g + (r % 8) / 2, register
-              // 2 ((r / 8) % 2) (high part) or + 1 (low part), half r % 2
-              __nv_bfloat16 phi, plo;
-              split_b(pr[i2] * scl, phi, plo);
-              pminv[i2] = fmaf(pr[i2], mn, pminv[i2]);
-              unsigned short* dst = reinterpret_cast<unsigned short*>(
-                  reinterpret_cast<uint8_t*>(pv) + grp16 * 512 + (4 * g + ((sl16 & 7) >> 1)) * 16 + ((sl16 >> 3) & 1) * 8 +
-                  (sl16 & 1) * 2);
-              dst[0] = __bfloat16_as_ushort(phi);
-              dst[2] = __bfloat16_as_ushort(plo);
-            }
-          }
-        }
-        // ---- anchor values: w^T V_A over the tile's staged slots (bf16, weights hi + lo) ----
-        const uint8_t* Vr = st + mt.staged;
-        const int nr = (int)mt.nrows;
-        const int mi = lane >> 3, ri = lane & 7;
-        for (int blk = 0; 16 * blk < nr; ++blk) {
-          const int ka = 16 * blk + 2 * c4;
-          uint32_t ah0 = 0, al0 = 0, ah2 = 0, al2 = 0;
-          if (r8 < GS) {
-            const int kk[4] = {ka, ka + 1, ka + 8, ka + 9};
             __nv_bfloat16 hi[4], lo_[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) split_b(kk[e] < nr ? W[kk[e] * GS + r8] : 0.f, hi[e], lo_[e]);
-            ah0 = pack_b2(hi[0], hi[1]);
-            al0 = pack_b2(lo_[0], lo_[1]);
-            ah2 = pack_b2(hi[2], hi[3]);
-            al2 = pack_b2(lo_[2], lo_[3]);
-          }
-          const uint32_t m0 = (ka < nr ? 0xFFFFu : 0u) | (ka + 1 < nr ? 0xFFFF0000u : 0u);
-          const uint32_t m1 = (ka + 8 < nr ? 0xFFFFu : 0u) | (ka + 9 < nr ? 0xFFFF0000u : 0u);
-          const int row = 16 * blk + (mi & 1) * 8 + ri;
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf) {
-            const int cc = (4 * wg + 2 * hf + (mi >> 1)) ^ (int)((mt.lo + (uint32_t)ri) & 7u);
-            uint32_t b00, b01, b10, b11;
-            ldsm_x4_trans(smem_u32(Vr + row * 256 + 16 * cc), b00, b01, b10, b11);
-            // rows past the staged slots hold other bytes: clear their halves of B
-            b00 &= m0;
-            b10 &= m0;
-            b01 &= m1;
-            b11 &= m1;
-            mma_bf16(accA[2 * hf], ah0, al0, ah2, al2, b00, b01);
-            mma_bf16(accA[2 * hf + 1], ah0, al0, ah2, al2, b10, b11);
+            for (int e = 0; e < 4; ++e) split_b(f[e], hi[e], lo_[e]);
+            __syncwarp();  // everything is read before it is overwritten
+            if (r8 < GS)
+              *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(src) + 16 * lane) =
+                  make_uint4(pack_b2(hi[0], hi[1]), pack_b2(lo_[0], lo_[1]), pack_b2(hi[2], hi[3]), pack_b2(lo_[2], lo_[3]));
           }
         }
-        {  // the warps' first and last runs: rows picked by their slots (k places 8 .. 15 are empty)
-          uint32_t ah0 = 0, al0 = 0;
-          if (r8 < GS) {
-            __nv_bfloat16 hi[2], lo_[2];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) split_b(W[(P.X + 2 * c4 + e) * GS + r8], hi[e], lo_[e]);
-            ah0 = pack_b2(hi[0], hi[1]);
-            al0 = pack_b2(lo_[0], lo_[1]);
-          }
-          const int2 vc = *reinterpret_cast<const int2*>(vs + 2 * c4);
-          const uint32_t m0 = (vc.x >= 0 ? 0xFFFFu : 0u) | (vc.y >= 0 ? 0xFFFF0000u : 0u);
-          const int slot = max(vs[ri], 0);
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf) {
-            const int cc = (4 * wg + 2 * hf + (mi >> 1)) ^ (int)((mt.lo + (uint32_t)slot) & 7u);
+        prod_sync();  // every operand is built
+        if (go) {
+          // ---- anchor values: w^T V_A over the tile's staged slots, then over the token warps' first and last
+          // runs, whose rows are picked by their slots ----
+          const uint8_t* Vr = st + mt.staged;
+          const int mi = lane >> 3, ri = lane & 7;
+          const int* vs = reinterpret_cast<const int*>(smem + P.o_vs) + (lt % 3) * kEnds;
+          for (int blk = 0; blk <= nb16; ++blk) {
+            const bool ends = blk == nb16;
+            const int ka = (ends ? 0 : 16 * blk) + 2 * c4;
+            const uint4 a = r8 < GS ? *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(ends ? W + P.X * GS : W + 16 * GS * blk) + 16 * lane)
+                                    : make_uint4(0u, 0u, 0u, 0u);
+            // rows past the staged slots, or of runs that are not there, hold other bytes: their halves of B are cleared
+            uint32_t m0, m1;
+            int slot;
+            if (ends) {
+              const int2 v0 = *reinterpret_cast<const int2*>(vs + ka), v1 = *reinterpret_cast<const int2*>(vs + ka + 8);
+              m0 = (v0.x >= 0 ? 0xFFFFu : 0u) | (v0.y >= 0 ? 0xFFFF0000u : 0u);
+              m1 = (v1.x >= 0 ? 0xFFFFu : 0u) | (v1.y >= 0 ? 0xFFFF0000u : 0u);
+              slot = max(vs[(mi & 1) * 8 + ri], 0);
+            } else {
+              m0 = (ka < nr ? 0xFFFFu : 0u) | (ka + 1 < nr ? 0xFFFF0000u : 0u);
+              m1 = (ka + 8 < nr ? 0xFFFFu : 0u) | (ka + 9 < nr ? 0xFFFF0000u : 0u);
+              slot = 16 * blk + (mi & 1) * 8 + ri;
+            }
+            const int cc = (2 * wi8 + (mi >> 1)) ^ (int)((mt.lo + (uint32_t)slot) & 7u);
             uint32_t b00, b01, b10, b11;
             ldsm_x4_trans(smem_u32(Vr + slot * 256 + 16 * cc), b00, b01, b10, b11);
-            mma_bf16(accA[2 * hf], ah0, al0, 0u, 0u, b00 & m0, 0u);
-            mma_bf16(accA[2 * hf + 1], ah0, al0, 0u, 0u, b10 & m0, 0u);
+            mma_bf16(accA[0], a.x, a.y, a.z, a.w, b00 & m0, b01 & m1);
+            mma_bf16(accA[1], a.x, a.y, a.z, a.w, b10 & m0, b11 & m1);
           }
-        }
-      }
-      gsync();  // (C) every value operand is built
-      if (go) {
-        // ---- value residuals: (p scale) c over the staged records, in the rotated domain;
-        // this lane's four code words hold dimensions 32 wg + 8 nb + r8 of 16 records ----
-        const uint32_t woff = tv.cd_v + 4u * (uint32_t)(32 * wg + 4 * r8);
-        const bool all_staged = tv.cd_v + 512u * (uint32_t)((nVs + 15) / 16) <= tv.staged;
-        for (int g16 = 0; g16 * 16 < nVs; g16 += 2) {
+          // ---- value residuals: (p scale) c over the staged records, in the rotated domain;
+          // this lane's two code words hold dimensions 16 wi8 + 8 nb + r8 of 16 records ----
+          const uint32_t woff = mt.cd_v + 4u * (uint32_t)(32 * (wi8 >> 1) + 4 * r8 + 2 * (wi8 & 1));
+          auto residual = [&](int g16, const uint2 w2) {
+            const uint4 a = r8 < GS ? *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(pv) + g16 * 512 + lane * 16)
+                                    : make_uint4(0u, 0u, 0u, 0u);
+            const uint32_t wd[2] = {w2.x, w2.y};
 #pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            if ((g16 + q) * 16 >= nVs) break;  // warp-uniform
-            const uint4 a = *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(pv) + (g16 + q) * 512 + lane * 16);
-            const uint32_t off = woff + 512u * (uint32_t)(g16 + q);
-            const uint4 w4 = all_staged ? *reinterpret_cast<const uint4*>(st + off) : *reinterpret_cast<const uint4*>(tv.at(off));
-            const uint32_t wd[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-            for (int nb = 0; nb < 4; ++nb) {
+            for (int nb = 0; nb < 2; ++nb) {
               // records 2c, 2c+1 at bits 2c and 2c + 16, records 2c+8, 2c+9 eight bits higher
               const uint32_t x = wd[nb] >> (2 * c4);
               mma_bf16(accR[nb], a.x, a.y, a.z, a.w, code_pair_b2<CODEC>(x), code_pair_b2<CODEC>(x >> 8));
             }
+          };
+          if (mt.fast & 2u) {
+#pragma unroll 4
+            for (int g16 = 0; g16 * 16 < nVs; ++g16) residual(g16, *reinterpret_cast<const uint2*>(st + woff + 512u * (uint32_t)g16));
+          } else {
+            const TileView tv = tile_view(st, mt, u);
+            for (int g16 = 0; g16 * 16 < nVs; ++g16)
+              residual(g16, *reinterpret_cast<const uint2*>(tv.at(P.arena, woff + 512u * (uint32_t)g16)));
           }
         }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_empty(lt % NSG));  // this warp is done with the tile
+        if (!ahead) key_phase(lt + 1, false);
       }
-      if (lastf[2]) {  // (written before barrier C by warp 0, the same for every warp)
-        gsync();
-        if (wg == 0) {
-          release_to(lt + 1);
-          issue_more();
+      prod_sync();  // every warp is done with the header, where the segment's sums go
+      static_assert(2 * GS * 512 <= hdr_bytes(GS), "a segment's sums fit its header's place");
+      if (r8 < GS) {
+#pragma unroll
+        for (int nb = 0; nb < 2; ++nb) {
+          const int col = 16 * wi8 + 8 * nb + 2 * c4;
+          *reinterpret_cast<float2*>(qp + r8 * 128 + col) = make_float2(accA[nb][0] + accA[nb][2], accA[nb][1] + accA[nb][3]);
+          *reinterpret_cast<float2*>(qp + (GS + r8) * 128 + col) = make_float2(accR[nb][0] + accR[nb][2], accR[nb][1] + accR[nb][3]);
         }
       }
+      pminv += __shfl_xor_sync(0xffffffffu, pminv, 1);
+      pminv += __shfl_xor_sync(0xffffffffu, pminv, 2);
+      if (c4 == 0) gsum[64 + wi8 * 8 + r8] = pminv;
     }
 
-    // ---- the group's sums for this unit into shared memory, where its query header was (anchor-value
-    // and rotated value-residual numerators [2][GS][128]; normaliser and sum of p min per warp) ----
-    static_assert(2 * GS * 512 <= hdr_bytes(GS), "a group's sums fit its header's place");
-    gsync();  // every warp is done with the header
-    if (r8 < GS) {
-#pragma unroll
-      for (int nb = 0; nb < 4; ++nb) {
-        const int col = 32 * wg + 8 * nb + 2 * c4;
-        *reinterpret_cast<float2*>(qp + r8 * 128 + col) = make_float2(accA[nb][0] + accA[nb][2], accA[nb][1] + accA[nb][3]);
-        *reinterpret_cast<float2*>(qp + (GS + r8) * 128 + col) = make_float2(accR[nb][0] + accR[nb][2], accR[nb][1] + accR[nb][3]);
-      }
-    }
-#pragma unroll
-    for (int g = 0; g < GS; ++g) {
-      const float sl = warp_sum((g & 1) ? l2[g >> 1].y : l2[g >> 1].x);
-      if (lane == 0) gsum[wg * 16 + g] = sl;
-    }
-#pragma unroll
-    for (int i2 = 0; i2 < HPL; ++i2) {
-      float v = pminv[i2];
-#pragma unroll
-      for (int o = 1; o < 16; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      const int g = (lane >> 4) + 2 * i2;
-      if ((lane & 15) == 0 && g < GS) gsum[wg * 16 + 8 + g] = v;
-    }
-    if (wg == 0) {  // the segment's last tile is done with: top the ring up
-      release_to(lt);
-      issue_more();
-    }
-    // ---- the group that finishes the segment last (the other has stored its sums) turns both
-    // groups' sums and the overflow's into the CTA's slot of the unit: the value-residual part gets its sum
-    // of p min and the inverse rotation (s o H(.) / 128, once per head and CTA), the anchor-value part
-    // is added; then it counts the slot in, and starts the next unit ----
-    gsync();
-    if (gt == 0) {
-      __threadfence_block();
-      lastf[1] = atomicAdd(segcnt, 1) % NG == NG - 1 ? 1 : 0;
-      __threadfence_block();
-    }
-    gsync();
-    const bool has_next = sg.t0 + sg.je < B1;
-    if (lastf[1]) {
-      float* dst = P.part + (size_t)(c + sg.u) * PF;
-      const uint8_t* G0 = smem + P.o_grp;  // the groups' blocks, summed in their order
-      auto group_sum = [&](int off, int i) {
+    // ---- the segment's end: a token warp per query head turns the sums into the CTA's slot of the unit (the
+    // value-residual part gets its sum of p min and the inverse rotation s o H(.) / 128, once per head and CTA;
+    // the anchor-value part and the overflow's sums are added), counts it in on the head's counter, and
+    // combines the head if that completes it ----
+    all_sync();
+    const bool has_next = sg->t0 + sg->je < B1;
+    if (tok) {
+      if (tid == 0) copy_more();
+      const int first = sg->first, nseg = sg->nseg;
+      float* dst = P.part + (size_t)(c + u) * PF;
+      auto warp_sums = [&](int off, int g) {
         float v = 0.f;
 #pragma unroll
-        for (int g = 0; g < NG; ++g)
-#pragma unroll
-          for (int x = 0; x < WPG; ++x) v += reinterpret_cast<const float*>(G0 + g * P.grp_bytes + off)[x * 16 + i];
+        for (int x = 0; x < 8; ++x) v += gsum[off + x * 8 + g];
         return v;
       };
-      for (int h = wg; h < GS; h += WPG) {
+      static_assert(GS <= NTW, "a warp per query head");
+      const int h = wi8;
+      if (h < GS) {
         float4* oa = reinterpret_cast<float4*>(ovf + h * 128 + 4 * lane);
         float4* orr = reinterpret_cast<float4*>(ovf + GS * 128 + h * 128 + 4 * lane);
-        float4 va = *oa, vr = *orr;
-#pragma unroll
-        for (int g = 0; g < NG; ++g) {
-          const float* sums = reinterpret_cast<const float*>(G0 + g * P.grp_bytes + P.g_qp);
-          const float4 a = *reinterpret_cast<const float4*>(sums + h * 128 + 4 * lane);
-          const float4 r = *reinterpret_cast<const float4*>(sums + (GS + h) * 128 + 4 * lane);
-          va.x += a.x; va.y += a.y; va.z += a.z; va.w += a.w;
-          vr.x += r.x; vr.y += r.y; vr.z += r.z; vr.w += r.w;
-        }
-        const float pm = group_sum(P.g_sum, 8 + h);
-        float x[4] = {vr.x + pm, vr.y + pm, vr.z + pm, vr.w + pm};
+        const float4 a = *reinterpret_cast<const float4*>(qp + h * 128 + 4 * lane);
+        const float4 r = *reinterpret_cast<const float4*>(qp + (GS + h) * 128 + 4 * lane);
+        const float4 oav = *oa, orv = *orr;
+        const float pm = warp_sums(64, h);
+        float x[4] = {r.x + orv.x + pm, r.y + orv.y + pm, r.z + orv.z + pm, r.w + orv.w + pm};
         if (P.rotate) {
           warp_wht128(x, lane);
           apply_signs(x, lane, P.sign_lo, P.sign_hi);
 #pragma unroll
           for (int e = 0; e < 4; ++e) x[e] *= (1.0f / 128.0f);
         }
-        *reinterpret_cast<float4*>(dst + h * 128 + 4 * lane) = make_float4(va.x + x[0], va.y + x[1], va.z + x[2], va.w + x[3]);
+        *reinterpret_cast<float4*>(dst + h * 128 + 4 * lane) =
+            make_float4(a.x + oav.x + x[0], a.y + oav.y + x[1], a.z + oav.z + x[2], a.w + oav.w + x[3]);
+        if (lane == 0) dst[part_l(GS) + h] = *failed ? __int_as_float(0x7FC00000) : warp_sums(0, h);
         *oa = make_float4(0.f, 0.f, 0.f, 0.f);
         *orr = make_float4(0.f, 0.f, 0.f, 0.f);
       }
-      if (gt < GS) dst[part_l(GS) + gt] = group_sum(P.g_sum, gt);
-      gsync();
-      if (gt == 0) {
-        dst[part_flag(GS)] = *failed ? 1.f : 0.f;
-        lastf[0] = count_in(P, sg.u, sg.nseg) ? 1 : 0;
-        if (has_next) start_unit(sg.u + 1);  // both groups' sums are read
-      }
-      gsync();
-      if (lastf[0]) {
-        __threadfence();
-        combine_unit<GS>(P, sg.u, sg.first, sg.nseg, wg, WPG);
+      const float m = rows[24 + (h & 7)];
+      tok_sync();  // the sums are read
+      if (tid == 0 && has_next) start_unit(u + 1);
+      if (h < GS) {
+        bool last = true;  // (a unit of one CTA: nothing to count)
+        if (nseg > 1) {
+          unsigned old = 0;
+          if (lane == 0) {
+            __threadfence();
+            old = atomicAdd(unit_counters(P.uh, P.uh_stride, u, GS) + h, 1u);
+          }
+          last = __shfl_sync(0xffffffffu, old, 0) == (unsigned)(nseg - 1);
+          if (last) __threadfence();
+        }
+        if (last) combine_head<GS>(P, u, first, nseg, h, m);
       }
     }
-    gsync();  // lastf and the set-up buffers are reused by the next segment
     if (!has_next) break;
-    seg_next(sg);
+    all_sync();
+    if (tid == 0) {
+      Seg s = *sg;
+      seg_next(s);
+      *sg = s;
+    }
+    all_sync();
   }
-  // every copy this group started has landed before the CTA may exit (bounded; they all have
-  // unless a wait ran out)
-  if (wg == 0 && lane == 0) {
-    for (int t = max(0, nis - NSG); t < nis; ++t)
-      if (!(gmeta[t % NSG].nrows >> 31)) mbar_wait(bar_full(grp, t % NSG), (uint32_t)(t / NSG) & 1u);
-    mbar_wait(bar_hdr(grp), (uint32_t)sigma & 1u);
-    if (grp == 0) mbar_wait(bar_sa_full, (uint32_t)sigma & 1u);
+  // every copy has landed before the CTA may exit (bounded; they all have unless a wait ran out)
+  if (tid == 0) {
+    for (int t = max(0, pr->ii - NSG); t < pr->ii; ++t)
+      if (!(meta[t % NSG].nrows >> 31)) mbar_wait(bar_full(t % NSG), (uint32_t)(t / NSG) & 1u);
+    mbar_wait(bar_hdr, (uint32_t)sigma & 1u);
+    mbar_wait(bar_sa_full, (uint32_t)sigma & 1u);
   }
 }
 
@@ -2191,7 +2312,7 @@ struct Plan {
 };
 
 // Shared-memory carve-up for (R, X, table in shared memory or not); false if the ring
-// would hold fewer than `min_tiles` of the largest staged tiles per group.
+// would hold fewer than `min_tiles` of the largest staged tiles.
 bool make_plan_rx(const Layout& L, int GS, int R, int X, bool smem_sa, int smem_optin, int min_tiles, Plan* out) {
   DecodeParams& P = out->P;
   P.R = R;
@@ -2205,49 +2326,41 @@ bool make_plan_rx(const Layout& L, int GS, int R, int X, bool smem_sa, int smem_
     off = align128(off + bytes);
     return (int)o;
   };
-  P.o_bar = take((NG * NSG + 1 + NG) * 8);
-  P.o_meta = take(NG * NSG * sizeof(Meta));
-  P.o_misc = take(16);
+  P.o_bar = take((2 * NSG + 6) * 8);
+  P.o_meta = take(NSG * sizeof(Meta));
+  P.o_misc = take(16 + sizeof(Seg));  // failure flag; the segment in work
   P.o_sa = take(smem_sa ? (size_t)P.ka_stride * GS * 4 : 0);
   P.o_ovf = take((size_t)2 * GS * 128 * 4);
-  // a group's block: q' rows, small rows, last flag, two weight tables, p rows / A operands
-  size_t g = 0;
-  auto gtake = [&](size_t bytes) {
-    const size_t o = g;
-    g = align128(g + bytes);
-    return (int)o;
-  };
-  P.g_qp = gtake((size_t)hdr_bytes(GS));  // the unit's query header: q', its sums, B fragments
-  P.g_qf = P.g_qp + GS * 512 + 32;
-  P.g_rows = gtake(32 * 4);
-  P.g_red = gtake(16);
-  P.g_wb = gtake((size_t)2 * (X + kEnds) * GS * 4);  // the slots' rows, then the warps' first and last runs
-  P.g_vs = gtake((size_t)2 * kEnds * 4);
-  P.g_sum = gtake((size_t)WPG * 16 * 4);
-  P.g_pv = gtake((size_t)R * 32);
-  P.g_ovl = gtake((size_t)(16 + 2 * kOvl * 9 * 4));  // the tile's overflow lists (counts, then entries)
-  P.grp_bytes = (int)g;
-  P.o_grp = take((size_t)NG * g);
+  P.o_qp = take((size_t)hdr_bytes(GS));  // the unit's query header: q', its sums, B fragments
+  P.o_rows = take(32 * 4);
+  P.o_gsum = take(2 * 8 * 8 * 4);
+  // three tiles' weights of their slots and of the warps' first and last runs, and the slots of those; two tiles'
+  // p rows (then A operands) and overflow lists
+  P.o_wb = take((size_t)3 * (X + kEnds) * GS * 4);
+  P.o_vs = take((size_t)3 * kEnds * 4);
+  P.o_pv = take((size_t)2 * R * 32);
+  P.o_ovl = take((size_t)2 * kOvlBytes);
+  P.o_prod = take(sizeof(Prod));
   P.o_ring = (int)off;
   const long long room = (long long)smem_optin - (long long)P.o_ring - kRingSlack;
   const long long tile_max = (long long)P.cap + 256LL * X;
-  if (((room / NG) & ~127LL) < (long long)min_tiles * tile_max) return false;  // each group's part of the ring
+  if ((room & ~127LL) < (long long)min_tiles * tile_max) return false;
   P.ring_bytes = (int)(room & ~127LL);
   out->smem = (size_t)P.o_ring + (size_t)P.ring_bytes + kRingSlack;
   return true;
 }
 
 // Preference: the anchor-score table in shared memory (the token gathers' fast path), with
-// room for two, then one of the largest staged tiles in each group's half of the ring, staged
+// room for three, then two of the largest staged tiles in the ring, staged
 // counts trimmed from their full values towards the mean (records first, then anchor-value
 // rows: a run beyond those takes the slowest fallback); then the table in global memory
-// (gathers through L1 and L2) the same way; then anything that holds one tile per group.
+// (gathers through L1 and L2) the same way; then anything that holds one tile.
 // table false: no anchor-score table is read (RoPE at decode), so none is placed in shared memory.
 bool make_plan(const Layout& L, int GS, int smem_optin, bool table, Plan* out, std::string* why) {
   const int R0 = full_r(L), X0 = full_x(L);
   const int Rmin = std::max(16, ((R0 * 3 / 4) + 15) & ~15), Xmin = std::max(16, ((X0 * 3 / 4) + 15) & ~15);
   for (int sa = table ? 1 : 0; sa >= 0; --sa)
-    for (int min_tiles : {2, 1})
+    for (int min_tiles : {3, 2})
       for (int X = X0; X >= Xmin; X -= 16)
         for (int R = R0; R >= Rmin; R -= 16)
           if (make_plan_rx(L, GS, R, X, sa == 1, smem_optin, min_tiles, out)) return true;
@@ -2263,10 +2376,14 @@ using DecodeFn = void (*)(const DecodeParams);
 using ScoreFn = void (*)(const ScoreParams);
 using ScoreTcFn = void (*)(const ScoreParams, const CUtensorMap, const CUtensorMap);
 using RopeFn = void (*)(const RopeParams);
+template <int GS, int MODE>
+DecodeFn decode_kernel_c(int codec) {
+  return codec ? akv_decode_kernel<GS, 1, MODE> : akv_decode_kernel<GS, 0, MODE>;
+}
 template <int GS>
-DecodeFn decode_kernel(int codec, int rope) {
-  if (rope) return codec ? akv_decode_kernel<GS, 1, 1> : akv_decode_kernel<GS, 0, 1>;
-  return codec ? akv_decode_kernel<GS, 1, 0> : akv_decode_kernel<GS, 0, 0>;
+DecodeFn decode_kernel(int codec, int rope, const DecodeParams& P) {
+  if (rope) return decode_kernel_c<GS, kRope>(codec);
+  return P.smem_sa ? decode_kernel_c<GS, kTableSmem>(codec) : decode_kernel_c<GS, kTableGlobal>(codec);
 }
 template <int GS>
 RopeFn rope_kernel(int codec) {
@@ -2276,6 +2393,9 @@ template <int GS>
 ScoreTcFn score_kernel() {
   return akv_scores_tc_kernel<GS>;
 }
+
+// 64-anchor chunks up to which the small score kernel takes the anchor scores: a few waves of its CTAs.
+constexpr int kSmallChunks = 1024;
 
 template <int GS>
 ScoreFn suffix_kernel(bool rope) {
@@ -2287,9 +2407,10 @@ ScoreFn suffix_kernel(bool rope) {
 struct LaunchKey {
   int dev, G, codec, rope, units, max_len, max_k, ctas;
   long long dens_key, adens_key, ttot;
+  std::vector<int32_t> tiles;  // per unit: the CTAs' ranges depend on the order of the lengths
   bool operator<(const LaunchKey& o) const {
-    return std::tie(dev, G, codec, rope, units, max_len, max_k, ctas, dens_key, adens_key, ttot) <
-           std::tie(o.dev, o.G, o.codec, o.rope, o.units, o.max_len, o.max_k, o.ctas, o.dens_key, o.adens_key, o.ttot);
+    return std::tie(dev, G, codec, rope, units, max_len, max_k, ctas, dens_key, adens_key, ttot, tiles) <
+           std::tie(o.dev, o.G, o.codec, o.rope, o.units, o.max_len, o.max_k, o.ctas, o.dens_key, o.adens_key, o.ttot, o.tiles);
   }
 };
 
@@ -2304,7 +2425,12 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   int dev = 0;
   cudaGetDevice(&dev);
   long long ttot = 0;
-  for (const auto& s : L.shape) ttot += s.nt;
+  std::vector<int32_t> tiles;
+  tiles.reserve(L.shape.size());
+  for (const auto& s : L.shape) {
+    ttot += s.nt;
+    tiles.push_back(s.nt);
+  }
   // testing controls (akv_decode_set_debug): a requested number of CTAs, and the failure-detection
   // hook with which every CTA withholds the last tile of its range, so the waits on it run out
   // after their bound and the outputs of its units become NaN
@@ -2313,7 +2439,7 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   const int codec = (p.flags & AKV_FLAG_LLOYD) ? 1 : 0;
   const int rope = (p.flags & AKV_FLAG_ROPE) ? 1 : 0;
   const LaunchKey key{dev, L.G, codec, rope, units, L.max_len, L.max_k, ctas, (long long)(max_density(L) * 1e6),
-                      (long long)(max_anchor_density(L) * 1e6), ttot};
+                      (long long)(max_anchor_density(L) * 1e6), ttot, std::move(tiles)};
   Plan pl;
   bool have = false;
   {
@@ -2326,10 +2452,10 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   }
   if (!have) {
     const DeviceInfo di = device_info();
-    cudaError_t e =
-        cudaFuncSetAttribute(decode_kernel<GS>(codec, rope), cudaFuncAttributeMaxDynamicSharedMemorySize, di.smem_optin);
-    if (e != cudaSuccess) return (int)e;
     if (!make_plan(L, GS, di.smem_optin, !rope, &pl, why)) return -1;
+    cudaError_t e =
+        cudaFuncSetAttribute(decode_kernel<GS>(codec, rope, pl.P), cudaFuncAttributeMaxDynamicSharedMemorySize, di.smem_optin);
+    if (e != cudaSuccess) return (int)e;
     if ((e = cudaFuncSetAttribute(score_kernel<GS>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)kScDynSmem)) != cudaSuccess)  // the score launch's stages
       return (int)e;
@@ -2364,7 +2490,6 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   P.sa = (const float*)(wsb + W.o_sa);
   P.cmax = (const float*)(wsb + W.o_cmax);
   P.part = (float*)(wsb + W.o_part);
-  P.cnt = (unsigned*)(wsb + W.o_cnt);
   P.uh = wsb + W.o_uh;
   P.uh_stride = (hdr_bytes(GS) + 255) & ~255;
   P.n_kv_heads = p.n_kv_heads;
@@ -2386,7 +2511,6 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   S.q = P.q;
   S.sa = (float*)(wsb + W.o_sa);
   S.cmax = (float*)(wsb + W.o_cmax);
-  S.cnt = P.cnt;
   S.n_kv_heads = p.n_kv_heads;
   S.n_q_heads = p.n_q_heads;
   S.G = L.G;
@@ -2413,13 +2537,15 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   get_decode_events(&ev_scores_p, &ev_decode_p);
   const cudaEvent_t ev_scores = (cudaEvent_t)ev_scores_p, ev_decode = (cudaEvent_t)ev_decode_p;
   cudaError_t e;
+  bool beside = false;  // the decode may start beside the launch before it
   if (rope) {  // the logits of every stored token (no anchor scores)
     RopeParams R;
     R.arena = P.arena;
     R.q = P.q;
     R.lg = (float*)(wsb + W.o_lg);
     R.cmax = (float*)(wsb + W.o_cmax);
-    R.cnt = P.cnt;
+    R.uh = P.uh;
+    R.uh_stride = P.uh_stride;
     R.n_kv_heads = p.n_kv_heads;
     R.n_q_heads = p.n_q_heads;
     R.rotate = P.rotate;
@@ -2436,6 +2562,12 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
     cfg.gridDim = dim3((unsigned)(units * P.n_ch), 1, 1);
     e = cudaLaunchKernelEx(&cfg, rope_kernel<GS>(codec), R);
     for (int j = 0; j < 64; ++j) S.turn[j] = R.turn[j];
+  } else if ((long long)units * P.n_ch <= kSmallChunks) {
+    S.units = units;
+    S.arena_rows = (long long)(arena_bytes / 256);
+    cfg.gridDim = dim3((unsigned)(units + units * P.n_ch), 1, 1);
+    e = cudaLaunchKernelEx(&cfg, akv_scores_small_kernel<GS>, S);
+    beside = true;
   } else {
     // anchor rows of every unit through one map over the caller's arena as 256-byte rows (each
     // unit's anchor-key section starts its 256-byte-aligned segment; a full-selection arena places
@@ -2471,10 +2603,17 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   cfg.gridDim = dim3((unsigned)pl.grid, 1, 1);
   cfg.blockDim = dim3(NT, 1, 1);
   cfg.dynamicSmemBytes = pl.smem;
-  e = cudaLaunchKernelEx(&cfg, decode_kernel<GS>(codec, rope), P);
+  cudaLaunchAttribute pdl;
+  pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  pdl.val.programmaticStreamSerializationAllowed = 1;
+  if (beside) {
+    cfg.attrs = &pdl;
+    cfg.numAttrs = 1;
+  }
+  e = cudaLaunchKernelEx(&cfg, decode_kernel<GS>(codec, rope, P), P);
   if (e != cudaSuccess) {
     cudaFuncAttributes fa{};
-    cudaFuncGetAttributes(&fa, decode_kernel<GS>(codec, rope));
+    cudaFuncGetAttributes(&fa, decode_kernel<GS>(codec, rope, P));
     *why = "(decode kernel: " + std::to_string(fa.numRegs) + " registers, max " + std::to_string(fa.maxThreadsPerBlock) +
            " threads, " + std::to_string(pl.smem) + " B dynamic shared memory of " +
            std::to_string(fa.maxDynamicSharedSizeBytes) + ", grid " + std::to_string(pl.grid) + ")";

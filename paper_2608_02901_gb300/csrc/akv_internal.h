@@ -133,10 +133,9 @@ constexpr int kSuffixChunk = 64;
 constexpr int kMaxGrid = 256;       // CTAs of the decode launch at most
 constexpr int CHA = 64;             // anchors per chunk maximum of the score launch
 // floats of one CTA's partial slot for a unit: numerator y [GS][128] (the inverse rotation already
-// applied), normaliser l [GS] (8 places), failure flag, pad to 16 bytes
+// applied), normaliser l [GS] (8 places), pad
 AKV_HD constexpr int part_floats(int GS) { return 128 * GS + 12; }
 AKV_HD constexpr int part_l(int GS) { return 128 * GS; }
-AKV_HD constexpr int part_flag(int GS) { return 128 * GS + 8; }
 
 // Bytes of a unit's query header (from the score kernel): the rotated query q' [GS][128] f32, its
 // sums [8] f32, and the key-residual mma B fragments [GS == 8 ? 2 : 1][8][32] uint2.
