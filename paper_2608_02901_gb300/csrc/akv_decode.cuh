@@ -1303,7 +1303,7 @@ struct TokTile {
   const float* SAt;   // anchor scores [k][GS]
   const float* rows;  // [0,8): -m, [8,16): -inf, [16,24): sum q'
   const float* qp;    // [GS][128] rotated query
-  float* pv;          // [R][8] p rows of the value records
+  float* pv;          // [R][GS] p rows of the value records
   float* W;           // [X][GS] the tile's value weights
   float* ovf;         // [2][GS][128] overflow sums
   const uint8_t* AV;  // the unit's anchor values (global)
@@ -1423,7 +1423,7 @@ __device__ __noinline__ LShare<(GS >= 2 ? GS / 2 : 1)> token_chunk_general(const
     rvn += (int)vb;
     if (vb && e < nvalid) {
       if (rv < nVs) {
-        store_row<GS>(pv + rv * 8, pe);
+        store_row<GS>(pv + rv * GS, pe);
       } else {  // beyond the staged records: listed for the group (else on CUDA cores here)
         const int en_i = atomicAdd(ovl_n, 1);
         if (en_i < kOvl) {
@@ -1652,7 +1652,6 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   for (int e = tid; e < 2 * GS * 128; e += NT) ovf[e] = 0.f;  // (the overflow's sums start at zero)
-  for (int e = tid; e < 2 * P.R * 8; e += NT) reinterpret_cast<float*>(smem + P.o_pv)[e] = 0.f;
   __syncthreads();
 
   if (tid == 0)
@@ -1739,7 +1738,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
           const bool fast_tile = mt.fast & 1u;
           float* W = reinterpret_cast<float*>(smem + P.o_wb) + (lt % 3) * (P.X + kEnds) * GS;
           int* vs = reinterpret_cast<int*>(smem + P.o_vs) + (lt % 3) * kEnds;
-          float* pv = reinterpret_cast<float*>(smem + P.o_pv) + b * P.R * 8;
+          float* pv = reinterpret_cast<float*>(smem + P.o_pv) + b * P.R * GS;
           // ---- tokens: lane -> stored tokens t0 .. t0 + 3, every head ----
           const int t0 = wi8 * (32 * LCH) + LCH * lane;
           TokLane tl;
@@ -1825,7 +1824,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
                   l2[i2] = __fadd2_rn(l2[i2], pe[i2]);
                 }
                 const bool vb = (tl.vbits >> e) & 1u;
-                if (vb) store_row<GS>(pv + rv * 8, pe);
+                if (vb) store_row<GS>(pv + rv * GS, pe);
                 rv += (int)vb;
                 // the run of `key` ends here when the slot changes (branch-free): the lane's first
                 // run is kept as its head (it may continue the previous lane's); a later one started
@@ -2026,7 +2025,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
         const Meta mt = meta[lt % NSG];
         const uint8_t* st = ring + mt.ring_off;
         float* W = reinterpret_cast<float*>(smem + P.o_wb) + (lt % 3) * (P.X + kEnds) * GS;
-        float* pv = reinterpret_cast<float*>(smem + P.o_pv) + b * P.R * 8;
+        float* pv = reinterpret_cast<float*>(smem + P.o_pv) + b * P.R * GS;
         const int nVs = mt.nVs, nr = (int)mt.nrows, nb16 = (nr + 15) / 16;
         if (go) {
           if (!(mt.fast & 1u)) {  // the overflow lists: thread mt_ takes dimension mt_ % 128 of every entry of one list
@@ -2074,13 +2073,12 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
           for (int x = wi8; x < n_vg + nb16 + 1; x += NMW) {
             const bool val = x < n_vg;
             const int blk = x - n_vg;  // block of slots; the last one: the token warps' first and last runs
-            float* src = val ? pv + 128 * x : (blk < nb16 ? W + 16 * GS * blk : W + P.X * GS);
-            const int stride = val ? 8 : GS;
+            float* src = val ? pv + 16 * GS * x : (blk < nb16 ? W + 16 * GS * blk : W + P.X * GS);
             const int lim = val ? nVs - 16 * x : (blk < nb16 ? nr - 16 * blk : kEnds);
             const int kk[4] = {2 * c4, 2 * c4 + 1, 2 * c4 + 8, 2 * c4 + 9};
             float f[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) f[e] = kk[e] < lim && r8 < GS ? src[kk[e] * stride + r8] : 0.f;
+            for (int e = 0; e < 4; ++e) f[e] = kk[e] < lim && r8 < GS ? src[kk[e] * GS + r8] : 0.f;
             if (val) {
               uint32_t smn[4];
               const uint32_t so = mt.sm_v + 64u * (uint32_t)x;  // (padded to 16 bytes: pairs may be read together)
@@ -2142,7 +2140,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
           // this lane's two code words hold dimensions 16 wi8 + 8 nb + r8 of 16 records ----
           const uint32_t woff = mt.cd_v + 4u * (uint32_t)(32 * (wi8 >> 1) + 4 * r8 + 2 * (wi8 & 1));
           auto residual = [&](int g16, const uint2 w2) {
-            const uint4 a = r8 < GS ? *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(pv) + g16 * 512 + lane * 16)
+            const uint4 a = r8 < GS ? *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(pv) + g16 * 64 * GS + lane * 16)
                                     : make_uint4(0u, 0u, 0u, 0u);
             const uint32_t wd[2] = {w2.x, w2.y};
 #pragma unroll
@@ -2291,16 +2289,28 @@ double max_anchor_density(const Layout& L) {
   return dens;
 }
 
-// Records staged per tile and side: 1.35x the densest unit's mean plus slack, at most 320;
-// records of a denser tile beyond these take the CUDA-core paths, which cost far more.
+double mean_density(const Layout& L) {
+  double n = 0.0, t = 0.0;
+  for (const auto& s : L.shape) {
+    n += (double)std::max(s.nk, s.nv);
+    t += (double)s.S;
+  }
+  return n / t;
+}
+
+// Value records per tile with p rows at least: 1.35x the densest unit's mean plus slack, at most 320; records of a
+// denser tile beyond the plan's count take the CUDA-core paths, which cost far more.  An encoder's tiles
+// are uneven (tokens of a cluster lie together and their residuals are alike), so a plan takes as many
+// more as shared memory has room for: a 32K layer of 656 anchors whose densest tile held more than 1.35x the mean
+// plus slack took 42 us with that count and 19 us with all its records staged.
 int full_r(const Layout& L) {
   const int R = (int)(T * max_density(L) * 1.35) + 32;
   return std::min(320, std::max(16, (R + 15) & ~15));
 }
-// Anchor-value rows staged per tile: 1.5x the mean number of value slots a tile covers plus
+// Anchor-value rows staged per tile: 2x the mean number of value slots a tile covers plus
 // slack, at most 256; runs on slots beyond these take a CUDA-core path.
 int full_x(const Layout& L) {
-  const int X = (int)(1.5 * (T * max_anchor_density(L) + 1.0)) + 16;
+  const int X = (int)(2.0 * (T * max_anchor_density(L) + 1.0)) + 16;
   return std::min(256, std::max(16, (X + 15) & ~15));
 }
 
@@ -2311,13 +2321,11 @@ struct Plan {
   int sms = 0;  // SMs of the device (the score launch: one CTA each)
 };
 
-// Shared-memory carve-up for (R, X, table in shared memory or not); false if the ring
-// would hold fewer than `min_tiles` of the largest staged tiles.
-bool make_plan_rx(const Layout& L, int GS, int R, int X, bool smem_sa, int smem_optin, int min_tiles, Plan* out) {
+// Shared-memory carve-up for X anchor-value rows, the table in shared memory or not, a ring of at least
+// `ring_min` bytes, and as many p rows as fit beside it, at least Rmin; false if they don't.
+bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, bool smem_sa, int smem_optin, long long ring_min, Plan* out) {
   DecodeParams& P = out->P;
-  P.R = R;
   P.X = X;
-  P.cap = (int)(F_MAX + 2 * round16(4u * (uint32_t)R) + 64u * (uint32_t)R);
   P.ka_stride = (L.max_k + 3) & ~3;
   P.smem_sa = smem_sa ? 1 : 0;
   size_t off = 0;
@@ -2338,36 +2346,41 @@ bool make_plan_rx(const Layout& L, int GS, int R, int X, bool smem_sa, int smem_
   // p rows (then A operands) and overflow lists
   P.o_wb = take((size_t)3 * (X + kEnds) * GS * 4);
   P.o_vs = take((size_t)3 * kEnds * 4);
-  P.o_pv = take((size_t)2 * R * 32);
   P.o_ovl = take((size_t)2 * kOvlBytes);
   P.o_prod = take(sizeof(Prod));
+  const long long room = (long long)smem_optin - (long long)off - kRingSlack - 128;
+  const long long fit = (room - ring_min) / (2 * GS * 4) & ~15LL;
+  if (fit < Rmin) return false;
+  P.R = (int)std::min<long long>(fit, T);
+  P.o_pv = take((size_t)2 * P.R * GS * 4);
   P.o_ring = (int)off;
-  const long long room = (long long)smem_optin - (long long)P.o_ring - kRingSlack;
-  const long long tile_max = (long long)P.cap + 256LL * X;
-  if ((room & ~127LL) < (long long)min_tiles * tile_max) return false;
-  P.ring_bytes = (int)(room & ~127LL);
+  P.ring_bytes = (int)(((long long)smem_optin - (long long)off - kRingSlack) & ~127LL);
+  // staged bytes of a tile block at most: all of one with R records per side, as far as the ring holds it
+  // beside its anchor-value rows
+  P.cap = (int)std::min<long long>((long long)(F_MAX + 2 * round16(4u * (uint32_t)P.R) + 64u * (uint32_t)P.R),
+                                   (P.ring_bytes - 256LL * X) & ~15LL);
+  if (P.cap < (int)F_MAX) return false;
   out->smem = (size_t)P.o_ring + (size_t)P.ring_bytes + kRingSlack;
   return true;
 }
 
-// Preference: the anchor-score table in shared memory (the token gathers' fast path), with
-// room for three, then two of the largest staged tiles in the ring, staged
-// counts trimmed from their full values towards the mean (records first, then anchor-value
-// rows: a run beyond those takes the slowest fallback); then the table in global memory
-// (gathers through L1 and L2) the same way; then anything that holds one tile.
+// Preference: the anchor-score table in shared memory (the token gathers' fast path), with a ring of four and
+// a half mean tiles (one in each role, one landing, and what wrapping around leaves unused), then less, the
+// least p rows and anchor-value rows trimmed towards 3/4 of their values with it; then the table in global
+// memory (gathers through L1 and L2) the same way; then anything that holds one tile.
 // table false: no anchor-score table is read (RoPE at decode), so none is placed in shared memory.
 bool make_plan(const Layout& L, int GS, int smem_optin, bool table, Plan* out, std::string* why) {
   const int R0 = full_r(L), X0 = full_x(L);
   const int Rmin = std::max(16, ((R0 * 3 / 4) + 15) & ~15), Xmin = std::max(16, ((X0 * 3 / 4) + 15) & ~15);
+  const double mean = (double)F_MAX + T * mean_density(L) * 72.0 + 256.0 + 256.0 * (T * max_anchor_density(L) + 2.0);
   for (int sa = table ? 1 : 0; sa >= 0; --sa)
-    for (int min_tiles : {3, 2})
-      for (int X = X0; X >= Xmin; X -= 16)
-        for (int R = R0; R >= Rmin; R -= 16)
-          if (make_plan_rx(L, GS, R, X, sa == 1, smem_optin, min_tiles, out)) return true;
-  for (int min_tiles : {1})
-    for (int X = X0; X >= 16; X -= 16)
-      for (int R = R0; R >= 16; R -= 16)
-        if (make_plan_rx(L, GS, R, X, false, smem_optin, min_tiles, out)) return true;
+    for (const double tiles : {4.5, 3.5, 2.5}) {
+      const bool trim = tiles < 4.0;
+      for (int X = X0; X >= (trim ? Xmin : X0); X -= 16)
+        if (make_plan_rx(L, GS, trim ? Rmin : R0, X, sa == 1, smem_optin, (long long)(tiles * mean), out)) return true;
+    }
+  for (int X = X0; X >= 16; X -= 16)
+    if (make_plan_rx(L, GS, 16, X, false, smem_optin, (long long)F_MAX + 2 * 16 * 36 + 256LL * X, out)) return true;
   *why = "shared memory: no room for the decode pipeline";
   return false;
 }
@@ -2406,11 +2419,11 @@ ScoreFn suffix_kernel(bool rope) {
 // call made during CUDA-graph capture only issues the launches.
 struct LaunchKey {
   int dev, G, codec, rope, units, max_len, max_k, ctas;
-  long long dens_key, adens_key, ttot;
+  long long dens_key, adens_key, mdens_key, ttot;
   std::vector<int32_t> tiles;  // per unit: the CTAs' ranges depend on the order of the lengths
   bool operator<(const LaunchKey& o) const {
-    return std::tie(dev, G, codec, rope, units, max_len, max_k, ctas, dens_key, adens_key, ttot, tiles) <
-           std::tie(o.dev, o.G, o.codec, o.rope, o.units, o.max_len, o.max_k, o.ctas, o.dens_key, o.adens_key, o.ttot, o.tiles);
+    return std::tie(dev, G, codec, rope, units, max_len, max_k, ctas, dens_key, adens_key, mdens_key, ttot, tiles) <
+           std::tie(o.dev, o.G, o.codec, o.rope, o.units, o.max_len, o.max_k, o.ctas, o.dens_key, o.adens_key, o.mdens_key, o.ttot, o.tiles);
   }
 };
 
@@ -2439,7 +2452,7 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   const int codec = (p.flags & AKV_FLAG_LLOYD) ? 1 : 0;
   const int rope = (p.flags & AKV_FLAG_ROPE) ? 1 : 0;
   const LaunchKey key{dev, L.G, codec, rope, units, L.max_len, L.max_k, ctas, (long long)(max_density(L) * 1e6),
-                      (long long)(max_anchor_density(L) * 1e6), ttot, std::move(tiles)};
+                      (long long)(max_anchor_density(L) * 1e6), (long long)(mean_density(L) * 1e6), ttot, std::move(tiles)};
   Plan pl;
   bool have = false;
   {
