@@ -1111,28 +1111,52 @@ __device__ __forceinline__ void head_probs(float gk, const float (&sa)[GS], cons
 // Keys are stored pre-RoPE, so a token's score no longer factors through its anchor's score:
 // q . R(p_i) x^_i with x^_i = gamma_i x_a(i) + r~_i (Eq. 3) and R(p) the rotate-half RoPE turn
 // of dimension pairs (j, j + 64) by p theta_j (Section 3.2; Appendix E.1's score kernel rebuilds
-// keys and applies RoPE from the stored positions the same way).  CTA (unit u, chunk c): stored
-// tokens 64 c .. 64 c + 63; warp w rebuilds tokens 16 w .. 16 w + 15, lane l holding dimensions
-// 4 l .. 4 l + 3 (pair partners sit 16 lanes apart), into shared memory; then its 16 x G logits
-// come from tensor-core products (keys as fp16 high + low parts, q exact).  The angle of pair j
-// at position p is taken as a binary fraction of a turn, p * turn_j mod 2^64 (exact integer
-// arithmetic), so the sine and cosine are evaluated on [0, 2 pi) whatever the position.
+// keys and applies RoPE from the stored positions the same way).  A warp takes 64 consecutive stored tokens
+// (a word of the bitmap), 16 at a time, in the layout of the products' A operand: lane (r8, c4) holds dimension
+// pairs 16 c4 .. 16 c4 + 15 of tokens r8 and r8 + 8, so a key is rebuilt, turned and split into fp16 high and
+// low parts in the registers that the products read (no shuffles, no shared memory; q exact).  The residuals of
+// the few tokens that have one are inverse-rotated by the whole warp into shared memory first.  The angle
+// of pair j at position p is taken as a binary fraction of a turn, p * turn_j mod 2^64 (exact integer
+// arithmetic; its upper 32 bits are kept, as a signed fraction), so the sine and cosine are evaluated on [-pi, pi)
+// whatever the position.
+// Bound: issue slots (51-57 % of them used, about 80 warp instructions per token: 2 x 64 x (angle, sine, cosine,
+// turn, split)) and the latencies between them at 3 blocks of 136 registers per SM; the special-function units are
+// next.  8 KV heads, requests of 40960, 20011, 65536 and 9001 tokens (1.08 M tokens), G = 4: 138 us; a warp per
+// token with four dimensions per lane, which traded angles and partners by shuffles and passed keys through shared
+// memory, took 322 us (163 warp instructions per token).  Of the whole decode, 179 us: with records read two tokens
+// ahead 198, with 96 registers and 5 blocks per SM 205 (spills).
+constexpr int kRopeWarps = 4;
 template <int GS, int CODEC>
-__global__ void __launch_bounds__(128) akv_rope_logits_kernel(const RopeParams P) {
-  __shared__ __align__(16) float ys[64][132];  // rows 16-byte aligned; 128-bit reads conflict-free
-  __shared__ __align__(16) float qsm[8][128];
-  __shared__ float wmx4[4][8];
-  __shared__ unsigned long long turn[64];
-  const int u = blockIdx.x / P.n_tch, c = blockIdx.x % P.n_tch;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+__global__ void __launch_bounds__(kRopeWarps * 32) akv_rope_logits_kernel(const RopeParams P) {
+  __shared__ __align__(16) float rs[kRopeWarps][17][132];  // a group's inverse-rotated residuals, and a row of zeros
+  __shared__ uint2 turn[64];                               // low and high words
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, r8 = lane >> 2, c4 = lane & 3;
+  const int n_blk = (P.n_tch + kRopeWarps - 1) / kRopeWarps;
+  const int u = blockIdx.x / n_blk, c = (blockIdx.x % n_blk) * kRopeWarps + warp;  // unit, 64-token chunk
   const akv_unit_desc* d = unit_desc(P.arena, u);
   const int S = d->len, k = d->n_anchors;
-  if (c == 0 && tid < 8) unit_counters(P.uh, P.uh_stride, u, GS)[tid] = 0u;
+  if (blockIdx.x % n_blk == 0 && tid < 8) unit_counters(P.uh, P.uh_stride, u, GS)[tid] = 0u;
+  if (tid < 64) turn[tid] = make_uint2((uint32_t)P.turn[tid], (uint32_t)(P.turn[tid] >> 32));
+  *reinterpret_cast<float4*>(&rs[warp][16][4 * lane]) = make_float4(0.f, 0.f, 0.f, 0.f);
+  __syncthreads();
   const int ts0 = 64 * c;
   if (ts0 >= S) return;  // past this unit's end (a shorter request)
   const size_t qb = qrow_base(u, P.n_kv_heads, P.n_q_heads);
-  for (int e = tid; e < GS * 128; e += 128) qsm[e / 128][e % 128] = __bfloat162float(P.q[qb + e]);
-  if (tid < 64) turn[tid] = P.turn[tid];
+  // B operand, head r8: k places (2 c4, 2 c4 + 1) of step ks are dims 16 c4 + 2 ks, + 1, those 8 on dims 64 higher
+  uint32_t bq[8][2];
+#pragma unroll
+  for (int ks = 0; ks < 8; ++ks)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float2 v = make_float2(0.f, 0.f);
+      if (r8 < GS) {
+        const uint32_t w = *reinterpret_cast<const uint32_t*>(P.q + qb + (size_t)r8 * 128 + 64 * h + 16 * c4 + 2 * ks);
+        v = make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+      }
+      const __half2 b = __float22half2_rn(v);
+      bq[ks][h] = *reinterpret_cast<const uint32_t*>(&b);
+    }
   // the chunk inside its tile block: one bitmap word (64 tokens) per side
   const int j = ts0 / T, tl0 = ts0 % T;
   const int n = min(T, S - j * T), nw = (int)tile_words(n), n64 = 64 * nw;
@@ -1146,148 +1170,120 @@ __global__ void __launch_bounds__(128) akv_rope_logits_kernel(const RopeParams P
   const uint64_t word = bm[tl0 / 64];
   const int rbase = rkk[tl0 / 64];
   const uint8_t* AK = P.arena + d->off_anchor_k;
-  const uint32_t* pos = reinterpret_cast<const uint32_t*>(P.arena + d->off_pos);
-  __syncthreads();
-  // per lane: the turns of the two pair angles it evaluates (lanes 0-15 pairs 0, 1 of their four,
-  // lanes 16-31 pairs 2, 3), the rotation signs of its dimensions with the 1/128 folded in
-  const bool low = lane < 16;
-  const unsigned long long tn0 = turn[(4 * lane + (low ? 0 : 2)) & 63], tn1 = turn[(4 * lane + (low ? 1 : 3)) & 63];
-  const float rsgn = low ? -1.f : 1.f;  // y = x cos - x' sin below the partner, x cos + x' sin above
+  const uint32_t* kst = reinterpret_cast<const uint32_t*>(blk) + tl0;
+  const uint32_t* pos = reinterpret_cast<const uint32_t*>(P.arena + d->off_pos) + ts0;
+  // rotation signs of dims 4 lane .. 4 lane + 3 with the 1/128 folded in (the residuals' layout)
   float sgn128[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
     const unsigned long long sb = lane < 16 ? P.sign_lo : P.sign_hi;
     sgn128[e] = (P.rotate ? (((sb >> ((4 * lane + e) & 63)) & 1ull) ? -1.f : 1.f) : 1.f) * (P.rotate ? 1.0f / 128.0f : 1.f);
   }
-  // the warp's 16 tokens: lane i < 16 fetches token i's stream word and position; every lane then
-  // loads its 8 bytes of all 16 anchor rows, and the records of the tokens with a residual, before
-  // any arithmetic (the loads do not wait on one another)
-  const int tw = tl0 + 16 * warp;
-  const int nwt = max(0, min(16, n - tw));  // the warp's tokens inside the tile
-  uint32_t ek_l = 0u, pos_l = 0u;
-  if (lane < nwt) {
-    ek_l = reinterpret_cast<const uint32_t*>(blk)[tw + lane];
-    pos_l = pos[j * T + tw + lane];
-  }
-  uint2 xa[16];
-  uint32_t smn[16], cbyte[16];
-  const uint32_t wbits = (uint32_t)(word >> (tw % 64)) & 0xFFFFu;  // residual flags of the 16 tokens
+  const int n_tok = min(64, S - ts0);  // the chunk's tokens
+  float mx[2] = {-INFINITY, -INFINITY};
+  // stream words and positions of the lane's tokens r8 and r8 + 8 of a group, read one group ahead
+  uint32_t ekn[2], psn[2];
+  auto read_words = [&](int g) {
 #pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const uint32_t ek = __shfl_sync(0xffffffffu, ek_l, i);
-    const int a = min((int)(ek & 0xFFFFu), k - 1);
-    xa[i] = i < nwt ? *reinterpret_cast<const uint2*>(AK + (size_t)a * 256 + 16 * ((lane >> 1) ^ (a & 7)) + 8 * (lane & 1))
-                    : make_uint2(0u, 0u);
-    smn[i] = 0u;
-    cbyte[i] = 0u;
-    if (i < nwt && ((wbits >> i) & 1u)) {
-      const int r = rbase + __popcll(word & ((1ull << ((tw % 64) + i)) - 1ull));
-      smn[i] = *reinterpret_cast<const uint32_t*>(blk + sm_k + 4u * (uint32_t)r);
-      cbyte[i] = blk[cd_k + 32u * (uint32_t)r + (uint32_t)lane];
+    for (int x = 0; x < 2; ++x) {
+      const int t = 16 * g + 8 * x + r8;
+      ekn[x] = t < n_tok ? kst[t] : 0u;
+      psn[x] = t < n_tok ? pos[t] : 0u;
     }
-  }
+  };
+  read_words(0);
+#pragma unroll 1  // (unrolled, the four groups' code does not fit the instruction cache: 251 us, not 138)
+  for (int g = 0; 16 * g < n_tok; ++g) {
+    const uint32_t ek[2] = {ekn[0], ekn[1]}, ps[2] = {psn[0], psn[1]};
+    read_words(g + 1);
+    // the anchor rows' 16-byte chunks 2 c4, 2 c4 + 1 and 8 + 2 c4, 9 + 2 c4 (stored at chunk ^ (slot % 8))
+    uint4 xr[2][4];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) {  // (fully unrolled: the per-token arrays stay in registers)
-    float y[4] = {0.f, 0.f, 0.f, 0.f};
-    const uint32_t ek = __shfl_sync(0xffffffffu, ek_l, i);
-    const uint32_t p = __shfl_sync(0xffffffffu, pos_l, i);
-    if (i < nwt) {  // (the same for the whole warp)
-      const float gk = half_hi(ek);
-      float x[4];
-      x[0] = gk * __bfloat162float(__ushort_as_bfloat16((unsigned short)(xa[i].x & 0xFFFFu)));
-      x[1] = gk * __bfloat162float(__ushort_as_bfloat16((unsigned short)(xa[i].x >> 16)));
-      x[2] = gk * __bfloat162float(__ushort_as_bfloat16((unsigned short)(xa[i].y & 0xFFFFu)));
-      x[3] = gk * __bfloat162float(__ushort_as_bfloat16((unsigned short)(xa[i].y >> 16)));
-      if ((wbits >> i) & 1u) {  // plus r~ = s o H(c^) / 128, c^ = min + scale L[code] (warp-uniform)
+    for (int x = 0; x < 2; ++x) {
+      const int a = min((int)(ek[x] & 0xFFFFu), k - 1);
+      const uint8_t* row = AK + (size_t)a * 256;
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        const int ch = (h >> 1) * 8 + 2 * c4 + (h & 1);
+        xr[x][h] = *reinterpret_cast<const uint4*>(row + 16 * (ch ^ (a & 7)));
+      }
+    }
+    // residuals of the group's tokens: r~ = s o H(c^) / 128, c^ = min + scale L[code], into shared memory
+    const uint32_t wbits = (uint32_t)(word >> (16 * g)) & 0xFFFFu;
+    if (wbits) {
+      __syncwarp();  // the last group's rows are read
+      for (uint32_t left = wbits; left; left &= left - 1u) {
+        const int i = __ffs(left) - 1;
+        const int r = rbase + __popcll(word & ((1ull << (16 * g + i)) - 1ull));
+        const uint32_t smn = *reinterpret_cast<const uint32_t*>(blk + sm_k + 4u * (uint32_t)r);
+        const uint32_t byte = blk[cd_k + 32u * (uint32_t)r + (uint32_t)lane];
         float cr[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-          cr[e] = fmaf(half_lo(smn[i]), code_level((cbyte[i] >> (2 * e)) & 3u, CODEC), half_hi(smn[i]));
+        for (int e = 0; e < 4; ++e) cr[e] = fmaf(half_lo(smn), code_level((byte >> (2 * e)) & 3u, CODEC), half_hi(smn));
         if (P.rotate) warp_wht128(cr, lane);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) x[e] = fmaf(cr[e], sgn128[e], x[e]);
+        *reinterpret_cast<float4*>(&rs[warp][i][4 * lane]) =
+            make_float4(cr[0] * sgn128[0], cr[1] * sgn128[1], cr[2] * sgn128[2], cr[3] * sgn128[3]);
       }
-      // RoPE at the token's position: lanes 0-15 hold dims j < 64, lanes 16-31 their partners j + 64;
-      // the two halves each evaluate two of the four pairs' angles and trade them
-      float sa[2], ca[2], sb[2], cb[2];
-      __sincosf((float)(uint32_t)(((unsigned long long)p * tn0) >> 40) * (6.2831853071795865f / 16777216.0f), &sa[0], &ca[0]);
-      __sincosf((float)(uint32_t)(((unsigned long long)p * tn1) >> 40) * (6.2831853071795865f / 16777216.0f), &sa[1], &ca[1]);
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {  // the partner half's two angles
-        sb[h] = __shfl_xor_sync(0xffffffffu, sa[h], 16);
-        cb[h] = __shfl_xor_sync(0xffffffffu, ca[h], 16);
-      }
-      // pair e of this lane: pairs 0, 1 from the lower half's angles, pairs 2, 3 from the upper half's
-      const float sn[4] = {low ? sa[0] : sb[0], low ? sa[1] : sb[1], low ? sb[0] : sa[0], low ? sb[1] : sa[1]};
-      const float cs[4] = {low ? ca[0] : cb[0], low ? ca[1] : cb[1], low ? cb[0] : ca[0], low ? cb[1] : ca[1]};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float xp = __shfl_xor_sync(0xffffffffu, x[e], 16);
-        y[e] = fmaf(x[e], cs[e], rsgn * xp * sn[e]);
-      }
+      __syncwarp();
     }
-    *reinterpret_cast<float4*>(&ys[16 * warp + i][4 * lane]) = make_float4(y[0], y[1], y[2], y[3]);
-  }
-  __syncwarp();
-  // the warp's 16 logits rows on tensor cores: A = its rotated keys (fp16 high and low parts, from
-  // shared memory), B = the query rows (exact in fp16), fp32 sums: D[token][head] (heads >= GS zero)
-  {
-    const int r8 = lane >> 2, c4 = lane & 3;
-    float d[4] = {0.f, 0.f, 0.f, 0.f};
+    float d4[4] = {0.f, 0.f, 0.f, 0.f};
+    const float gk[2] = {half_hi(ek[0]), half_hi(ek[1])};
+    // a token's residual row, or the zeros
+    const float* rrow[2] = {rs[warp][((wbits >> r8) & 1u) ? r8 : 16] + 16 * c4, rs[warp][((wbits >> (r8 + 8)) & 1u) ? r8 + 8 : 16] + 16 * c4};
 #pragma unroll
-    for (int ks = 0; ks < 8; ++ks) {
-      const float* y0 = &ys[16 * warp + r8][16 * ks + 2 * c4];
-      const float* y1 = &ys[16 * warp + r8 + 8][16 * ks + 2 * c4];
-      const float2 v[4] = {*reinterpret_cast<const float2*>(y0), *reinterpret_cast<const float2*>(y1),
-                           *reinterpret_cast<const float2*>(y0 + 8), *reinterpret_cast<const float2*>(y1 + 8)};
-      uint32_t hi[4], lo[4];
+    for (int ks = 0; ks < 8; ++ks) {  // pairs 16 c4 + 2 ks, + 1
+      uint32_t hi[4], lo[4];          // A: token r8 lower dims, token r8 + 8 lower, r8 upper, r8 + 8 upper
+      const uint2 tn0 = turn[16 * c4 + 2 * ks], tn1 = turn[16 * c4 + 2 * ks + 1];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const __half2 h = __float22half2_rn(v[e]);
-        const float2 hf = __half22float2(h);
-        const __half2 l = __float22half2_rn(make_float2(v[e].x - hf.x, v[e].y - hf.y));
-        hi[e] = *reinterpret_cast<const uint32_t*>(&h);
-        lo[e] = *reinterpret_cast<const uint32_t*>(&l);
+      for (int x = 0; x < 2; ++x) {
+        const uint4 cl = xr[x][ks >> 2], cu = xr[x][2 + (ks >> 2)];
+        const uint32_t wl = (ks & 3) == 0 ? cl.x : ((ks & 3) == 1 ? cl.y : ((ks & 3) == 2 ? cl.z : cl.w));
+        const uint32_t wu = (ks & 3) == 0 ? cu.x : ((ks & 3) == 1 ? cu.y : ((ks & 3) == 2 ? cu.z : cu.w));
+        const float2 rl = *reinterpret_cast<const float2*>(rrow[x] + 2 * ks), ru = *reinterpret_cast<const float2*>(rrow[x] + 64 + 2 * ks);
+        const float a0 = fmaf(gk[x], __uint_as_float(wl << 16), rl.x), a1 = fmaf(gk[x], __uint_as_float(wl & 0xFFFF0000u), rl.y);
+        const float b0 = fmaf(gk[x], __uint_as_float(wu << 16), ru.x), b1 = fmaf(gk[x], __uint_as_float(wu & 0xFFFF0000u), ru.y);
+        const uint32_t p = ps[x];
+        float s0, c0, s1, c1;
+        __sincosf((float)(int)(__umulhi(p, tn0.x) + p * tn0.y) * (6.2831853071795865f / 4294967296.0f), &s0, &c0);
+        __sincosf((float)(int)(__umulhi(p, tn1.x) + p * tn1.y) * (6.2831853071795865f / 4294967296.0f), &s1, &c1);
+        const float2 yl = make_float2(fmaf(a0, c0, -b0 * s0), fmaf(a1, c1, -b1 * s1));
+        const float2 yu = make_float2(fmaf(b0, c0, a0 * s0), fmaf(b1, c1, a1 * s1));
+        const __half2 hl = __float22half2_rn(yl), hu = __float22half2_rn(yu);
+        const float2 fl = __half22float2(hl), fu = __half22float2(hu);
+        const __half2 ll = __float22half2_rn(make_float2(yl.x - fl.x, yl.y - fl.y));
+        const __half2 lu = __float22half2_rn(make_float2(yu.x - fu.x, yu.y - fu.y));
+        hi[x] = *reinterpret_cast<const uint32_t*>(&hl);
+        hi[2 + x] = *reinterpret_cast<const uint32_t*>(&hu);
+        lo[x] = *reinterpret_cast<const uint32_t*>(&ll);
+        lo[2 + x] = *reinterpret_cast<const uint32_t*>(&lu);
       }
-      const bool hv = r8 < GS;  // column n = r8 of B: head r8
-      const __half2 b0 = __float22half2_rn(hv ? make_float2(qsm[hv ? r8 : 0][16 * ks + 2 * c4], qsm[hv ? r8 : 0][16 * ks + 2 * c4 + 1])
-                                              : make_float2(0.f, 0.f));
-      const __half2 b1 = __float22half2_rn(hv ? make_float2(qsm[hv ? r8 : 0][16 * ks + 2 * c4 + 8], qsm[hv ? r8 : 0][16 * ks + 2 * c4 + 9])
-                                              : make_float2(0.f, 0.f));
-      const uint32_t ub0 = *reinterpret_cast<const uint32_t*>(&b0), ub1 = *reinterpret_cast<const uint32_t*>(&b1);
-      mma_f16(d, make_uint4(hi[0], hi[1], hi[2], hi[3]), ub0, ub1);
-      mma_f16(d, make_uint4(lo[0], lo[1], lo[2], lo[3]), ub0, ub1);
+      mma_f16(d4, make_uint4(hi[0], hi[1], hi[2], hi[3]), bq[ks][0], bq[ks][1]);
+      mma_f16(d4, make_uint4(lo[0], lo[1], lo[2], lo[3]), bq[ks][0], bq[ks][1]);
     }
     // D rows r8, r8 + 8 (tokens), columns 2 c4, 2 c4 + 1 (heads)
-    float mx[2] = {-INFINITY, -INFINITY};
 #pragma unroll
     for (int hr = 0; hr < 2; ++hr) {
-      const int ts = ts0 + 16 * warp + r8 + 8 * hr;
-      const bool ok = ts < S;
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int g = 2 * c4 + e;
-        const float l = d[2 * hr + e] * P.scale_log2;
-        if (ok && g < GS) {
-          P.lg[((size_t)u * P.s_stride + ts) * GS + g] = l;
-          mx[e] = fmaxf(mx[e], l);
-        }
+      const int ts = ts0 + 16 * g + r8 + 8 * hr;
+      const float l0 = d4[2 * hr] * P.scale_log2, l1 = d4[2 * hr + 1] * P.scale_log2;
+      if (ts < S && 2 * c4 < GS) {
+        float* o = P.lg + ((size_t)u * P.s_stride + ts) * GS + 2 * c4;
+        if constexpr (GS == 1) o[0] = l0;
+        else *reinterpret_cast<float2*>(o) = make_float2(l0, l1);
+        mx[0] = fmaxf(mx[0], l0);
+        mx[1] = fmaxf(mx[1], l1);
       }
     }
-#pragma unroll
-    for (int o = 4; o < 32; o <<= 1) {
-      mx[0] = fmaxf(mx[0], __shfl_xor_sync(0xffffffffu, mx[0], o));
-      mx[1] = fmaxf(mx[1], __shfl_xor_sync(0xffffffffu, mx[1], o));
-    }
-    if (lane < 4) {
-      wmx4[warp][2 * lane] = mx[0];
-      wmx4[warp][2 * lane + 1] = mx[1];
-    }
   }
-  __syncthreads();
-  if (tid < GS)
-    P.cmax[((size_t)u * P.n_tch + c) * GS + tid] =
-        fmaxf(fmaxf(wmx4[0][tid], wmx4[1][tid]), fmaxf(wmx4[2][tid], wmx4[3][tid]));
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) {
+    mx[0] = fmaxf(mx[0], __shfl_xor_sync(0xffffffffu, mx[0], o));
+    mx[1] = fmaxf(mx[1], __shfl_xor_sync(0xffffffffu, mx[1], o));
+  }
+  if (lane < 4) {
+    float* o = P.cmax + ((size_t)u * P.n_tch + c) * GS;
+    if (2 * lane < GS) o[2 * lane] = mx[0];
+    if (2 * lane + 1 < GS) o[2 * lane + 1] = mx[1];
+  }
 }
 
 // A lane's tokens of a tile: bitmap bytes and first record indices.
@@ -2572,9 +2568,12 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
     for (int j = 0; j < 64; ++j)
       R.turn[j] = (unsigned long long)std::ldexp(
           std::pow((double)p.rope_theta, -2.0 * (double)j / 128.0) / 6.283185307179586476925, 64);
-    cfg.gridDim = dim3((unsigned)(units * P.n_ch), 1, 1);
+    cfg.gridDim = dim3((unsigned)(units * ((P.n_ch + kRopeWarps - 1) / kRopeWarps)), 1, 1);
+    cfg.blockDim = dim3(kRopeWarps * 32, 1, 1);
     e = cudaLaunchKernelEx(&cfg, rope_kernel<GS>(codec), R);
+    cfg.blockDim = dim3(128, 1, 1);
     for (int j = 0; j < 64; ++j) S.turn[j] = R.turn[j];
+    beside = true;
   } else if ((long long)units * P.n_ch <= kSmallChunks) {
     S.units = units;
     S.arena_rows = (long long)(arena_bytes / 256);

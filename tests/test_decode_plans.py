@@ -38,3 +38,13 @@ def test_partial_tiles(dev, S, lloyd):  # noqa: F811
             d["min_k"] = d["min_k"] * 0
             d["min_v"] = d["min_v"] * 0
     _run_seeded(dev, p, [S], mutate=mutate)
+
+
+@pytest.mark.parametrize("S", [1, 8, 9, 15, 16, 17, 48, 64, 65, 255, 256, 257, 1023, 1025, 1281])
+@pytest.mark.parametrize("G,fr,rotate", [(1, 0.1, True), (2, 1.0, True), (4, 0.0, True), (4, 0.3, False), (8, 0.5, True)])
+def test_rope_chunks(dev, S, G, fr, rotate):  # noqa: F811
+    """Rotary keys at the edges of a warp's pieces (16 tokens), its bitmap word (64), a block (256) and a tile (1024),
+    with no, some and only residual tokens, beside a longer request."""
+    p = akv.Params(batch=2, n_kv_heads=2, n_q_heads=2 * G, res_frac_k=fr, res_frac_v=0.1, window=4, seed=6, rotate=rotate,
+                   rope=True, rope_theta=10000.0)
+    _run_seeded(dev, p, [S, 1300], sm_scale=0.1)
