@@ -474,21 +474,25 @@ __global__ void __launch_bounds__(256) enc_rows(const EncArgs A) {
 // anchor may be the nearest.
 //
 // One persistent CTA per SM takes items of 256 positions of one unit and side (two M = 128 tiles
-// that share every anchor chunk, which halves the L2 reads of the anchors), anchor chunks of 192.
-// Warp 8 copies (three position tiles and two anchor chunks in flight), warp 9 issues the
-// products (two accumulators of 192 TMEM columns), warps 10 and 11 take the positions' norms one
-// item ahead, warps 0-3 and 4-7 are the two tiles' epilogues:
-// a thread owns one position and takes 32 columns at a time without branches on single columns (those
-// diverge: in the first chunks nearly every column is some lane's new maximum, and the kernel took
-// 293 us that way): scores with the column number in their lowest bits give the largest and its
-// column, and a clamped sum how many come near it.  Waits are bounded; after a failure every remaining position gets the word that lets
+// that share every anchor chunk, which halves the L2 reads of the anchors), anchor chunks of 128.
+// Warp 16 copies (three position tiles and three anchor chunks in flight), warp 17 issues the products (two
+// accumulators of 128 TMEM columns per tile, taken by alternate chunks), warps 18 and 19 take the positions' norms one
+// item ahead, warps 0-15 are the epilogues, four per tile and accumulator: a thread owns one position and half of its
+// chunks, and takes 32 columns at a time without branches on single columns (those diverge: in the first chunks
+// nearly every column is some lane's new maximum, and the kernel took 293 us that way): scores with the column number
+// in their lowest bits give the largest and its column, and a clamped sum how many come near it.  The halves' candidates are put together at the
+// item's end.  Waits are bounded; after a failure every remaining position gets the word that lets
 // enc_finish decide it alone, so the result stays right.
-constexpr int kAtN = 192;
-constexpr int kAtA = 3, kAtB = 2;  // stages
+// Bound: the epilogues' latencies, some 190 instructions per 32 columns and warp (56 % of the issue slots, ALU pipe
+// 48 %, tensor pipe 28 %).  8 units of 32768 positions, 656 anchors: 126 us; 2 of 131072, 2621: 405 us.  With one
+// accumulator of 192 columns per tile and eight epilogue warps, loads a step ahead: 143 and 480 us; eight warps that
+// each take both tiles (inverse norms read once for them): 136 us.
+constexpr int kAtN = 128;
+constexpr int kAtA = 3, kAtB = 3;  // stages
 constexpr uint32_t kAtHalfA = 128 * 128, kAtHalfB = kAtN * 128;  // bytes of 64 of the 128 dimensions
 constexpr int kAtI = 4;  // chunks of inverse norms in flight
-constexpr uint32_t kAtSmem = kAtA * 2 * kAtHalfA + kAtB * 2 * kAtHalfB + kAtI * kAtN * 4 + 2 * 256 * 4 + 1024;
-constexpr int kAtThreads = 384;
+constexpr uint32_t kAtSmem = kAtA * 2 * kAtHalfA + kAtB * 2 * kAtHalfB + kAtI * kAtN * 4 + 2 * 256 * 4 + 2 * 256 * 8 + 1024;
+constexpr int kAtThreads = 640;
 constexpr float kAtMargin = 0x1p-14f;  // 2 x 2^-15, relative to |x|
 
 __device__ __forceinline__ float max3(float a, float b, float c) {
@@ -502,20 +506,22 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c) {
   asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
-// 32 columns of the thread's TMEM lane: the load is started, and waited for through the registers it fills,
-// so that nothing can read them in between.
-__device__ __forceinline__ void tc_ld32_start(uint32_t taddr, float2 (&v)[16]) {
+// a with its five lowest bits replaced by col, without the sign (one instruction: the mask is a register, since an
+// instruction holds one immediate)
+__device__ __forceinline__ float tagged(float a, uint32_t mask, uint32_t col) {
+  uint32_t r;
+  asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(r) : "r"(__float_as_uint(a)), "r"(mask), "r"(col));
+  return __uint_as_float(r);
+}
+// 32 columns of the thread's TMEM lane.  One statement with its wait: registers that a load fills before a separate
+// wait were copied, some 70 moves per 32 columns.
+__device__ __forceinline__ void tc_ld32(uint32_t taddr, float2 (&v)[16]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n"
+      " tcgen05.wait::ld.sync.aligned;"
       : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[2].x), "=f"(v[2].y), "=f"(v[3].x), "=f"(v[3].y), "=f"(v[4].x), "=f"(v[4].y), "=f"(v[5].x), "=f"(v[5].y), "=f"(v[6].x), "=f"(v[6].y), "=f"(v[7].x), "=f"(v[7].y), "=f"(v[8].x), "=f"(v[8].y), "=f"(v[9].x), "=f"(v[9].y), "=f"(v[10].x), "=f"(v[10].y), "=f"(v[11].x), "=f"(v[11].y), "=f"(v[12].x), "=f"(v[12].y), "=f"(v[13].x), "=f"(v[13].y), "=f"(v[14].x), "=f"(v[14].y), "=f"(v[15].x), "=f"(v[15].y)
       : "r"(taddr)
       : "memory");
-}
-__device__ __forceinline__ void tc_ld32_wait(float2 (&v)[16]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+f"(v[0].x), "+f"(v[0].y), "+f"(v[1].x), "+f"(v[1].y), "+f"(v[2].x), "+f"(v[2].y), "+f"(v[3].x), "+f"(v[3].y), "+f"(v[4].x), "+f"(v[4].y), "+f"(v[5].x), "+f"(v[5].y), "+f"(v[6].x), "+f"(v[6].y), "+f"(v[7].x), "+f"(v[7].y), "+f"(v[8].x), "+f"(v[8].y), "+f"(v[9].x), "+f"(v[9].y), "+f"(v[10].x), "+f"(v[10].y), "+f"(v[11].x), "+f"(v[11].y), "+f"(v[12].x), "+f"(v[12].y), "+f"(v[13].x), "+f"(v[13].y), "+f"(v[14].x), "+f"(v[14].y), "+f"(v[15].x), "+f"(v[15].y)
-               :
-               : "memory");
 }
 
 __global__ void __launch_bounds__(kAtThreads, 1)
@@ -523,7 +529,7 @@ __global__ void __launch_bounds__(kAtThreads, 1)
                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmA, long long items,
                   int max_t) {
   extern __shared__ __align__(1024) uint8_t as_dyn[];
-  __shared__ __align__(8) uint64_t bars[2 * kAtA + 2 * kAtB + 8 + kAtI];
+  __shared__ __align__(8) uint64_t bars[2 * kAtA + 2 * kAtB + 12 + kAtI];
   __shared__ uint32_t tmem_sh;
   __shared__ int failed_sh;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -532,21 +538,22 @@ __global__ void __launch_bounds__(kAtThreads, 1)
   auto a_free = [&](int s) { return smem_u32(bars + kAtA + s); };
   auto b_full = [&](int s) { return smem_u32(bars + 2 * kAtA + s); };
   auto b_free = [&](int s) { return smem_u32(bars + 2 * kAtA + kAtB + s); };
-  auto acc_full = [&](int m) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + m); };
-  auto acc_empty = [&](int m) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + 2 + m); };
-  auto nrm_full = [&](int b) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + 4 + b); };
-  auto nrm_free = [&](int b) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + 6 + b); };
-  auto inv_free = [&](int s) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + 8 + s); };
+  auto acc_full = [&](int a) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + a); };  // a = 2 h + m
+  auto acc_empty = [&](int a) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + 4 + a); };
+  auto nrm_full = [&](int b) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + 8 + b); };
+  auto nrm_free = [&](int b) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + 10 + b); };
+  auto inv_free = [&](int s) { return smem_u32(bars + 2 * kAtA + 2 * kAtB + 12 + s); };
   const uint32_t sI = sB + kAtB * 2 * kAtHalfB;
   float* inv_sm = reinterpret_cast<float*>(as_dyn + (sI - smem_u32(as_dyn)));  // [kAtI][kAtN]
   float* nrm_sm = inv_sm + kAtI * kAtN;                                        // [2][256] squared norms
+  uint2* part_sm = reinterpret_cast<uint2*>(nrm_sm + 2 * 256);                 // [2][256] half 0's candidates
   volatile int* failed = &failed_sh;
   if (tid == 0) {
-    for (int i = 0; i < 2 * kAtA + 2 * kAtB + 2; ++i) mbar_init(smem_u32(bars + i), 1);
-    for (int m = 0; m < 2; ++m) {
-      mbar_init(acc_empty(m), 4);  // one arrival per epilogue warp
-      mbar_init(nrm_full(m), 2);   // per norm warp
-      mbar_init(nrm_free(m), 8);   // per epilogue warp
+    for (int i = 0; i < 2 * kAtA + 2 * kAtB + 4; ++i) mbar_init(smem_u32(bars + i), 1);
+    for (int a = 0; a < 4; ++a) mbar_init(acc_empty(a), 4);  // one arrival per epilogue warp
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(nrm_full(b), 2);   // per norm warp
+      mbar_init(nrm_free(b), 16);  // per epilogue warp
     }
     for (int s = 0; s < kAtI; ++s) mbar_init(inv_free(s), 8);
     *failed = 0;
@@ -576,7 +583,7 @@ __global__ void __launch_bounds__(kAtThreads, 1)
   };
   auto n_tiles = [](const Item& it) { return it.S - it.t * 256 > 128 ? 2 : 1; };
 
-  if (warp == 8) {
+  if (warp == 16) {
     if (lane == 0) {  // ---- copies
       int na = 0, nb = 0;
       auto load_a = [&](const Item& it, int m) {
@@ -622,33 +629,38 @@ __global__ void __launch_bounds__(kAtThreads, 1)
       for (int j = max(0, nb - kAtB); j < nb; ++j) mbar_wait(b_full(j % kAtB), (uint32_t)(j / kAtB) & 1u);
     }
     __syncwarp();
-  } else if (warp == 9) {
+  } else if (warp == 17) {
     if (lane == 0) {  // ---- products
-      int na = 0, nb = 0, nacc[2] = {0, 0};
+      int na = 0, nb = 0, ni = 0;
+      uint32_t nacc[4] = {0u, 0u, 0u, 0u};
       bool ok = true;
       Item it;
-      for (long long i = blockIdx.x; ok && next_item(i, it); i += gridDim.x) {
+      for (long long i = blockIdx.x; ok && next_item(i, it); i += gridDim.x, ++ni) {
         const int nm = n_tiles(it);
-        for (int c0 = 0; ok && c0 < it.k; c0 += kAtN, ++nb) {
+        for (int c = 0, c0 = 0; ok && c0 < it.k; c0 += kAtN, ++nb, ++c) {
+          const int h = (c + ni) & 1;
           const int sb = nb % kAtB;
           const uint32_t n = (uint32_t)min(kAtN, (it.k - c0 + 15) & ~15);
           const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((128u >> 4) << 24);
           ok = !*failed && mbar_wait(b_full(sb), (uint32_t)(nb / kAtB) & 1u);
-          for (int m = 0; ok && m < nm; ++m) {
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            if (!ok || m >= nm) break;
             const int sa = (na + m) % kAtA;
             ok = (c0 > 0 || mbar_wait(a_full(sa), (uint32_t)((na + m) / kAtA) & 1u)) &&
-                 mbar_wait(acc_empty(m), (uint32_t)(nacc[m] & 1) ^ 1u);
+                 mbar_wait(acc_empty(2 * h + m), ((h ? nacc[2 + m] : nacc[m]) & 1u) ^ 1u);
             if (!ok) break;
             tc_fence_after();
-            const uint32_t a = sA + sa * 2 * kAtHalfA, b = sB + sb * 2 * kAtHalfB;
+            const uint64_t da = sw128_desc(sA + sa * 2 * kAtHalfA), db = sw128_desc(sB + sb * 2 * kAtHalfB);
 #pragma unroll
             for (int kk = 0; kk < 8; ++kk) {
               const uint32_t ka = (uint32_t)(kk >> 2) * kAtHalfA + (uint32_t)(kk & 3) * 32;
               const uint32_t kb = (uint32_t)(kk >> 2) * kAtHalfB + (uint32_t)(kk & 3) * 32;
-              tc_mma(tmem + 256u * (uint32_t)m, sw128_desc(a + ka), sw128_desc(b + kb), idesc, kk > 0 ? 1u : 0u);
+              tc_mma(tmem + 128u * (uint32_t)(2 * h + m), da + (ka >> 4), db + (kb >> 4), idesc, kk > 0 ? 1u : 0u);
             }
-            ++nacc[m];
-            tc_commit(acc_full(m));
+            if (h) ++nacc[2 + m];
+            else ++nacc[m];
+            tc_commit(acc_full(2 * h + m));
             if (c0 + kAtN >= it.k) tc_commit(a_free(sa));
           }
           if (ok) tc_commit(b_free(sb));
@@ -657,15 +669,16 @@ __global__ void __launch_bounds__(kAtThreads, 1)
       }
       if (!ok) *failed = 1;
       // (bounded) every product has completed before the CTA may exit: the last commits have arrived
-      for (int m = 0; m < 2; ++m)
-        if (nacc[m] > 0) mbar_wait(acc_full(m), (uint32_t)(nacc[m] - 1) & 1u);
+#pragma unroll
+      for (int a = 0; a < 4; ++a)
+        if (nacc[a] > 0) mbar_wait(acc_full(a), (nacc[a] - 1u) & 1u);
     }
     __syncwarp();
-  } else if (warp >= 10) {  // ---- squared norms of the item's 256 positions, four per thread
+  } else if (warp >= 18) {  // ---- squared norms of the item's 256 positions, four per thread
     int j = 0;
     Item it;
     for (long long i = blockIdx.x; next_item(i, it); i += gridDim.x, ++j) {
-      const int t = tid - 320, b = j & 1;
+      const int t = tid - 576, b = j & 1;
       const uint4* X = reinterpret_cast<const uint4*>((it.side ? A.V : A.K) + ((size_t)it.u * A.s_max + it.t * 256) * 128);
       float nx2[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -692,8 +705,10 @@ __global__ void __launch_bounds__(kAtThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(nrm_full(b));
     }
-  } else {  // ---- epilogue of tile m
-    const int m = warp >> 2, q = warp & 3;
+  } else {  // ---- epilogue of tile m, half h of its chunks
+    const int m = (warp >> 2) & 1, h = warp >> 3, q = warp & 3;
+    uint32_t tag_mask;
+    asm volatile("mov.b32 %0, 0x7FFFFFE0;" : "=r"(tag_mask));
     int nacc = 0, ni = 0, nc = 0;  // accumulators, items and anchor chunks so far
     bool ok = true;
     Item it;
@@ -706,7 +721,8 @@ __global__ void __launch_bounds__(kAtThreads, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(nrm_free(ni & 1));
       if (m >= n_tiles(it)) {  // no positions of this tile: its chunks pass by
-        for (int c0 = 0; c0 < it.k; c0 += kAtN, ++nc) {
+        for (int c = 0, c0 = 0; c0 < it.k; c0 += kAtN, ++nc, ++c) {
+          if (((c + ni) & 1) != h) continue;
           if (ok && nc >= kAtI) ok = mbar_wait_w(inv_free(nc % kAtI), (uint32_t)(nc / kAtI - 1) & 1u);
           if (lane == 0) mbar_arrive(inv_free(nc % kAtI));
         }
@@ -727,10 +743,10 @@ __global__ void __launch_bounds__(kAtThreads, 1)
         for (int e = 0; e < 8; ++e) {
           const float4 f = *reinterpret_cast<const float4*>(iv + 4 * e);
           const float2 x = __fmul2_rn(s[2 * e], make_float2(f.x, f.y)), y = __fmul2_rn(s[2 * e + 1], make_float2(f.z, f.w));
-          v[4 * e] = __uint_as_float((__float_as_uint(x.x) & 0x7FFFFFE0u) | (uint32_t)(4 * e));
-          v[4 * e + 1] = __uint_as_float((__float_as_uint(x.y) & 0x7FFFFFE0u) | (uint32_t)(4 * e + 1));
-          v[4 * e + 2] = __uint_as_float((__float_as_uint(y.x) & 0x7FFFFFE0u) | (uint32_t)(4 * e + 2));
-          v[4 * e + 3] = __uint_as_float((__float_as_uint(y.y) & 0x7FFFFFE0u) | (uint32_t)(4 * e + 3));
+          v[4 * e] = tagged(x.x, tag_mask, (uint32_t)(4 * e));
+          v[4 * e + 1] = tagged(x.y, tag_mask, (uint32_t)(4 * e + 1));
+          v[4 * e + 2] = tagged(y.x, tag_mask, (uint32_t)(4 * e + 2));
+          v[4 * e + 3] = tagged(y.y, tag_mask, (uint32_t)(4 * e + 3));
         }
         float mx[11];
 #pragma unroll
@@ -751,37 +767,46 @@ __global__ void __launch_bounds__(kAtThreads, 1)
         i1 = alone ? idx : i1;
         m1 = top;
       };
-      for (int c0 = 0; c0 < it.k; c0 += kAtN, ++nc) {
+      for (int c = 0, c0 = 0; c0 < it.k; c0 += kAtN, ++nc, ++c) {
+        if (((c + ni) & 1) != h) continue;
         __syncwarp();
-        ok = ok && __shfl_sync(0xffffffffu, *failed, 0) == 0 && mbar_wait_w(acc_full(m), (uint32_t)nacc & 1u);
-        if (!ok) break;  // (the same for the whole warp)
+        ok = ok && __shfl_sync(0xffffffffu, *failed, 0) == 0 && mbar_wait_w(acc_full(2 * h + m), (uint32_t)nacc & 1u);
+        if (!ok) continue;  // (the same for the whole warp)
         ++nacc;
         tc_fence_after();
         const int n = min(kAtN, it.k - c0);
-        const uint32_t tcol = tmem + ((uint32_t)(32 * q) << 16) + 256u * (uint32_t)m;
+        const uint32_t tcol = tmem + ((uint32_t)(32 * q) << 16) + 128u * (uint32_t)(2 * h + m);
         const float* iv = inv_sm + (nc % kAtI) * kAtN;
-        auto done = [&]() {  // the tile's last read of the accumulator has come back
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(acc_empty(m));
-        };
-        float2 sa[16], sb[16];
-        tc_ld32_start(tcol, sa);
-        for (int sc = 0; sc < n; sc += 64) {
-          tc_ld32_wait(sa);
-          if (sc + 32 < n) tc_ld32_start(tcol + (uint32_t)(sc + 32), sb);
-          else done();
-          step(sa, iv + sc, (uint32_t)(c0 + sc));
-          if (sc + 32 >= n) break;
-          tc_ld32_wait(sb);
-          if (sc + 64 < n) tc_ld32_start(tcol + (uint32_t)(sc + 64), sa);
-          else done();
-          step(sb, iv + sc + 32, (uint32_t)(c0 + sc + 32));
+        for (int sc = 0; sc < n; sc += 32) {
+          float2 s[16];
+          tc_ld32(tcol + (uint32_t)sc, s);
+          if (sc + 32 >= n) {  // the tile's last read of the accumulator has come back
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty(2 * h + m));
+          }
+          step(s, iv + sc, (uint32_t)(c0 + sc));
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(inv_free(nc % kAtI));
       }
-      if (p < it.S) (it.side ? w.st[1] : w.st[0])[p] = ok && usable && m1 > marg && !more ? i1 | (i2 << 16) : 0xFFFFFFFFu;
+      // the two halves' candidates together (a barrier of the two warps that share these positions; half 0 writes
+      // the other buffer for the next item)
+      uint2* part = part_sm + 256 * (ni & 1) + 128 * m + 32 * q + lane;
+      more = more || !ok;
+      if (h == 0) *part = make_uint2(__float_as_uint(more ? -1.f : m1), i1 | (i2 << 16));
+      asm volatile("bar.sync %0, 64;" ::"r"(1 + 4 * m + q) : "memory");
+      if (h == 1 && p < it.S) {
+        const uint2 o = *part;
+        const float om = __uint_as_float(o.x);
+        uint32_t word = 0xFFFFFFFFu;
+        if (usable && !more && om >= 0.f) {
+          if (m1 > om + marg) word = i1 | (i2 << 16);
+          else if (om > m1 + marg) word = o.y;
+          else if (i2 == 0xFFFFu && (o.y >> 16) == 0xFFFFu && fmaxf(m1, om) > marg) word = min(i1, o.y & 0xFFFFu) | (max(i1, o.y & 0xFFFFu) << 16);
+        }
+        (it.side ? w.st[1] : w.st[0])[p] = word;
+      }
     }
     if (!ok) *failed = 1;
   }

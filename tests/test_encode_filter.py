@@ -48,6 +48,21 @@ def test_equal_rows(dev, kinds, k1):  # noqa: F811
     _encode_both(dev, p, [S], K[:, :, pick], V[:, :, pick])
 
 
+@pytest.mark.parametrize("k", [1, 31, 33, 127, 129, 256, 300, 640])
+def test_near_ties_across_anchor_chunks(dev, k):  # noqa: F811
+    """Every row again half the positions later, one bit apart in one dimension: the nearest anchors' scores differ by
+    less than the filter tells, mostly in different anchor chunks (of 128, in turn to two accumulators)."""
+    S = 1300
+    p = akv.Params(batch=1, n_kv_heads=1, n_q_heads=1, anchor_frac=(k - 0.5) / S, window=0, res_frac_k=0.1,
+                   res_frac_v=0.1, seed=14)
+    assert akv.akv_unit_shapes(p, [S])[0][1] == k
+    K, V = gen.clustered_batch(1, 1, [S], seed=15)
+    for X in (K, V):
+        X[:, :, S // 2:] = X[:, :, :S // 2]
+        X[:, :, S // 2:, 7] ^= 1
+    _encode_both(dev, p, [S], K, V)
+
+
 @pytest.mark.parametrize("kinds,e", [(30, 0), (0, 40), (300, 0)])
 def test_selection_left_to_fp64(dev, kinds, e):  # noqa: F811
     """The full selection where the paired sums cannot rank: positions drawn from a few distinct rows (equal scores
