@@ -1085,7 +1085,12 @@ __device__ void paired_dot(const uint4* x, const uint4* row, int a, float& s, fl
 // anchor of a group of 32, or any at all, a block each.  Scores are told apart in fp32, then in twice its
 // precision (as squares: dot^2 |other|^2), duplicates by their bytes; fp64 chains run only for what is
 // left, since one of 128 steps takes about 10 us here.
-constexpr int kUndFirst = 8, kUndBlocks = 72, kUndThreads = 128;  // blocks of the first list; blocks per unit and side
+constexpr int kUndThreads = 128;
+// Blocks per unit and side, a ninth of them for the first list: 72 in a large batch (24 units already start 3456),
+// up to 576 for fewer than 8 units, whose lists are as long as their requests.  2 units of 131072 positions: 76 us with
+// the 288 of this rule, 122 us with 72.
+__host__ __device__ constexpr int und_first(int blocks) { return blocks / 9; }
+inline int und_blocks(int units) { return 72 * std::min(8, std::max(1, 8 / std::max(1, units))); }
 __global__ void __launch_bounds__(kUndThreads) enc_undecided(const EncArgs A) {
   __shared__ __align__(16) float xs[128];
   __shared__ float red[kUndThreads / 32];
@@ -1098,8 +1103,9 @@ __global__ void __launch_bounds__(kUndThreads) enc_undecided(const EncArgs A) {
   const EncUnitWs w = unit_ws(A, u, d);
   const int n_todo = (int)w.ctrl[8 + side], n_full = (int)w.ctrl[10 + side];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool second = blockIdx.x >= kUndFirst;
-  if (second ? n_full <= (int)blockIdx.x - kUndFirst : n_todo <= (int)blockIdx.x * kUndThreads) return;
+  const int n_first = und_first((int)gridDim.x), b = (int)blockIdx.x;
+  const bool second = b >= n_first;
+  if (second ? n_full <= b - n_first : n_todo <= b * kUndThreads) return;
   const uint4* X = reinterpret_cast<const uint4*>((side ? A.V : A.K) + (size_t)u * A.s_max * 128);
   const uint4* AR = reinterpret_cast<const uint4*>(A.arena_c + (side ? d->off_anchor_v : d->off_anchor_k));
   uint32_t* stream = w.st[side];
@@ -1154,7 +1160,7 @@ __global__ void __launch_bounds__(kUndThreads) enc_undecided(const EncArgs A) {
     return same;
   };
   if (!second) {
-    for (int t = blockIdx.x * kUndThreads + tid; t < n_todo; t += kUndFirst * kUndThreads) {
+    for (int t = b * kUndThreads + tid; t < n_todo; t += n_first * kUndThreads) {
       const int p = list[t];
       const uint32_t word = stream[p];
       const int a1 = (int)(word & 0xFFFFu), a2 = (int)(word >> 16);
@@ -1183,7 +1189,7 @@ __global__ void __launch_bounds__(kUndThreads) enc_undecided(const EncArgs A) {
     }
     return;
   }
-  for (int t = (int)blockIdx.x - kUndFirst; t < n_full; t += kUndBlocks - kUndFirst) {
+  for (int t = b - n_first; t < n_full; t += (int)gridDim.x - n_first) {
     const int p = list[S - 1 - t];
     const uint32_t word = stream[p];
     const int a_lo = word == 0xFFFFFFFFu ? 0 : (int)(word & 0xFFE0u), a_hi = word == 0xFFFFFFFFu ? k : min(k, a_lo + 32);
@@ -2888,7 +2894,7 @@ int launch_encode(const Layout& L, const EncodeWs& W, const akv_params& p, const
   const long long items = 2ll * units * max_t;
   enc_assign_tc<<<(unsigned)std::min<long long>(items, sms), kAtThreads, kAtSmem, st>>>(A, tmK, tmV, tmA, items, max_t);
   enc_finish<<<dim3((maxS + kFinPos - 1) / kFinPos, units, 2), 256, 0, st>>>(A);
-  enc_undecided<<<dim3(kUndBlocks, units, 2), kUndThreads, 0, st>>>(A);
+  enc_undecided<<<dim3((unsigned)und_blocks((int)units), units, 2), kUndThreads, 0, st>>>(A);
   if (full) {  // Eq. 6 utilities, then each side's pooled top-N per request
     const unsigned m = (unsigned)m_obs;
     if ((e = cudaFuncSetAttribute(enc_util_f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(UtilSmem))) !=
