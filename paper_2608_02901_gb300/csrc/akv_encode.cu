@@ -1355,21 +1355,35 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) 
   for (int i = tid; i < 3 * 2048; i += kSelThreads) (&hist[0][0])[i] = 0u;
   if (tid == 0) cnt_hi = cnt_band = n_app = n_list = 0u;
   __syncthreads();
+  // f(position, its key or 0 past the share), by whole warps; eight keys are read at a time (one at a time, the five
+  // passes' reads took most of the kernel: 70 us, not 47, for 2 units of 131072 positions, 36, not 31, for 8 of 32768)
+  auto each_key = [&](auto&& f) {
+    for (int p0 = lo; p0 < hi; p0 += 8 * kSelThreads) {
+      uint32_t v[8];
+#pragma unroll
+      for (int x = 0; x < 8; ++x) {
+        const int p = p0 + x * kSelThreads + tid;
+        v[x] = p < hi ? key[p] : 0u;
+      }
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+        if (p0 + x * kSelThreads < hi) f(p0 + x * kSelThreads + tid, v[x]);
+    }
+  };
   uint32_t prefix = 0, want = (uint32_t)N;
 #pragma unroll 1
   for (int dg = 0; dg < 3; ++dg) {
     const int sh = dg == 0 ? 21 : (dg == 1 ? 10 : 0), bits = dg == 2 ? 10 : 11;
-    for (int p = lo + tid; p < hi; p += kSelThreads) {
-      const uint32_t v = key[p];
-      const bool in = dg == 0 || (v >> (sh + bits)) == prefix;
+    each_key([&](int p, uint32_t v) {
+      const bool in = p < hi && (dg == 0 || (v >> (sh + bits)) == prefix);
       const uint32_t digit = (v >> sh) & ((1u << bits) - 1u);
       if (dg == 0) {  // a few digits hold all the energies: equal ones of a warp are counted at once
-        const unsigned peers = __match_any_sync(__activemask(), digit);
-        if ((peers & ((1u << lane) - 1u)) == 0u) atomicAdd(&hist[dg][digit], (uint32_t)__popc(peers));
+        const unsigned peers = __match_any_sync(0xffffffffu, in ? digit : 0xFFFFFFFFu);
+        if (in && (peers & ((1u << lane) - 1u)) == 0u) atomicAdd(&hist[dg][digit], (uint32_t)__popc(peers));
       } else if (in) {
         atomicAdd(&hist[dg][digit], 1u);
       }
-    }
+    });
     cl.sync();
     uint32_t inside;
     prefix = (prefix << bits) | cluster_digit<true>(cl, hist[dg], wsum, found, want, &inside);
@@ -1378,16 +1392,14 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) 
   const float eT = __uint_as_float(T - 1u);
   const uint32_t k_lo = __float_as_uint(__fmul_rn(eT, 1.0f - 0x1p-16f)) + 1u;
   const uint32_t k_hi = __float_as_uint(__fmul_rn(eT, 1.0f + 0x1p-16f)) + 1u;
-  for (int p0 = lo; p0 < hi; p0 += kSelThreads) {
-    const int p = p0 + tid;
-    const uint32_t v = p < hi ? key[p] : 0u;
+  each_key([&](int p, uint32_t v) {
     const unsigned above = __ballot_sync(0xffffffffu, v > k_hi);
     if (lane == 0 && above) atomicAdd(&cnt_hi, (uint32_t)__popc(above));
     if (v >= k_lo && v <= k_hi) {
       const uint32_t i = atomicAdd(&cnt_band, 1u);
       if (i < kSelBand) band[i] = p;
     }
-  }
+  });
   cl.sync();
   uint32_t n_hi = 0, n_band = 0, hi_before = 0, band_before = 0;
   for (int r = 0; r < kSelCtas; ++r) {
@@ -1409,16 +1421,15 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) 
   }
   const uint32_t k_in = all ? k_lo : k_hi + 1u;
   const uint32_t at = all ? hi_before + band_before : hi_before;
-  for (int p0 = lo; p0 < hi; p0 += kSelThreads) {
-    const int p = p0 + tid;
-    const bool sel = p < hi && key[p] >= k_in;
+  each_key([&](int p, uint32_t v) {
+    const bool sel = p < hi && v >= k_in;
     const unsigned bal = __ballot_sync(0xffffffffu, sel);
     uint32_t i = 0;
     if (lane == 0 && bal) i = atomicAdd(&n_app, (uint32_t)__popc(bal));
     i = __shfl_sync(0xffffffffu, i, 0);
     if (p < hi) flag[p] = sel ? 1 : 0;
     if (sel) rp[at + i + __popc(bal & ((1u << lane) - 1u))] = p;
-  }
+  });
   if (!all && tied) {  // in position order
     __syncthreads();
     if (tid == 0) {
@@ -1581,15 +1592,20 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) 
   const int lo = row < n_rows ? (int)min((long long)S, (long long)row * per) : S;
   const int hi = (int)min((long long)S, (long long)lo + per);
   uint32_t* mine = mat + (size_t)row * k;
+  auto slot_at = [&](int p) { return p < hi ? (st[p] & 0xFFFFu) : 0xFFFFFFFFu; };  // of position p
   if (row < n_rows) {
     for (int a = lane; a < k; a += 32) mine[a] = 0u;
     __threadfence();
     __syncwarp();
-    for (int p0 = lo; p0 < hi; p0 += 32) {
-      const int p = p0 + lane;
-      const uint32_t a = p < hi ? (st[p] & 0xFFFFu) : 0xFFFFFFFFu;
-      const unsigned peers = __match_any_sync(0xffffffffu, a);
-      if (p < hi && (peers & ((1u << lane) - 1u)) == 0u) atomicAdd(&mine[a], (uint32_t)__popc(peers));
+    for (int p0 = lo; p0 < hi; p0 += 128) {
+      uint32_t a[4];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) a[x] = slot_at(p0 + 32 * x + lane);
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const unsigned peers = __match_any_sync(0xffffffffu, a[x]);
+        if (a[x] != 0xFFFFFFFFu && (peers & ((1u << lane) - 1u)) == 0u) atomicAdd(&mine[a[x]], (uint32_t)__popc(peers));
+      }
     }
   }
   cl.sync();
@@ -1646,19 +1662,29 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) 
     }
   }
   __syncthreads();
-  for (int p0 = lo; p0 < hi; p0 += 32) {
-    const int p = p0 + lane;
-    const uint32_t a = p < hi ? (st[p] & 0xFFFFu) : 0xFFFFFFFFu;
-    const unsigned peers = __match_any_sync(0xffffffffu, a);
-    const int before = __popc(peers & ((1u << lane) - 1u));
-    uint32_t at = 0;
-    if (p < hi && before == 0) at = atomicAdd(&mine[a], (uint32_t)__popc(peers)) + __ldcg(w.cursor + a) + part[1][a / kper];
-    at = __shfl_sync(0xffffffffu, at, __ffs(peers) - 1) + (uint32_t)before;
-    if (p < hi) {
-      w.perm[at] = p;
-      w.at[p] = (int32_t)at;
+  // 128 positions at a time, so that four updates are under way together: a row's updates of successive 32 positions
+  // are ordered by the warp barrier between them, not by the values they return (2 units of 131072: 72 -> 65 us)
+  for (int p0 = lo; p0 < hi; p0 += 128) {
+    uint32_t a[4], at[4] = {0u, 0u, 0u, 0u};
+    unsigned peers[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) a[x] = slot_at(p0 + 32 * x + lane);
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      peers[x] = __match_any_sync(0xffffffffu, a[x]);
+      if (a[x] != 0xFFFFFFFFu && (peers[x] & ((1u << lane) - 1u)) == 0u) at[x] = atomicAdd(&mine[a[x]], (uint32_t)__popc(peers[x]));
+      __syncwarp();
     }
-    __syncwarp();  // (orders the rows' updates of successive steps)
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const int p = p0 + 32 * x + lane;
+      at[x] = __shfl_sync(0xffffffffu, at[x], __ffs(peers[x]) - 1) + (uint32_t)__popc(peers[x] & ((1u << lane) - 1u));
+      if (p < hi) {
+        at[x] += __ldcg(w.cursor + a[x]) + part[1][a[x] / kper];
+        w.perm[at[x]] = p;
+        w.at[p] = (int32_t)at[x];
+      }
+    }
   }
   cl.sync();  // no CTA leaves while another may still read its total
 }
