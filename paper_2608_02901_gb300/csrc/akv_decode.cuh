@@ -684,6 +684,9 @@ __global__ void __launch_bounds__(128) akv_suffix_kernel(const ScoreParams P) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (a decode that waits for it where it needs it)
   suffix_chunk<GS, ROPE>(P, blockIdx.x / P.n_sch, blockIdx.x % P.n_sch,
                          reinterpret_cast<__nv_bfloat16 (*)[128]>(score_dyn));
+  // nothing above reads what the launch before this one (the scores) writes, so the two run beside each other; the
+  // decode waits for this launch alone, which therefore ends after that one
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // The arrival counters of unit u's query heads, behind its query header.
@@ -789,6 +792,7 @@ __global__ void __launch_bounds__(kScThreads) akv_scores_tc_kernel(const __grid_
   auto acc_full = [&](int b) { return smem_u32(bars + 2 * kScStages + b); };
   auto acc_empty = [&](int b) { return smem_u32(bars + 2 * kScStages + 2 + b); };
   volatile int* failed = &failed_sh;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int n_tiles = P.units * P.n_t;
   const int n_my = n_tiles > (int)blockIdx.x ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
   for (int i = tid; i < n_my && i < kScMaxTiles; i += kScThreads) {  // all descriptors in one round trip
@@ -2546,7 +2550,6 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   get_decode_events(&ev_scores_p, &ev_decode_p);
   const cudaEvent_t ev_scores = (cudaEvent_t)ev_scores_p, ev_decode = (cudaEvent_t)ev_decode_p;
   cudaError_t e;
-  bool beside = false;  // the decode may start beside the launch before it
   if (rope) {  // the logits of every stored token (no anchor scores)
     RopeParams R;
     R.arena = P.arena;
@@ -2573,13 +2576,11 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
     e = cudaLaunchKernelEx(&cfg, rope_kernel<GS>(codec), R);
     cfg.blockDim = dim3(128, 1, 1);
     for (int j = 0; j < 64; ++j) S.turn[j] = R.turn[j];
-    beside = true;
   } else if ((long long)units * P.n_ch <= kSmallChunks) {
     S.units = units;
     S.arena_rows = (long long)(arena_bytes / 256);
     cfg.gridDim = dim3((unsigned)(units + units * P.n_ch), 1, 1);
     e = cudaLaunchKernelEx(&cfg, akv_scores_small_kernel<GS>, S);
-    beside = true;
   } else {
     // anchor rows of every unit through one map over the caller's arena as 256-byte rows (each
     // unit's anchor-key section starts its 256-byte-aligned segment; a full-selection arena places
@@ -2604,6 +2605,12 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
     cfg.blockDim = dim3(128, 1, 1);
     cfg.dynamicSmemBytes = 0;
   }
+  // the launches after the first may start beside the one before them and wait for it where they need it
+  cudaLaunchAttribute pdl;
+  pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  pdl.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &pdl;
+  cfg.numAttrs = 1;
   if (e == cudaSuccess && n_sch) {  // the dense suffix's chunks (with RoPE: keys turned to positions S + t)
     cfg.gridDim = dim3((unsigned)(units * n_sch), 1, 1);
     cfg.dynamicSmemBytes = (size_t)SCH * 256;  // a chunk's value rows
@@ -2615,13 +2622,6 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   cfg.gridDim = dim3((unsigned)pl.grid, 1, 1);
   cfg.blockDim = dim3(NT, 1, 1);
   cfg.dynamicSmemBytes = pl.smem;
-  cudaLaunchAttribute pdl;
-  pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  pdl.val.programmaticStreamSerializationAllowed = 1;
-  if (beside) {
-    cfg.attrs = &pdl;
-    cfg.numAttrs = 1;
-  }
   e = cudaLaunchKernelEx(&cfg, decode_kernel<GS>(codec, rope, P), P);
   if (e != cudaSuccess) {
     cudaFuncAttributes fa{};
