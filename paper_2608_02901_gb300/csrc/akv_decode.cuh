@@ -2490,6 +2490,7 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
     // chunk maxima per unit: of 64 anchors, or with RoPE of 64 stored tokens
     pl.P.n_ch = rope ? (L.max_len + 63) / 64 : (L.max_k + CHA - 1) / CHA;
     std::lock_guard<std::mutex> lk(mu);
+    if (cache.size() >= 64) cache.clear();  // (bounded: a server's calls come in many combinations of lengths)
     cache[key] = pl;
   }
   const DecodeWs W = decode_ws_layout(L, sfx.cap);

@@ -48,3 +48,64 @@ def test_rope_chunks(dev, S, G, fr, rotate):  # noqa: F811
     p = akv.Params(batch=2, n_kv_heads=2, n_q_heads=2 * G, res_frac_k=fr, res_frac_v=0.1, window=4, seed=6, rotate=rotate,
                    rope=True, rope_theta=10000.0)
     _run_seeded(dev, p, [S, 1300], sm_scale=0.1)
+
+
+@pytest.mark.parametrize("before", ["nothing", "copy", "kernel", "join"])
+@pytest.mark.parametrize("rope,lens", [(False, [3000]), (False, [9000] * 20), (True, [2500, 700])])
+def test_queries_written_just_before(dev, before, rope, lens):  # noqa: F811
+    """Calls in a row on one workspace, each behind what writes its queries (a copy, a kernel, another stream's
+    kernel): every launch may be set up while the one before it runs, and must see all of it.  In the stream and as
+    a replayed graph, where each kind of predecessor is another kind of edge."""
+    import gen
+    import torch
+    from helpers import seeded_units, to_dev_u16
+    p = akv.Params(batch=len(lens), n_kv_heads=4, n_q_heads=16, seed=9, anchor_frac=0.04, rope=rope, rope_theta=10000.0)
+    units = seeded_units(p, lens, seed=3)
+    arena = torch.from_numpy(akv.akv_cache_pack_host(p, lens, [akv.unit_host_from_logical(u) for u in units])).to(dev)
+    shape = (p.batch, p.n_q_heads, 128)
+    qs = [to_dev_u16(gen.queries(p.batch * p.n_q_heads, seed=s).reshape(shape), torch, dev) for s in (1, 2)]
+    ws = torch.empty(akv.akv_decode_workspace_size(p, lens), dtype=torch.uint8, device=dev)
+    q = torch.empty_like(qs[0])
+    outs = [torch.empty(shape, dtype=torch.float32, device=dev) for _ in range(6)]
+    out = torch.empty(shape, dtype=torch.bfloat16, device=dev)
+    want = []
+    for x in qs:
+        o = torch.empty_like(outs[0])
+        akv.akv_decode_attn(p, lens, arena, x, out, o, sm_scale=1.0, ws=ws)
+        torch.cuda.synchronize()
+        want.append(o)
+    assert (want[0] - want[1]).abs().max() > 0.1
+    main, other = torch.cuda.Stream(device=dev), torch.cuda.Stream(device=dev)
+
+    def calls():
+        for i, o in enumerate(outs):
+            x = qs[i & 1]
+            if before == "copy":
+                q.copy_(x)
+            elif before == "kernel":
+                torch.mul(x, 1.0, out=q)
+            elif before == "join":
+                other.wait_stream(main)
+                with torch.cuda.stream(other):
+                    torch.mul(x, 1.0, out=q)
+                main.wait_stream(other)
+            akv.akv_decode_attn(p, lens, arena, x if before == "nothing" else q, out, o, sm_scale=1.0, ws=ws, stream=main)
+
+    def check():
+        torch.cuda.synchronize()
+        for i, o in enumerate(outs):
+            assert torch.allclose(o, want[i & 1], rtol=1e-4, atol=1e-4)
+            o.zero_()
+        torch.cuda.synchronize()
+
+    with torch.cuda.stream(main):
+        for _ in range(5):
+            calls()
+    check()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=main):
+        calls()
+    for _ in range(3):
+        with torch.cuda.stream(main):
+            g.replay()
+        check()
