@@ -959,11 +959,21 @@ __global__ void __launch_bounds__(256) enc_finish(const EncArgs A) {
       ab += __shfl_xor_sync(0xffffffffu, ab, o);
     }
   };
+  // a position's slot and candidate word are read one step ahead, so that its rows don't wait for them (8 units of
+  // 32768 positions: 61 -> 55 us)
+  int sl_n = 0;
+  uint32_t word_n = 0u;
+  auto read_word = [&](int q) {
+    const bool in = q < kFinPos && p0 + q < S;
+    sl_n = in ? w.slot_of[p0 + q] : 0;
+    word_n = in ? stream[p0 + q] : 0u;
+  };
+  read_word(tid >> 3);
   for (int q = tid >> 3; q < kFinPos; q += 32) {
     const int p = p0 + q;
     const bool in = p < S;
-    const int sl = in ? w.slot_of[p] : 0;
-    const uint32_t word = in ? stream[p] : 0u;
+    const int sl = sl_n;
+    const uint32_t word = word_n;
     int a = (int)(word & 0xFFFFu);
     const int a2 = (int)(word >> 16);
     const bool some = in && sl < 0, lone = some && a2 != a;  // lone: one candidate, or two
@@ -974,6 +984,7 @@ __global__ void __launch_bounds__(256) enc_finish(const EncArgs A) {
       load_anchor(a, aw);
     }
     float iv = lone ? inv[a] : 0.f;
+    read_word(q + 32);
     float dd, ab;
     dot(xw, aw, dd, ab);
     const bool two = lone && a2 != 0xFFFF;
