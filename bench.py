@@ -527,7 +527,7 @@ def run_akv(args, rank, world, local):
                 "frac_of_8tbs": round(achieved / 8000.0, 4),
                 "step": {"bytes": round(step_bytes), "achieved": round(step_bytes / (sec / args.steps) / 1e9, 2),
                          "frac": round(step_bytes / (sec / args.steps) / 1e9 / peak, 4)},
-                "scores_kernel": {"kernel": ("akv_rope_logits_kernel" if args.rope else "akv_scores_tc_kernel")
+                "scores_kernel": {"kernel": ("akv_rope_logits_kernel" if args.rope else "akv_scores_kernel")
                                   + (" + akv_suffix_kernel" if args.suffix > 0 else ""),
                                   "launch_us": round(us_scores, 3),
                                   "bytes_per_launch": round(scores_bytes),

@@ -154,11 +154,13 @@ akv_status make_layout(const akv_params* p, const int32_t* ctx_lens, Layout* out
 }
 
 void encode_ws_layout(const Layout& L, EncodeWs* ws, int32_t m_obs) {
-  // Per unit: two u64 key arrays [S] (anchor hashes, then residual energies
-  // per side), slot map i32 [S], residual positions i32 [N_K + N_V],
-  // anchor norms (squared, and square roots) f64 [k] per side, 256 B control,
-  // stream words u32 [S] per side, flags u8 [S], stored order and inverse
-  // i32 [S], run starts u32 [k + 1], record counts u32 [2 n_tiles].
+  // Per unit: two u64 key arrays [S] (selector scores, then residual energies
+  // per side with the lists of undecided positions behind them, then the
+  // counting sort's rows), slot map i32 [S] (then a side's flags), residual
+  // positions i32 [N_K + N_V], squared anchor norms f64 [k] per side (and as
+  // much again that nothing uses), 256 B control, stream words u32 [S] per
+  // side, flags u8 [S], stored order and inverse i32 [S] (before that the
+  // anchors' inverse norms), run starts u32 [k + 1], record counts u32 [2 n_tiles].
   // A table of per-unit byte offsets (u64 each) leads the workspace.
   ws->unit_off.resize(L.shape.size());
   uint64_t off = align_up((uint64_t)L.shape.size() * 8, 256);

@@ -1,16 +1,17 @@
 // Decode attention read directly from the AnchorKV compressed cache (Eq. 3 folded into
-// Eq. 4: no key or value row is ever rebuilt in memory).  Two launches per call, in stream
-// order (three with a dense suffix, whose chunks take a launch of their own between them):
+// Eq. 4: no key or value row is ever rebuilt in memory).  Two launches per call (three with a dense suffix, whose
+// chunks take a launch of their own between them).  Each launch after the first is a programmatic dependent of the one
+// before it: it may start once that one's CTAs have, and waits where it needs its results.  So the decode is set up and
+// its first tiles are on their way beside the scores, and the suffix's chunks run beside them (16 ragged requests, 8B
+// shape: 87.5 -> 85.6 us; 8 x 131072, 70B shape: 170.4 -> 169.7).  The first launch is an ordinary one (as a dependent
+// of the call before, its wait cost more than the gap: 18.4 -> 20.5 us a call at 8 units of 32768).
 //
 // 1. The anchor scores S_A[a][g] = q_g . k_a of every anchor of every unit, once per anchor (Eq. 2-3),
 //    in log2 units with sm_scale folded in, into the workspace, with the largest score per query head of
 //    each chunk of 64 anchors; also each unit's query header (the rotated query q' = H(s o q)/128 of
 //    Appendix A.1 Eq. 12, its sums per head, and q' as tensor-core fragments for the key residuals) and
-//    zeroed arrival counters behind it.  akv_scores_tc_kernel: tiles of 128 anchors brought by tensor
-//    copies (TMA), products by tcgen05.mma into tensor memory, one persistent warp-specialised CTA per SM.
-//    akv_scores_small_kernel, for calls of at most kSmallChunks chunks: one short-lived CTA per chunk, beside
-//    which the decode sets itself up (programmatic dependent launch).  (With RoPE at decode
-//    akv_rope_logits_kernel takes their place.)
+//    zeroed arrival counters behind it.  akv_scores_kernel: a short-lived CTA per chunk, tensor-core products.  (With
+//    RoPE at decode akv_rope_logits_kernel takes its place.)
 //
 // 2. akv_decode_kernel.  Persistent: one CTA per SM.  The tile blocks of all units, in unit
 //    order, are split into equal contiguous ranges, one per CTA (stream-K): a unit's tiles may
@@ -45,7 +46,7 @@
 // per tile), each about half used; the rest is the latency of the phases' dependent chains.  Two groups
 // of four warps that took a tile through all phases (255 registers, two warps per sub-partition) spent
 // 2.8 us per tile pair-wise; token and product warps side by side spend 2.7 us and leave each other's
-// latencies covered where tiles are few (8B shape, 32K: 24.6 -> 18.9 us per call with the small score launch).
+// latencies covered where tiles are few (8B shape, 32K: 24.6 -> 18.4 us per call with the small score launch).
 //
 // The exponent reference m is the largest anchor score of each query row.  Anchors are
 // tokens of the unit, so it is a lower bound of the largest logit (sums cannot overflow unless
@@ -86,20 +87,6 @@ constexpr int T = kTile;            // tokens per tile block
 constexpr int LCH = T / (NTW * 32); // consecutive stored tokens per lane
 static_assert(LCH == 4, "a lane's tokens are half a byte of a bitmap word and 16 bytes of a stream");
 constexpr int NSG = 6;              // tiles in flight at most (their descriptors)
-// Score launch on tensor cores: a tile of 128 anchors (TMEM lanes) x 16 query rows (columns),
-// anchor rows and query rows brought by tensor copies into two 128-byte halves each
-constexpr int kScTile = 128;
-constexpr uint32_t kScHalfA = kScTile * 128;             // 128 rows x 64 bf16
-constexpr uint32_t kScHalfB = 16 * 128;                  // 16 rows x 64 bf16
-constexpr uint32_t kScStage = 2 * kScHalfA + 2 * kScHalfB;  // 36 KB, a multiple of 1024
-constexpr int kScStages = 6;                             // tiles in flight (one CTA per SM)
-constexpr int kScThreads = 192;  // warps 0-3 epilogue (TMEM lanes 32 w ..), 4 copies and products, 5 query headers
-constexpr int kScMaxTiles = 512;  // tiles of one CTA (its table in shared memory); the grid grows past this
-constexpr uint32_t kScDynSmem = kScStages * kScStage + 1024;  // + alignment of the first stage
-constexpr uint32_t kScTmemCols = 32;                     // two accumulators of 16 fp32 columns
-// Instruction descriptor of kind::f16: fp32 accumulator (bits 4-5 = 1), bf16 A and B (7-9 = 1,
-// 10-12 = 1), both K-major (15, 16 = 0), N / 8 (17-22), M / 16 (24-28).
-constexpr uint32_t kScIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((16u >> 3) << 17) | ((uint32_t)(kScTile >> 4) << 24);
 constexpr int kEnds = 2 * NTW;       // a tile's runs that may go on in a neighbour warp: each warp's first and last
 constexpr int kOvl = 32;            // a tile's entries per overflow list (value records, anchor-value runs)
 constexpr int kOvlBytes = 16 + 2 * kOvl * 9 * 4;  // a tile's two lists: counts, then entries
@@ -127,8 +114,8 @@ struct ScoreParams {
   const int32_t* suf_len;
   float* suf_part;
   int suf_cap, n_sch;
-  int units, n_t;  // units; tiles of kScTile anchors per unit (the largest unit's)
-  long long arena_rows;  // 256-byte rows of the arena the anchor map covers
+  int units;
+  long long arena_rows;  // 256-byte rows of the arena
   // RoPE at decode (the suffix launch): suffix token t of a unit sits at position S + t
   unsigned long long turn[64];  // theta_j / (2 pi) as a 64-bit binary fraction of a turn
 };
@@ -754,216 +741,17 @@ __device__ __noinline__ void unit_query_header_warp(const ScoreParams& P, int u,
   __syncwarp();  // the next unit's rows may overwrite qs
 }
 
-// Anchor scores on tensor cores (Eq. 2-3: S_A = q . k_a once per anchor).  One persistent CTA per
-// SM takes tiles T = blockIdx.x, + gridDim.x, ... of units x n_t; tile (u, t) is anchors
-// 128 t .. 128 t + 127 of unit u (tile 0 of every unit is taken even when empty).  Warps have
-// roles, coupled only by mbarriers:
-//  * warp 4, lane 0, copies and products: it keeps kScStages tiles in flight (two tensor copies
-//    bring the anchor rows' 128-byte halves, stored with the 16-byte chunks of row a at chunk
-//    j ^ (a & 7), which is the 128-byte swizzled operand layout as it is; two bring the query
-//    rows, swizzled by the copy, with the next 16 - G rows of q or zeros in columns that are not
-//    read), and as each tile lands and one of two TMEM accumulators is free it issues the 8 K steps
-//    of D[128 anchors][16 columns] and commits them to that accumulator's "full" barrier and to the
-//    stage's "free" barrier; the stage of the previous tile is refilled once its products are done;
-//  * warps 0-3, the epilogue: warp w reads TMEM lanes 32 w .. 32 w + 31 (one anchor per thread),
-//    frees the accumulator, writes S_A in log2 units and, after a named barrier of the four warps,
-//    the maxima of the tile's two 64-anchor chunks;
-//  * warp 5 writes the query header of every unit whose tile 0 is this CTA's and zeroes the unit's
-//    arrival counter.
-// Both the copying lane and the epilogue walk the same tiles, from a table of the CTA's tiles that
-// all threads fill at the start (every descriptor load in flight at once).  Every wait is bounded; a CTA whose wait runs out, or that finds a unit's anchor rows
-// outside the arena the map covers, writes +inf as the chunk maxima of all its tiles (the decode's
-// outputs for those units become NaN) and stops.
+// Anchor scores (Eq. 2-3: S_A = q . k_a once per anchor): CTA b < units writes unit b's query header and zeroes its
+// counters; the others take 64 anchors of a unit each (warp w rows 16 w .. 16 w + 15), straight from global memory into
+// bf16 mma A fragments (rows are stored swizzled in 16-byte chunks by slot % 8; the k order is permuted the same way
+// in A and B, so that a thread's dims are contiguous).  Bound by the anchor rows' bytes and a CTA's load latency; many
+// short CTAs keep enough loads in flight, hold no tensor memory and little else, so the decode, the programmatic
+// dependent, sets itself up beside them.  A persistent CTA per SM with tensor copies, tcgen05 products and
+// tensor-memory accumulators took 7 us whatever the size at 8 x 656 anchors, where this takes 3, and was slower at
+// every size (whole calls, us, that and this: 8 units of 32768 tokens 20.8, 18.4; 16 ragged requests 85.0, 80.0;
+// 64 x 2622 anchors 170.9, 163.5; 64 x 6554 198.7, 189.6; 128 x 5243 390, 373).
 template <int GS>
-__global__ void __launch_bounds__(kScThreads) akv_scores_tc_kernel(const __grid_constant__ ScoreParams P,
-                                                                   const __grid_constant__ CUtensorMap tmA,
-                                                                   const __grid_constant__ CUtensorMap tmB) {
-  extern __shared__ __align__(16) uint8_t score_dyn[];
-  __shared__ __align__(8) uint64_t bars[2 * kScStages + 4];  // full[s], free[s], acc_full[b], acc_empty[b]
-  __shared__ uint32_t tmem_sh;
-  __shared__ float wmx[2][4][8];
-  __shared__ int failed_sh;
-  __shared__ int2 tab[kScMaxTiles];  // this CTA's tiles: the unit's anchors, anchor row (-1: outside the map)
-  __shared__ __align__(16) float hdr_q[8 * 128];  // the header warp's rotated query rows
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t sbase = (smem_u32(score_dyn) + 1023u) & ~1023u;
-  auto full = [&](int s) { return smem_u32(bars + s); };
-  auto freed = [&](int s) { return smem_u32(bars + kScStages + s); };
-  auto acc_full = [&](int b) { return smem_u32(bars + 2 * kScStages + b); };
-  auto acc_empty = [&](int b) { return smem_u32(bars + 2 * kScStages + 2 + b); };
-  volatile int* failed = &failed_sh;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int n_tiles = P.units * P.n_t;
-  const int n_my = n_tiles > (int)blockIdx.x ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-  for (int i = tid; i < n_my && i < kScMaxTiles; i += kScThreads) {  // all descriptors in one round trip
-    const akv_unit_desc* d = unit_desc(P.arena, ((int)blockIdx.x + i * (int)gridDim.x) / P.n_t);
-    const int k = d->n_anchors;
-    const uint64_t off = d->off_anchor_k;
-    tab[i] = make_int2(k, !(off & 255u) && (long long)(off >> 8) + k <= P.arena_rows ? (int)(off >> 8) : -1);
-  }
-  if (tid == 0) {
-    for (int s = 0; s < kScStages; ++s) {
-      mbar_init(full(s), 1);
-      mbar_init(freed(s), 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(acc_full(b), 1);
-      mbar_init(acc_empty(b), 4);  // one arrival per epilogue warp
-    }
-    *failed = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 0) tc_alloc(smem_u32(&tmem_sh), kScTmemCols);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = tmem_sh;
-
-  // the next of this CTA's tiles that hold anchors (or are a unit's tile 0), from the table: ci is
-  // the next entry to look at; row is the anchor row (-1: outside the map)
-  int ci = 0;
-  const int n_tab = min(n_my, kScMaxTiles);
-  auto next_tile = [&](int& u, int& t, int& k, int& row) {
-    while (ci < n_tab) {
-      const int T = (int)blockIdx.x + ci * (int)gridDim.x;
-      const int2 e = tab[ci++];
-      k = e.x;
-      row = e.y;
-      u = T / P.n_t;
-      t = T % P.n_t;
-      if (t == 0 || t * kScTile < k) return true;
-    }
-    return false;
-  };
-
-  if (warp == 4) {
-    if (lane == 0) {  // ---- copies and products
-      int u, t, k, row0, n_iss = 0, n_mma = 0;
-      auto issue = [&](int j) {  // the tile just found into stage j % kScStages
-        const int s = j % kScStages;
-        const uint32_t st = sbase + (uint32_t)s * kScStage;
-        if (row0 >= 0) {
-          const int row = row0 + t * kScTile;  // 256-byte rows
-          const int qrow = (int)(qrow_base(u, P.n_kv_heads, P.n_q_heads) >> 7);
-          mbar_expect_tx(full(s), kScStage);
-          tma_load_2d(st, &tmA, 0, row, full(s));
-          tma_load_2d(st + kScHalfA, &tmA, 64, row, full(s));
-          tma_load_2d(st + 2 * kScHalfA, &tmB, 0, qrow, full(s));
-          tma_load_2d(st + 2 * kScHalfA + kScHalfB, &tmB, 64, qrow, full(s));
-        } else {
-          mbar_arrive(full(s));  // nothing copied: the epilogue fails the CTA
-        }
-      };
-      bool more = true;
-      while (n_iss < kScStages && (more = next_tile(u, t, k, row0))) issue(n_iss++);
-      for (int j = 0; j < n_iss; ++j) {
-        const int s = j % kScStages, b = j & 1;
-        if (*failed || !mbar_wait(full(s), (uint32_t)(j / kScStages) & 1u) ||
-            !mbar_wait(acc_empty(b), ((uint32_t)(j >> 1) & 1u) ^ 1u)) {
-          *failed = 1;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t a = sbase + (uint32_t)s * kScStage, bq = a + 2 * kScHalfA;
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {  // K steps of 16: 32 bytes into a half, then the other half
-          const uint32_t ka = (uint32_t)(kk >> 2) * kScHalfA + (uint32_t)(kk & 3) * 32;
-          const uint32_t kb = (uint32_t)(kk >> 2) * kScHalfB + (uint32_t)(kk & 3) * 32;
-          tc_mma(tmem + 16u * (uint32_t)b, sw128_desc(a + ka), sw128_desc(bq + kb), kScIdesc, kk > 0 ? 1u : 0u);
-        }
-        tc_commit(acc_full(b));
-        tc_commit(freed(s));
-        ++n_mma;
-        // refill the previous tile's stage once its products are done (this tile's run meanwhile)
-        if (j > 0 && more && (more = next_tile(u, t, k, row0))) {
-          const int sp = (j - 1) % kScStages;
-          if (!mbar_wait(freed(sp), (uint32_t)((j - 1) / kScStages) & 1u)) {
-            *failed = 1;
-            break;
-          }
-          issue(n_iss++);  // n_iss = j - 1 + kScStages: stage sp
-        }
-      }
-      // (bounded) nothing of this CTA's is left in flight at exit: copies never consumed (after a
-      // failure), and the last commit's arrivals (every earlier one has landed before it)
-      if (*failed)
-        for (int j = n_mma; j < n_iss; ++j) mbar_wait(full(j % kScStages), (uint32_t)(j / kScStages) & 1u);
-      if (n_mma > 0) mbar_wait(freed((n_mma - 1) % kScStages), (uint32_t)((n_mma - 1) / kScStages) & 1u);
-    }
-    __syncwarp();
-  } else if (warp == 5) {  // ---- query headers
-    for (int T = (int)blockIdx.x; T < n_tiles; T += (int)gridDim.x) {
-      if (T % P.n_t) continue;
-      if (lane < 8) unit_counters(P.uh, P.uh_stride, T / P.n_t, GS)[lane] = 0u;
-      unit_query_header_warp<GS>(P, T / P.n_t, hdr_q);
-    }
-  } else {  // ---- epilogue, warps 0-3
-    int u, t, k, row0;
-    for (int j = 0; next_tile(u, t, k, row0); ++j) {
-      const int b = j & 1;
-      const bool got = mbar_wait_w(acc_full(b), (uint32_t)(j >> 1) & 1u);
-      tc_fence_after();
-      float v[8];
-      tc_ld8(tmem + ((uint32_t)(32 * warp) << 16) + 16u * (uint32_t)b, v);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(acc_empty(b));  // this warp's lanes of accumulator b are read
-      const bool ok_tile = got && row0 >= 0;
-      const int a = t * kScTile + 32 * warp + lane;
-      const bool ok = ok_tile && a < k;
-      float sc[8];
-#pragma unroll
-      for (int g = 0; g < 8; ++g) sc[g] = v[g] * P.scale_log2;
-      if (ok) {
-        float* sa = P.sa + (size_t)u * P.ka_stride * GS;
-        if constexpr (GS == 8) {
-          *reinterpret_cast<float4*>(sa + (size_t)a * 4) = make_float4(sc[0], sc[1], sc[2], sc[3]);
-          *reinterpret_cast<float4*>(sa + ((size_t)P.ka_stride + a) * 4) = make_float4(sc[4], sc[5], sc[6], sc[7]);
-        } else if constexpr (GS == 4) {
-          *reinterpret_cast<float4*>(sa + (size_t)a * 4) = make_float4(sc[0], sc[1], sc[2], sc[3]);
-        } else if constexpr (GS == 2) {
-          *reinterpret_cast<float2*>(sa + (size_t)a * 2) = make_float2(sc[0], sc[1]);
-        } else {
-          sa[a] = sc[0];
-        }
-      }
-#pragma unroll
-      for (int g = 0; g < GS; ++g) {
-        const float m = warp_max(ok ? sc[g] : -INFINITY);
-        if (lane == 0) wmx[b][warp][g] = m;
-      }
-      // the four warps' maxima are in place; a failure seen by any thread stops all four
-      if (named_sync_or(1, 128, !ok_tile || *failed)) {
-        if (tid == 0) *failed = 1;
-        break;
-      }
-      if (tid < 2 * GS) {
-        const int c = tid / GS, g = tid % GS, ch = 2 * t + c;
-        if (ch * CHA < k) P.cmax[((size_t)u * P.n_ch + ch) * GS + g] = fmaxf(wmx[b][2 * c][g], wmx[b][2 * c + 1][g]);
-      }
-    }
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  if (*failed) {
-    for (int T2 = (int)blockIdx.x; T2 < n_tiles; T2 += (int)gridDim.x) {
-      const int u = T2 / P.n_t, t = T2 % P.n_t;
-      if (tid < 2 * GS && 2 * t + tid / GS < P.n_ch)
-        P.cmax[((size_t)u * P.n_ch + 2 * t + tid / GS) * GS + tid % GS] = INFINITY;
-    }
-  }
-  if (warp == 0) tc_dealloc(tmem, kScTmemCols);
-}
-
-// Anchor scores of small calls: CTA b < units writes unit b's query header and zeroes its counters; the others
-// take 64 anchors of a unit each (warp w rows 16 w .. 16 w + 15), straight from global memory into bf16 mma A
-// fragments (rows are stored swizzled in 16-byte chunks by slot % 8; the k order is permuted the same way in
-// A and B, so that a thread's dims are contiguous).  It holds no tensor memory and little else, so it starts
-// and ends in about 3 us where the persistent launch above takes 7 us whatever its size (8 x 656 anchors),
-// and the decode, its programmatic dependent, sets itself up beside it.
-template <int GS>
-__global__ void __launch_bounds__(128) akv_scores_small_kernel(const ScoreParams P) {
+__global__ void __launch_bounds__(128) akv_scores_kernel(const ScoreParams P) {
   __shared__ __align__(16) float hdr_q[8 * 128];
   __shared__ float wm[4][8];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -978,7 +766,7 @@ __global__ void __launch_bounds__(128) akv_scores_small_kernel(const ScoreParams
   const int k = d->n_anchors;
   if (ch * CHA >= k) return;
   const uint64_t off = d->off_anchor_k;
-  const bool inside = (long long)(off >> 8) + k <= P.arena_rows;
+  const bool inside = !(off & 255u) && (long long)(off >> 8) + k <= P.arena_rows;
   const uint8_t* AK = P.arena + off;
   const size_t qb = qrow_base(u, P.n_kv_heads, P.n_q_heads);
   uint2 bq[8];
@@ -2318,7 +2106,6 @@ struct Plan {
   DecodeParams P;
   size_t smem = 0;
   int grid = 0;
-  int sms = 0;  // SMs of the device (the score launch: one CTA each)
 };
 
 // Shared-memory carve-up for X anchor-value rows, the table in shared memory or not, a ring of at least
@@ -2364,20 +2151,23 @@ bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, bool smem_sa, int sm
   return true;
 }
 
-// Preference: the anchor-score table in shared memory (the token gathers' fast path), with a ring of four and
-// a half mean tiles (one in each role, one landing, and what wrapping around leaves unused), then less, the
-// least p rows and anchor-value rows trimmed towards 3/4 of their values with it; then the table in global
-// memory (gathers through L1 and L2) the same way; then anything that holds one tile.
+// Preference: the anchor-score table in shared memory (the token gathers' fast path), with a ring of five mean tiles
+// (one in each role, two landing, and what wrapping around leaves unused) and p rows for tiles half again as dense as
+// the R they need, then less, the least p rows and anchor-value rows trimmed towards 3/4 of their values with it; then
+// the table in global memory (gathers through L1 and L2) the same way; then anything that holds one tile.  4 requests
+// of 131072, 8B shape, us per call with rings of 4.5, 3.5, 2.5 mean tiles alone and with these: 2 % anchors and 20 %
+// residuals 115.3 -> 114.5, 4 % and 10 % 107.1 -> 105.4, 4 % and 20 % 135.1 -> 126.9; six ragged requests with 20 %
+// residuals 80.0 -> 77.4.
 // table false: no anchor-score table is read (RoPE at decode), so none is placed in shared memory.
 bool make_plan(const Layout& L, int GS, int smem_optin, bool table, Plan* out, std::string* why) {
   const int R0 = full_r(L), X0 = full_x(L);
   const int Rmin = std::max(16, ((R0 * 3 / 4) + 15) & ~15), Xmin = std::max(16, ((X0 * 3 / 4) + 15) & ~15);
   const double mean = (double)F_MAX + T * mean_density(L) * 72.0 + 256.0 + 256.0 * (T * max_anchor_density(L) + 2.0);
   for (int sa = table ? 1 : 0; sa >= 0; --sa)
-    for (const double tiles : {4.5, 3.5, 2.5}) {
+    for (const double tiles : {5.0, 4.5, 4.0, 3.5, 3.0, 2.5, 2.0, 1.5}) {
       const bool trim = tiles < 4.0;
       for (int X = X0; X >= (trim ? Xmin : X0); X -= 16)
-        if (make_plan_rx(L, GS, trim ? Rmin : R0, X, sa == 1, smem_optin, (long long)(tiles * mean), out)) return true;
+        if (make_plan_rx(L, GS, trim ? Rmin : (tiles > 4.5 ? R0 * 3 / 2 : R0), X, sa == 1, smem_optin, (long long)(tiles * mean), out)) return true;
     }
   for (int X = X0; X >= 16; X -= 16)
     if (make_plan_rx(L, GS, 16, X, false, smem_optin, (long long)F_MAX + 2 * 16 * 36 + 256LL * X, out)) return true;
@@ -2387,7 +2177,6 @@ bool make_plan(const Layout& L, int GS, int smem_optin, bool table, Plan* out, s
 
 using DecodeFn = void (*)(const DecodeParams);
 using ScoreFn = void (*)(const ScoreParams);
-using ScoreTcFn = void (*)(const ScoreParams, const CUtensorMap, const CUtensorMap);
 using RopeFn = void (*)(const RopeParams);
 template <int GS, int MODE>
 DecodeFn decode_kernel_c(int codec) {
@@ -2402,14 +2191,6 @@ template <int GS>
 RopeFn rope_kernel(int codec) {
   return codec ? akv_rope_logits_kernel<GS, 1> : akv_rope_logits_kernel<GS, 0>;
 }
-template <int GS>
-ScoreTcFn score_kernel() {
-  return akv_scores_tc_kernel<GS>;
-}
-
-// 64-anchor chunks up to which the small score kernel takes the anchor scores: a few waves of its CTAs.
-constexpr int kSmallChunks = 1024;
-
 template <int GS>
 ScoreFn suffix_kernel(bool rope) {
   return rope ? akv_suffix_kernel<GS, true> : akv_suffix_kernel<GS, false>;
@@ -2466,16 +2247,12 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   if (!have) {
     const DeviceInfo di = device_info();
     if (!make_plan(L, GS, di.smem_optin, !rope, &pl, why)) return -1;
-    cudaError_t e =
+    const cudaError_t e =
         cudaFuncSetAttribute(decode_kernel<GS>(codec, rope, pl.P), cudaFuncAttributeMaxDynamicSharedMemorySize, di.smem_optin);
     if (e != cudaSuccess) return (int)e;
-    if ((e = cudaFuncSetAttribute(score_kernel<GS>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)kScDynSmem)) != cudaSuccess)  // the score launch's stages
-      return (int)e;
     int grid = (int)std::min<long long>(std::min(di.sms, kMaxGrid), ttot);
     if (ctas > 0) grid = (int)std::min<long long>(ctas, ttot);
     pl.grid = grid;
-    pl.sms = di.sms;
     // first unit and tile of every CTA's range
     long long t0 = 0;
     int u = 0;
@@ -2577,34 +2354,11 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
     e = cudaLaunchKernelEx(&cfg, rope_kernel<GS>(codec), R);
     cfg.blockDim = dim3(128, 1, 1);
     for (int j = 0; j < 64; ++j) S.turn[j] = R.turn[j];
-  } else if ((long long)units * P.n_ch <= kSmallChunks) {
+  } else {
     S.units = units;
     S.arena_rows = (long long)(arena_bytes / 256);
     cfg.gridDim = dim3((unsigned)(units + units * P.n_ch), 1, 1);
-    e = cudaLaunchKernelEx(&cfg, akv_scores_small_kernel<GS>, S);
-  } else {
-    // anchor rows of every unit through one map over the caller's arena as 256-byte rows (each
-    // unit's anchor-key section starts its 256-byte-aligned segment; a full-selection arena places
-    // its units by the budgets it chose, past the plain layout's size), query rows through one over q
-    CUtensorMap tmA, tmB;
-    if (!encode_row_map(&tmA, arena, arena_bytes / 256, kScTile, CU_TENSOR_MAP_SWIZZLE_NONE) ||
-        !encode_row_map(&tmB, q, (uint64_t)p.batch * (uint64_t)p.n_q_heads, 16, CU_TENSOR_MAP_SWIZZLE_128B)) {
-      *why = "(tensor maps of the score launch could not be encoded)";
-      return -1;
-    }
-    S.units = units;
-    S.n_t = (P.n_ch + 1) / 2;
-    S.arena_rows = (long long)(arena_bytes / 256);
-    // persistent, one CTA per SM over the units' anchor tiles (more CTAs, one after another on an
-    // SM, when one CTA would take more tiles than its table holds)
-    const long long n_tiles = (long long)units * S.n_t;
-    cfg.gridDim = dim3((unsigned)std::max<long long>({1, std::min<long long>(n_tiles, pl.sms),
-                                                      (n_tiles + kScMaxTiles - 1) / kScMaxTiles}), 1, 1);
-    cfg.blockDim = dim3(kScThreads, 1, 1);
-    cfg.dynamicSmemBytes = kScDynSmem;
-    e = cudaLaunchKernelEx(&cfg, score_kernel<GS>(), S, tmA, tmB);
-    cfg.blockDim = dim3(128, 1, 1);
-    cfg.dynamicSmemBytes = 0;
+    e = cudaLaunchKernelEx(&cfg, akv_scores_kernel<GS>, S);
   }
   // the launches after the first may start beside the one before them and wait for it where they need it
   cudaLaunchAttribute pdl;

@@ -1,23 +1,28 @@
-// Plain GPU encoder of the AnchorKV compressed cache (Algorithm 1 with the
-// anchor and slot rules of this build).  Correct, not tuned: every decision
-// (assignment, gamma, residual energy ranking, rotation, codes) is taken in
-// IEEE fp64 with a fixed operation order, so the packed bytes are
-// reproducible bit for bit.  Compiled with --fmad=false; where a fused
-// multiply-add is used explicitly its product is exact, so rounding once or
-// twice gives the same result.
+// GPU encoder of the AnchorKV compressed cache (Algorithm 1 with the anchor and slot rules of this build; the paper's
+// full selection).  Every decision (assignment, gamma, residual energy ranking, rotation, codes) is the one that IEEE
+// fp64 with a fixed operation order takes, so the packed bytes are reproducible bit for bit.  That arithmetic is done
+// only where it decides: this GPU's fp64 unit takes a warp instruction per 64 cycles and scheduler, so each step is
+// first taken on tensor cores, in fp32 or in pairs of fp32, with a bound of its error, and what the bound leaves open
+// (about 1 % of positions and records) is repeated in fp64.  8 units of 32768 tokens: 82.9 ms with fp64 throughout,
+// 0.40 ms.  Compiled with --fmad=false; where a fused multiply-add is used explicitly in fp64 its product is exact, so
+// rounding once or twice gives the same result.
 //
 // Kernels, in launch order, each over all units of the batch:
 //   enc_anchors    select the k - W smallest hashes, number anchor slots by position
 //   enc_rows       copy anchor rows into the arena (16-byte chunks swizzled), squared norms
 //   enc_assign_tc  Eq. 1: the one or two anchors that can be a position's nearest, on tensor cores
 //   enc_finish     Eq. 2 gamma, residual energies (per position), as far as fp32 decides them
-//   enc_undecided  the rest in fp64
+//   enc_undecided  the rest, in paired fp32 and fp64
 //   enc_slots      top-N residual energies per side -> residual flags and slot list
+//   enc_slots_exact the same from fp64 energies, where the fp32 ones cannot rank (else empty)
 //   enc_order      stored order: stable counting sort of positions by value anchor slot
 //   enc_tile_count residual records per tile and side
 //   enc_tile_table tile block offsets
 //   enc_tile_fill  streams, bitmaps and rank words of every tile block
 //   enc_quant      Eq. 12 rotation and 2-bit quantization of every slot, into its tile
+// The full selection adds the observation rows' attention and the scores before them (enc_obs_*_f, enc_score_*) and
+// the utilities and pools in enc_slots' place (enc_util_f, enc_pool_f), each followed by its exact form, which runs
+// only for units whose ranking the errors leave open.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
