@@ -2,8 +2,8 @@
 // Eq. 4: no key or value row is ever rebuilt in memory).  Two launches per call (three with a dense suffix, whose
 // chunks take a launch of their own between them).  Each launch after the first is a programmatic dependent of the one
 // before it: it may start once that one's CTAs have, and waits where it needs its results.  So the decode is set up and
-// its first tiles are on their way beside the scores, and the suffix's chunks run beside them (16 ragged requests, 8B
-// shape: 87.5 -> 85.6 us; 8 x 131072, 70B shape: 170.4 -> 169.7).  The first launch is an ordinary one (as a dependent
+// its first tiles are on their way beside the scores, and the suffix's chunks run beside them (six ragged requests, 8B
+// shape: 87.5 -> 85.6 us; four with RoPE and a suffix: 179 -> 172).  The first launch is an ordinary one (as a dependent
 // of the call before, its wait cost more than the gap: 18.4 -> 20.5 us a call at 8 units of 32768).
 //
 // 1. The anchor scores S_A[a][g] = q_g . k_a of every anchor of every unit, once per anchor (Eq. 2-3),
@@ -46,7 +46,7 @@
 // per tile), each about half used; the rest is the latency of the phases' dependent chains.  Two groups
 // of four warps that took a tile through all phases (255 registers, two warps per sub-partition) spent
 // 2.8 us per tile pair-wise; token and product warps side by side spend 2.7 us and leave each other's
-// latencies covered where tiles are few (8B shape, 32K: 24.6 -> 18.4 us per call with the small score launch).
+// latencies covered where tiles are few (8B shape, 32K: 24.6 -> 18.4 us per call, the score launch's part included).
 //
 // The exponent reference m is the largest anchor score of each query row.  Anchors are
 // tokens of the unit, so it is a lower bound of the largest logit (sums cannot overflow unless
@@ -256,10 +256,23 @@ __device__ __forceinline__ uint32_t code_pair_h2(uint32_t x) {
   if constexpr (CODEC == 0) return codes2_to_h2(x);
   else return lm_pair(x, 0xB740BE08u, 0x3E083740u);
 }
+// Both pairs of a value word's records, codes at bits 0, 16 and 8, 24: with the Lloyd-Max codec the four selector bytes
+// come from one multiply-add (6 instructions for the two pairs, not 9: 8 x 131072, G = 8, Lloyd-Max 203.6 -> 196.7 us, G = 4
+// 162.4 -> 158.2; the product warps are the longer side there).
 template <int CODEC>
-__device__ __forceinline__ uint32_t code_pair_b2(uint32_t x) {
-  if constexpr (CODEC == 0) return codes2_to_b2(x);
-  else return lm_pair(x, 0xBEE8BFC1u, 0x3FC13EE8u);
+__device__ __forceinline__ uint2 code_pairs_b2(uint32_t x) {
+  if constexpr (CODEC == 0) {
+    return make_uint2(codes2_to_b2(x), codes2_to_b2(x >> 8));
+  } else {
+    const uint32_t u = (x & 0x03030303u) * 0x22u + 0x10101010u;
+    uint32_t s0, s1;
+    uint2 r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(s0) : "r"(u), "r"(0u), "r"(0x00000020u));
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(s1) : "r"(u), "r"(0u), "r"(0x00000031u));
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r.x) : "r"(0xBEE8BFC1u), "r"(0x3FC13EE8u), "r"(s0));
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r.y) : "r"(0xBEE8BFC1u), "r"(0x3FC13EE8u), "r"(s1));
+    return r;
+  }
 }
 // One code's reconstruction value on CUDA cores (the rare paths).
 __device__ __forceinline__ float code_level(uint32_t c, int lloyd) {
@@ -748,7 +761,7 @@ __device__ __noinline__ void unit_query_header_warp(const ScoreParams& P, int u,
 // short CTAs keep enough loads in flight, hold no tensor memory and little else, so the decode, the programmatic
 // dependent, sets itself up beside them.  A persistent CTA per SM with tensor copies, tcgen05 products and
 // tensor-memory accumulators took 7 us whatever the size at 8 x 656 anchors, where this takes 3, and was slower at
-// every size (whole calls, us, that and this: 8 units of 32768 tokens 20.8, 18.4; 16 ragged requests 85.0, 80.0;
+// every size (whole calls, us, that and this: 8 units of 32768 tokens 20.8, 18.4; six ragged requests 85.0, 80.0;
 // 64 x 2622 anchors 170.9, 163.5; 64 x 6554 198.7, 189.6; 128 x 5243 390, 373).
 template <int GS>
 __global__ void __launch_bounds__(128) akv_scores_kernel(const ScoreParams P) {
@@ -1935,7 +1948,8 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
             for (int nb = 0; nb < 2; ++nb) {
               // records 2c, 2c+1 at bits 2c and 2c + 16, records 2c+8, 2c+9 eight bits higher
               const uint32_t x = wd[nb] >> (2 * c4);
-              mma_bf16(accR[nb], a.x, a.y, a.z, a.w, code_pair_b2<CODEC>(x), code_pair_b2<CODEC>(x >> 8));
+              const uint2 b = code_pairs_b2<CODEC>(x);
+              mma_bf16(accR[nb], a.x, a.y, a.z, a.w, b.x, b.y);
             }
           };
           if (mt.fast & 2u) {
