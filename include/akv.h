@@ -242,9 +242,9 @@ akv_status akv_cache_header_host(const akv_params* p, const int32_t* ctx_lens_ho
  *   arena : device, arena_bytes >= akv_cache_size(...).arena_bytes, 256-byte aligned
  *   ws    : device scratch, ws_bytes >= encode_ws_bytes, 256-byte aligned;
  *           contents on entry are ignored and on exit are unspecified
- * Decisions (assignment, gamma, slot ranking, codes) are taken in IEEE fp64
- * with a fixed operation order, so the packed bytes are reproducible bit for
- * bit.  Errors: AKV_ERR_INVALID (null, misaligned, s_max < max S_b),
+ * Decisions (assignment, gamma, slot ranking, codes) are those of IEEE fp64
+ * with a fixed operation order (taken in it where faster arithmetic leaves them
+ * open), so the packed bytes are reproducible bit for bit.  Errors: AKV_ERR_INVALID (null, misaligned, s_max < max S_b),
  * AKV_ERR_TOO_SMALL (arena or ws short), AKV_ERR_CUDA (launch failure).
  */
 akv_status akv_encode(const akv_params* p, const int32_t* ctx_lens_host, const void* K, const void* V,
@@ -409,7 +409,7 @@ akv_status akv_pack_table1_host(const akv_params* p, const int32_t* ctx_lens_hos
 /*
  * Bytes of device workspace akv_decode_attn needs for these parameters and
  * context lengths: the anchor scores of every unit (4 G bytes per anchor),
- * their maxima per chunk of 64 anchors, one arrival counter per unit, and
+ * their maxima per chunk of 64 anchors, one arrival counter per query head, and
  * the partial sums of the CTAs that share a unit (about 8.5 KB per query head
  * and (CTA or unit) slot, at most 256 CTAs).  Contents on entry are ignored.
  */
@@ -425,22 +425,22 @@ akv_status akv_decode_workspace_size(const akv_params* p, const int32_t* ctx_len
  *   arena     : device, as written by akv_encode or copied from akv_cache_pack_host
  *               for the same (p, ctx_lens_host), or by akv_encode_select
  *   arena_bytes : the arena's whole size (akv_cache_size, or akv_cache_size_select
- *               for a full-selection arena): the score launch reads anchor rows
- *               through a tensor map of exactly this many bytes, and a unit whose
- *               anchor rows lie outside it gets NaN outputs
+ *               for a full-selection arena): a unit whose anchor rows lie outside
+ *               it gets NaN outputs
  *   q         : device bf16 [B][H_q][128]
  *   out       : device bf16 [B][H_q][128], round-to-nearest-even of the fp32 result
  *   out_f32   : device fp32 [B][H_q][128] or NULL
  *   ws        : device workspace, 256-byte aligned, of >= akv_decode_workspace_size
  *               bytes; calls that overlap on the GPU need separate workspaces
- * Two launches: the anchor scores of every unit (persistent, tensor cores with
- * tensor-memory accumulators, tiles of 128 anchors brought by tensor copies), then
- * the decode itself, one CTA per SM over equal shares of all units' tile blocks.
+ * Two launches: the anchor scores of every unit (with AKV_FLAG_ROPE the logits of
+ * every stored token instead), then the decode itself, one CTA per SM over equal
+ * shares of all units' tile blocks.
  * Errors: AKV_ERR_INVALID (null/misaligned pointers, bad sizes), AKV_ERR_TOO_SMALL
  * (arena or workspace short), AKV_ERR_UNSUPPORTED (no shared-memory plan fits),
  * AKV_ERR_CUDA (launch failure).
- * Ordering: both launches are ordinary launches on `stream`: they start after all
- * preceding work in the stream and complete before any later work starts.
+ * Ordering: the first launch starts after all preceding work in the stream; the
+ * second may be set up beside it and waits for it (a programmatic dependent
+ * launch); both complete before any later work starts.
  */
 akv_status akv_decode_attn(const akv_params* p, const int32_t* ctx_lens_host, const void* arena,
                            size_t arena_bytes, const void* q, void* out, float* out_f32, float sm_scale,
