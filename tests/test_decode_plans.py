@@ -109,3 +109,26 @@ def test_queries_written_just_before(dev, before, rope, lens):  # noqa: F811
         with torch.cuda.stream(main):
             g.replay()
         check()
+
+
+@pytest.mark.parametrize("G", [1, 4, 8])
+@pytest.mark.parametrize("fa,fr", [(0.01, 0.0), (0.02, 0.3), (0.04, 0.2), (0.08, 0.1), (0.15, 0.2), (0.27, 0.1)])
+def test_plans_by_anchor_share(dev, G, fa, fr):  # noqa: F811
+    """From rings of five mean tiles with the score table in shared memory to two tiles with the table in global
+    memory, and tiles with more runs than the staged anchor-value rows; two units, so that ranges cross them."""
+    p = akv.Params(batch=2, n_kv_heads=1, n_q_heads=G, anchor_frac=fa, res_frac_k=fr, res_frac_v=fr, seed=8)
+    _run_seeded(dev, p, [41000, 20011], sm_scale=0.2)
+
+
+@pytest.mark.parametrize("G", [2, 8])
+@pytest.mark.parametrize("nv", [1, 15, 16, 17, 31, 33, 200])
+def test_lloyd_max_record_groups(dev, G, nv):  # noqa: F811
+    """Value records around the edges of their groups of 16, Lloyd-Max levels."""
+    S = 1000
+    p = akv.Params(batch=1, n_kv_heads=1, n_q_heads=G, res_frac_k=0.05, res_frac_v=(nv + 0.5) / S, seed=10, lloyd=True)
+    assert akv.akv_unit_shapes(p, [S])[0][3] == nv
+
+    def mutate(u, d):
+        d["min_k"] = d["min_k"] * 0
+        d["min_v"] = d["min_v"] * 0
+    _run_seeded(dev, p, [S], mutate=mutate)
