@@ -27,7 +27,7 @@ void get_decode_events(void** after_scores, void** after_decode) {
   *after_decode = (void*)g_ev_decode;
 }
 
-// Workspace of a decode call: anchor scores, chunk maxima, arrival counters, partial slots.
+// Workspace of a decode call: anchor scores, query headers and arrival counters, chunk maxima, partial slots.
 DecodeWs decode_ws_layout(const Layout& L, int32_t suffix_cap) {
   DecodeWs w;
   const size_t units = L.shape.size();
@@ -42,11 +42,10 @@ DecodeWs decode_ws_layout(const Layout& L, int32_t suffix_cap) {
   const bool rope = (L.header.params.flags & AKV_FLAG_ROPE) != 0;
   const size_t s_stride = (size_t)((L.max_len + 63) & ~63);
   w.o_sa = take(rope ? 0 : units * ka * (size_t)L.G * 4);
-  w.o_uh = take(units * (size_t)((hdr_bytes(L.G) + 255) & ~255));
+  w.o_uh = take(units * (size_t)((hdr_bytes(L.G) + 255) & ~255));  // with the heads' arrival counters in the padding
   // chunk maxima: of 64 anchors, or with RoPE of 64 stored tokens
   w.o_cmax = take(units * (rope ? s_stride / 64 : nch) * (size_t)L.G * 4);
   w.o_lg = take(rope ? units * s_stride * (size_t)L.G * 4 : 0);  // RoPE: every token's logits
-  w.o_cnt = take(units * 4);
   w.o_part = take((size_t)(kMaxGrid + units) * (size_t)part_floats(L.G) * 4);
   w.o_suf = take(units * (size_t)((suffix_cap + kSuffixChunk - 1) / kSuffixChunk) * (size_t)suf_floats(L.G) * 4);
   w.total = off;

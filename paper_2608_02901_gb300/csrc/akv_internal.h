@@ -115,10 +115,10 @@ void encode_ws_layout(const Layout& L, EncodeWs* ws, int32_t m_obs = 0);
 int launch_encode(const Layout& L, const EncodeWs& W, const akv_params& p, const void* K, const void* V, int32_t s_max,
                   void* arena, void* ws, void* stream, const akv_select_params* sel = nullptr,
                   const void* Q = nullptr, int32_t m_obs = 0);
-// Decode workspace (device): anchor scores [units][ka][G] f32, query headers, chunk maxima,
-// arrival counters, partial slots; byte offsets from the workspace base (256-byte aligned).
+// Decode workspace (device): anchor scores [units][ka][G] f32, query headers with the heads' arrival counters,
+// chunk maxima, partial slots; byte offsets from the workspace base (256-byte aligned).
 struct DecodeWs {
-  size_t o_sa = 0, o_uh = 0, o_cmax = 0, o_cnt = 0, o_part = 0, o_suf = 0, o_lg = 0, total = 0;
+  size_t o_sa = 0, o_uh = 0, o_cmax = 0, o_part = 0, o_suf = 0, o_lg = 0, total = 0;
 };
 // The dense suffix of a decode call (akv_suffix): bf16 rows [B][H_kv][cap][128] and the tokens
 // held per request (device int32 [B]); null K = no suffix.
@@ -140,6 +140,9 @@ AKV_HD constexpr int part_l(int GS) { return 128 * GS; }
 // Bytes of a unit's query header (from the score kernel): the rotated query q' [GS][128] f32, its
 // sums [8] f32, and the key-residual mma B fragments [GS == 8 ? 2 : 1][8][32] uint2.
 AKV_HD constexpr int hdr_bytes(int GS) { return GS * 512 + 32 + (GS == 8 ? 2 : 1) * 2048; }
+static_assert(hdr_bytes(1) % 256 && hdr_bytes(1) % 256 <= 224 && hdr_bytes(2) % 256 <= 224 && hdr_bytes(4) % 256 <= 224 && hdr_bytes(8) % 256 <= 224 &&
+                  hdr_bytes(2) % 256 && hdr_bytes(4) % 256 && hdr_bytes(8) % 256,
+              "eight arrival counters fit the padding of a header to 256 bytes");
 
 // Dense suffix: tokens per chunk, and the floats of a chunk's partial slot: the value sum
 // o [GS][128] under the chunk's own maximum, its normaliser l [8] and that maximum m [8] (log2 units).
