@@ -1875,20 +1875,21 @@ __device__ Quantized quantize_exact(const EncArgs& A, const __nv_bfloat16* X, co
 
 // The same in fp32, where its error bounds decide every rounding; false (for the whole warp) where one does
 // not.  r is one exactly rounded step; each of the seven butterfly stages rounds values whose sum of
-// magnitudes is at most L1 = sum |r|, so v is within 8 x 2^-24 L1 of the exact transform: err = 2^-20 L1
-// below is twice that.  A value within err of a rounding boundary (fp16 min and scale, code regions) leaves
-// the record to quantize_exact, about one record in a hundred.  (fp64 for every record took 457 us for
-// 52,000 records: the fp64 units issue one warp instruction in 64 cycles.)
+// magnitudes is at most L1 = sum |r|, so v is within 8 x 2^-24 L1 of the exact transform (err below: 2 % more).  A value
+// within err of a rounding boundary (fp16 min and scale, code regions) leaves the record to quantize_exact, about one
+// record in a hundred.  (fp64 for every record took 457 us for 52,000 records: the fp64 units issue one warp instruction
+// in 64 cycles; this takes 58, Lloyd-Max records of 24 short units 31, not 36 with their scales from the rotated sums.)
 __device__ bool quantize_fast(const EncArgs& A, const uint2 xr, const uint2 ar, float g, bool valid, Quantized* q) {
   const int lane = threadIdx.x & 31;
   const uint32_t xw[4] = {xr.x << 16, xr.x & 0xFFFF0000u, xr.y << 16, xr.y & 0xFFFF0000u};
   const uint32_t aw[4] = {ar.x << 16, ar.x & 0xFFFF0000u, ar.y << 16, ar.y & 0xFFFF0000u};
-  float v[4], l1 = 0.f;
+  float v[4], l1 = 0.f, rr = 0.f;
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
     v[e] = __uint_as_float(xw[e]);
     if (valid) v[e] = __fmaf_rn(-g, __uint_as_float(aw[e]), v[e]);
     l1 += fabsf(v[e]);
+    rr = __fmaf_rn(v[e], v[e], rr);
     if (A.rotate) {
       const unsigned long long sb = lane < 16 ? A.sign_lo : A.sign_hi;
       if ((sb >> ((4 * lane + e) & 63)) & 1ull) v[e] = -v[e];
@@ -1896,8 +1897,10 @@ __device__ bool quantize_fast(const EncArgs& A, const uint2 xr, const uint2 ar, 
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) l1 += __shfl_xor_sync(0xffffffffu, l1, o);
-  if (!(l1 >= 0x1p-60f && l1 <= 0x1p60f)) return false;
-  const float err = l1 * 0x1p-20f;
+  if (!(l1 >= 0x1p-40f && l1 <= 0x1p60f)) return false;  // (sums of squares stay normal)
+  // one rounding of the residual and seven of the butterflies, each at most 2^-24 of the sum of magnitudes that it is
+  // part of; the rest for l1's own and second-order terms
+  const float err = l1 * (1.02f * 0x1p-21f);
   if (A.rotate) {
     const float b0 = v[0] + v[1], b1 = v[0] - v[1], b2 = v[2] + v[3], b3 = v[2] - v[3];
     v[0] = b0 + b2;
@@ -1914,22 +1917,15 @@ __device__ bool quantize_fast(const EncArgs& A, const uint2 xr, const uint2 ar, 
   bool sure = true;
   q->byte = 0;
   if (A.lloyd) {
-    float ss = 0.f, sa = 0.f;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      ss = __fmaf_rn(v[e], v[e], ss);
-      sa += fabsf(v[e]);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      ss += __shfl_xor_sync(0xffffffffu, ss, o);
-      sa += __shfl_xor_sync(0xffffffffu, sa, o);
-    }
-    // sum v^2 off by 2 err sum |v| + 128 err^2 and ten roundings; the root adds two more
-    const float es = 2.001f * err * sa + 128.f * err * err + ss * 0x1p-20f;
+    for (int o = 16; o > 0; o >>= 1) rr += __shfl_xor_sync(0xffffffffu, rr, o);
+    // sum v^2 / 128 is sum r^2 (the transform keeps it, times 128; without it the mean is taken): each residual rounded
+    // once, nine roundings of the sum, so off by 2^-20.4 of it; the root adds two more.  (Summed after the rotation, whose
+    // errors are not each value's own, 10 % of the scales were left to fp64.)
+    const float ms = A.rotate ? rr : rr * 0.0078125f, es = ms * 0x1p-20f;
     q->min = 0u;
-    q->scale = f32_to_fp16_bits(__fsqrt_rn(fmaxf(ss - es, 0.f) * 0.0078125f) * (1.f - 0x1p-22f));
-    sure = q->scale == f32_to_fp16_bits(__fsqrt_rn((ss + es) * 0.0078125f) * (1.f + 0x1p-22f));
+    q->scale = f32_to_fp16_bits(__fsqrt_rn(ms - es) * (1.f - 0x1p-22f));
+    sure = q->scale == f32_to_fp16_bits(__fsqrt_rn(ms + es) * (1.f + 0x1p-22f));
     const float sc = __half2float(__ushort_as_half((unsigned short)q->scale));
     const float T = (float)kLloydT;
     if (sc == 0.f) {

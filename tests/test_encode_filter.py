@@ -36,6 +36,19 @@ def test_rows_outside_the_filter_range(dev, e):  # noqa: F811
     _encode_both(dev, p, lens, K, V)
 
 
+@pytest.mark.parametrize("lloyd,rotate", [(True, True), (True, False), (False, True)])
+@pytest.mark.parametrize("e", [-60, -46, -44, -42, -40, 20, 52])
+def test_record_magnitudes(dev, e, lloyd, rotate):  # noqa: F811
+    """Residuals on both sides of the range in which the fp32 quantiser's sums of squares stay normal."""
+    lens = [400]
+    p = akv.Params(batch=1, n_kv_heads=1, n_q_heads=1, anchor_frac=0.05, res_frac_k=0.5, res_frac_v=0.5, seed=16,
+                   lloyd=lloyd, rotate=rotate)
+    K, V = gen.clustered_batch(1, 1, lens, seed=17)
+    K[0, 0] = _scaled(K[0, 0], e)
+    V[0, 0, ::2] = _scaled(V[0, 0, ::2], e)
+    _encode_both(dev, p, lens, K, V)
+
+
 @pytest.mark.parametrize("kinds,k1", [(1, False), (4, True), (4, False), (40, False)])
 def test_equal_rows(dev, kinds, k1):  # noqa: F811
     """Positions drawn from a few distinct rows: equal scores (the lowest slot wins), energies that are exactly 0, and
