@@ -61,7 +61,7 @@ struct EncUnitWs {
   uint32_t* st[2];    // [S] stream word (slot | fp16 gamma << 16) per position and side
   uint8_t* flag[2];   // [S] residual flag per side (values: over slot_of, which is read no more by then)
   float* inv[2];      // [k to a multiple of 32] 1 / anchor norm, 0 for a zero anchor (over perm and inv)
-  int32_t* perm;      // [S] position of stored token t
+  int32_t* perm;      // [S] position of stored token t (full selection, before that: errors of u^K, fp64, over perm and at)
   int32_t* at;        // [S] stored index of position i
   uint32_t* cursor;   // [k + 1] value-anchor counts, then start of each run
   uint32_t* tcnt;     // [2 * n_tiles] residual records per tile (keys, values)
@@ -2223,8 +2223,8 @@ __global__ void __launch_bounds__(128) enc_obs_y_f(const EncArgs A) {
   }
 }
 
-// Eq. 6 utilities of 32 positions: key0 = bits(u^K) + 1, key1 = bits(u^V) + 1, anchors 0, and the relative error
-// of u^K (fp32, over perm).  Thread (position, group g of eight): rows g and g + 8 of every sixteen.  With r the
+// Eq. 6 utilities of 32 positions: key0 = bits(u^K) + 1, key1 = bits(u^V) + 1, anchors 0, and the error of u^K (fp64,
+// over perm and at; absolute, since |V - y|^2 may come out at or below 0 where V is close to y; infinite: no bound).  Thread (position, group g of eight): rows g and g + 8 of every sixteen.  With r the
 // key residual as an exact pair, u^K sums alpha^2 (q . r)^2 / D (|V|^2 - 2 V . y + |y|^2).
 constexpr int kUtPos = 32, kUtRows = 16;
 struct UtilSmem {
@@ -2384,7 +2384,7 @@ __global__ void __launch_bounds__(256) enc_util_f(const EncArgs A) {
         // errors of q . r and of dv: paired chains of 128 steps, and y's
         const float hq = 0x1p-32f * s.qn[r] * rnorm, sum = vnorm + s.yn[r] + ey;
         const float hv = sum * (0x1p-31f * sum + 2.f * ey);
-        ek = fma(a2, (double)(0.0078125f * (2.f * fabsf((float)dq) + hq) * hq * ((float)dv + hv)), fma(aq, (double)hv, ek));
+        ek = fma(a2, (double)(0.0078125f * (2.f * fabsf((float)dq) + hq) * hq * (fabsf((float)dv) + hv)), fma(aq, (double)hv, ek));
       }
     }
   }
@@ -2394,10 +2394,10 @@ __global__ void __launch_bounds__(256) enc_util_f(const EncArgs A) {
   s.red[g][lane][2] = ek;
   __syncthreads();
   if (g != 0 || p >= S) return;
-  float* err = reinterpret_cast<float*>(w.perm);
+  double* err = reinterpret_cast<double*>(w.perm);
   if (w.slot_of[p] >= 0) {
     w.key0[p] = w.key1[p] = 0ull;
-    err[p] = 0.f;
+    err[p] = 0.0;
     return;
   }
   for (int x = 1; x < 8; ++x) {
@@ -2412,7 +2412,7 @@ __global__ void __launch_bounds__(256) enc_util_f(const EncArgs A) {
   const bool bounded = (rnorm2 == 0.f || norm_ok(rnorm2)) && (vnorm2 == 0.f || norm_ok(vnorm2));
   w.key0[p] = (uint64_t)__double_as_longlong(uk > 0.0 ? uk : 0.0) + 1ull;
   w.key1[p] = (uint64_t)__double_as_longlong(uv > 0.0 ? uv : 0.0) + 1ull;
-  err[p] = !bounded ? INFINITY : (ek > 0.0 ? (float)(1.001 * ek * rm / uk) : 0.f);  // relative to u^K
+  err[p] = bounded ? 1.001 * ek * rm : (double)INFINITY;
 }
 
 // Whether a ranking by values v with errors e stands: the lowest selected v - e above the largest
@@ -2518,7 +2518,7 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) 
   __shared__ uint32_t wsum[kSelThreads / 32], found[3];
   __shared__ unsigned long long slot[2];
   __shared__ const uint64_t* keys[256];
-  __shared__ const float* errs[256];
+  __shared__ const double* errs[256];
   __shared__ float rel[256];
   __shared__ int32_t* lists[256];
   __shared__ uint32_t* ctrls[256];
@@ -2532,7 +2532,7 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) 
     const akv_unit_desc* d = unit_desc(A, u0 + h);
     const EncUnitWs w = unit_ws(A, u0 + h, d);
     keys[h] = side ? w.key1 : w.key0;
-    errs[h] = reinterpret_cast<const float*>(w.perm);
+    errs[h] = reinterpret_cast<const double*>(w.perm);
     rel[h] = 2.5f * alpha_error(w) + 0x1p-30f;
     lists[h] = w.res_pos + (side ? d->n_res_k : 0);
     ctrls[h] = w.ctrl;
@@ -2554,9 +2554,10 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) 
       const uint64_t key = keys[h][p];
       if (key == 0ull) continue;  // an anchor
       const double v = __longlong_as_double((long long)(key - 1ull));
-      const double e = v * (double)(rel[h] + (side ? 0.f : errs[h][p])) + 1e-300;
-      if ((key >> sh) >= prefix) in_lo = max(in_lo, ~f64_order(v - e));
-      else out_hi = max(out_hi, f64_order(v + e));
+      const double e = v * (double)rel[h] + (side ? 0.0 : errs[h][p]) + 1e-300;
+      const bool known = v + e < (double)INFINITY;  // (an error without a bound, or a NaN, leaves the ranking open)
+      if ((key >> sh) >= prefix) in_lo = max(in_lo, known ? ~f64_order(v - e) : ~(uint64_t)0);
+      else out_hi = max(out_hi, known ? f64_order(v + e) : ~(uint64_t)0);
     }
     in_lo = cluster_max(cl, in_lo, &slot[0]);
     out_hi = cluster_max(cl, out_hi, &slot[1]);
