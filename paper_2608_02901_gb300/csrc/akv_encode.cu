@@ -2056,8 +2056,10 @@ __device__ __forceinline__ double pair_f64(float s, float c) { return (double)s 
 __device__ __forceinline__ float alpha_error(const EncUnitWs& w) {
   return 4.f * 0x1p-34f * 0.0885f * __fsqrt_rn(__uint_as_float(w.ctrl[17])) * __fsqrt_rn(__uint_as_float(w.ctrl[18])) + 0x1p-34f;
 }
-// Squared norms that keep every fp32 product of the kernels below inside the range.
-__device__ __forceinline__ bool norm_ok(float n2) { return n2 >= 0x1p-80f && n2 <= 0x1p60f; }
+// Squared norms that keep every fp32 product of the kernels below from overflowing; and a norm from its fp32 square,
+// rounded up by what squares below the fp32 range (2^-149 each) may have lost.
+__device__ __forceinline__ bool norm_ok(float n2) { return n2 <= 0x1p60f; }
+__device__ __forceinline__ float norm_up(float n2) { return __fsqrt_rn(n2 + 0x1p-140f); }
 
 // Logits q_w . K_t / sqrt(D): a thread takes one position and eight rows at a time.
 __global__ void __launch_bounds__(128) enc_obs_logit_f(const EncArgs A) {
@@ -2309,9 +2311,9 @@ __global__ void __launch_bounds__(256) enc_util_f(const EncArgs A) {
   const double v2 = s.red[0][lane][0], ev = s.red[1][lane][0];
   const float rnorm2 = s.red_n[0][lane], vnorm2 = s.red_n[1][lane];
   __syncthreads();
-  const float ea = alpha_error(w), vmax = __fsqrt_rn(__uint_as_float(w.ctrl[19]));
+  const float ea = alpha_error(w), vmax = norm_up(__uint_as_float(w.ctrl[19]));
   const float ey = (0x1p-29f + ea) * vmax;  // |error of y| (256 paired steps of three additions, and alpha's)
-  const float rnorm = __fsqrt_rn(rnorm2), vnorm = __fsqrt_rn(vnorm2);
+  const float rnorm = norm_up(rnorm2), vnorm = norm_up(vnorm2);
   double uk = 0.0, uv = 0.0, ek = 0.0;
   for (int w0 = 0; w0 < A.m_obs; w0 += kUtRows) {
     const int nr = min(kUtRows, A.m_obs - w0);
@@ -2340,8 +2342,8 @@ __global__ void __launch_bounds__(256) enc_util_f(const EncArgs A) {
       }
       if (lane == 0) {
         s.y2[r] = pair_f64(ys, yc);
-        s.qn[r] = __fsqrt_rn(qn);
-        s.yn[r] = __fsqrt_rn(ys);
+        s.qn[r] = norm_up(qn);
+        s.yn[r] = norm_up(ys);
       }
     }
     __syncthreads();
@@ -2381,10 +2383,12 @@ __global__ void __launch_bounds__(256) enc_util_f(const EncArgs A) {
         const double aq = a2 * (dq * dq) * 0.0078125;
         uk = fma(aq, dv, uk);
         uv += a2;
-        // errors of q . r and of dv: paired chains of 128 steps, and y's
-        const float hq = 0x1p-32f * s.qn[r] * rnorm, sum = vnorm + s.yn[r] + ey;
-        const float hv = sum * (0x1p-31f * sum + 2.f * ey);
-        ek = fma(a2, (double)(0.0078125f * (2.f * fabsf((float)dq) + hq) * hq * (fabsf((float)dv) + hv)), fma(aq, (double)hv, ek));
+        // errors of q . r and of dv: paired chains of 128 steps, and y's; products below the fp32 range (2^-149 each)
+        // by their own terms
+        const float hq = __fmaf_rn(0x1p-32f * s.qn[r], rnorm, 0x1p-138f), sum = vnorm + s.yn[r] + ey;
+        const float hv = __fmaf_rn(sum, __fmaf_rn(0x1p-31f, sum, 2.f * ey), 0x1p-136f);
+        const float sq = __fmaf_rn(__fmaf_rn(2.f, fabsf((float)dq), hq), 0.0078125f * hq, 0x1p-148f);  // of (q . r)^2 / D
+        ek = fma(a2, (double)__fmaf_rn(sq, fabsf((float)dv) + hv, 0x1p-148f), fma(aq, (double)hv, ek));
       }
     }
   }
@@ -2408,8 +2412,7 @@ __global__ void __launch_bounds__(256) enc_util_f(const EncArgs A) {
   const double rm = 1.0 / (double)A.m_obs;
   uk *= rm;
   uv *= ev * rm;
-  // fp32 norms outside the safe range (and not exactly 0): no bound
-  const bool bounded = (rnorm2 == 0.f || norm_ok(rnorm2)) && (vnorm2 == 0.f || norm_ok(vnorm2));
+  const bool bounded = norm_ok(rnorm2) && norm_ok(vnorm2);
   w.key0[p] = (uint64_t)__double_as_longlong(uk > 0.0 ? uk : 0.0) + 1ull;
   w.key1[p] = (uint64_t)__double_as_longlong(uv > 0.0 ? uv : 0.0) + 1ull;
   err[p] = bounded ? 1.001 * ek * rm : (double)INFINITY;

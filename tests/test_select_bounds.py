@@ -44,3 +44,13 @@ def test_token_that_takes_all_the_attention(dev, seed):  # noqa: F811
     K[:, :, at] *= np.sqrt(128.0) / np.linalg.norm(K[:, :, at], axis=-1, keepdims=True)
     Q = 3.2 * K[:, :, at:at + 1] + 0.1 * r.standard_normal((1, H, W * G, 128))
     _encode_both(dev, K, V, Q, [S], theta=0.12)
+
+
+@pytest.mark.parametrize("eq,ek", [(-126, -18), (-66, -79)])
+def test_products_below_the_fp32_range(dev, eq, ek):  # noqa: F811
+    """Queries and key residuals whose products, or whose squares, fall below what fp32 holds: the sums of q . r are
+    then off by far more than their relative error."""
+    S, r = 500, np.random.Generator(np.random.PCG64(7))
+    K, V = r.standard_normal((2, 1, H, S, 128))
+    Q = r.standard_normal((1, H, W * G, 128))
+    _encode_both(dev, np.ldexp(K, ek), V, np.ldexp(Q, eq), [S], theta=0.08)
