@@ -2226,8 +2226,9 @@ __global__ void __launch_bounds__(128) enc_obs_y_f(const EncArgs A) {
 }
 
 // Eq. 6 utilities of 32 positions: key0 = bits(u^K) + 1, key1 = bits(u^V) + 1, anchors 0, and the error of u^K (fp64,
-// over perm and at; absolute, since |V - y|^2 may come out at or below 0 where V is close to y; infinite: no bound).  Thread (position, group g of eight): rows g and g + 8 of every sixteen.  With r the
-// key residual as an exact pair, u^K sums alpha^2 (q . r)^2 / D (|V|^2 - 2 V . y + |y|^2).
+// over perm and at; absolute, since |V - y|^2 may come out at or below 0 where V is close to y; infinite: no bound for
+// either utility).  Thread (position, group g of eight): rows g and g + 8 of every sixteen.  With r the key residual as
+// an exact pair, u^K sums alpha^2 (q . r)^2 / D (|V|^2 - 2 V . y + |y|^2).
 constexpr int kUtPos = 32, kUtRows = 16;
 struct UtilSmem {
   float rh[128][kUtPos], rl[128][kUtPos], v[128][kUtPos];  // residual pairs and values, by dimension
@@ -2302,7 +2303,12 @@ __global__ void __launch_bounds__(256) enc_util_f(const EncArgs A) {
     if (sub == 0) {  // handed to the position's threads below through the sums' places
       s.red[0][lp][0] = pair_f64(vs, vc);
       s.red[1][lp][0] = pair_f64(es, ec);
-      s.red_n[0][lp] = rn;
+      // u^V has no bound but that of its factors: the value residual's energy has to be exactly 0 or inside the fp32
+      // range, or the norm that goes with it is handed on as infinite
+      const bool ev_ok = (es >= 0x1p-100f && es <= 0x1p100f) ||
+                         (es == 0.f && (!in || exactly_zero_residual(reinterpret_cast<const uint4*>(A.V + ((size_t)u * A.s_max + pl) * 128),
+                                                                     AV + (size_t)av * 16, av, gv)));
+      s.red_n[0][lp] = ev_ok ? rn : INFINITY;
       s.red_n[1][lp] = vn;
     }
   }
@@ -2557,7 +2563,7 @@ __global__ void __cluster_dims__(kSelCtas, 1, 1) __launch_bounds__(kSelThreads) 
       const uint64_t key = keys[h][p];
       if (key == 0ull) continue;  // an anchor
       const double v = __longlong_as_double((long long)(key - 1ull));
-      const double e = v * (double)rel[h] + (side ? 0.0 : errs[h][p]) + 1e-300;
+      const double ek = errs[h][p], e = v * (double)rel[h] + (side == 0 || !(ek < (double)INFINITY) ? ek : 0.0) + 1e-300;
       const bool known = v + e < (double)INFINITY;  // (an error without a bound, or a NaN, leaves the ranking open)
       if ((key >> sh) >= prefix) in_lo = max(in_lo, known ? ~f64_order(v - e) : ~(uint64_t)0);
       else out_hi = max(out_hi, known ? f64_order(v + e) : ~(uint64_t)0);

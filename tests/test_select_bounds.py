@@ -54,3 +54,14 @@ def test_products_below_the_fp32_range(dev, eq, ek):  # noqa: F811
     K, V = r.standard_normal((2, 1, H, S, 128))
     Q = r.standard_normal((1, H, W * G, 128))
     _encode_both(dev, np.ldexp(K, ek), V, np.ldexp(Q, eq), [S], theta=0.08)
+
+
+@pytest.mark.parametrize("e", [-73, -74])
+def test_value_residuals_below_the_fp32_range(dev, e):  # noqa: F811
+    """Values of ordinary norm that differ from their anchors by amounts whose squares fp32 does not hold."""
+    S, r = 500, np.random.Generator(np.random.PCG64(8))
+    K, V = r.standard_normal((2, 1, H, S, 128))
+    V = np.ldexp(V, e)
+    V[..., 0] = 4.0
+    Q = 1e-3 * r.standard_normal((1, H, W * G, 128))
+    _encode_both(dev, K, V, Q, [S], theta=0.08)
