@@ -1961,6 +1961,9 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
               residual(g16, *reinterpret_cast<const uint2*>(tv.at(P.arena, woff + 512u * (uint32_t)g16)));
           }
         }
+        // (the key terms were written over the tile's bytes: ordered before the copy that takes their place, which goes
+        // through the asynchronous proxy)
+        if constexpr (!ROPE) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_empty(lt % NSG));  // this warp is done with the tile
         if (!ahead) key_phase(lt + 1, false);
