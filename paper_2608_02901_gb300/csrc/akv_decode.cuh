@@ -138,8 +138,10 @@ struct __align__(16) Meta {  // a staged tile: as it was copied, then its shape 
   uint32_t ring_off, blk_off, staged, lo, nrows, j, bytes, pad;
   uint32_t sm_v, cd_k, cd_v, sm_k;  // byte offsets of scales and codes in the block
   int n, nKs, nVs;                  // tokens; key records with terms, value records on tensor cores
-  uint32_t fast;                    // every record and anchor-value row staged: the token path without rare cases; bit 1: value records staged
+  uint32_t fast;                    // every record and anchor-value row staged: the token path without rare cases; bit 1: value records staged;
+                                    // kNoShape: the wait for the tile ran out, the shape is another tile's
 };
+constexpr uint32_t kNoShape = 4u;
 struct Seg {  // a CTA's tiles of one unit
   int u, jb, je, ib;  // unit, its tiles [jb, je), CTA-local index of tile jb
   long long t0;       // global index of the unit's tile 0
@@ -1531,7 +1533,9 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
             }
           }
         }
-        const bool go = wait_or_fail(bar_kdone(b), (uint32_t)(lt >> 1) & 1u) && wait_or_fail(bar_full(lt % NSG), (uint32_t)(lt / NSG) & 1u);
+        // (its shape comes with the key terms; without one, a tile that lands late after all is left alone)
+        const bool go = wait_or_fail(bar_kdone(b), (uint32_t)(lt >> 1) & 1u) && wait_or_fail(bar_full(lt % NSG), (uint32_t)(lt / NSG) & 1u) &&
+                        !(meta[lt % NSG].fast & kNoShape);
         if (go) {
           const Meta mt = meta[lt % NSG];
           const uint8_t* st = ring + mt.ring_off;
@@ -1807,6 +1811,8 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
               }
             }
           }
+        } else if (wi8 == 0 && lane == 0) {
+          meta[t % NSG].fast = kNoShape;
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_kdone(b));
@@ -1822,8 +1828,9 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
           key_phase(lt + 1, true);
           ahead = true;
         }
-        const bool go = wait_or_fail(bar_tdone(b), (uint32_t)(lt >> 1) & 1u);
+        const bool waited = wait_or_fail(bar_tdone(b), (uint32_t)(lt >> 1) & 1u);
         const Meta mt = meta[lt % NSG];
+        const bool go = waited && !(mt.fast & kNoShape);
         const uint8_t* st = ring + mt.ring_off;
         float* W = reinterpret_cast<float*>(smem + P.o_wb) + (lt % 3) * (P.X + kEnds) * GS;
         float* pv = reinterpret_cast<float*>(smem + P.o_pv) + b * P.R * GS;
