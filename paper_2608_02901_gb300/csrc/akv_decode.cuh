@@ -2110,14 +2110,14 @@ double mean_density(const Layout& L) {
   return n / t;
 }
 
-// Value records per tile with p rows at least: 1.35x the densest unit's mean plus slack, at most 320; records of a
+// Value records per tile with p rows at least: 1.35x the densest unit's mean plus slack; records of a
 // denser tile beyond the plan's count take the CUDA-core paths, which cost far more.  An encoder's tiles
 // are uneven (tokens of a cluster lie together and their residuals are alike), so a plan takes as many
 // more as shared memory has room for: a 32K layer of 656 anchors whose densest tile held more than 1.35x the mean
 // plus slack took 42 us with that count and 19 us with all its records staged.
 int full_r(const Layout& L) {
   const int R = (int)(T * max_density(L) * 1.35) + 32;
-  return std::min(320, std::max(16, (R + 15) & ~15));
+  return std::max(16, (R + 15) & ~15);
 }
 // Anchor-value rows staged per tile: 2x the mean number of value slots a tile covers plus
 // slack, at most 256; runs on slots beyond these take a CUDA-core path.
@@ -2125,6 +2125,8 @@ int full_x(const Layout& L) {
   const int X = (int)(2.0 * (T * max_anchor_density(L) + 1.0)) + 16;
   return std::min(256, std::max(16, (X + 15) & ~15));
 }
+// bytes of a full tile's block with r records per side, at most
+long long block_bytes_at_most(int r) { return (long long)F_MAX + 2 * round16(4u * (uint32_t)r) + 64LL * r; }
 
 struct Plan {
   DecodeParams P;
@@ -2132,8 +2134,9 @@ struct Plan {
   int grid = 0;
 };
 
-// Shared-memory carve-up for X anchor-value rows, the table in shared memory or not, a ring of at least
-// `ring_min` bytes, and as many p rows as fit beside it, at least Rmin; false if they don't.
+// Shared-memory carve-up for X anchor-value rows, the table in shared memory or not, a ring of at
+// least `ring_min` bytes that holds a block of Rmin records per side beside its anchor-value rows, and as many p rows as fit
+// beside it, at least Rmin; false if they don't.
 bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, bool smem_sa, int smem_optin, long long ring_min, Plan* out) {
   DecodeParams& P = out->P;
   P.X = X;
@@ -2168,9 +2171,8 @@ bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, bool smem_sa, int sm
   P.ring_bytes = (int)(((long long)smem_optin - (long long)off - kRingSlack) & ~127LL);
   // staged bytes of a tile block at most: all of one with R records per side, as far as the ring holds it
   // beside its anchor-value rows
-  P.cap = (int)std::min<long long>((long long)(F_MAX + 2 * round16(4u * (uint32_t)P.R) + 64u * (uint32_t)P.R),
-                                   (P.ring_bytes - 256LL * X) & ~15LL);
-  if (P.cap < (int)F_MAX) return false;
+  P.cap = (int)std::min<long long>(block_bytes_at_most(P.R), (P.ring_bytes - 256LL * X) & ~15LL);
+  if (P.cap < block_bytes_at_most(Rmin)) return false;
   out->smem = (size_t)P.o_ring + (size_t)P.ring_bytes + kRingSlack;
   return true;
 }
@@ -2178,23 +2180,29 @@ bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, bool smem_sa, int sm
 // Preference: the anchor-score table in shared memory (the token gathers' fast path), with a ring of five mean tiles
 // (one in each role, two landing, and what wrapping around leaves unused) and p rows for tiles half again as dense as
 // the R they need, then less, the least p rows and anchor-value rows trimmed towards 3/4 of their values with it; then
-// the table in global memory (gathers through L1 and L2) the same way; then anything that holds one tile.  4 requests
+// the table in global memory (gathers through L1 and L2) the same way; then a ring of one such tile with ever fewer
+// anchor-value rows staged; then anything that holds one tile.  4 requests
 // of 131072, 8B shape, us per call with rings of 4.5, 3.5, 2.5 mean tiles alone and with these: 2 % anchors and 20 %
 // residuals 115.3 -> 114.5, 4 % and 10 % 107.1 -> 105.4, 4 % and 20 % 135.1 -> 126.9; six ragged requests with 20 %
-// residuals 80.0 -> 77.4.
+// residuals 80.0 -> 77.4.  Every choice but the last keeps the records of a mean tile, and some more, on the tensor-core paths
+// (16 units of 60000 tokens, 2 % anchors and 35, 50, 90 % residuals, G = 8: 52, 64, 95 us; with p rows for 320 records at
+// most 10283, 8568, 39697; 12 % and 10 %, G = 4, where the ring was too short for a mean tile's records: 533 -> 52).
 // table false: no anchor-score table is read (RoPE at decode), so none is placed in shared memory.
 bool make_plan(const Layout& L, int GS, int smem_optin, bool table, Plan* out, std::string* why) {
   const int R0 = full_r(L), X0 = full_x(L);
-  const int Rmin = std::max(16, ((R0 * 3 / 4) + 15) & ~15), Xmin = std::max(16, ((X0 * 3 / 4) + 15) & ~15);
+  const int Rmin = std::min(T, std::max(16, ((R0 * 3 / 4) + 15) & ~15)), Xmin = std::max(16, ((X0 * 3 / 4) + 15) & ~15);
   const double mean = (double)F_MAX + T * mean_density(L) * 72.0 + 256.0 + 256.0 * (T * max_anchor_density(L) + 2.0);
   for (int sa = table ? 1 : 0; sa >= 0; --sa)
     for (const double tiles : {5.0, 4.5, 4.0, 3.5, 3.0, 2.5, 2.0, 1.5}) {
       const bool trim = tiles < 4.0;
+      const int R = trim ? Rmin : std::min(T, tiles > 4.5 ? R0 * 3 / 2 : R0);
       for (int X = X0; X >= (trim ? Xmin : X0); X -= 16)
-        if (make_plan_rx(L, GS, trim ? Rmin : (tiles > 4.5 ? R0 * 3 / 2 : R0), X, sa == 1, smem_optin, (long long)(tiles * mean), out)) return true;
+        if (make_plan_rx(L, GS, R, X, sa == 1, smem_optin, (long long)(tiles * mean), out)) return true;
     }
   for (int X = X0; X >= 16; X -= 16)
-    if (make_plan_rx(L, GS, 16, X, false, smem_optin, (long long)F_MAX + 2 * 16 * 36 + 256LL * X, out)) return true;
+    if (make_plan_rx(L, GS, Rmin, X, false, smem_optin, block_bytes_at_most(Rmin) + 256LL * X, out)) return true;
+  for (int X = X0; X >= 16; X -= 16)
+    if (make_plan_rx(L, GS, 16, X, false, smem_optin, block_bytes_at_most(16) + 256LL * X, out)) return true;
   *why = "shared memory: no room for the decode pipeline";
   return false;
 }

@@ -132,3 +132,43 @@ def test_lloyd_max_record_groups(dev, G, nv):  # noqa: F811
         d["min_k"] = d["min_k"] * 0
         d["min_v"] = d["min_v"] * 0
     _run_seeded(dev, p, [S], mutate=mutate)
+
+
+@pytest.mark.parametrize("G", [1, 4, 8])
+@pytest.mark.parametrize("fa,fr", [(0.12, 0.1), (0.1, 0.4), (0.02, 0.35), (0.02, 0.5), (0.02, 0.95)])
+@pytest.mark.parametrize("rope", [False, True])
+def test_plans_at_large_shares(dev, G, fa, fr, rope):  # noqa: F811
+    """Records up to one per token; lengths that end tiles early, a range that crosses units."""
+    p = akv.Params(batch=2, n_kv_heads=2, n_q_heads=2 * G, anchor_frac=fa, res_frac_k=fr, res_frac_v=fr, seed=11, rope=rope,
+                   rope_theta=10000.0)
+    _run_seeded(dev, p, [9001, 3333], sm_scale=0.2)
+
+
+@pytest.mark.parametrize("G", [2, 8])
+def test_time_at_large_shares(dev, G):  # noqa: F811
+    """No cliff: a call with many records takes a few times what one at 20 % anchors takes, as its bytes do (at most 2.3
+    times as many), not a hundred times (tiles off the tensor-core paths)."""
+    import torch
+    from helpers import seeded_units
+
+    def us(fa, fr):
+        p = akv.Params(batch=1, n_kv_heads=8, n_q_heads=8 * G, anchor_frac=fa, res_frac_k=fr, res_frac_v=fr, seed=12)
+        lens = [20000]
+        units = [akv.unit_host_from_logical(u) for u in seeded_units(p, lens)]
+        arena = torch.from_numpy(akv.akv_cache_pack_host(p, lens, units)).to(dev)
+        q = torch.randn((1, 8 * G, 128), device=dev).to(torch.bfloat16)
+        out, ws = torch.empty_like(q), torch.empty(akv.akv_decode_workspace_size(p, lens), dtype=torch.uint8, device=dev)
+        best = 1e9
+        for _ in range(4):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(5):
+                akv.akv_decode_attn(p, lens, arena, q, out, ws=ws)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) / 5 * 1e3)
+        return best
+
+    base = us(0.2, 0.1)
+    for fa, fr in ((0.12, 0.1), (0.02, 0.35), (0.02, 0.5)):
+        assert us(fa, fr) < 8 * base, (fa, fr)
