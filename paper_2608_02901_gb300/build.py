@@ -21,6 +21,10 @@ SOURCES = {
     "akv_decode_g2.cu": [],
     "akv_decode_g4.cu": [],
     "akv_decode_g8.cu": [],
+    "akv_decode_g1w.cu": [],  # with more weight rows than staged rows
+    "akv_decode_g2w.cu": [],
+    "akv_decode_g4w.cu": [],
+    "akv_decode_g8w.cu": [],
     "akv_encode.cu": ["--fmad=false"],  # fp64 decisions: no contraction
 }
 

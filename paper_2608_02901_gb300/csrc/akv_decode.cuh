@@ -77,6 +77,12 @@
 #include "akv_internal.h"
 
 namespace akv {
+
+// The decode kernels with more weight rows than staged anchor-value rows, the table in global memory: in translation units
+// of their own, so that they compile beside the others.
+template <int GS>
+const void* wide_decode_kernel(int codec, int rope);
+
 namespace {
 
 constexpr int NTW = 8;              // token warps
@@ -135,10 +141,11 @@ struct RopeParams {
 };
 
 struct __align__(16) Meta {  // a staged tile: as it was copied, then its shape (product warp 0, before the key terms are announced)
-  uint32_t ring_off, blk_off, staged, lo, nrows, j, bytes, pad;
+  uint32_t ring_off, blk_off, staged, lo, nrows, j, bytes;  // nrows: anchor-value rows staged
+  uint32_t nw;                      // WIDE: value slots with a weight row
   uint32_t sm_v, cd_k, cd_v, sm_k;  // byte offsets of scales and codes in the block
   int n, nKs, nVs;                  // tokens; key records with terms, value records on tensor cores
-  uint32_t fast;                    // every record and anchor-value row staged: the token path without rare cases; bit 1: value records staged;
+  uint32_t fast;                    // every record staged, every slot has a weight row: the token path without rare cases; bit 1: value records staged;
                                     // kNoShape: the wait for the tile ran out, the shape is another tile's
 };
 constexpr uint32_t kNoShape = 4u;
@@ -173,7 +180,7 @@ struct DecodeParams {
   float scale_log2;
   unsigned long long sign_lo, sign_hi;
   int R;           // value records per tile handled on tensor cores (their p rows); sizes the staging cap
-  int X;           // anchor-value rows per tile that are staged (the weight table's rows)
+  int X;           // anchor-value rows per tile that are staged, and the weight table's rows (WIDE: XW)
   int cap;         // staged bytes of a tile block at most
   int ring_bytes, drop_last, smem_sa;
   int o_bar, o_meta, o_misc, o_sa, o_ovf, o_qp, o_rows, o_gsum, o_wb, o_vs, o_pv, o_ovl, o_prod, o_ring;
@@ -184,6 +191,7 @@ struct DecodeParams {
   int suf_cap, n_sch;
   int cta_unit[kMaxGrid];  // first unit of each CTA's range
   int cta_tile[kMaxGrid];  // its first tile inside that unit
+  int XW;                  // WIDE: the weight table's rows, more than X (else X)
 };
 
 // ---- device helpers ---------------------------------------------------------------
@@ -442,7 +450,7 @@ __device__ __noinline__ void value_record_add(const uint8_t* st, const uint8_t* 
   }
 }
 // acc[g] x the anchor's value row (global memory, swizzled by the slot), added into ov[g][:]:
-// a run whose value slot lies beyond the tile's staged anchor-value rows (rare).
+// a run whose value slot lies beyond the tile's weight rows (rare).
 template <int GS>
 __device__ __noinline__ void anchor_value_add(const uint8_t* AV, int anchor, const float* acc, float* ov) {
   const uint8_t* row = AV + (size_t)anchor * 256;
@@ -1107,17 +1115,17 @@ struct TokTile {
   const float* rows;  // [0,8): -m, [8,16): -inf, [16,24): sum q'
   const float* qp;    // [GS][128] rotated query
   float* pv;          // [R][GS] p rows of the value records
-  float* W;           // [X][GS] the tile's value weights
+  float* W;           // [nrows][GS] the tile's value weights
   float* ovf;         // [2][GS][128] overflow sums
   const uint8_t* AV;  // the unit's anchor values (global)
   const float* lgt;   // RoPE at decode: the tile's logit rows [T][GS] (global), else null
   int* ovl_n;         // the tile's overflow lists: value records beyond the staged ones, and runs
-  float* ovl;         // beyond the staged anchor-value rows, applied by the whole group after the tokens
+  float* ovl;         // beyond the weight rows, applied by the whole group after the tokens
   int k, nKs, nVs, ka, lloyd;
 };
 
-// The general token path (kept out of line: a tile with records beyond the staged ones, runs
-// beyond the staged anchor-value rows, or a lane past the tile's end): the same arithmetic as
+// The general token path (kept out of line: a tile with records beyond the staged ones, or runs
+// beyond its weight rows): the same arithmetic as
 // the fast path, with the rare cases on CUDA cores; it returns the lane's share of the
 // normaliser (a shared-memory sum would take every lane's addition on the same words).  The
 // arguments arrive by value and are copied into locals first: the shared-memory reductions below clobber memory, so a field read
@@ -1171,7 +1179,7 @@ __device__ __noinline__ LShare<(GS >= 2 ? GS / 2 : 1)> token_chunk_general(const
       float* w = W + ix * GS;
 #pragma unroll
       for (int g = 0; g < GS; ++g) red_local(w + g, vv[g]);
-    } else {  // beyond the staged anchor-value rows: listed for the group (else on CUDA cores here)
+    } else {  // beyond the weight rows: listed for the group (else on CUDA cores here)
       const int e = atomicAdd(ovl_n + 1, 1);
       if (e < kOvl) {
         float* en = ovl + (kOvl + e) * 9;
@@ -1261,6 +1269,43 @@ __device__ __noinline__ LShare<(GS >= 2 ? GS / 2 : 1)> token_chunk_general(const
   return ls;
 }
 
+// w^T V_A over the value slots of a tile that have a weight row but no staged anchor-value row (slots nr .. nw - 1, and those
+// among the token warps' first and last runs), their rows read from global memory, on CUDA cores, added into the overflow's
+// sums ov[g][:]: product thread t takes dimension t % 128 of every other slot.  A tile has such slots where a unit's
+// anchors are more than one token in five or so, and staging all their rows would leave the ring no room.
+// W: the weights; ends: the runs' weights as the operand built from them; vs: their slots; AV: slot 0's row.
+template <int GS>
+__device__ __forceinline__ void unstaged_rows(const float* W, const uint32_t* ends, const int* vs, const uint8_t* AV, uint32_t lo, int nr, int nw,
+                                          int t, float* ov) {
+  const int dim = t & 127;
+  float av[GS];
+#pragma unroll
+  for (int g = 0; g < GS; ++g) av[g] = 0.f;
+  auto value = [&](int slot) {  // (rows are stored swizzled by the slot)
+    return __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(AV + (size_t)slot * 256 + 16 * ((uint32_t)(dim >> 3) ^ ((lo + (uint32_t)slot) & 7u)) + 2 * (dim & 7)));
+  };
+#pragma unroll 4
+  for (int slot = nr + (t >> 7); slot < nw; slot += 2) {
+    float w[GS];
+    load_row<GS>(W + slot * GS, w);
+    const float x = value(slot);
+#pragma unroll
+    for (int g = 0; g < GS; ++g) av[g] = fmaf(w[g], x, av[g]);
+  }
+  for (int e = t >> 7; e < kEnds; e += 2) {
+    if (vs[e] < nr) continue;
+    const float x = value(vs[e]);
+#pragma unroll
+    for (int g = 0; g < GS; ++g) {  // head g's place e of the operand: bf16 high and low parts
+      const uint32_t* f = ends + 4 * (4 * g + (e & 7) / 2) + 2 * (e >> 3);
+      const int sh = 16 * (e & 1);
+      av[g] = fmaf(__uint_as_float((f[0] >> sh) << 16) + __uint_as_float((f[1] >> sh) << 16), x, av[g]);
+    }
+  }
+#pragma unroll
+  for (int g = 0; g < GS; ++g) red_local(ov + g * 128 + dim, av[g]);
+}
+
 // ================================ decode ============================================
 // CODEC: 0 = uniform codes (c^ = min + c scale), 1 = Lloyd-Max levels (c^ = scale L[c]).
 // MODE: where a unit's anchor scores are.  kTableSmem: copied from the score launch into shared memory;
@@ -1268,7 +1313,9 @@ __device__ __noinline__ LShare<(GS >= 2 ? GS / 2 : 1)> token_chunk_general(const
 // token's logit comes from the RoPE logits launch (P.lg) instead of gamma S_A plus its key-residual
 // term, and the key-residual phase has nothing to do.
 enum Mode { kTableSmem = 0, kTableGlobal = 1, kRope = 2 };
-template <int GS, int CODEC, int MODE>
+// WIDE: tiles may cover more value slots than have their anchor-value rows staged (P.XW > P.X); kernels of their own,
+// since the same code as a branch, inline or called, made the others slower (8 x 131072, G = 8: 164 -> 178, 193 us).
+template <int GS, int CODEC, int MODE, bool WIDE = false>
 __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P) {
   extern __shared__ __align__(128) uint8_t smem[];
   constexpr int NP = GS >= 2 ? GS / 2 : 1;      // pairs of heads for the packed arithmetic
@@ -1416,6 +1463,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
       mt.nrows = nrows;
       mt.j = (uint32_t)(pr->s.jb + (ii - pr->s.ib));
       mt.bytes = sz;
+      if constexpr (WIDE) mt.nw = min(hi - lo + 1u, (uint32_t)P.XW);
       // (drop_last: a test withholds the last tile of the range)
       if (P.drop_last > 0 && ii == n_cta_tiles - P.drop_last) {
         mt.nrows |= 0x80000000u;  // withheld: nothing in flight
@@ -1541,7 +1589,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
           const uint8_t* st = ring + mt.ring_off;
           const TileView tv = tile_view(st, mt, u);
           const bool fast_tile = mt.fast & 1u;
-          float* W = reinterpret_cast<float*>(smem + P.o_wb) + (lt % 3) * (P.X + kEnds) * GS;
+          float* W = reinterpret_cast<float*>(smem + P.o_wb) + (lt % 3) * ((WIDE ? P.XW : P.X) + kEnds) * GS;
           int* vs = reinterpret_cast<int*>(smem + P.o_vs) + (lt % 3) * kEnds;
           float* pv = reinterpret_cast<float*>(smem + P.o_pv) + b * P.R * GS;
           // ---- tokens: lane -> stored tokens t0 .. t0 + 3, every head ----
@@ -1559,7 +1607,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
             tl.rv = tv.rk(1, wi) + __popcll(wv & ((1ull << sh) - 1ull));
           }
           if (fast_tile) {  // warp-uniform
-            // Every record staged, every run on a staged anchor-value row.  No shared atomics: a run
+            // Every record staged, every run with a weight row.  No shared atomics: a run
             // that starts and ends inside a lane's tokens is stored as it is (no other lane has its
             // slot); runs that cross lanes are merged by a segmented scan.  Places past the end of a unit's
             // last tile join its last run with weight 0.
@@ -1675,7 +1723,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
             // the warp's first run may continue the previous warp's last one and its last run go on in the
             // next: both get rows of their own past the slots' (a shared-memory float addition is a
             // compare-and-swap loop, and would meet the neighbour's)
-            float* w_ends = W + (P.X + 2 * wi8) * GS;
+            float* w_ends = W + ((WIDE ? P.XW : P.X) + 2 * wi8) * GS;
             if (multi && !(lane > 0 && ptk == hk)) {
               if (lane == 0) vs[2 * wi8] = (int)(hk - lo);
               store_row<GS>(lane == 0 ? w_ends : W + (int)(hk - lo) * GS, hs);
@@ -1706,7 +1754,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
             int* ovl_n = reinterpret_cast<int*>(smem + P.o_ovl + b * kOvlBytes);
             float* ovl = reinterpret_cast<float*>(ovl_n + 4);
             const auto ls = token_chunk_general<GS>(
-                TokTile{tv, tv.gb(P.arena), mt.lo, mt.nrows, SAt, rows, qp, pv, W, ovf, P.arena + unit_desc(P.arena, u)->off_anchor_v,
+                TokTile{tv, tv.gb(P.arena), mt.lo, WIDE ? mt.nw : mt.nrows, SAt, rows, qp, pv, W, ovf, P.arena + unit_desc(P.arena, u)->off_anchor_v,
                         ROPE ? P.lg + ((size_t)u * P.s_stride + (size_t)mt.j * T) * GS : nullptr, ovl_n, ovl, k, mt.nKs, mt.nVs, P.ka_stride,
                         CODEC}, tl);
 #pragma unroll
@@ -1749,7 +1797,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
           if (wi8 == 0 && lane == 0) {
             const int nVs = min(tv.nv, P.R);
             const bool fast = (ROPE || nKs == tv.nk) && nVs == tv.nv &&
-                              (int)(((reinterpret_cast<const uint32_t*>(st + 4 * tv.n64))[tv.n - 1] & 0xFFFFu) - mt.lo) < (int)mt.nrows;
+                              (int)(((reinterpret_cast<const uint32_t*>(st + 4 * tv.n64))[tv.n - 1] & 0xFFFFu) - mt.lo) < (int)(WIDE ? mt.nw : mt.nrows);
             Meta& w = meta[t % NSG];
             w.sm_v = tv.sm_v;
             w.cd_k = tv.cd_k;
@@ -1760,8 +1808,8 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
             w.nVs = nVs;
             w.fast = (fast ? 1u : 0u) | (tv.cd_v + 512u * (uint32_t)((nVs + 15) / 16) <= tv.staged ? 2u : 0u);
           }
-          float* W = reinterpret_cast<float*>(smem + P.o_wb) + (t % 3) * (P.X + kEnds) * GS;
-          for (int e = 4 * mt_; e < (P.X + kEnds) * GS; e += 4 * NMW * 32) *reinterpret_cast<float4*>(W + e) = make_float4(0.f, 0.f, 0.f, 0.f);
+          float* W = reinterpret_cast<float*>(smem + P.o_wb) + (t % 3) * ((WIDE ? P.XW : P.X) + kEnds) * GS;
+          for (int e = 4 * mt_; e < ((WIDE ? P.XW : P.X) + kEnds) * GS; e += 4 * NMW * 32) *reinterpret_cast<float4*>(W + e) = make_float4(0.f, 0.f, 0.f, 0.f);
           if (mt_ < kEnds) reinterpret_cast<int*>(smem + P.o_vs)[(t % 3) * kEnds + mt_] = -1;
           if (mt_ < 2) reinterpret_cast<int*>(smem + P.o_ovl + b * kOvlBytes)[mt_] = 0;
           float* rsb = reinterpret_cast<float*>(const_cast<uint8_t*>(st) + tv.cd_k);
@@ -1832,7 +1880,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
         const Meta mt = meta[lt % NSG];
         const bool go = waited && !(mt.fast & kNoShape);
         const uint8_t* st = ring + mt.ring_off;
-        float* W = reinterpret_cast<float*>(smem + P.o_wb) + (lt % 3) * (P.X + kEnds) * GS;
+        float* W = reinterpret_cast<float*>(smem + P.o_wb) + (lt % 3) * ((WIDE ? P.XW : P.X) + kEnds) * GS;
         float* pv = reinterpret_cast<float*>(smem + P.o_pv) + b * P.R * GS;
         const int nVs = mt.nVs, nr = (int)mt.nrows, nb16 = (nr + 15) / 16;
         if (go) {
@@ -1881,7 +1929,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
           for (int x = wi8; x < n_vg + nb16 + 1; x += NMW) {
             const bool val = x < n_vg;
             const int blk = x - n_vg;  // block of slots; the last one: the token warps' first and last runs
-            float* src = val ? pv + 16 * GS * x : (blk < nb16 ? W + 16 * GS * blk : W + P.X * GS);
+            float* src = val ? pv + 16 * GS * x : (blk < nb16 ? W + 16 * GS * blk : W + (WIDE ? P.XW : P.X) * GS);
             const int lim = val ? nVs - 16 * x : (blk < nb16 ? nr - 16 * blk : kEnds);
             const int kk[4] = {2 * c4, 2 * c4 + 1, 2 * c4 + 8, 2 * c4 + 9};
             float f[4];
@@ -1923,7 +1971,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
           for (int blk = 0; blk <= nb16; ++blk) {
             const bool ends = blk == nb16;
             const int ka = (ends ? 0 : 16 * blk) + 2 * c4;
-            const uint4 a = r8 < GS ? *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(ends ? W + P.X * GS : W + 16 * GS * blk) + 16 * lane)
+            const uint4 a = r8 < GS ? *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(ends ? W + (WIDE ? P.XW : P.X) * GS : W + 16 * GS * blk) + 16 * lane)
                                     : make_uint4(0u, 0u, 0u, 0u);
             // rows past the staged slots, or of runs that are not there, hold other bytes: their halves of B are cleared
             uint32_t m0, m1;
@@ -1933,6 +1981,11 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
               m0 = (v0.x >= 0 ? 0xFFFFu : 0u) | (v0.y >= 0 ? 0xFFFF0000u : 0u);
               m1 = (v1.x >= 0 ? 0xFFFFu : 0u) | (v1.y >= 0 ? 0xFFFF0000u : 0u);
               slot = max(vs[(mi & 1) * 8 + ri], 0);
+              if constexpr (WIDE) {  // (those past the staged rows are taken below)
+                m0 &= (v0.x < nr ? 0xFFFFu : 0u) | (v0.y < nr ? 0xFFFF0000u : 0u);
+                m1 &= (v1.x < nr ? 0xFFFFu : 0u) | (v1.y < nr ? 0xFFFF0000u : 0u);
+                slot = min(slot, nr - 1);
+              }
             } else {
               m0 = (ka < nr ? 0xFFFFu : 0u) | (ka + 1 < nr ? 0xFFFF0000u : 0u);
               m1 = (ka + 8 < nr ? 0xFFFFu : 0u) | (ka + 9 < nr ? 0xFFFF0000u : 0u);
@@ -1966,6 +2019,11 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
             const TileView tv = tile_view(st, mt, u);
             for (int g16 = 0; g16 * 16 < nVs; ++g16)
               residual(g16, *reinterpret_cast<const uint2*>(tv.at(P.arena, woff + 512u * (uint32_t)g16)));
+          }
+          if constexpr (WIDE) {
+            if (mt.nw > mt.nrows)
+              unstaged_rows<GS>(W, reinterpret_cast<const uint32_t*>(W + (WIDE ? P.XW : P.X) * GS), vs,
+                                P.arena + unit_desc(P.arena, u)->off_anchor_v + (size_t)mt.lo * 256, mt.lo, nr, (int)mt.nw, mt_, ovf);
           }
         }
         // (the key terms were written over the tile's bytes: ordered before the copy that takes their place, which goes
@@ -2119,12 +2177,14 @@ int full_r(const Layout& L) {
   const int R = (int)(T * max_density(L) * 1.35) + 32;
   return std::max(16, (R + 15) & ~15);
 }
-// Anchor-value rows staged per tile: 2x the mean number of value slots a tile covers plus
-// slack, at most 256; runs on slots beyond these take a CUDA-core path.
-int full_x(const Layout& L) {
+// Weight rows of a tile wanted: 2x the mean number of value slots it covers plus slack; runs on slots beyond a plan's
+// take a CUDA-core path.
+int full_w(const Layout& L) {
   const int X = (int)(2.0 * (T * max_anchor_density(L) + 1.0)) + 16;
-  return std::min(256, std::max(16, (X + 15) & ~15));
+  return std::min(T, std::max(16, (X + 15) & ~15));
 }
+// Anchor-value rows staged per tile: those slots', at most 256; the rest are read from global memory.
+int full_x(const Layout& L) { return std::min(256, full_w(L)); }
 // bytes of a full tile's block with r records per side, at most
 long long block_bytes_at_most(int r) { return (long long)F_MAX + 2 * round16(4u * (uint32_t)r) + 64LL * r; }
 
@@ -2134,12 +2194,13 @@ struct Plan {
   int grid = 0;
 };
 
-// Shared-memory carve-up for X anchor-value rows, the table in shared memory or not, a ring of at
+// Shared-memory carve-up for X staged anchor-value rows of XW weight rows, the table in shared memory or not, a ring of at
 // least `ring_min` bytes that holds a block of Rmin records per side beside its anchor-value rows, and as many p rows as fit
 // beside it, at least Rmin; false if they don't.
-bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, bool smem_sa, int smem_optin, long long ring_min, Plan* out) {
+bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, int XW, bool smem_sa, int smem_optin, long long ring_min, Plan* out) {
   DecodeParams& P = out->P;
   P.X = X;
+  P.XW = XW;
   P.ka_stride = (L.max_k + 3) & ~3;
   P.smem_sa = smem_sa ? 1 : 0;
   size_t off = 0;
@@ -2158,7 +2219,7 @@ bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, bool smem_sa, int sm
   P.o_gsum = take(2 * 8 * 8 * 4);
   // three tiles' weights of their slots and of the warps' first and last runs, and the slots of those; two tiles'
   // p rows (then A operands) and overflow lists
-  P.o_wb = take((size_t)3 * (X + kEnds) * GS * 4);
+  P.o_wb = take((size_t)3 * (XW + kEnds) * GS * 4);
   P.o_vs = take((size_t)3 * kEnds * 4);
   P.o_ovl = take((size_t)2 * kOvlBytes);
   P.o_prod = take(sizeof(Prod));
@@ -2187,35 +2248,41 @@ bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, bool smem_sa, int sm
 // residuals 80.0 -> 77.4.  Every choice but the last keeps the records of a mean tile, and some more, on the tensor-core paths
 // (16 units of 60000 tokens, 2 % anchors and 35, 50, 90 % residuals, G = 8: 52, 64, 95 us; with p rows for 320 records at
 // most 10283, 8568, 39697; 12 % and 10 %, G = 4, where the ring was too short for a mean tile's records: 533 -> 52).
+// Where the slots of tiles near the mean (15 % and 16 over it: fa above 0.2) are more than the rows staged at most, tiles
+// have more weight rows than those, 2x the mean (the WIDE kernels, table in global memory): 16 x 60000 tokens, 25 % anchors,
+// G = 1, 2, 4, 8: 59, 62, 65, 77 us per
+// call; with such tiles on the general token path 97, 147, 241, 428.  30 %: 81, 84, 88, 116 (1809, 3487, 5965, 11632).
 // table false: no anchor-score table is read (RoPE at decode), so none is placed in shared memory.
 bool make_plan(const Layout& L, int GS, int smem_optin, bool table, Plan* out, std::string* why) {
   const int R0 = full_r(L), X0 = full_x(L);
+  const bool wide = 1.15 * (T * max_anchor_density(L) + 1.0) + 16.0 > 256.0;
   const int Rmin = std::min(T, std::max(16, ((R0 * 3 / 4) + 15) & ~15)), Xmin = std::max(16, ((X0 * 3 / 4) + 15) & ~15);
-  const double mean = (double)F_MAX + T * mean_density(L) * 72.0 + 256.0 + 256.0 * (T * max_anchor_density(L) + 2.0);
-  for (int sa = table ? 1 : 0; sa >= 0; --sa)
+  const double rows = std::min(256.0, T * max_anchor_density(L) + 2.0);
+  const double mean = (double)F_MAX + T * mean_density(L) * 72.0 + 256.0 + 256.0 * rows;
+  for (int sa = table && !wide ? 1 : 0; sa >= 0; --sa)
     for (const double tiles : {5.0, 4.5, 4.0, 3.5, 3.0, 2.5, 2.0, 1.5}) {
       const bool trim = tiles < 4.0;
       const int R = trim ? Rmin : std::min(T, tiles > 4.5 ? R0 * 3 / 2 : R0);
       for (int X = X0; X >= (trim ? Xmin : X0); X -= 16)
-        if (make_plan_rx(L, GS, R, X, sa == 1, smem_optin, (long long)(tiles * mean), out)) return true;
+        if (make_plan_rx(L, GS, R, X, wide ? full_w(L) : X, sa == 1, smem_optin, (long long)(tiles * mean), out)) return true;
     }
   for (int X = X0; X >= 16; X -= 16)
-    if (make_plan_rx(L, GS, Rmin, X, false, smem_optin, block_bytes_at_most(Rmin) + 256LL * X, out)) return true;
+    if (make_plan_rx(L, GS, Rmin, X, wide ? full_w(L) : X, false, smem_optin, block_bytes_at_most(Rmin) + 256LL * X, out)) return true;
   for (int X = X0; X >= 16; X -= 16)
-    if (make_plan_rx(L, GS, 16, X, false, smem_optin, block_bytes_at_most(16) + 256LL * X, out)) return true;
+    if (make_plan_rx(L, GS, 16, X, X, false, smem_optin, block_bytes_at_most(16) + 256LL * X, out)) return true;
   *why = "shared memory: no room for the decode pipeline";
   return false;
 }
 
-using DecodeFn = void (*)(const DecodeParams);
 using ScoreFn = void (*)(const ScoreParams);
 using RopeFn = void (*)(const RopeParams);
 template <int GS, int MODE>
-DecodeFn decode_kernel_c(int codec) {
-  return codec ? akv_decode_kernel<GS, 1, MODE> : akv_decode_kernel<GS, 0, MODE>;
+const void* decode_kernel_c(int codec) {
+  return codec ? (const void*)akv_decode_kernel<GS, 1, MODE> : (const void*)akv_decode_kernel<GS, 0, MODE>;
 }
 template <int GS>
-DecodeFn decode_kernel(int codec, int rope, const DecodeParams& P) {
+const void* decode_kernel(int codec, int rope, const DecodeParams& P) {
+  if (P.XW > P.X) return wide_decode_kernel<GS>(codec, rope);
   if (rope) return decode_kernel_c<GS, kRope>(codec);
   return P.smem_sa ? decode_kernel_c<GS, kTableSmem>(codec) : decode_kernel_c<GS, kTableGlobal>(codec);
 }
@@ -2409,7 +2476,8 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   cfg.gridDim = dim3((unsigned)pl.grid, 1, 1);
   cfg.blockDim = dim3(NT, 1, 1);
   cfg.dynamicSmemBytes = pl.smem;
-  e = cudaLaunchKernelEx(&cfg, decode_kernel<GS>(codec, rope, P), P);
+  void* args[] = {&P};
+  e = cudaLaunchKernelExC(&cfg, decode_kernel<GS>(codec, rope, P), args);
   if (e != cudaSuccess) {
     cudaFuncAttributes fa{};
     cudaFuncGetAttributes(&fa, decode_kernel<GS>(codec, rope, P));

@@ -1,0 +1,10 @@
+// The decode kernels for one query head per KV head whose tiles have more weight rows than staged anchor-value rows.
+#include "akv_decode.cuh"
+
+namespace akv {
+template <>
+const void* wide_decode_kernel<1>(int codec, int rope) {
+  if (rope) return codec ? (const void*)akv_decode_kernel<1, 1, kRope, true> : (const void*)akv_decode_kernel<1, 0, kRope, true>;
+  return codec ? (const void*)akv_decode_kernel<1, 1, kTableGlobal, true> : (const void*)akv_decode_kernel<1, 0, kTableGlobal, true>;
+}
+}  // namespace akv

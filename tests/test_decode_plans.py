@@ -135,10 +135,11 @@ def test_lloyd_max_record_groups(dev, G, nv):  # noqa: F811
 
 
 @pytest.mark.parametrize("G", [1, 4, 8])
-@pytest.mark.parametrize("fa,fr", [(0.12, 0.1), (0.1, 0.4), (0.02, 0.35), (0.02, 0.5), (0.02, 0.95)])
+@pytest.mark.parametrize("fa,fr", [(0.12, 0.1), (0.1, 0.4), (0.33, 0.1), (0.6, 0.3), (1.0, 0.0), (0.02, 0.35), (0.02, 0.5), (0.02, 0.95)])
 @pytest.mark.parametrize("rope", [False, True])
 def test_plans_at_large_shares(dev, G, fa, fr, rope):  # noqa: F811
-    """Records up to one per token; lengths that end tiles early, a range that crosses units."""
+    """Tiles that cover more value slots than have their anchor-value rows staged, up to one per token, and records up to
+    one per token; lengths that end tiles early, a range that crosses units."""
     p = akv.Params(batch=2, n_kv_heads=2, n_q_heads=2 * G, anchor_frac=fa, res_frac_k=fr, res_frac_v=fr, seed=11, rope=rope,
                    rope_theta=10000.0)
     _run_seeded(dev, p, [9001, 3333], sm_scale=0.2)
@@ -146,8 +147,8 @@ def test_plans_at_large_shares(dev, G, fa, fr, rope):  # noqa: F811
 
 @pytest.mark.parametrize("G", [2, 8])
 def test_time_at_large_shares(dev, G):  # noqa: F811
-    """No cliff: a call with many records takes a few times what one at 20 % anchors takes, as its bytes do (at most 2.3
-    times as many), not a hundred times (tiles off the tensor-core paths)."""
+    """No cliff: a call with many anchors or many records takes a few times what one at 20 % anchors takes, as its bytes
+    do (at most 2.3 times as many), not a hundred times (tiles off the tensor-core paths)."""
     import torch
     from helpers import seeded_units
 
@@ -170,5 +171,5 @@ def test_time_at_large_shares(dev, G):  # noqa: F811
         return best
 
     base = us(0.2, 0.1)
-    for fa, fr in ((0.12, 0.1), (0.02, 0.35), (0.02, 0.5)):
+    for fa, fr in ((0.12, 0.1), (0.25, 0.0), (0.3, 0.1), (0.5, 0.0), (0.02, 0.35), (0.02, 0.5)):
         assert us(fa, fr) < 8 * base, (fa, fr)
