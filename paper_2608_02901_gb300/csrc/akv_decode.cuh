@@ -182,7 +182,7 @@ struct DecodeParams {
   int R;           // value records per tile handled on tensor cores (their p rows); sizes the staging cap
   int X;           // anchor-value rows per tile that are staged, and the weight table's rows (WIDE: XW)
   int cap;         // staged bytes of a tile block at most
-  int ring_bytes, drop_last, smem_sa;
+  int ring_bytes, drop_last, smem_sa;  // smem_sa: score table in shared memory (1), half of it (2)
   int o_bar, o_meta, o_misc, o_sa, o_ovf, o_qp, o_rows, o_gsum, o_wb, o_vs, o_pv, o_ovl, o_prod, o_ring;
   const float* lg;         // RoPE at decode: logits [units][s_stride][G] in stored order (else null)
   int s_stride;
@@ -1309,10 +1309,11 @@ __device__ __forceinline__ void unstaged_rows(const float* W, const uint32_t* en
 // ================================ decode ============================================
 // CODEC: 0 = uniform codes (c^ = min + c scale), 1 = Lloyd-Max levels (c^ = scale L[c]).
 // MODE: where a unit's anchor scores are.  kTableSmem: copied from the score launch into shared memory;
-// kTableGlobal: read from global memory where the score launch left them; kRope: pre-RoPE keys, every
+// kTableGlobal: read from global memory where the score launch left them; kTableHalf (GS = 8): heads 0-3 in shared, heads 4-7
+// in global memory; kRope: pre-RoPE keys, every
 // token's logit comes from the RoPE logits launch (P.lg) instead of gamma S_A plus its key-residual
 // term, and the key-residual phase has nothing to do.
-enum Mode { kTableSmem = 0, kTableGlobal = 1, kRope = 2 };
+enum Mode { kTableSmem = 0, kTableGlobal = 1, kRope = 2, kTableHalf = 3 };
 // WIDE: tiles may cover more value slots than have their anchor-value rows staged (P.XW > P.X); kernels of their own,
 // since the same code as a branch, inline or called, made the others slower (8 x 131072, G = 8: 164 -> 178, 193 us).
 template <int GS, int CODEC, int MODE, bool WIDE = false>
@@ -1383,7 +1384,10 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
     } else {
       mbar_arrive(bar_hdr);
     }
-    if (MODE == kTableSmem && ok) {
+    if (MODE == kTableHalf && ok) {
+      mbar_expect_tx(bar_sa_full, 16u * (uint32_t)k);
+      bulk_g2s(smem_u32(SAs), P.sa + (size_t)u * P.ka_stride * GS, 16u * (uint32_t)k, bar_sa_full);
+    } else if (MODE == kTableSmem && ok) {
       const float* src = P.sa + (size_t)u * P.ka_stride * GS;
       if (GS == 8) {  // the two four-head arrays, k rows of each
         const uint32_t half = 16u * (uint32_t)k;
@@ -1649,7 +1653,13 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
                 } else {
                   const int a = min((int)(ek[e] & 0xFFFFu), km1);  // indices are < k by construction
                   float sa[GS];
-                  load_sa_row<GS>(SAtab, a, P.ka_stride, sa);
+                  if constexpr (MODE == kTableHalf) {
+                    const float4 v = *reinterpret_cast<const float4*>(SAs + a * 4), w = *reinterpret_cast<const float4*>(SAtab + (P.ka_stride + a) * 4);
+                    sa[0] = v.x; sa[1] = v.y; sa[2] = v.z; sa[3] = v.w;
+                    sa[4] = w.x; sa[5] = w.y; sa[6] = w.z; sa[7] = w.w;
+                  } else {
+                    load_sa_row<GS>(SAtab, a, P.ka_stride, sa);
+                  }
                   const bool kb = (tl.kbits >> e) & 1u;
                   const float gk = half_hi(ek[e]);
                   // logits gamma S_A - m, plus the key-residual term for the lanes whose token has one
@@ -2197,12 +2207,12 @@ struct Plan {
 // Shared-memory carve-up for X staged anchor-value rows of XW weight rows, the table in shared memory or not, a ring of at
 // least `ring_min` bytes that holds a block of Rmin records per side beside its anchor-value rows, and as many p rows as fit
 // beside it, at least Rmin; false if they don't.
-bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, int XW, bool smem_sa, int smem_optin, long long ring_min, Plan* out) {
+bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, int XW, int smem_sa, int smem_optin, long long ring_min, Plan* out) {
   DecodeParams& P = out->P;
   P.X = X;
   P.XW = XW;
   P.ka_stride = (L.max_k + 3) & ~3;
-  P.smem_sa = smem_sa ? 1 : 0;
+  P.smem_sa = smem_sa;
   size_t off = 0;
   auto take = [&](size_t bytes) {
     const size_t o = off;
@@ -2212,7 +2222,7 @@ bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, int XW, bool smem_sa
   P.o_bar = take((2 * NSG + 6) * 8);
   P.o_meta = take(NSG * sizeof(Meta));
   P.o_misc = take(16 + sizeof(Seg));  // failure flag; the segment in work
-  P.o_sa = take(smem_sa ? (size_t)P.ka_stride * GS * 4 : 0);
+  P.o_sa = take(smem_sa == 1 ? (size_t)P.ka_stride * GS * 4 : (smem_sa == 2 ? (size_t)P.ka_stride * 16 : 0));
   P.o_ovf = take((size_t)2 * GS * 128 * 4);
   P.o_qp = take((size_t)hdr_bytes(GS));  // the unit's query header: q', its sums, B fragments
   P.o_rows = take(32 * 4);
@@ -2252,6 +2262,10 @@ bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, int XW, bool smem_sa
 // have more weight rows than those, 2x the mean (the WIDE kernels, table in global memory): 16 x 60000 tokens, 25 % anchors,
 // G = 1, 2, 4, 8: 59, 62, 65, 77 us per
 // call; with such tiles on the general token path 97, 147, 241, 428.  30 %: 81, 84, 88, 116 (1809, 3487, 5965, 11632).
+// Half the table in shared memory (G = 8) where it does not fit and records are many, if the ring still holds two mean
+// tiles: 4 requests of 131072, 8 KV heads, 4 % anchors, all in global memory and this: 20 % residuals 182.7, 171.9 us, 30 %
+// 203, 193; with fewer records the ring's length is worth more: 10 % 136, 142, 5 % even; with a ring of 1.5 tiles (2
+// requests, 5 % and 20 %) 99.9, 105.4.
 // table false: no anchor-score table is read (RoPE at decode), so none is placed in shared memory.
 bool make_plan(const Layout& L, int GS, int smem_optin, bool table, Plan* out, std::string* why) {
   const int R0 = full_r(L), X0 = full_x(L);
@@ -2259,17 +2273,20 @@ bool make_plan(const Layout& L, int GS, int smem_optin, bool table, Plan* out, s
   const int Rmin = std::min(T, std::max(16, ((R0 * 3 / 4) + 15) & ~15)), Xmin = std::max(16, ((X0 * 3 / 4) + 15) & ~15);
   const double rows = std::min(256.0, T * max_anchor_density(L) + 2.0);
   const double mean = (double)F_MAX + T * mean_density(L) * 72.0 + 256.0 + 256.0 * rows;
-  for (int sa = table && !wide ? 1 : 0; sa >= 0; --sa)
+  for (const int sa : {1, 2, 0}) {
+    if (sa && (!table || wide || (sa == 2 && GS != 8))) continue;
     for (const double tiles : {5.0, 4.5, 4.0, 3.5, 3.0, 2.5, 2.0, 1.5}) {
+      if (sa == 2 && (tiles < 2.0 || mean_density(L) < 0.15)) break;
       const bool trim = tiles < 4.0;
       const int R = trim ? Rmin : std::min(T, tiles > 4.5 ? R0 * 3 / 2 : R0);
       for (int X = X0; X >= (trim ? Xmin : X0); X -= 16)
-        if (make_plan_rx(L, GS, R, X, wide ? full_w(L) : X, sa == 1, smem_optin, (long long)(tiles * mean), out)) return true;
+        if (make_plan_rx(L, GS, R, X, wide ? full_w(L) : X, sa, smem_optin, (long long)(tiles * mean), out)) return true;
     }
+  }
   for (int X = X0; X >= 16; X -= 16)
-    if (make_plan_rx(L, GS, Rmin, X, wide ? full_w(L) : X, false, smem_optin, block_bytes_at_most(Rmin) + 256LL * X, out)) return true;
+    if (make_plan_rx(L, GS, Rmin, X, wide ? full_w(L) : X, 0, smem_optin, block_bytes_at_most(Rmin) + 256LL * X, out)) return true;
   for (int X = X0; X >= 16; X -= 16)
-    if (make_plan_rx(L, GS, 16, X, X, false, smem_optin, block_bytes_at_most(16) + 256LL * X, out)) return true;
+    if (make_plan_rx(L, GS, 16, X, X, 0, smem_optin, block_bytes_at_most(16) + 256LL * X, out)) return true;
   *why = "shared memory: no room for the decode pipeline";
   return false;
 }
@@ -2284,6 +2301,8 @@ template <int GS>
 const void* decode_kernel(int codec, int rope, const DecodeParams& P) {
   if (P.XW > P.X) return wide_decode_kernel<GS>(codec, rope);
   if (rope) return decode_kernel_c<GS, kRope>(codec);
+  if constexpr (GS == 8)
+    if (P.smem_sa == 2) return decode_kernel_c<GS, kTableHalf>(codec);
   return P.smem_sa ? decode_kernel_c<GS, kTableSmem>(codec) : decode_kernel_c<GS, kTableGlobal>(codec);
 }
 template <int GS>

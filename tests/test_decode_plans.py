@@ -145,6 +145,21 @@ def test_plans_at_large_shares(dev, G, fa, fr, rope):  # noqa: F811
     _run_seeded(dev, p, [9001, 3333], sm_scale=0.2)
 
 
+@pytest.mark.parametrize("S", [60001, 70000])
+@pytest.mark.parametrize("lloyd", [False, True])
+@pytest.mark.parametrize("fa,fr", [(0.08, 0.2), (0.06, 0.3)])
+def test_half_of_the_score_table_in_shared_memory(dev, S, lloyd, fa, fr):  # noqa: F811
+    """Eight query heads, a score table that does not fit into shared memory and many records: heads 0-3 gather from shared,
+    heads 4-7 from global memory; anchor counts that are and are not a multiple of four."""
+    p = akv.Params(batch=1, n_kv_heads=2, n_q_heads=16, anchor_frac=fa, res_frac_k=fr, res_frac_v=fr, seed=13, lloyd=lloyd)
+
+    def mutate(u, d):
+        if lloyd:
+            d["min_k"] = d["min_k"] * 0
+            d["min_v"] = d["min_v"] * 0
+    _run_seeded(dev, p, [S], mutate=mutate, sm_scale=0.2)
+
+
 @pytest.mark.parametrize("G", [2, 8])
 def test_time_at_large_shares(dev, G):  # noqa: F811
     """No cliff: a call with many anchors or many records takes a few times what one at 20 % anchors takes, as its bytes
