@@ -1585,9 +1585,8 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
             }
           }
         }
-        // (its shape comes with the key terms; without one, a tile that lands late after all is left alone)
-        const bool go = wait_or_fail(bar_kdone(b), (uint32_t)(lt >> 1) & 1u) && wait_or_fail(bar_full(lt % NSG), (uint32_t)(lt / NSG) & 1u) &&
-                        !(meta[lt % NSG].fast & kNoShape);
+        // (its shape comes with the key terms; without one it has no tokens)
+        const bool go = wait_or_fail(bar_kdone(b), (uint32_t)(lt >> 1) & 1u) && wait_or_fail(bar_full(lt % NSG), (uint32_t)(lt / NSG) & 1u);
         if (go) {
           const Meta mt = meta[lt % NSG];
           const uint8_t* st = ring + mt.ring_off;
@@ -1871,6 +1870,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
           }
         } else if (wi8 == 0 && lane == 0) {
           meta[t % NSG].fast = kNoShape;
+          meta[t % NSG].n = 0;
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_kdone(b));

@@ -24,12 +24,12 @@ def test_key_terms_are_ordered_before_the_copy_that_takes_their_place():
 
 
 def test_a_tile_without_its_shape_is_left_alone():
-    """A tile's shape (fast, nVs, offsets) is written by the product warp that waited for it.  If that wait runs out, the
-    descriptor holds the shape of an older tile, which must not be used with the bytes of one that lands late: the
-    warp marks it before it arrives on bar_kdone, and both roles look at the mark before they touch the tile."""
+    """A tile's shape (tokens, fast, nVs, offsets) is written by the product warp that waited for it.  If that wait runs
+    out, the descriptor holds the shape of an older tile, which must not be used with the bytes of one that lands late: the
+    warp takes its tokens away and marks it before it arrives on bar_kdone; the token warps have nothing to do then, and
+    the product warps look at the mark before they touch the tile."""
     phase = KERNEL[KERNEL.index("auto key_phase"):KERNEL.index("mbar_arrive(bar_kdone(b))")]
-    assert re.search(r"else if \(wi8 == 0 && lane == 0\) \{\s*meta\[t % NSG\]\.fast = kNoShape;", phase)
-    uses = re.findall(r"const bool go = [^;]*;", KERNEL)
-    assert len(uses) == 3  # the key phase's own, the token warps' and the product warps'
-    for go in uses:
-        assert "landed" in go or "kNoShape" in go, go
+    assert re.search(r"else if \(wi8 == 0 && lane == 0\) \{\s*meta\[t % NSG\]\.fast = kNoShape;\s*meta\[t % NSG\]\.n = 0;", phase)
+    tokens = KERNEL[KERNEL.index("mt.fast & 1u"):KERNEL.index("mbar_arrive(bar_tdone(b))")]
+    assert re.search(r"constexpr uint32_t kNoShape = 4u;", SRC) and re.search(r"else if \(t0 < tv\.n\)", tokens)
+    assert re.search(r"const bool go = waited && !\(mt\.fast & kNoShape\);", KERNEL)
