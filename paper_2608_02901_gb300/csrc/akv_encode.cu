@@ -1097,10 +1097,41 @@ __device__ void paired_dot(const uint4* x, const uint4* row, int a, float& s, fl
   }
 }
 
+// |x . x_a| / |x_a| in fp32 for rows of any finite size, as enc_undecided's own score, within 2^-19 |x|: x comes scaled by
+// a power of two to a largest component in [1, 2), and again by 2^64 and 2^-64 (xs[0 .. 2][128]) for anchors whose norm
+// would take the products out of the range; the anchor's norm from the leading bits of its square.  0 for an anchor that
+// cannot be the nearest (zero, or not finite).
+__device__ __noinline__ float scaled_score(const float (*xs)[128], const uint4* row, int a, double n2) {
+  const uint32_t hi = (uint32_t)__double2hiint(n2), lo = (uint32_t)__double2loint(n2);
+  if (hi == 0u || hi >= 0x7FF00000u) return 0.f;
+  const int e = (int)(hi >> 20) - 1023, h = e >> 1;  // |x_a| = sqrt(m) 2^h, m in [1, 4)
+  const float m = __uint_as_float((uint32_t)(127 + (e & 1)) << 23 | (hi & 0xFFFFFu) << 3 | lo >> 29);
+  const int cls = h < -60 ? 1 : (h > 60 ? 2 : 0), c = cls == 1 ? 64 : (cls == 2 ? -64 : 0);
+  const float* x = xs[cls];
+  float s = 0.f;
+#pragma unroll 8
+  for (int g = 0; g < 16; ++g) {
+    const uint4 v = __ldg(row + (g ^ (a & 7)));
+    const float* xc = x + 8 * g;
+    float t = xc[0] * bf_lo(v.x);
+    t = __fmaf_rn(xc[1], bf_hi(v.x), t);
+    t = __fmaf_rn(xc[2], bf_lo(v.y), t);
+    t = __fmaf_rn(xc[3], bf_hi(v.y), t);
+    t = __fmaf_rn(xc[4], bf_lo(v.z), t);
+    t = __fmaf_rn(xc[5], bf_hi(v.z), t);
+    t = __fmaf_rn(xc[6], bf_lo(v.w), t);
+    t = __fmaf_rn(xc[7], bf_hi(v.w), t);
+    s += t;
+  }
+  return fabsf(s) * __frsqrt_rn(m) * __uint_as_float((uint32_t)(127 - h - c) << 23);
+}
+
 // The positions that enc_finish left.  First list: one or two candidate anchors, a thread each; second list: any
 // anchor of a group of 32, or any at all, a block each.  Scores are told apart in fp32, then in twice its
 // precision (as squares: dot^2 |other|^2), duplicates by their bytes; fp64 chains run only for what is
-// left, since one of 128 steps takes about 10 us here.
+// left, since one of 128 steps takes about 10 us here.  Rows outside the filter's range are scaled first (8 units of 32768
+// positions with one anchor of norm 2^-32 each, so that the filter is off: 11 ms; with fp64 scores for every
+// position and anchor 160).
 constexpr int kUndThreads = 128;
 // Blocks per unit and side, a ninth of them for the first list: 72 in a large batch (24 units already start 3456),
 // up to 576 for fewer than 8 units, whose lists are as long as their requests.  2 units of 131072 positions: 76 us with
@@ -1108,7 +1139,7 @@ constexpr int kUndThreads = 128;
 __host__ __device__ constexpr int und_first(int blocks) { return blocks / 9; }
 inline int und_blocks(int units) { return 72 * std::min(8, std::max(1, 8 / std::max(1, units))); }
 __global__ void __launch_bounds__(kUndThreads) enc_undecided(const EncArgs A) {
-  __shared__ __align__(16) float xs[128];
+  __shared__ __align__(16) float xs[128], xs3[3][128];  // a position's row; scaled
   __shared__ float red[kUndThreads / 32];
   __shared__ int lowest;
   __shared__ double bcs[kUndThreads], bds[kUndThreads];
@@ -1219,9 +1250,30 @@ __global__ void __launch_bounds__(kUndThreads) enc_undecided(const EncArgs A) {
     if (lane == 0) red[warp] = nx2;
     __syncthreads();
     nx2 = (red[0] + red[1]) + (red[2] + red[3]);
-    const bool filter = !zero && nx2 >= (float)kNormLo && nx2 <= (float)kNormHi && w.ctrl[4 + side] == 0u;
+    bool filter = !zero && nx2 >= (float)kNormLo && nx2 <= (float)kNormHi && w.ctrl[4 + side] == 0u;
+    const bool scaled = !filter && !zero && __syncthreads_and(fabsf(xs[tid]) < INFINITY);
+    if (scaled) {
+      const uint32_t top = __reduce_max_sync(0xffffffffu, __float_as_uint(xs[tid]) & 0x7FFFFFFFu);
+      __syncthreads();
+      if (lane == 0) red[warp] = __uint_as_float(top);
+      __syncthreads();
+      int e;
+      frexpf(fmaxf(fmaxf(red[0], red[1]), fmaxf(red[2], red[3])), &e);
+      const float v = ldexpf(xs[tid], 1 - e);  // (exact, or far below 2^-100)
+      xs3[0][tid] = v;
+      xs3[1][tid] = v * 0x1p64f;
+      xs3[2][tid] = v * 0x1p-64f;
+      nx2 = v * v;
+      for (int o = 16; o > 0; o >>= 1) nx2 += __shfl_xor_sync(0xffffffffu, nx2, o);
+      __syncthreads();
+      if (lane == 0) red[warp] = nx2;
+      __syncthreads();
+      nx2 = (red[0] + red[1]) + (red[2] + red[3]);
+      filter = true;
+    }
     auto score = [&](int a) {  // fp32, within 2^-19 |x| of |x . x_a| / |x_a| (sums per chunk: 26 roundings)
       const uint4* row = AR + (size_t)a * 16;
+      if (scaled) return scaled_score(xs3, row, a, n2[a]);
       float s = 0.f;
 #pragma unroll 8
       for (int c = 0; c < 16; ++c) {

@@ -104,3 +104,48 @@ def test_selection_left_to_fp64(dev, kinds, e):  # noqa: F811
     for u, (g, w) in enumerate(zip(got, want)):
         assert (g.S, g.k, g.nk, g.nv) == (w.S, w.k, w.nk, w.nv), u
         assert_same_unit(g, stored_order(w), f"unit {u}")
+
+
+@pytest.mark.parametrize("e", [-125, -90, 62, 64, 110])
+def test_rows_far_outside_the_filter_range(dev, e):  # noqa: F811
+    """The same with rows whose products fp32 does not hold unscaled, of subnormal components among them, both sides at
+    once, near ties (rows that differ by a bit), and one such anchor in a unit of ordinary rows."""
+    lens = [700]
+    p = akv.Params(batch=1, n_kv_heads=4, n_q_heads=4, anchor_frac=0.1, res_frac_k=0.2, res_frac_v=0.2, seed=21)
+    K, V = gen.clustered_batch(1, 4, lens, seed=22)
+    K[0, 0], V[0, 0] = _scaled(K[0, 0], e), _scaled(V[0, 0], e)
+    K[0, 1, 350:] = K[0, 1, :350]
+    K[0, 1, 350:, 5] ^= 1
+    K[0, 1] = _scaled(K[0, 1], e)
+    K[0, 2, 5:300:7] = _scaled(K[0, 2, 5:300:7], e)
+    V[0, 2, 699:] = _scaled(V[0, 2, 699:], e)
+    V[0, 3, ::3] = _scaled(V[0, 3, ::3], -e // 2)
+    V[0, 3, 1::3] = _scaled(V[0, 3, 1::3], e)
+    _encode_both(dev, p, lens, K, V)
+
+
+def test_time_with_an_anchor_outside_the_filter_range(dev):  # noqa: F811
+    """One tiny anchor per unit turns the filter off for it: the scores are then fp32 of scaled rows (some 25 times the
+    call's time), not fp64 (350 times)."""
+    import torch
+    p = akv.Params(batch=1, n_kv_heads=8, n_q_heads=8, seed=23)
+    lens = [32768]
+    K = torch.randn((1, 8, lens[0], 128), device=dev).to(torch.bfloat16)
+    V = torch.randn_like(K)
+    a, w = akv.akv_cache_size(p, lens)
+    arena, ws = torch.empty(a, dtype=torch.uint8, device=dev), torch.empty(w, dtype=torch.uint8, device=dev)
+
+    def ms():
+        best = 1e9
+        for _ in range(3):
+            x, y = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            x.record()
+            akv.akv_encode(p, lens, K, V, arena, ws)
+            y.record()
+            torch.cuda.synchronize()
+            best = min(best, x.elapsed_time(y))
+        return best
+
+    plain = ms()
+    K[:, :, -1] *= 1e-11  # (a window position)
+    assert ms() < 100 * plain
