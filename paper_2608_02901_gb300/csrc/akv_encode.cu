@@ -2652,12 +2652,19 @@ __device__ __forceinline__ bool gated(const EncArgs& A, int u) {
   return (c[12] | c[13]) != 0u;
 }
 
+// The attention of unit u is taken in fp64: for its scores (GATE 1), or for its request's utilities (GATE 2) where that has
+// not been done for the scores.
+template <int GATE>
+__device__ __forceinline__ bool gated_alpha(const EncArgs& A, int u) {
+  return gated<GATE>(A, u) && (GATE == 1 || !gated<1>(A, u));
+}
+
 // Logits q_w . K_t / sqrt(D) of every observation row and position (Eq. 4), into alpha.
 template <int GATE>
 __global__ void __launch_bounds__(128) enc_obs_logit(const EncArgs A) {
   __shared__ double qs[128];
   const int u = blockIdx.y;
-  if (!gated<GATE>(A, u)) return;
+  if (!gated_alpha<GATE>(A, u)) return;
   const akv_unit_desc* d = unit_desc(A, u);
   const int S = d->len;
   const int t = blockIdx.x * 128 + threadIdx.x;
@@ -2680,7 +2687,7 @@ __global__ void __launch_bounds__(1024) enc_obs_softmax(const EncArgs A) {
   __shared__ double red[32];
   __shared__ double den_s;
   const int u = blockIdx.y, wr = blockIdx.x;
-  if (!gated<GATE>(A, u)) return;
+  if (!gated_alpha<GATE>(A, u)) return;
   const akv_unit_desc* d = unit_desc(A, u);
   const int S = d->len;
   EncUnitWs w = unit_ws(A, u, d);

@@ -65,3 +65,29 @@ def test_value_residuals_below_the_fp32_range(dev, e):  # noqa: F811
     V[..., 0] = 4.0
     Q = 1e-3 * r.standard_normal((1, H, W * G, 128))
     _encode_both(dev, K, V, Q, [S], theta=0.08)
+
+
+def test_attention_taken_in_fp64_once(dev):  # noqa: F811
+    """Where the scores and the utilities are both left to fp64 (keys whose norms leave the fp32 range), the attention is
+    taken in fp64 once: the call takes little longer than one without scored anchors."""
+    S, heads = 4096, 8
+    p = akv.Params(batch=1, n_kv_heads=heads, n_q_heads=4 * heads, anchor_frac=0.02, res_frac_k=0.0, res_frac_v=0.0, seed=3)
+    g = torch.Generator(device=dev).manual_seed(5)
+    K, V = ((torch.randn((1, heads, S, 128), generator=g, device=dev) * f).to(torch.bfloat16) for f in (1e12, 1.0))
+    Q = torch.randn((1, heads, 128, 128), generator=g, device=dev).to(torch.bfloat16)
+
+    def ms(rho):
+        sel = akv.SelectParams(theta=0.05, rho=rho, kappa=7)
+        a, w = akv.akv_cache_size_select(p, sel, [S])
+        arena, ws = torch.empty(a, dtype=torch.uint8, device=dev), torch.empty(w, dtype=torch.uint8, device=dev)
+        best = 1e9
+        for _ in range(3):
+            x, y = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            x.record()
+            akv.akv_encode_select(p, sel, [S], K, V, Q, arena, ws)
+            y.record()
+            torch.cuda.synchronize()
+            best = min(best, x.elapsed_time(y))
+        return best
+
+    assert ms(0.7) < 1.08 * ms(0.0)  # (1.00; 1.17 with it taken twice)
