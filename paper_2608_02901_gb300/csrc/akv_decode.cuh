@@ -165,6 +165,9 @@ struct Prod {
   uint32_t head, used;        // ring bytes: next free place, bytes in flight
 };
 
+constexpr int kTurnGroup = 2;  // copies in turn: query groups at most,
+constexpr int kTurnTiles = 12;  // and tiles per CTA at least
+
 struct DecodeParams {
   const uint8_t* arena;
   const __nv_bfloat16* q;
@@ -1314,9 +1317,14 @@ __device__ __forceinline__ void unstaged_rows(const float* W, const uint32_t* en
 // token's logit comes from the RoPE logits launch (P.lg) instead of gamma S_A plus its key-residual
 // term, and the key-residual phase has nothing to do.
 enum Mode { kTableSmem = 0, kTableGlobal = 1, kRope = 2, kTableHalf = 3 };
+// TURN: the token warps copy the tiles in turn.  With small query groups a tile's tokens take so little that copying the next
+// one, some 1500 cycles of one lane, is what every other warp waits for: 4 requests of 131072, 8 KV heads, no residuals, G = 1
+// and 2, 1 % anchors 59.8 -> 55.6 us and 61.8 -> 57.6, 2 % 63.6 -> 59.7 and 64.8 -> 61.7.  Calls of a few tiles per CTA lose by its
+// set-up (3 requests of 16001, 9000 and 4173, G = 1: 18.57 -> 18.88; even at 7 and 9 tiles per CTA, 39.5 -> 38.4 and 50.0 -> 47.6 at 13),
+// hence kTurnTiles.
 // WIDE: tiles may cover more value slots than have their anchor-value rows staged (P.XW > P.X); kernels of their own,
 // since the same code as a branch, inline or called, made the others slower (8 x 131072, G = 8: 164 -> 178, 193 us).
-template <int GS, int CODEC, int MODE, bool WIDE = false>
+template <int GS, int CODEC, int MODE, bool WIDE = false, bool TURN = false>
 __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P) {
   extern __shared__ __align__(128) uint8_t smem[];
   constexpr int NP = GS >= 2 ? GS / 2 : 1;      // pairs of heads for the packed arithmetic
@@ -1407,30 +1415,37 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
   // ---- copies: lane 0 of token warp 0.  Each tile goes, with the anchor-value rows of the value slots it
   // covers, into the ring, oldest first, as places come free; the table entries of the next tile are read
   // one tile ahead ----
+  // TURN: tile ii by lane 0 of token warp ii % 8, except that warp 0 copies the first three; each such lane has a segment
+  // and table entries of its own (read a turn, eight tiles, ahead), the state common to all is warp 0's and is handed on by
+  // its ii: whoever finds its own tile there sees what the turns before left.
   Prod* pr = reinterpret_cast<Prod*>(smem + P.o_prod);
+  Prod* pw = TURN ? pr + (warp & (NTW - 1)) : pr;
+  int mine = warp < 3 && warp > 0 ? warp + NTW : warp;  // TURN: this lane's next tile
   uint32_t pe0 = 0, pe1 = 0, pe2 = 0;  // table entries of the next tile to copy: block offset, next offset, slot range
   auto read_entry = [&](int ii) {
     if (ii >= n_cta_tiles) return;
-    if (ii >= pr->end) {  // (and at the start)
-      Seg s = pr->s;
+    if (ii >= pw->end) {  // (and at the start)
+      Seg s = pw->s;
       while (ii >= s.ib + (s.je - s.jb)) seg_next(s);
       const akv_unit_desc* d = unit_desc(P.arena, s.u);
-      pr->s = s;
-      pr->end = s.ib + (s.je - s.jb);
-      pr->tiles = P.arena + d->off_tiles;
-      pr->av = P.arena + d->off_anchor_v;
-      pr->table = reinterpret_cast<const uint32_t*>(P.arena + d->off_tile_table);
+      pw->s = s;
+      pw->end = s.ib + (s.je - s.jb);
+      pw->tiles = P.arena + d->off_tiles;
+      pw->av = P.arena + d->off_anchor_v;
+      pw->table = reinterpret_cast<const uint32_t*>(P.arena + d->off_tile_table);
     }
-    const int pj = pr->s.jb + (ii - pr->s.ib);
-    const uint32_t* table = pr->table;
+    const int pj = pw->s.jb + (ii - pw->s.ib);
+    const uint32_t* table = pw->table;
     pe0 = table[pj];
     pe1 = table[pj + 1];
-    pe2 = table[pr->s.nt + 1 + pj];
+    pe2 = table[pw->s.nt + 1 + pj];
   };
   // (one tile a call: the entries read after it are not waited for)
   auto copy_more = [&]() {  // the next tile, if it fits now (never waits)
-    const int ii = pr->ii;
+    const int ii = TURN ? *(volatile int*)&pr->ii : pr->ii;
+    if (TURN && ii != mine) return;
     if (ii < n_cta_tiles && !*failed) {
+      if constexpr (TURN) __threadfence_block();  // what the turns before left
       const uint32_t RB = (uint32_t)P.ring_bytes;
       const uint32_t lo = pe2 & 0xFFFFu, hi = pe2 >> 16;
       const uint32_t staged = min(pe1 - pe0, (uint32_t)P.cap);
@@ -1465,7 +1480,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
       mt.staged = staged;
       mt.lo = lo;
       mt.nrows = nrows;
-      mt.j = (uint32_t)(pr->s.jb + (ii - pr->s.ib));
+      mt.j = (uint32_t)(pw->s.jb + (ii - pw->s.ib));
       mt.bytes = sz;
       if constexpr (WIDE) mt.nw = min(hi - lo + 1u, (uint32_t)P.XW);
       // (drop_last: a test withholds the last tile of the range)
@@ -1473,13 +1488,20 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
         mt.nrows |= 0x80000000u;  // withheld: nothing in flight
       } else {
         mbar_expect_tx(bar_full(sl), sz);
-        bulk_g2s(smem_u32(ring + at), pr->tiles + pe0, staged, bar_full(sl));
-        if (nrows) bulk_g2s(smem_u32(ring + at + staged), pr->av + (size_t)lo * 256, 256u * nrows, bar_full(sl));
+        bulk_g2s(smem_u32(ring + at), pw->tiles + pe0, staged, bar_full(sl));
+        if (nrows) bulk_g2s(smem_u32(ring + at + staged), pw->av + (size_t)lo * 256, 256u * nrows, bar_full(sl));
       }
       pr->head = at + sz;
       pr->used = used + sz;
-      pr->ii = ii + 1;
-      read_entry(ii + 1);
+      if constexpr (TURN) {
+        __threadfence_block();
+        *(volatile int*)&pr->ii = ii + 1;
+        mine += mine < 2 ? 1 : (mine == 2 ? NTW - 2 : NTW);
+        read_entry(mine);
+      } else {
+        pr->ii = ii + 1;
+        read_entry(ii + 1);
+      }
     }
   };
   if (tid == 0) {  // the first tile's table entries are on their way while shared memory is set up
@@ -1511,6 +1533,15 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
 
   if (tid == 0)
     for (int i = 0; i < 3; ++i) copy_more();
+  if constexpr (TURN) {
+    if (warp > 0 && warp < NTW && lane == 0 && mine < n_cta_tiles) {
+      Seg s;
+      seg_begin(s);
+      pw->s = s;
+      pw->end = 0;
+      read_entry(mine);
+    }
+  }
 
   // =========================== token warps, product warps ==========================
   const bool tok = warp < NTW;
@@ -1572,12 +1603,12 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
       for (int i = 0; i < n_seg; ++i, ++lt) {
         const int b = lt & 1;
         // (the tile itself too: its bytes came through the asynchronous proxy)
-        if (warp == 0) {  // the copying lane's warp: the ring is topped up, and this tile certainly on its way
+        if (warp == 0 || (TURN && n_cta_tiles > 3)) {  // the copying lanes' warps: the ring is topped up, and this tile certainly on its way
           unsigned long long t_0 = 0;
           for (unsigned n = 0;; ++n) {
             if (lane == 0) copy_more();
             __syncwarp();
-            if (__shfl_sync(0xffffffffu, pr->ii, 0) > lt || warp_failed(failed)) break;
+            if (__shfl_sync(0xffffffffu, TURN ? *(volatile int*)&pr->ii : pr->ii, 0) > lt || warp_failed(failed)) break;
             if ((n & 63u) == 63u) {  // (bounded; the clock is read now and then)
               const unsigned long long now = __shfl_sync(0xffffffffu, global_ns(), 0);
               if (t_0 == 0) t_0 = now;
@@ -2065,7 +2096,7 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
     all_sync();
     const bool has_next = sg->t0 + sg->je < B1;
     if (tok) {
-      if (tid == 0) copy_more();
+      if (TURN ? lane == 0 && mine < n_cta_tiles : tid == 0) copy_more();
       const int first = sg->first, nseg = sg->nseg;
       float* dst = P.part + (size_t)(c + u) * PF;
       auto warp_sums = [&](int off, int g) {
@@ -2200,6 +2231,7 @@ long long block_bytes_at_most(int r) { return (long long)F_MAX + 2 * round16(4u 
 
 struct Plan {
   DecodeParams P;
+  bool turn = false;  // the token warps copy in turn
   size_t smem = 0;
   int grid = 0;
 };
@@ -2232,7 +2264,7 @@ bool make_plan_rx(const Layout& L, int GS, int Rmin, int X, int XW, int smem_sa,
   P.o_wb = take((size_t)3 * (XW + kEnds) * GS * 4);
   P.o_vs = take((size_t)3 * kEnds * 4);
   P.o_ovl = take((size_t)2 * kOvlBytes);
-  P.o_prod = take(sizeof(Prod));
+  P.o_prod = take((GS <= kTurnGroup ? NTW : 1) * sizeof(Prod));
   const long long room = (long long)smem_optin - (long long)off - kRingSlack - 128;
   const long long fit = (room - ring_min) / (2 * GS * 4) & ~15LL;
   if (fit < Rmin) return false;
@@ -2298,7 +2330,10 @@ const void* decode_kernel_c(int codec) {
   return codec ? (const void*)akv_decode_kernel<GS, 1, MODE> : (const void*)akv_decode_kernel<GS, 0, MODE>;
 }
 template <int GS>
-const void* decode_kernel(int codec, int rope, const DecodeParams& P) {
+const void* decode_kernel(int codec, int rope, const Plan& pl) {
+  const DecodeParams& P = pl.P;
+  if constexpr (GS <= kTurnGroup)
+    if (pl.turn) return codec ? (const void*)akv_decode_kernel<GS, 1, kTableSmem, false, true> : (const void*)akv_decode_kernel<GS, 0, kTableSmem, false, true>;
   if (P.XW > P.X) return wide_decode_kernel<GS>(codec, rope);
   if (rope) return decode_kernel_c<GS, kRope>(codec);
   if constexpr (GS == 8)
@@ -2365,12 +2400,13 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   if (!have) {
     const DeviceInfo di = device_info();
     if (!make_plan(L, GS, di.smem_optin, !rope, &pl, why)) return -1;
-    const cudaError_t e =
-        cudaFuncSetAttribute(decode_kernel<GS>(codec, rope, pl.P), cudaFuncAttributeMaxDynamicSharedMemorySize, di.smem_optin);
-    if (e != cudaSuccess) return (int)e;
     int grid = (int)std::min<long long>(std::min(di.sms, kMaxGrid), ttot);
     if (ctas > 0) grid = (int)std::min<long long>(ctas, ttot);
     pl.grid = grid;
+    pl.turn = GS <= kTurnGroup && !rope && pl.P.smem_sa == 1 && pl.P.XW == pl.P.X && ttot >= (long long)kTurnTiles * grid;
+    const cudaError_t e =
+        cudaFuncSetAttribute(decode_kernel<GS>(codec, rope, pl), cudaFuncAttributeMaxDynamicSharedMemorySize, di.smem_optin);
+    if (e != cudaSuccess) return (int)e;
     // first unit and tile of every CTA's range
     long long t0 = 0;
     int u = 0;
@@ -2496,10 +2532,10 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   cfg.blockDim = dim3(NT, 1, 1);
   cfg.dynamicSmemBytes = pl.smem;
   void* args[] = {&P};
-  e = cudaLaunchKernelExC(&cfg, decode_kernel<GS>(codec, rope, P), args);
+  e = cudaLaunchKernelExC(&cfg, decode_kernel<GS>(codec, rope, pl), args);
   if (e != cudaSuccess) {
     cudaFuncAttributes fa{};
-    cudaFuncGetAttributes(&fa, decode_kernel<GS>(codec, rope, P));
+    cudaFuncGetAttributes(&fa, decode_kernel<GS>(codec, rope, pl));
     *why = "(decode kernel: " + std::to_string(fa.numRegs) + " registers, max " + std::to_string(fa.maxThreadsPerBlock) +
            " threads, " + std::to_string(pl.smem) + " B dynamic shared memory of " +
            std::to_string(fa.maxDynamicSharedSizeBytes) + ", grid " + std::to_string(pl.grid) + ")";

@@ -2,7 +2,7 @@
 import pytest
 
 import paper_2608_02901_gb300 as akv
-from test_decode_parity import _run_seeded, dev  # noqa: F401
+from test_decode_parity import _run_seeded, debug_controls, dev  # noqa: F401
 
 pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -143,6 +143,41 @@ def test_plans_at_large_shares(dev, G, fa, fr, rope):  # noqa: F811
     p = akv.Params(batch=2, n_kv_heads=2, n_q_heads=2 * G, anchor_frac=fa, res_frac_k=fr, res_frac_v=fr, seed=11, rope=rope,
                    rope_theta=10000.0)
     _run_seeded(dev, p, [9001, 3333], sm_scale=0.2)
+
+
+@pytest.mark.parametrize("G", [1, 2])
+@pytest.mark.parametrize("lloyd,fa,fr", [(False, 0.02, 0.1), (True, 0.02, 0.2), (False, 0.01, 0.0), (False, 0.06, 0.6)])
+@pytest.mark.parametrize("ctas", [1, 2, 5, 6])
+def test_copies_in_turn(dev, debug_controls, G, lloyd, fa, fr, ctas):  # noqa: F811
+    """Small query groups and many tiles per CTA: the token warps copy in turn; ranges that cross units, rings of a dozen
+    tiles and of two (whose first three tiles do not fit at once), on both sides of the line (63 tiles, 12 per CTA)."""
+    p = akv.Params(batch=3, n_kv_heads=1, n_q_heads=G, anchor_frac=fa, res_frac_k=fr, res_frac_v=fr, seed=14, lloyd=lloyd)
+
+    def mutate(u, d):
+        if lloyd:
+            d["min_k"] = d["min_k"] * 0
+            d["min_v"] = d["min_v"] * 0
+    akv.akv_decode_set_debug(ctas=ctas)
+    _run_seeded(dev, p, [33333, 3000, 27000], mutate=mutate, sm_scale=0.2)
+
+
+def test_withheld_tile_with_copies_in_turn(dev, debug_controls):  # noqa: F811
+    """The last tile of each range withheld: NaN outputs after the bounded wait, and the next call is right."""
+    import numpy as np
+    import torch
+    from helpers import check_outputs, decode_on_gpu, oracle_decode, oracle_unit, seeded_units
+    import gen
+    p = akv.Params(batch=1, n_kv_heads=1, n_q_heads=1, seed=15)
+    lens = [40000]
+    units = seeded_units(p, lens, seed=5)
+    arena = torch.from_numpy(akv.akv_cache_pack_host(p, lens, [akv.unit_host_from_logical(u) for u in units])).to(dev)
+    q = gen.queries(1, seed=17)
+    akv.akv_decode_set_debug(ctas=2, withhold_last=1)
+    out, out32 = decode_on_gpu(torch, p, lens, arena, q, 1.0)
+    assert np.all(np.isnan(out32)) and np.all(np.isnan(out))
+    akv.akv_decode_set_debug(ctas=2)
+    out, out32 = decode_on_gpu(torch, p, lens, arena, q, 1.0)
+    check_outputs(out, out32, oracle_decode(p, [oracle_unit(u) for u in units], q, 1.0), where="after the timed-out call in turn")
 
 
 @pytest.mark.parametrize("S", [60001, 70000])
