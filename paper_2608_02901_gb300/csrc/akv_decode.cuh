@@ -165,7 +165,7 @@ struct Prod {
   uint32_t head, used;        // ring bytes: next free place, bytes in flight
 };
 
-constexpr int kTurnGroup = 2;  // copies in turn: query groups at most,
+constexpr int kTurnGroup = 2;   // copies in turn: query groups at most
 constexpr int kTurnTiles = 12;  // and tiles per CTA at least
 
 struct DecodeParams {
@@ -1317,11 +1317,12 @@ __device__ __forceinline__ void unstaged_rows(const float* W, const uint32_t* en
 // token's logit comes from the RoPE logits launch (P.lg) instead of gamma S_A plus its key-residual
 // term, and the key-residual phase has nothing to do.
 enum Mode { kTableSmem = 0, kTableGlobal = 1, kRope = 2, kTableHalf = 3 };
-// TURN: the token warps copy the tiles in turn.  With small query groups a tile's tokens take so little that copying the next
-// one, some 1500 cycles of one lane, is what every other warp waits for: 4 requests of 131072, 8 KV heads, no residuals, G = 1
-// and 2, 1 % anchors 59.8 -> 55.6 us and 61.8 -> 57.6, 2 % 63.6 -> 59.7 and 64.8 -> 61.7.  Calls of a few tiles per CTA lose by its
-// set-up (3 requests of 16001, 9000 and 4173, G = 1: 18.57 -> 18.88; even at 7 and 9 tiles per CTA, 39.5 -> 38.4 and 50.0 -> 47.6 at 13),
-// hence kTurnTiles.
+// TURN: the token warps copy the tiles in turn.  With small query groups and no residual records a tile's tokens and values
+// take so little that copying the next one, some 1500 cycles of one lane, is what every other warp waits for: 4 requests of
+// 131072, 8 KV heads, G = 1 and 2, 1 % anchors 59.8 -> 55.6 us and 61.8 -> 57.6, 2 % 63.6 -> 59.7 and 64.8 -> 61.7.  With
+// records the product warps are the longer side, and the other lanes' looks at the state cost 0 to 3 % (1 % of records
+// already); calls of a few tiles per CTA lose by its set-up (3 requests of 16001, 9000 and 4173, 5 % records, G = 1: 18.57 ->
+// 18.88; no records, even at 7 and 9 tiles per CTA, 39.5 -> 38.4 at 13), hence kTurnTiles.
 // WIDE: tiles may cover more value slots than have their anchor-value rows staged (P.XW > P.X); kernels of their own,
 // since the same code as a branch, inline or called, made the others slower (8 x 131072, G = 8: 164 -> 178, 193 us).
 template <int GS, int CODEC, int MODE, bool WIDE = false, bool TURN = false>
@@ -2403,7 +2404,7 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
     int grid = (int)std::min<long long>(std::min(di.sms, kMaxGrid), ttot);
     if (ctas > 0) grid = (int)std::min<long long>(ctas, ttot);
     pl.grid = grid;
-    pl.turn = GS <= kTurnGroup && !rope && pl.P.smem_sa == 1 && pl.P.XW == pl.P.X && ttot >= (long long)kTurnTiles * grid;
+    pl.turn = GS <= kTurnGroup && !rope && max_density(L) == 0.0 && pl.P.smem_sa == 1 && pl.P.XW == pl.P.X && ttot >= (long long)kTurnTiles * grid;
     const cudaError_t e =
         cudaFuncSetAttribute(decode_kernel<GS>(codec, rope, pl), cudaFuncAttributeMaxDynamicSharedMemorySize, di.smem_optin);
     if (e != cudaSuccess) return (int)e;

@@ -146,19 +146,38 @@ def test_plans_at_large_shares(dev, G, fa, fr, rope):  # noqa: F811
 
 
 @pytest.mark.parametrize("G", [1, 2])
-@pytest.mark.parametrize("lloyd,fa,fr", [(False, 0.02, 0.1), (True, 0.02, 0.2), (False, 0.01, 0.0), (False, 0.06, 0.6)])
+@pytest.mark.parametrize("fa", [0.01, 0.04, 0.15])
 @pytest.mark.parametrize("ctas", [1, 2, 5, 6])
-def test_copies_in_turn(dev, debug_controls, G, lloyd, fa, fr, ctas):  # noqa: F811
-    """Small query groups and many tiles per CTA: the token warps copy in turn; ranges that cross units, rings of a dozen
-    tiles and of two (whose first three tiles do not fit at once), on both sides of the line (63 tiles, 12 per CTA)."""
-    p = akv.Params(batch=3, n_kv_heads=1, n_q_heads=G, anchor_frac=fa, res_frac_k=fr, res_frac_v=fr, seed=14, lloyd=lloyd)
-
-    def mutate(u, d):
-        if lloyd:
-            d["min_k"] = d["min_k"] * 0
-            d["min_v"] = d["min_v"] * 0
+def test_copies_in_turn(dev, debug_controls, G, fa, ctas):  # noqa: F811
+    """Small query groups, no records and many tiles per CTA: the token warps copy in turn; ranges that cross units, rings of
+    a dozen tiles and of two or three (whose first three do not fit at once), on both sides of the line (63 tiles, 12 per
+    CTA)."""
+    p = akv.Params(batch=3, n_kv_heads=1, n_q_heads=G, anchor_frac=fa, res_frac_k=0.0, res_frac_v=0.0, seed=14)
     akv.akv_decode_set_debug(ctas=ctas)
-    _run_seeded(dev, p, [33333, 3000, 27000], mutate=mutate, sm_scale=0.2)
+    _run_seeded(dev, p, [33333, 3000, 27000], sm_scale=0.2)
+
+
+@pytest.mark.parametrize("lloyd", [False, True])
+def test_copies_in_turn_with_records(dev, debug_controls, lloyd):  # noqa: F811
+    """An arena of the full selection holds records that the parameters do not tell of."""
+    import gen
+    import oracle
+    import torch
+    from helpers import check_outputs, decode_on_gpu, oracle_decode, to_dev_u16
+    lens, W = [14000], 32
+    p = akv.Params(batch=1, n_kv_heads=1, n_q_heads=1, res_frac_k=0.0, res_frac_v=0.0, window=W, seed=16, lloyd=lloyd)
+    sel = akv.SelectParams(theta=0.1)
+    K, V = gen.clustered_batch(1, 1, lens, seed=17)
+    Q = gen.observation_queries(K, lens, W, seed=18)
+    a, w = akv.akv_cache_size_select(p, sel, lens)
+    arena, ws = (torch.empty(n, dtype=torch.uint8, device=dev) for n in (a, w))
+    akv.akv_encode_select(p, sel, lens, to_dev_u16(K, torch, dev), to_dev_u16(V, torch, dev), to_dev_u16(Q, torch, dev), arena, ws)
+    units = oracle.unpack_arena(arena.cpu().numpy())
+    assert units[0].nk > 1000 and units[0].nv > 1000
+    q = gen.queries(1, seed=19)
+    akv.akv_decode_set_debug(ctas=1)
+    out, out32 = decode_on_gpu(torch, p, lens, arena, q, 0.2)
+    check_outputs(out, out32, oracle_decode(p, units, q, 0.2), where="in turn with records")
 
 
 def test_withheld_tile_with_copies_in_turn(dev, debug_controls):  # noqa: F811
@@ -167,7 +186,7 @@ def test_withheld_tile_with_copies_in_turn(dev, debug_controls):  # noqa: F811
     import torch
     from helpers import check_outputs, decode_on_gpu, oracle_decode, oracle_unit, seeded_units
     import gen
-    p = akv.Params(batch=1, n_kv_heads=1, n_q_heads=1, seed=15)
+    p = akv.Params(batch=1, n_kv_heads=1, n_q_heads=1, res_frac_k=0.0, res_frac_v=0.0, seed=15)
     lens = [40000]
     units = seeded_units(p, lens, seed=5)
     arena = torch.from_numpy(akv.akv_cache_pack_host(p, lens, [akv.unit_host_from_logical(u) for u in units])).to(dev)
