@@ -410,8 +410,8 @@ akv_status akv_pack_table1_host(const akv_params* p, const int32_t* ctx_lens_hos
  * Bytes of device workspace akv_decode_attn needs for these parameters and
  * context lengths: the anchor scores of every unit (4 G bytes per anchor),
  * their maxima per chunk of 64 anchors, one arrival counter per query head, and
- * the partial sums of the CTAs that share a unit (about 8.5 KB per query head
- * and (CTA or unit) slot, at most 256 CTAs).  Contents on entry are ignored.
+ * the partial sums of the CTAs that share a unit (512 G + 48 bytes per CTA, 256
+ * at most, and unit).  Contents on entry are ignored.
  */
 akv_status akv_decode_workspace_size(const akv_params* p, const int32_t* ctx_lens_host, size_t* ws_bytes);
 

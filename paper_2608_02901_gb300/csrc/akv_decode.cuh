@@ -18,7 +18,8 @@
 //    lie in several CTAs and a CTA's range may cross units (its segments).  A CTA has eight token warps
 //    and eight product warps (four warps per SM sub-partition at 128 registers), coupled by mbarriers, which
 //    work on neighbouring tiles at the same time:
-//      copies         a lane of token warp 0 brings the tiles into a byte ring of shared memory: one bulk
+//      copies         a lane of token warp 0 (small query groups and long ranges: of each token warp in
+//                     turn) brings the tiles into a byte ring of shared memory: one bulk
 //                     asynchronous copy of the tile block and one of the anchor-value rows of the value
 //                     slots the tile covers (the tile table records the range); table entries are read
 //                     one tile ahead;
@@ -39,7 +40,8 @@
 //    the CTA's partial numerator and normaliser into its workspace slot for the unit, and counts it in
 //    on the head's counter; the warp that completes the count sums the head's slots in a fixed
 //    order and writes the output.  Tiles denser than the staged counts, and runs on value
-//    slots beyond a tile's staged anchor-value rows, take CUDA-core paths.
+//    slots beyond a tile's weight rows, take CUDA-core paths; where anchors are many, tiles have more
+//    weight rows than staged anchor-value rows, and the rest are read from global memory.
 //
 // What bounds the decode (70B shape, 128K: 54 tiles per SM): shared-memory wavefronts (about 3100 per tile, the
 // gathers of score rows by random slots a quarter of them) and issue slots (about 11000 warp instructions
@@ -56,7 +58,6 @@
 #pragma once
 
 #include <cuda.h>
-#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -111,7 +112,7 @@ struct ScoreParams {
   unsigned long long sign_lo, sign_hi;
   float* sa;      // [units][ka_stride][G] anchor scores (log2 units)
   float* cmax;    // [units][n_ch][G] largest score of each chunk of CHA anchors
-  int n_kv_heads, n_q_heads, G, ka_stride, n_ch;
+  int n_kv_heads, n_q_heads, ka_stride, n_ch;
   float scale_log2;
   // dense suffix (null ksuf: none): rows [units][suf_cap][128], lengths per request, n_sch
   // chunks of SCH tokens per unit, each a partial slot of suf_floats(G) floats
@@ -134,7 +135,7 @@ struct RopeParams {
   float* cmax;    // [units][n_tch][G] largest logit of each chunk of 64 stored tokens
   const uint8_t* uh;  // query headers: only their arrival counters are used (zeroed here)
   int uh_stride;
-  int n_kv_heads, n_q_heads, rotate, lloyd, s_stride, n_tch;
+  int n_kv_heads, n_q_heads, rotate, s_stride, n_tch;
   float scale_log2;
   unsigned long long sign_lo, sign_hi;
   unsigned long long turn[64];  // theta_j / (2 pi) as a 64-bit binary fraction of a turn
@@ -170,7 +171,6 @@ constexpr int kTurnTiles = 12;  // and tiles per CTA at least
 
 struct DecodeParams {
   const uint8_t* arena;
-  const __nv_bfloat16* q;
   __nv_bfloat16* out;
   float* out_f32;
   const float* sa;
@@ -2166,7 +2166,6 @@ __global__ void __launch_bounds__(NT, 1) akv_decode_kernel(const DecodeParams P)
 struct DeviceInfo {
   int sms = 0;
   int smem_optin = 0;
-  int smem_sm = 0;  // shared memory per SM
 };
 
 DeviceInfo device_info() {
@@ -2180,7 +2179,6 @@ DeviceInfo device_info() {
   DeviceInfo d;
   cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&d.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  cudaDeviceGetAttribute(&d.smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
   if (dev >= 0 && dev < 64) {
     cache[dev] = d;
     have[dev] = true;
@@ -2430,7 +2428,6 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   uint8_t* wsb = (uint8_t*)ws;
   DecodeParams& P = pl.P;
   P.arena = (const uint8_t*)arena;
-  P.q = (const __nv_bfloat16*)q;
   P.out = (__nv_bfloat16*)out;
   P.out_f32 = out_f32;
   P.sa = (const float*)(wsb + W.o_sa);
@@ -2454,12 +2451,11 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
 
   ScoreParams S;
   S.arena = P.arena;
-  S.q = P.q;
+  S.q = (const __nv_bfloat16*)q;
   S.sa = (float*)(wsb + W.o_sa);
   S.cmax = (float*)(wsb + W.o_cmax);
   S.n_kv_heads = p.n_kv_heads;
   S.n_q_heads = p.n_q_heads;
-  S.G = L.G;
   S.ksuf = (const __nv_bfloat16*)sfx.K;
   S.vsuf = (const __nv_bfloat16*)sfx.V;
   S.suf_len = sfx.len;
@@ -2486,7 +2482,7 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
   if (rope) {  // the logits of every stored token (no anchor scores)
     RopeParams R;
     R.arena = P.arena;
-    R.q = P.q;
+    R.q = S.q;
     R.lg = (float*)(wsb + W.o_lg);
     R.cmax = (float*)(wsb + W.o_cmax);
     R.uh = P.uh;
@@ -2494,7 +2490,6 @@ int launch_g(const Layout& L, const akv_params& p, const void* arena, size_t are
     R.n_kv_heads = p.n_kv_heads;
     R.n_q_heads = p.n_q_heads;
     R.rotate = P.rotate;
-    R.lloyd = codec;
     R.s_stride = P.s_stride;
     R.n_tch = P.n_ch;
     R.scale_log2 = P.scale_log2;

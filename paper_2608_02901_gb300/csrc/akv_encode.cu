@@ -472,8 +472,9 @@ __global__ void __launch_bounds__(256) enc_rows(const EncArgs A) {
 // As a GEMM (positions x anchors x 128) the fp64 units need 81 ms for a layer of 8 x 32768 positions
 // and 656 anchors; the tensor cores' fp32 sums of the exact bf16 products take the same scores to
 // within 2^-15 |x| (128 exact products, fp32 accumulation; 4 times the worst bound of eight truncated
-// steps, the column bits below included), so only the anchors within 2 x 2^-15 |x| of a position's
-// largest score can be its nearest.  That leaves one anchor for about 99 % of positions; enc_finish and
+// steps, the column bits below included: how the hardware adds the products of a step is not documented, so this is an
+// assumption, with that factor of 4 to spare and the tests' near ties to support it), so only the anchors within 2 x 2^-15 |x| of a
+// position's largest score can be its nearest.  That leaves one anchor for about 99 % of positions; enc_finish and
 // enc_undecided decide the rest.  The candidate word of a position: first candidate in bits 0-15, second
 // in bits 16-31 (0xFFFF: none; the first again: the anchors of its group of 32), or 0xFFFFFFFF: any
 // anchor may be the nearest.
